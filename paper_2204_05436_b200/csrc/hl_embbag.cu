@@ -2,6 +2,7 @@
 // distinct row.  Rows are fp32 [*, D]; a group of G lanes owns one row at a time, each lane NV float4 columns,
 // so that a row is read with 128-bit loads that coalesce into whole sectors.
 #include <mutex>
+#include <type_traits>
 
 #include "hl_common.cuh"
 
@@ -18,12 +19,17 @@ __device__ __forceinline__ void red_add_f4(float4* p, float4 v) {
                  : "memory");
 }
 
-template <int N>
-__device__ __forceinline__ int32_t pick(const int32_t (&a)[N], int i) {      // a[i] without indexing registers
-    int32_t r = a[0];
-#pragma unroll
-    for (int k = 1; k < N; ++k) r = i == k ? a[k] : r;
-    return r;
+// acc = (restart ? 0 : acc) + r.  A restart clears the upper word only: what is left of acc is below 2^-1041, which an
+// fp32 value absorbs when it is added (and if that value is a zero, rounds to zero with the sum), and it costs one
+// select per column where clearing both words, which the compiler turns into predicated moves, costs two.
+__device__ __forceinline__ double unless(bool restart, double acc) {
+    return __hiloint2double(restart ? 0 : __double2hiint(acc), __double2loint(acc));
+}
+__device__ __forceinline__ void add_row(double (&acc)[4], float4 r, bool restart = false) {
+    acc[0] = unless(restart, acc[0]) + (double)r.x;
+    acc[1] = unless(restart, acc[1]) + (double)r.y;
+    acc[2] = unless(restart, acc[2]) + (double)r.z;
+    acc[3] = unless(restart, acc[3]) + (double)r.w;
 }
 
 __device__ __forceinline__ int clamp_samples(const int32_t* d_n_samples, int max_batch) {
@@ -204,26 +210,30 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pairs(const int32_t* __restric
     }
 }
 
-// The sorted lookups are cut into chunks of kBwdChunk.  One group per chunk sums, in order, the gradient rows of
-// each run of equal slots inside its chunk.  A run that lies wholly inside the chunk is finished here (one
-// reduction into its row).  A run that crosses a chunk border leaves a partial sum: part[chunk][0] for the
-// piece that continues a run from the previous chunk, part[chunk][1] for the piece that starts a run continuing
-// into the next chunk.  k_bwd_spans adds those up.
+// The sorted lookups are cut into chunks of 32.  One WARP per chunk sums, in order, the gradient rows of each run of
+// equal slots inside its chunk.  A run that lies wholly inside the chunk is finished here (one reduction into its row).
+// A run that crosses a chunk border leaves a partial sum: part[chunk][0] for the piece that continues a run from the
+// previous chunk, part[chunk][1] for the piece that starts a run continuing into the next chunk.  k_bwd_spans adds
+// those up.
 //
-// The group reads its chunk's 32 (slot, bag) pairs with one coalesced load per lane.  Where runs begin and end is
-// then settled once for the whole chunk: every lane compares its pairs' slots with their neighbours' (shuffles, the
-// slots just outside the chunk for the ends) and two ballots per 32 pairs give a mask of run heads and a mask of
-// run tails.  The loop over the lookups is driven by those two masks alone, and a lookup costs two shuffles, one
-// address, one 128-bit load per column and the additions; everything that checks a pair (position inside the call,
-// bag inside the gradient array) is done by the lane that loaded the pair, once.  Gradient rows are loaded U at a
-// time.  The instruction count matters: this kernel issues about as many cycles as it waits for memory.
+// Every lane loads one (slot, bag) pair and the 32 / G groups of the warp take G consecutive lookups each, so that the
+// gradient rows of a chunk are requested by all groups at once: a chunk of narrow rows (64 bytes: G = 4) is a chain of
+// four dependent steps, not of 32, which is what bounds a call of few lookups (4-row groups: 7.6 K lookups 18.4 -> 4.6
+// us, 86 K lookups 21.1 -> 6.3 us).  Where runs begin and end is settled by two ballots (a mask of run heads and one of
+// run tails).  Runs that lie inside a group's lookups are finished by the group; a run over several groups is put
+// together by a segmented scan of the groups' sums, in fixed order.  Everything that checks a pair (position inside
+// the call, bag inside the gradient array) is done by the lane that loaded it, once.  Rows that fill the warp (G = 32)
+// are bound by the float -> double conversions, the additions and the row updates in DRAM together (2.6 M lookups of
+// 512 bytes: 183 -> 173 us; chunks of 64 / 128 / 256 lookups 177 / 190 / 197 us: the row updates of the warps at work
+// then lie further apart).
 //
-// A run that starts in one chunk and ends in the next (most runs that cross a border do) is finished by the group of
-// the chunk it starts in, which reads on into the next chunk; the group of that next chunk leaves the run's lookups
+// A run that starts in one chunk and ends in the next (most runs that cross a border do) is finished by the warp of
+// the chunk it starts in, which reads on into the next chunk; the warp of that next chunk leaves the run's lookups
 // alone.  Both decide from the sorted slots alone and by the same test -- the run's head lies in the first of the two
 // chunks, and the chunk after the second does not begin with the run's slot -- so exactly one of them sums each
 // lookup.  Only runs over three or more chunks go through partial sums and k_bwd_spans.
-static_assert(kBwdChunk == 32, "the head and tail masks of a chunk are 32-bit words");
+constexpr int kSpanLookahead = 32;      // chunks k_bwd_chunks looks ahead for the end of a run
+static_assert(kBwdChunk == 32, "one lookup of a chunk per lane");
 
 template <int G, int NV>
 __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float* __restrict__ cache,
@@ -239,228 +249,255 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
     // the lookups of this call are positions [first, first + *d_n_lookups) of the sorted arrays; their keys are
     // slot + key_bias.  A chunk in which a run starts that goes on into the next chunk is appended to span_list
     // (in any order): k_bwd_spans finishes those runs.
-    constexpr int KPL = kBwdChunk / G;                       // pairs held per lane
+    static_assert(NV == 1 || G == 32, "several columns per lane only when a row fills the warp");
+    constexpr int NG = 32 / G;                                              // groups per warp
     constexpr int U = NV >= 4 ? 2 : (NV >= 2 ? 4 : (G >= 8 ? 8 : 4));       // lookups in flight per lane
     static_assert(G % U == 0, "batch must divide the group");
-    const int64_t first = d_first ? d_first[0] : 0;
-    const int64_t n = first + d_n_lookups[0];
-    const int lane = threadIdx.x & 31;
-    const int sub = lane % G;
-    const unsigned gshift = G == 32 ? 0u : (unsigned)(lane / G * G);
+    // (positions are below 2^30: 32-bit arithmetic)
+    const int first = d_first ? d_first[0] : 0;
+    const int count = d_n_lookups[0], n = first + count;
+    const int n_chunks = (count + kBwdChunk - 1) / kBwdChunk;
+    const int lane = threadIdx.x & 31, sub = lane % G, g0 = lane - sub;     // g0: first lane (= lookup) of my group
     constexpr unsigned gbits = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
-    const unsigned gmask = gbits << gshift;
-    const int64_t group = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G;
-    const int64_t n_groups = (int64_t)gridDim.x * kThreads / G;
-    float4* cache4 = reinterpret_cast<float4*>(cache);
+    const unsigned gmask = gbits << g0;
+    const unsigned before_group = (1u << g0) - 1u;                          // lookups of the groups before mine
+    const int n_warps = gridDim.x * (kThreads / 32);
     float4* __restrict__ part4 = reinterpret_cast<float4*>(part);
     // slots and bags are 32-bit numbers, so one unsigned comparison tells whether one lies inside its array
     const uint32_t n_rows_u = (uint32_t)(n_slots < 0x7fffffff ? n_slots : 0x7fffffff);
     const uint32_t n_grad_u = (uint32_t)(n_grad_rows < 0x7fffffff ? n_grad_rows : 0x7fffffff);
     // this lane's columns; a lane beyond the row's width reads column 0 and writes nothing
+    // (row addresses: one wide multiply-add of the 32-bit row number and the row's bytes)
     bool on[NV];
-    const float4* gcol[NV];
+    const char* gcol[NV];
+    const uint32_t row_bytes = (uint32_t)D4 * 16u;
+    __shared__ double2 s_first[G == 32 ? 1 : 2][G == 32 ? 1 : kThreads];      // sums of the groups' first runs
+    const float minus_lr = -lr;               // -(lr * G) and (-lr) * G are the same number
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const int c = sub + v * G;
         on[v] = c < D4;
-        gcol[v] = reinterpret_cast<const float4*>(grad_out) + (on[v] ? c : 0);
+        gcol[v] = reinterpret_cast<const char*>(grad_out) + (on[v] ? c : 0) * 16;
     }
+    char* cache_col = reinterpret_cast<char*>(cache) + sub * 16;
+    auto grad_row = [&](int v, int32_t b) {
+        return __ldg(reinterpret_cast<const float4*>(gcol[v] + (uint64_t)(uint32_t)b * row_bytes));
+    };
 
-    for (int64_t chunk = group; first + chunk * kBwdChunk < n; chunk += n_groups) {
-        const int64_t start = first + chunk * kBwdChunk;
-        const int64_t end = min(start + (int64_t)kBwdChunk, n);
-        int32_t kk[KPL], vv[KPL];
-#pragma unroll
-        for (int i = 0; i < KPL; ++i) {
-            const int64_t p = start + i * G + sub;
-            const bool in = p < end;
-            kk[i] = in ? keys[p] : -1;                       // -1: past the end; no slot has this key
-            const int32_t bag = in ? vals[p] : 0;
-            // (a bag id outside the gradient array can only be what a given-up chain poll of the sort left behind;
-            // such a call has its error status set, and reads bag 0 instead)
-            vv[i] = (uint32_t)bag < n_grad_u ? bag : 0;
-        }
-        const int32_t prev_key = start > first ? keys[start - 1] : -3;   // -3: equal to no key
+    for (int chunk = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); chunk < n_chunks; chunk += n_warps) {
+        const int start = first + chunk * kBwdChunk;
+        const int end = min(start + kBwdChunk, n);
+        const int32_t key = start + lane < end ? keys[start + lane] : -1;     // -1: past the end; no slot has this key
+        int32_t bag = start + lane < end ? vals[start + lane] : 0;
+        const int32_t prev_key = start > first ? keys[start - 1] : -3;        // -3: equal to no key
         const int32_t next_key = end < n ? keys[end] : -2;
         // the slot before the previous chunk, and the first slot of the chunk after the next one
         const int32_t prev2_key = start - kBwdChunk > first ? keys[start - kBwdChunk - 1] : -3;
         const int32_t next2_key = start + 2 * kBwdChunk < n ? keys[start + 2 * kBwdChunk] : -2;
+        // (a bag id outside the gradient array can only be what a given-up chain poll of the sort left behind; such a
+        // call has its error status set, and reads bag 0 instead)
+        bag = (uint32_t)bag < n_grad_u ? bag : 0;
 
-        // bit q of `heads`: lookup q of the chunk begins a run; of `tails`: it ends one
-        uint32_t heads = 0, tails = 0;
-#pragma unroll
-        for (int i = 0; i < KPL; ++i) {
-            const int32_t up = __shfl_up_sync(gmask, kk[i], 1, G);
-            const int32_t dn = __shfl_down_sync(gmask, kk[i], 1, G);
-            const int32_t before = i > 0 ? __shfl_sync(gmask, kk[i > 0 ? i - 1 : 0], G - 1, G) : prev_key;
-            const int32_t after = i + 1 < KPL ? __shfl_sync(gmask, kk[i + 1 < KPL ? i + 1 : i], 0, G) : next_key;
-            const int32_t pred = sub > 0 ? up : before;
-            const int32_t succ = sub < G - 1 ? dn : after;
-            const uint32_t hb = (__ballot_sync(gmask, kk[i] != pred) >> gshift) & gbits;
-            const uint32_t tb = (__ballot_sync(gmask, kk[i] != succ) >> gshift) & gbits;
-            heads |= hb << (i * G);
-            tails |= tb << (i * G);
-        }
-
-        const bool ends_open = !((tails >> (kBwdChunk - 1)) & 1u);   // the last run goes on in the next chunk
-        // A run that comes in from the previous chunk, began there and ends here was finished by that chunk's group:
-        // its lookups (up to its tail, the lowest tail bit) are not summed here -- their loads are pointed at the bag
-        // of the chunk's last lookup, which is loaded anyway, and the tail bit is cleared so that nothing is applied.
-        {
-            const int32_t key0 = __shfl_sync(gmask, kk[0], 0, G);
-            if (chunk >= 1 && !(heads & 1u) && tails != 0u && prev2_key != key0) {
-                const int t = __ffs((int)tails) - 1;
-                tails &= tails - 1u;
-                const int32_t last_bag = __shfl_sync(gmask, vv[KPL - 1], G - 1, G);
-#pragma unroll
-                for (int i = 0; i < KPL; ++i)
-                    if (i * G + sub <= t) vv[i] = last_bag;
-            }
-        }
-
-        // the run being summed continues one from the previous chunk until the first head
-        bool left_open = true;
         // a segment's sum is kept in fp64: a popular row can collect tens of thousands of gradient rows, and the
-        // rounding of many fp32 partial sums would show in the updated row
-        double acc[NV][4];
+        // rounding of many fp32 partial sums would show in the updated row.
+        double acc[NV][4];            // of the group's run that is not over yet
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v][0] = acc[v][1] = acc[v][2] = acc[v][3] = 0.0;
 
-        // the run whose last lookup in this chunk has key `key` is complete in acc
-        auto emit = [&](int32_t key, bool right_open) {
-            const uint32_t row = (uint32_t)(key - key_bias);
-            if (row >= n_rows_u) return;                     // a skipped lookup's sentinel, or past the end
-            if (!left_open && !right_open) {
+        // a run is complete in acc: one reduction into its row
+        auto apply = [&](uint32_t row, const double (&acc)[NV][4]) {
+            float4* to = reinterpret_cast<float4*>(cache_col + (uint64_t)row * row_bytes);
 #pragma unroll
-                for (int v = 0; v < NV; ++v)
-                    if (on[v])
-                        red_add_f4(&cache4[(int64_t)row * D4 + sub + v * G],
-                                   make_float4(-(lr * (float)acc[v][0]), -(lr * (float)acc[v][1]),
-                                               -(lr * (float)acc[v][2]), -(lr * (float)acc[v][3])));
-            } else {
-                const int64_t slot = chunk * 2 + (left_open ? 0 : 1);
+            for (int v = 0; v < NV; ++v)
+                if (on[v])
+                    red_add_f4(to + v * G,
+                               make_float4(minus_lr * (float)acc[v][0], minus_lr * (float)acc[v][1],
+                                           minus_lr * (float)acc[v][2], minus_lr * (float)acc[v][3]));
+        };
+        // a piece of a run that crosses the chunk's border (which: 0 = it comes in from the left, 1 = it starts here)
+        auto store_piece = [&](int which, const double (&acc)[NV][4]) {
 #pragma unroll
-                for (int v = 0; v < NV; ++v)
-                    if (on[v])
-                        part4[slot * D4 + sub + v * G] =
-                            make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]);
-                if (right_open && !left_open) {
-                    // a run starts here and goes on: list it, with its last chunk if that is among the next G (chunk
-                    // c > chunk holds a piece of the run iff its first slot is the run's; sorted keys: those chunks
-                    // form a prefix).  Nearly every run ends there, and k_bwd_spans then has nothing to search.
-                    const int64_t n_chunks = (n - first + kBwdChunk - 1) / kBwdChunk;
-                    const int64_t cc = chunk + 1 + sub;
-                    const bool goes_on = cc < n_chunks && keys[first + cc * kBwdChunk] == key;
-                    const uint32_t m = (__ballot_sync(gmask, goes_on) >> gshift) & gbits;
-                    const int cnt = __ffs((int)~m) - 1;      // m == gbits (all G go on): -1 for G == 32, else G
-                    if (sub == 0) {
-                        const int32_t pos = atomicAdd(span_count, 1);
-                        // (one entry per chunk at most, and the count is zero when a call starts: the list cannot
-                        // overflow unless an earlier call was cut short between its two kernels)
-                        if (pos >= 0 && pos < max_entries)
-                            reinterpret_cast<int4*>(span_list)[pos] =
-                                make_int4((int32_t)chunk, key, (cnt >= 1 && cnt < G) ? (int32_t)(chunk + cnt) : -1, 0);
-                        else
-                            set_status(status, HL_ECAPACITY);
-                    }
-                }
-            }
+            for (int v = 0; v < NV; ++v)
+                if (on[v])
+                    part4[(int64_t)(chunk * 2 + which) * D4 + sub + v * G] =
+                        make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]);
         };
 
-#pragma unroll
-        for (int i = 0; i < KPL; ++i) {
+        int32_t l = __shfl_up_sync(0xffffffffu, key, 1), r = __shfl_down_sync(0xffffffffu, key, 1);
+        if (lane == 0) l = prev_key;
+        if (lane == 31) r = next_key;
+        // bit q of `heads`: lookup q of the chunk begins a run; of `tails`: it ends one
+        const unsigned heads = __ballot_sync(0xffffffffu, key != l), tails = __ballot_sync(0xffffffffu, key != r);
+        // A run that comes in from the previous chunk, began there and ends here was finished by that chunk's warp: its
+        // lookups count for nothing here, and a row that is loaded anyway stands in for theirs.
+        const bool skip = chunk >= 1 && !(heads & 1u) && tails != 0u && prev2_key != prev_key;
+        if (skip) {
+            const int32_t other = __shfl_sync(0xffffffffu, bag, 31);
+            if (key == prev_key) bag = other;
+        }
+        // Tails that end a run of a row inside the cache, begun in this chunk: one reduction each.  (A row outside is a
+        // skipped lookup's sentinel, or past the end.)  The first tail of a chunk that begins inside a run leaves a
+        // piece instead, or nothing if the chunk before has seen to it.
+        const uint32_t row = (uint32_t)(key - key_bias);
+        const unsigned valid = __ballot_sync(0xffffffffu, row < n_rows_u);
+        unsigned piece = (heads & 1u) ? 0u : tails & (0u - tails);
+        const unsigned done = tails & valid & ~piece;
+        piece = skip ? 0u : piece & valid;
+
+        if constexpr (G == 32) {
+            unsigned hs = heads, ds = done, es = done | piece;
             // (kept rolled: with all 32 lookups unrolled the kernel is tens of KB of straight-line code that every
             // warp runs through about once, and it waits for instructions)
 #pragma unroll 1
-            for (int j = 0; j < G; j += U) {
-                int32_t k[U];
-                float4 g[U][NV];
+            for (int j = 0; j < 32; j += U) {
+                float4 x[U][NV];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    k[u] = __shfl_sync(gmask, kk[i], j + u, G);
-                    const int32_t bag = __shfl_sync(gmask, vv[i], j + u, G);
+                    const int32_t b = __shfl_sync(0xffffffffu, bag, j + u);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) g[u][v] = __ldg(gcol[v] + (int64_t)bag * D4);
+                    for (int v = 0; v < NV; ++v) x[u][v] = grad_row(v, b);
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int q = i * G + j + u;
-                    if ((heads >> q) & 1u) {
-                        left_open = false;
 #pragma unroll
-                        for (int v = 0; v < NV; ++v) acc[v][0] = acc[v][1] = acc[v][2] = acc[v][3] = 0.0;
+                    for (int v = 0; v < NV; ++v) add_row(acc[v], x[u][v], hs & (1u << u));
+                    if (es & (1u << u)) {
+                        if (ds & (1u << u)) apply(__shfl_sync(0xffffffffu, row, j + u), acc);
+                        else store_piece(0, acc);
                     }
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        acc[v][0] += (double)g[u][v].x;
-                        acc[v][1] += (double)g[u][v].y;
-                        acc[v][2] += (double)g[u][v].z;
-                        acc[v][3] += (double)g[u][v].w;
-                    }
-                    if ((tails >> q) & 1u) emit(k[u], false);
                 }
+                hs >>= U;
+                ds >>= U;
+                es >>= U;
             }
-        }
-        // the chunk's last lookup does not end its run: the run goes on in the next chunk (only a full chunk has a
-        // next one)
-        if (ends_open) {
-            const int32_t key = __shfl_sync(gmask, kk[KPL - 1], G - 1, G);
-            if (!left_open && next2_key != key && (uint32_t)(key - key_bias) < n_rows_u) {
-                // it began in this chunk and ends in the next: its lookups there are summed here as well (they are a
-                // prefix of that chunk: m of them), and the row gets its one update
-                const int64_t start2 = start + kBwdChunk;
-                const int64_t end2 = min(start2 + (int64_t)kBwdChunk, n);
-                int32_t vv2[KPL];
-                uint32_t same = 0;
+        } else {
+            const unsigned h = (heads >> g0) & gbits, t = (tails >> g0) & gbits;
+            // my first tail, if it ends a run that began further left: finished below
+            const unsigned late = (h & 1u) ? 0u : t & (0u - t);
+            const unsigned d = (done >> g0) & gbits & ~late;
+            const unsigned ends = d | late;
 #pragma unroll
-                for (int i = 0; i < KPL; ++i) {
-                    const int64_t p = start2 + i * G + sub;
-                    const bool in = p < end2;
-                    const int32_t k2 = in ? keys[p] : -1;
-                    const int32_t bag = in ? vals[p] : 0;
-                    vv2[i] = (uint32_t)bag < n_grad_u ? bag : 0;
-                    same |= ((__ballot_sync(gmask, k2 == key) >> gshift) & gbits) << (i * G);
-                }
-                const int m = same == 0xffffffffu ? kBwdChunk : __ffs((int)~same) - 1;
-#pragma unroll 1
-                for (int q0 = 0; q0 < m; q0 += U) {
-                    float4 g[U][NV];
+            for (int j = 0; j < G; j += U) {
+                float4 x[U];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int q = q0 + u < m ? q0 + u : m - 1;       // (past the run's end: a row already asked for)
-                        const int32_t bag = __shfl_sync(gmask, pick(vv2, q / G), q % G, G);
+                for (int u = 0; u < U; ++u) x[u] = grad_row(0, __shfl_sync(0xffffffffu, bag, j + u, G));
 #pragma unroll
-                        for (int v = 0; v < NV; ++v) g[u][v] = __ldg(gcol[v] + (int64_t)bag * D4);
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        if (q0 + u >= m) continue;
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) {
-                            acc[v][0] += (double)g[u][v].x;
-                            acc[v][1] += (double)g[u][v].y;
-                            acc[v][2] += (double)g[u][v].z;
-                            acc[v][3] += (double)g[u][v].w;
+                for (int u = 0; u < U; ++u) {
+                    add_row(acc[0], x[u], h & (1u << (j + u)));
+                    if (ends & (1u << (j + u))) {
+                        if (late & (1u << (j + u))) {      // (kept in shared memory: registers would cost eight moves a step)
+                            s_first[0][threadIdx.x] = make_double2(acc[0][0], acc[0][1]);
+                            s_first[1][threadIdx.x] = make_double2(acc[0][2], acc[0][3]);
+                        } else {
+                            apply(__shfl_sync(gmask, row, j + u, G), acc);
                         }
                     }
                 }
-                emit(key, false);
-            } else {
-                emit(key, true);
+            }
+            // What the run open at the right edge of every group has collected: an inclusive scan of the groups'
+            // trailing sums that restarts at groups with a head.
+            const unsigned upto = heads & (before_group | gmask);
+            const int from = upto ? (31 - __clz((int)upto)) / G : 0, gi = g0 / G;
+#pragma unroll
+            for (int s = 1; s < NG; s <<= 1) {
+                const bool add = gi - s >= from;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const double o = __shfl_up_sync(0xffffffffu, acc[0][e], s * G);
+                    if (add) acc[0][e] += o;
+                }
+            }
+            double in[1][4];          // what the run has collected in the groups before mine
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                in[0][e] = __shfl_up_sync(0xffffffffu, acc[0][e], G);
+                acc[0][e] = __shfl_sync(0xffffffffu, acc[0][e], 32 - G + sub);
+            }
+            const uint32_t row0 = __shfl_sync(0xffffffffu, row, 0, G);
+            if (late) {
+                const double2 p = s_first[0][threadIdx.x], q = s_first[1][threadIdx.x];
+                const bool from_left = gi > 0;
+                in[0][0] = p.x + (from_left ? in[0][0] : 0.0);
+                in[0][1] = p.y + (from_left ? in[0][1] : 0.0);
+                in[0][2] = q.x + (from_left ? in[0][2] : 0.0);
+                in[0][3] = q.y + (from_left ? in[0][3] : 0.0);
+                if (late & (done >> g0)) apply(row0, in);
+                else if (late & (piece >> g0)) store_piece(0, in);
+            }
+        }
+        // the chunk's last lookup does not end its run: the run goes on in the next chunk (only a full chunk has a
+        // next one), and acc holds what it has collected here
+        const int32_t last_key = __shfl_sync(0xffffffffu, key, 31);
+        if ((tails >> 31) || (uint32_t)(last_key - key_bias) >= n_rows_u) continue;
+        if (!heads) {
+            if (lane < G) store_piece(0, acc);
+        } else if (next2_key != last_key) {
+            // it began in this chunk and ends in the next: its lookups there are summed here as well (they are a prefix
+            // of that chunk: m of them), and the row gets its one update
+            double more[NV][4];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) more[v][0] = more[v][1] = more[v][2] = more[v][3] = 0.0;
+            const int p = end + lane;
+            const int32_t k2 = p < n ? keys[p] : -1;
+            int32_t b2 = p < n ? vals[p] : 0;
+            b2 = (uint32_t)b2 < n_grad_u ? b2 : 0;
+            const int m = __popc(__ballot_sync(0xffffffffu, k2 == last_key));
+            const int mine = m - g0;             // lookups of my group that belong to the run
+#pragma unroll 1
+            for (int j = 0; j < (G == 32 ? m : G); j += U) {
+                float4 x[U][NV];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int32_t b = __shfl_sync(0xffffffffu, b2, j + u, G);
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) x[u][v] = j + u < mine ? grad_row(v, b) : f4_zero();
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) add_row(more[v], x[u][v]);
+            }
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+#pragma unroll
+                    for (int off = G; off < 32; off <<= 1) more[v][e] += __shfl_xor_sync(0xffffffffu, more[v][e], off);
+                    more[v][e] += acc[v][e];
+                }
+            if (lane < G) apply((uint32_t)(last_key - key_bias), more);
+        } else {
+            if (lane < G) store_piece(1, acc);
+            // List it, with its last chunk if that is among the next 32 (chunk c > chunk holds a piece of the run iff
+            // its first slot is the run's; sorted keys: those chunks form a prefix).  Nearly every run ends there, and
+            // k_bwd_spans then has nothing to search; the longer ones go to the list's other end.
+            const int cc = chunk + 1 + lane;
+            const bool goes_on = cc < n_chunks && keys[first + cc * kBwdChunk] == last_key;
+            const int cnt = __popc(__ballot_sync(0xffffffffu, goes_on));
+            if (lane == 0) {
+                const bool is_long = cnt == kSpanLookahead;
+                const int32_t i = atomicAdd(&span_count[is_long ? 1 : 0], 1);
+                // (one entry per chunk at most, and the counts are zero when a call starts: the list cannot overflow
+                // unless an earlier call was cut short between its two kernels)
+                if (i >= 0 && i < max_entries)
+                    reinterpret_cast<int4*>(span_list)[is_long ? max_entries - 1 - i : i] =
+                        make_int4(chunk, last_key, is_long ? -1 : chunk + cnt, 0);
+                else
+                    set_status(status, HL_ECAPACITY);
             }
         }
     }
 }
 
-// One WARP per chunk; it acts only if a run STARTS in its chunk and continues into the next one.  The lanes look
-// at the first slot of the next 32 chunks at once to find where the run ends (and, if it goes on, close in on the end
-// with a 32-way search over the rest of the list).  A run of up to kLongRun chunks is summed by its warp: the 32/G
-// groups add the run's continuation pieces in an interleaved, fixed order in fp64 (runs of many thousands of lookups
-// occur), the group sums are combined by shuffles in a fixed order, and group 0 applies the single SGD update of the
-// row.  Longer runs (a popular row can own hundreds of chunks) are queued in shared memory and then summed by the
-// whole CTA, every group taking every (8 * 32/G)-th piece, the group sums combined in a fixed order by one group.
-constexpr int kLongRun = 32;
-
+// Finishes the listed runs: those that start in a chunk and go on over at least two more.  Two lists share one array.
+//
+// From its front: runs whose last chunk is known (up to kSpanLookahead chunks on).  One WARP per run: the 32/G groups add
+// the run's continuation pieces in an interleaved, fixed order in fp64, the group sums are combined by shuffles in a
+// fixed order, and group 0 applies the single SGD update of the row.
+// From its back: longer runs (a popular row can own hundreds of chunks).  One CTA per run, because they are what the
+// kernel's length depends on: its warps close in on the end with a 32-way search over the sorted keys, every group takes
+// every (8 * 32/G)-th piece, and one group combines the group sums in a fixed order.  (With both kinds in one list a CTA
+// met up to eight long runs one after the other: 2.6 M lookups of 512 bytes took 36.6 us.)
 template <int G, int NV>
 __global__ void __launch_bounds__(kThreads) k_bwd_spans(float* __restrict__ cache, const int32_t* __restrict__ keys,
                                                         const int32_t* __restrict__ d_n_lookups, int D4,
@@ -470,179 +507,118 @@ __global__ void __launch_bounds__(kThreads) k_bwd_spans(float* __restrict__ cach
                                                         const int32_t* __restrict__ span_list, int64_t max_entries) {
     constexpr int GW = 32 / G;   // groups per warp
     constexpr int kWarps = kThreads / 32;
-    constexpr int U = NV >= 4 ? 2 : (NV >= 2 ? 4 : 8);   // partial sums in flight per lane
-    constexpr int UC = 8;                // the same in the CTA-wide sum
-    constexpr bool kCtaPath = NV == 1;   // the CTA-wide sum keeps one float4 column per lane
-    __shared__ int64_t q_chunk[kWarps], q_last[kWarps], q_row[kWarps];
-    __shared__ double s_sum[kCtaPath ? kThreads : 1][4];
+    constexpr int U = NV >= 4 ? 2 : (NV >= 2 ? 4 : 8);   // pieces in flight per lane
+    __shared__ double s_sum[kThreads][4];
     const int64_t first = d_first ? d_first[0] : 0;
     const int64_t n = first + d_n_lookups[0];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int sub = lane % G, gi = lane / G;
     const float4* __restrict__ part4 = reinterpret_cast<const float4*>(part);
+    const int4* __restrict__ list = reinterpret_cast<const int4*>(span_list);
     float4* cache4 = reinterpret_cast<float4*>(cache);
     const int64_t n_chunks = (n - first + kBwdChunk - 1) / kBwdChunk;
+    const int64_t most = n_chunks < max_entries ? n_chunks : max_entries;
+    auto clamped = [&](int32_t c) { return c < 0 ? (int64_t)0 : ((int64_t)c < most ? (int64_t)c : most); };
+    const int64_t n_short = clamped(span_count[0]), n_long = clamped(span_count[1]);
 
-    int64_t n_owned = span_count[0];     // chunks in which a run starts that goes on into the next chunk
-    n_owned = n_owned < 0 ? 0 : (n_owned < n_chunks ? n_owned : n_chunks);
-    n_owned = n_owned < max_entries ? n_owned : max_entries;
-
-    // every warp of the CTA makes the same number of trips (there are block barriers inside)
-    for (int64_t base = (int64_t)blockIdx.x * kWarps; base < n_owned; base += (int64_t)gridDim.x * kWarps) {
-        if (kCtaPath && lane == 0) q_chunk[wib] = -1;
-        bool mine = false;
-        int32_t key = 0;
-        int64_t chunk = 0, row = 0, last_chunk = 0;
-        int64_t known_last = -1;
-        if (base + wib < n_owned) {
-            // (chunk, slot key of the run, its last chunk if the sum kernel has found it)
-            const int4 e = reinterpret_cast<const int4*>(span_list)[base + wib];
-            chunk = e.x;
-            key = e.y;
-            row = (int64_t)key - key_bias;
-            mine = chunk >= 0 && chunk + 1 < n_chunks && row >= 0 && row < n_slots;
-            if (e.z > e.x && e.z < n_chunks) known_last = e.z;
-        }
-        // the run's first piece is asked for now; it is needed after the search
-        float4 piece0[NV];
+    // sum over pieces from + step * {first, first + groups, ...} <= last of this lane's columns
+    auto add_pieces = [&](double (&acc)[NV][4], int64_t from, int64_t last, int64_t groups) {
+        for (int64_t c2 = from; c2 <= last; c2 += groups * U) {
+            float4 t[U][NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int c = sub + v * G;
-            const bool ld = mine && gi == 0 && c < D4;
-            piece0[v] = ld ? part4[(chunk * 2 + 1) * D4 + c] : f4_zero();
-        }
-        if (mine) {
-            // last chunk that holds a piece of the run: chunk c > chunk holds one iff its first slot is the run's
-            int64_t lo = chunk + 1, hi = n_chunks;      // chunk lo holds a piece, chunk hi (if any) does not
-            if (known_last >= 0) {
-                lo = known_last;
-                hi = known_last + 1;
-            } else {
-                const int64_t cc = lo + 1 + lane;       // the 32 chunks after lo
-                const bool t = cc < hi && keys[first + cc * kBwdChunk] == key;
-                const unsigned m = __ballot_sync(0xffffffffu, t);
-                const int cnt = __popc(m);              // sorted keys: the lanes that see the run form a prefix
-                lo += cnt;
-                if (cnt < 32) hi = min(hi, lo + 1);
-            }
-            while (hi - lo > 1) {
-                const int64_t step = (hi - lo + 31) / 32;
-                const int64_t cc = lo + (lane + 1) * step;
-                const bool t = cc < hi && keys[first + cc * kBwdChunk] == key;
-                const int cnt = __popc(__ballot_sync(0xffffffffu, t));
-                const int64_t new_hi = min(hi, lo + (cnt + 1) * step);
-                lo += cnt * step;
-                hi = new_hi;
-            }
-            last_chunk = lo;
-            if (kCtaPath && last_chunk - chunk > kLongRun) {
-                if (lane == 0) {
-                    q_chunk[wib] = chunk;
-                    q_last[wib] = last_chunk;
-                    q_row[wib] = row;
-                }
-                mine = false;        // summed by the whole CTA below
-            }
-        }
-        if (mine) {
-            double dacc[NV][4];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                dacc[v][0] = piece0[v].x;
-                dacc[v][1] = piece0[v].y;
-                dacc[v][2] = piece0[v].z;
-                dacc[v][3] = piece0[v].w;
-            }
-            for (int64_t c2 = chunk + 1 + gi; c2 <= last_chunk; c2 += (int64_t)GW * U) {
-                float4 t[U][NV];
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        const int c = sub + v * G;
-                        const int64_t cc = c2 + (int64_t)u * GW;
-                        t[u][v] = (cc <= last_chunk && c < D4) ? part4[(cc * 2) * D4 + c] : f4_zero();
-                    }
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-#pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        dacc[v][0] += (double)t[u][v].x;
-                        dacc[v][1] += (double)t[u][v].y;
-                        dacc[v][2] += (double)t[u][v].z;
-                        dacc[v][3] += (double)t[u][v].w;
-                    }
-            }
-#pragma unroll
-            for (int off = G; off < 32; off <<= 1)
-#pragma unroll
-                for (int v = 0; v < NV; ++v)
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) dacc[v][e] += __shfl_xor_sync(0xffffffffu, dacc[v][e], off);
-            if (gi == 0) {
+            for (int u = 0; u < U; ++u)
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     const int c = sub + v * G;
-                    if (c < D4)
-                        red_add_f4(&cache4[row * D4 + c],
-                                   make_float4(-(lr * (float)dacc[v][0]), -(lr * (float)dacc[v][1]),
-                                               -(lr * (float)dacc[v][2]), -(lr * (float)dacc[v][3])));
+                    const int64_t cc = c2 + u * groups;
+                    t[u][v] = (cc <= last && c < D4) ? part4[(cc * 2) * D4 + c] : f4_zero();
                 }
-            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int v = 0; v < NV; ++v) add_row(acc[v], t[u][v]);
         }
-        if (kCtaPath) {
+    };
+    auto apply = [&](int64_t row, int v, double x, double y, double z, double w) {
+        const int c = sub + v * G;
+        if (c < D4)
+            red_add_f4(&cache4[row * D4 + c],
+                       make_float4(-(lr * (float)x), -(lr * (float)y), -(lr * (float)z), -(lr * (float)w)));
+    };
+
+    for (int64_t i = blockIdx.x; i < n_long; i += gridDim.x) {
+        const int4 e = list[max_entries - 1 - i];            // (chunk, slot key of the run, -, -)
+        const int64_t chunk = e.x, row = (int64_t)e.y - key_bias;
+        if (chunk < 0 || chunk + 1 >= n_chunks || row < 0 || row >= n_slots) continue;     // the same for all threads
+        // last chunk that holds a piece of the run: chunk c > chunk holds one iff its first slot is the run's; chunk lo
+        // does, chunk hi (if any) does not
+        int64_t lo = chunk + 1, hi = n_chunks;
+        while (hi - lo > 1) {
+            const int64_t step = (hi - lo + 31) / 32;
+            const int64_t cc = lo + (lane + 1) * step;
+            const bool t = cc < hi && keys[first + cc * kBwdChunk] == e.y;
+            const int cnt = __popc(__ballot_sync(0xffffffffu, t));     // sorted keys: a prefix of the lanes
+            const int64_t new_hi = min(hi, lo + (cnt + 1) * step);
+            lo += cnt * step;
+            hi = new_hi;
+        }
+        double acc[NV][4];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v][0] = acc[v][1] = acc[v][2] = acc[v][3] = 0.0;
+        add_pieces(acc, chunk + 1 + wib * GW + gi, lo, (int64_t)kWarps * GW);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s_sum[threadIdx.x][k] = acc[v][k];
             __syncthreads();
-            for (int qi = 0; qi < kWarps; ++qi) {
-                const int64_t qc = q_chunk[qi];
-                if (qc < 0) continue;                    // the same for all threads
-                const int64_t ql = q_last[qi], qrow = q_row[qi];
-                const int gg = wib * GW + gi;            // this group among the CTA's kWarps * GW groups
-                double d0 = 0.0, d1 = 0.0, d2 = 0.0, d3 = 0.0;
-                for (int64_t c2 = qc + 1 + gg; c2 <= ql; c2 += (int64_t)kWarps * GW * UC) {
-                    float4 t[UC];
+            const int c = sub + v * G;
+            if (threadIdx.x < G && c < D4) {       // group 0 of warp 0: lane sub owns column c
+                const float4 p = part4[(chunk * 2 + 1) * D4 + c];      // the piece in the run's first chunk
+                double a[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll 8
+                for (int g2 = 0; g2 < kWarps * GW; ++g2)
 #pragma unroll
-                    for (int u = 0; u < UC; ++u) {
-                        const int64_t cc = c2 + (int64_t)u * kWarps * GW;
-                        t[u] = (cc <= ql && sub < D4) ? part4[(cc * 2) * D4 + sub] : f4_zero();
-                    }
-#pragma unroll
-                    for (int u = 0; u < UC; ++u) {
-                        d0 += (double)t[u].x;
-                        d1 += (double)t[u].y;
-                        d2 += (double)t[u].z;
-                        d3 += (double)t[u].w;
-                    }
-                }
-                s_sum[threadIdx.x][0] = d0;
-                s_sum[threadIdx.x][1] = d1;
-                s_sum[threadIdx.x][2] = d2;
-                s_sum[threadIdx.x][3] = d3;
-                __syncthreads();
-                if (threadIdx.x < G && sub < D4) {       // group 0 of warp 0: lane sub owns column sub
-                    const float4 p = part4[(qc * 2 + 1) * D4 + sub];      // the piece in the run's first chunk
-                    double a0 = p.x, a1 = p.y, a2 = p.z, a3 = p.w;
-                    for (int g2 = 0; g2 < kWarps * GW; ++g2) {
-                        a0 += s_sum[g2 * G + sub][0];
-                        a1 += s_sum[g2 * G + sub][1];
-                        a2 += s_sum[g2 * G + sub][2];
-                        a3 += s_sum[g2 * G + sub][3];
-                    }
-                    red_add_f4(&cache4[qrow * D4 + sub], make_float4(-(lr * (float)a0), -(lr * (float)a1),
-                                                                     -(lr * (float)a2), -(lr * (float)a3)));
-                }
-                __syncthreads();
+                    for (int k = 0; k < 4; ++k) a[k] += s_sum[g2 * G + sub][k];
+                apply(row, v, a[0], a[1], a[2], a[3]);
             }
-            __syncthreads();     // every warp has read the whole queue before any warp clears its entry again
+            __syncthreads();
         }
     }
-    // The list is empty again for the next call: the last CTA to get here clears the count (word 0) and the tally of
-    // finished CTAs (word 2).  Every CTA read the count when it started, and the next call's kernels start after this
-    // grid has ended.
+
+    for (int64_t i = (int64_t)blockIdx.x * kWarps + wib; i < n_short; i += (int64_t)gridDim.x * kWarps) {
+        const int4 e = list[i];                              // (chunk, slot key of the run, its last chunk, -)
+        const int64_t chunk = e.x, last = e.z, row = (int64_t)e.y - key_bias;
+        if (chunk < 0 || last <= chunk || last >= n_chunks || row < 0 || row >= n_slots) continue;
+        double acc[NV][4];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int c = sub + v * G;
+            const float4 p = gi == 0 && c < D4 ? part4[(chunk * 2 + 1) * D4 + c] : f4_zero();
+            acc[v][0] = p.x;
+            acc[v][1] = p.y;
+            acc[v][2] = p.z;
+            acc[v][3] = p.w;
+        }
+        add_pieces(acc, chunk + 1 + gi, last, GW);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                for (int off = G; off < 32; off <<= 1) acc[v][k] += __shfl_xor_sync(0xffffffffu, acc[v][k], off);
+            if (gi == 0) apply(row, v, acc[v][0], acc[v][1], acc[v][2], acc[v][3]);
+        }
+    }
+
+    // The lists are empty again for the next call: the last CTA to get here clears the counts (words 0 and 1) and the
+    // tally of finished CTAs (word 2).  Every CTA read the counts when it started, and the next call's kernels start
+    // after this grid has ended.
     __syncthreads();
     if (threadIdx.x == 0) {
         const int32_t finished = atomicAdd(&span_count[2], 1);
         if (finished == (int32_t)gridDim.x - 1) {
             span_count[0] = 0;
+            span_count[1] = 0;
             span_count[2] = 0;
         }
     }
@@ -671,7 +647,7 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
     const int64_t max_chunks = div_up(ctx->max_nnz, kBwdChunk);
     // a fixed number of CTAs per multiprocessor (the groups stride over the chunks), so that kernels of other
     // streams find room beside this one
-    const int grid = grid_for(max_chunks * G, kThreads, bwd_ctas_per_sm(ctx) * ctx_sms(ctx));
+    const int grid = grid_for(max_chunks * 32, kThreads, bwd_ctas_per_sm(ctx) * ctx_sms(ctx));
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 0, stream);
     // the list of runs that cross a chunk border sits behind the partial sums: [count words (8 ints)] [entries].
