@@ -161,8 +161,8 @@ HL_API int32_t hl_set_mover_ctas(hl_ctx* ctx, int32_t read_ctas, int32_t write_c
  * than 128 fp32; 6 for the sum kernel). */
 HL_API int32_t hl_set_kernel_width(hl_ctx* ctx, int32_t fwd_ctas_per_sm, int32_t bwd_ctas_per_sm);
 
-/* Test aid for the bounded device-side waits (the tile chaining of the scan inside hl_fragment and of the sorts
- * inside hl_embbag_bwd_* / hl_gather_cold, the wait of a row mover for a stage of bulk copies).  In production these
+/* Test aid for the bounded device-side waits (the tile chaining of the prefix sums inside hl_fragment and
+ * hl_gather_cold and of the sorts inside hl_embbag_bwd_*, the wait of a row mover for a stage of bulk copies).  In production these
  * waits poll for about a second before they give up, which never happens.  poll_limit > 0 makes them give up after
  * that many polls, and makes ONE participant withhold what the others wait for: tile `stall_tile` of every chained scan
  * and sort pass publishes nothing, and (stall_tile >= 0) the first stage of the movers' first CTA issues no copies.
@@ -171,8 +171,7 @@ HL_API int32_t hl_set_kernel_width(hl_ctx* ctx, int32_t fwd_ctas_per_sm, int32_t
  * poll_limit = 0 restores production behaviour.  Nothing here can hang or fault the device. */
 HL_API int32_t hl_test_bounded_waits(hl_ctx* ctx, int32_t poll_limit, int64_t stall_tile);
 
-/* Number of kernels this library has launched from the host in this process so far (all contexts; the general cold-row
- * search that a kernel launches from the device is not counted). */
+/* Number of kernels this library has launched in this process so far (all contexts). */
 HL_API uint64_t hl_launch_count(void);
 
 /* ---------------------------------------------------------------------------------------------------------
@@ -353,14 +352,10 @@ HL_API int32_t hl_index_cold(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non
                              const int32_t* d_prev_cold_rows, const int64_t* d_n_prev, int32_t* d_fwd_src,
                              void* stream);
 /* hl_index_cold in two halves.  hl_index_cold_begin classifies X's lookups and finds the distinct cold rows and the
- * slots: with at most 40 960 cold lookups (20 480 on a device that cannot place a cluster of 16 CTAs) one
- * thread-block cluster does all of it in one kernel; with more, that
- * kernel launches the general search (tile sort, head flags, scan, assignment) from the device, behind itself and
- * ahead of whatever the host queued next -- so the host queues the same two kernels for every mini-batch and never
- * needs to know the count.  The device word hl_index_cold_verdict(ctx) says afterwards which it was: 0 = the cluster
- * kernel, else the number of cold lookups handed on.  hl_index_cold_end does the match against the previous cold rows
- * (general_not_needed is ignored; it dates from when the host queued the general search).  Same arguments as
- * hl_index_cold; both halves on one stream, nothing else of this context's cold-row search between them. */
+ * slots (a bitmap of the model's rows, ranked in row order: the same kernels however many cold lookups there are).
+ * hl_index_cold_end does the match against the previous cold rows.  The device word hl_index_cold_verdict(ctx), which
+ * once said whether a second search had to be queued in between, reads 0, and general_not_needed is ignored.  Same
+ * arguments as hl_index_cold; both halves on one stream, nothing else of this context's cold-row search between them. */
 HL_API int32_t hl_index_cold_begin(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, int64_t stage_row0,
                                    int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold, void* stream);
 HL_API const int32_t* hl_index_cold_verdict(hl_ctx* ctx);
@@ -422,7 +417,7 @@ HL_API hl_pipe* hl_pipe_create(hl_ctx* ctx, float* d_cache, float* host_table, i
  * caller's; to put the bandwidth-bound main work above the ahead-work, create main_stream with a higher priority
  * than the ones given here. */
 typedef struct {
-    int32_t index_priority;          /* the three streams of index-only ahead-work (fragment, cold-row search, sort) */
+    int32_t index_priority;          /* the two streams of index-only ahead-work (fragment and cold-row search; sort) */
     int32_t link_priority;           /* the two streams of host-link transfers (host read, write-back)              */
     int32_t write_back;              /* HL_PIPE_WB_x: when the write-back of mini-batch j runs                       */
 } hl_pipe_options;
@@ -474,8 +469,8 @@ HL_API int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float* d_
  * of host time per call and no device memory).  Kinds HL_SPAN_KERNEL + HL_TIMER_x bracket single kernels inside those
  * calls: the movers' kernels, the backward's sum kernel, the forward kernel.  hl_pipe_trace_end waits for everything
  * queued (host-side), then writes the recorded spans, in the order they were issued, with times in milliseconds
- * relative to the earliest one; *n_spans = how many.  stream: 0 = main, 1-3 = fragment / sort / cold-row search,
- * 4 = host reads, 5 = write-backs. */
+ * relative to the earliest one; *n_spans = how many.  stream: 0 = main, 1 = index-only work, 2 = its sorts of
+ * many lookups, 4 = host reads, 5 = write-backs. */
 #define HL_SPAN_FRAGMENT     0
 #define HL_SPAN_INDEX_BEGIN  1
 #define HL_SPAN_INDEX_END    2

@@ -51,23 +51,19 @@ size_t carve(char* base, const hl_geometry* g, int64_t N, int32_t max_batch, int
     r->sel = c.take<SelectState>(1);
     r->sel_gt = c.take<uint32_t>(*n_sel_tiles + 2);
     r->sel_eq = c.take<uint32_t>(*n_sel_tiles + 2);
-    r->frag_flags = c.take<uint8_t>(max_batch);
-    r->frag_scan = c.take<int32_t>(max_bags + 2);
-    r->frag_tiles = c.take<int32_t>(scan_tile_words(max_bags));
+    r->frag_words = c.take<uint32_t>(max_batch / 32 + 1);
+    r->frag_chain = c.take<unsigned long long>(frag_chain_words(max_bags));
     for (int i = 0; i < 2; ++i) {
         r->bwd_keys[i] = c.take<int32_t>(nnz);
         r->bwd_vals[i] = c.take<int32_t>(nnz);
     }
-    r->bwd_hist = c.take<uint32_t>(hist_words(nnz));
+    for (int i = 0; i < 2; ++i) r->bwd_hist[i] = c.take<uint32_t>(hist_words(nnz));
     r->bwd_part = c.take<float>(2 * div_up(nnz, kBwdChunk) * D + bwd_span_list_words(nnz));
     r->bwd_n = c.take<int32_t>(4);
-    for (int i = 0; i < 2; ++i) {
-        r->cold_keys[i] = c.take<int32_t>(nnz);
-        r->cold_vals[i] = c.take<int32_t>(nnz);
-    }
-    r->cold_hist = c.take<uint32_t>(hist_words(nnz));
-    r->cold_rank = c.take<int32_t>(nnz + 2);
-    r->cold_tiles = c.take<int32_t>(scan_tile_words(nnz));
+    r->cold_bits = c.take<uint32_t>(cold_bitmap_words(N));
+    r->cold_summary = c.take<uint32_t>(N > kColdDirectRows ? cold_summary_words(N) : 1);
+    r->cold_ranked = c.take<uint2>(cold_bitmap_words(N));
+    r->cold_chain = c.take<unsigned long long>(cold_chain_words(N));
     r->cold_n = c.take<int32_t>(4);
     (void)hot_cap;
     (void)staging_cap;
@@ -140,7 +136,13 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
     if (e == cudaSuccess) e = cudaMemset(ctx->r.remap, 0, sizeof(RemapBlock) * ctx->n_remap_blocks);
     if (e == cudaSuccess) e = cudaMemset(ctx->r.counts, 0, sizeof(uint32_t) * N);
     if (e == cudaSuccess) e = cudaMemset(ctx->r.sel, 0, sizeof(SelectState));
-    if (e == cudaSuccess) e = cudaMemset(ctx->r.frag_tiles, 0, sizeof(int32_t) * scan_tile_words(max_bags));
+    if (e == cudaSuccess)
+        e = cudaMemset(ctx->r.frag_chain, 0, sizeof(unsigned long long) * frag_chain_words(max_bags));
+    if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_bits, 0, sizeof(uint32_t) * cold_bitmap_words(N));
+    if (e == cudaSuccess && N > kColdDirectRows)
+        e = cudaMemset(ctx->r.cold_summary, 0, sizeof(uint32_t) * cold_summary_words(N));
+    if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_chain, 0, sizeof(unsigned long long) * cold_chain_words(N));
+    if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_n, 0, 4 * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(span_count_of(ctx), 0, 8 * sizeof(int32_t));   // kept zero between backward calls
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {

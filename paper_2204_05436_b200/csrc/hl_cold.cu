@@ -1,319 +1,143 @@
-// The non-popular micro-batch's working set: classify its lookups, find the distinct cold rows, stage them from
-// the host-DRAM table (bulk copies over the host link, row by row) behind the hot cache, and write them back.
+// The non-popular micro-batch's working set: classify its lookups, find the distinct cold rows, stage them from the
+// host-DRAM table (bulk copies over the host link, row by row) behind the hot cache, and write them back.
 #include "hl_common.cuh"
-#include <cooperative_groups.h>
 
 namespace hl {
 namespace {
 
 constexpr int kThreads = 256;
 
-// Lookups of X: popular rows resolve to their cache slot at once; cold ones are appended (row, position) to
-// the list that is sorted next.  Append order is arbitrary; the sort and the final slots do not depend on it.
+// ---- the distinct cold rows, in ascending order --------------------------------------------------------------
+// One bit per row of the model: classifying X's lookups sets the bits of its cold rows (classify_cold), k_cold_rank
+// reads the bitmap in row order -- which is ascending order without a sort -- and hands out the ranks, and k_cold_assign
+// turns every cold lookup into the slot of its row's rank.  The work depends on the lookups and (a 32nd or a 1024th of
+// a word per row) on the size of the model, not on how many cold lookups there are, so there is one path for all
+// mini-batches: three kernels where a sort of the cold lookups took a cluster of 16 CTAs 21-43 us (up to 40 960 lookups)
+// or ten device-launched kernels and 0.3-0.7 ms (above).
 __global__ void __launch_bounds__(kThreads) k_cold_classify(int32_t* __restrict__ ids,
                                                             const int32_t* __restrict__ offsets,
                                                             const int32_t* __restrict__ d_n_non, int max_batch,
                                                             int bags_per_sample_all, int64_t cap_ids, int64_t N,
-                                                            const RemapBlock* __restrict__ remap,
-                                                            int32_t* __restrict__ keys, int32_t* __restrict__ vals,
-                                                            int32_t* __restrict__ d_n_cold_lookups, int64_t max_nnz,
-                                                            int32_t* status) {
+                                                            BitmapProbe remap, ColdMarks marks, int32_t* status) {
     int n_non = *d_n_non;
     n_non = n_non < 0 ? 0 : (n_non > max_batch ? max_batch : n_non);
     int64_t L = offsets[(int64_t)n_non * bags_per_sample_all];
     if (L > cap_ids) L = cap_ids;
-    const unsigned lt = lanemask_lt();
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // whole warps iterate together (the ballot below needs every lane)
-    for (int64_t j0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~int64_t(31); j0 < L; j0 += stride) {
-        const int64_t j = j0 + (threadIdx.x & 31);
-        bool cold = false;
-        int32_t g = -1;
-        if (j < L) {
-            g = ids[j];
-            if (g >= N) {
-                set_status(status, HL_EBOUNDS);
-                ids[j] = -1;
-            } else if (g >= 0) {
-                const int32_t slot = remap_slot(remap, g);
-                if (slot >= 0) ids[j] = slot;
-                else cold = true;
-            }
-        }
-        const unsigned vote = __ballot_sync(0xffffffffu, cold);
-        if (vote) {
-            int32_t base = 0;
-            if ((threadIdx.x & 31) == 0) base = atomicAdd(d_n_cold_lookups, __popc(vote));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (cold) {
-                const int64_t pos = (int64_t)base + __popc(vote & lt);
-                if (pos < max_nnz) {
-                    keys[pos] = g;
-                    vals[pos] = (int32_t)j;
-                }
-            }
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < L; j += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t g = ids[j];
+        if (g >= N) {
+            set_status(status, HL_EBOUNDS);
+            ids[j] = -1;
+        } else if (g >= 0) {
+            ids[j] = classify_cold(remap, g, marks);
         }
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_cold_heads(const int32_t* __restrict__ keys, int64_t n,
-                                                         int32_t* __restrict__ heads) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        heads[i] = (i == 0 || keys[i] != keys[i - 1]) ? 1 : 0;
-}
-
-// rank_excl[i] = number of run heads before i; the row at i has rank rank_excl[i] if it is a head, else
-// rank_excl[i] - 1.  A row of rank r is staged at cache slot slot0 + r (slot0 = start of the staging window).
-__global__ void __launch_bounds__(kThreads) k_cold_assign(const int32_t* __restrict__ keys,
-                                                          const int32_t* __restrict__ vals, int64_t n,
-                                                          const int32_t* __restrict__ rank_excl, int64_t slot0,
-                                                          int64_t staging_cap, int32_t* __restrict__ ids,
-                                                          int32_t* __restrict__ cold_rows,
-                                                          int64_t* __restrict__ d_n_cold, int32_t* status,
-                                                          int64_t cap_ids) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        int64_t distinct = rank_excl[n];
+// Tiles of kThreads * ITEMS words, chained (chain_before; chain[0] =
+// tally of finished CTAs, [1 + tile] = status word; zero on entry, and the CTA that finishes last clears them again).
+// SUMMARY: the words are those of the summary, which has a bit for every bitmap word that is not zero (models above
+// kColdDirectRows rows, whose bitmap would be megabytes of zeros to read); otherwise the bitmap's own.  Bitmap and summary
+// are left cleared; marks.ranked[word] keeps what k_cold_assign needs: the word's bits and the rank of its first one.
+template <bool SUMMARY, int ITEMS>
+__global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_words, int64_t staging_cap,
+                                                        int32_t* __restrict__ cold_rows, int64_t* __restrict__ d_n_cold,
+                                                        int32_t* __restrict__ verdict, unsigned long long* chain,
+                                                        int32_t* status, int max_polls, uint32_t* __restrict__ clear,
+                                                        int64_t n_clear) {
+    constexpr int NW = kThreads / 32;
+    __shared__ int s_sum[NW];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n_clear / 4; i += (int64_t)gridDim.x * kThreads)
+        reinterpret_cast<uint4*>(clear)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const int tile = blockIdx.x;
+    const int first = tile * kThreads * ITEMS;
+    uint32_t word[ITEMS];
+    int start[ITEMS], all = 0;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int w = first + (warp * ITEMS + i) * 32 + lane;
+        word[i] = w < n_words ? (SUMMARY ? marks.summary[w] : marks.bits[w]) : 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int w = first + (warp * ITEMS + i) * 32 + lane;
+        int n = 0;
+        if (SUMMARY) {
+            for (uint32_t m = word[i]; m; m &= m - 1) n += __popc(marks.bits[(int64_t)w * 32 + __ffs((int)m) - 1]);
+        } else {
+            n = __popc(word[i]);
+        }
+        int incl = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        start[i] = all + incl - n;
+        all += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) s_sum[warp] = all;
+    __syncthreads();
+    int tile_sum = 0, warp_start = 0;
+#pragma unroll
+    for (int k = 0; k < NW; ++k) {
+        if (k < warp) warp_start += s_sum[k];
+        tile_sum += s_sum[k];
+    }
+    chain_publish(chain + 1, tile, (unsigned long long)tile_sum);
+    const int before = (int)chain_before<kThreads>(chain + 1, tile, (unsigned long long)tile_sum, true, max_polls, status);
+    if (threadIdx.x == 0 && first + kThreads * ITEMS >= n_words) {       // the last tile knows the total
+        int64_t distinct = (int64_t)before + tile_sum;
         if (distinct > staging_cap) {
             set_status(status, HL_ECAPACITY);
             distinct = staging_cap;
         }
         *d_n_cold = distinct;
+        *verdict = 0;
     }
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const bool head = i == 0 || keys[i] != keys[i - 1];
-        const int64_t rank = head ? rank_excl[i] : rank_excl[i] - 1;
-        const int64_t where = vals[i];
-        if (where < 0 || where >= cap_ids || rank < 0) continue;   // only after a chain poll gave up (HL_ETIMEOUT)
-        if (rank < staging_cap) {
-            if (head) cold_rows[rank] = keys[i];
-            ids[where] = (int32_t)(slot0 + rank);
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int w = first + (warp * ITEMS + i) * 32 + lane;
+        int rank = before + warp_start + start[i];
+        auto take = [&](int64_t at, uint32_t bits) {         // bitmap word `at`
+            marks.bits[at] = 0u;
+            marks.ranked[at] = make_uint2(bits, (unsigned)rank);
+            for (uint32_t m = bits; m; m &= m - 1, ++rank)
+                if (rank < staging_cap) cold_rows[rank] = (int32_t)(at * 32 + __ffs((int)m) - 1);
+        };
+        if (word[i] == 0u) continue;
+        if (SUMMARY) {
+            marks.summary[w] = 0u;
+            for (uint32_t m = word[i]; m; m &= m - 1) {
+                const int64_t at = (int64_t)w * 32 + __ffs((int)m) - 1;
+                take(at, marks.bits[at]);
+            }
         } else {
-            ids[where] = -1;   // no room to stage this row: the lookup is dropped and the status word says so
+            take(w, word[i]);
         }
     }
+    if (threadIdx.x == 0) s_last = atomicAdd(&chain[0], 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (s_last)                                              // (nobody reads the status words any more)
+        for (int i = threadIdx.x; i < (int)gridDim.x + 1; i += kThreads) chain[i] = 0ull;
 }
 
-// ---- few cold lookups: one thread-block cluster does sort, distinct-row ranking and slot assignment ----------------
-// With at most CTAS * kSmallPerCta cold lookups (a DLRM-large mini-batch has about 18 K) the chain of radix passes,
-// head flags, scan and assignment -- nine launches that each take longer to start than to run -- is one kernel of
-// one cluster of CTAS CTAs: 16 (40 960 lookups; a cluster size the kernel has to opt in to) where the device can
-// place such a cluster, else 8 (20 480).  CTA c owns positions [c * kSmallPerCta, (c + 1) * kSmallPerCta) of the list.  Every pass ranks
-// the pairs, held in registers, by one digit (per-warp digit counters, as in the tile kernel of the general sort),
-// adds up the digit counts of the cluster's CTAs through distributed shared memory, and writes each pair into the shared
-// memory of the CTA that owns its new position.  The sorted list is then ranked and assigned in place.
-// Order of a CTA's items: position = warp * (32 * kSmallItems) + round * 32 + lane.
-// Larger inputs: the kernel launches the general path itself (tile sort, head flags, scan, assignment) as tail
-// launches, which run after this grid and before anything the host queued behind it -- so the host queues the same
-// two kernels for every mini-batch and never needs to know which path ran.  *d_n_general = the number of cold lookups
-// handed to the general path (0: none).
-constexpr int kSmallThreads = 256;
-constexpr int kSmallItems = 10;
-constexpr int kSmallPerCta = kSmallThreads * kSmallItems;       // 2560
-constexpr int kSmallWarps = kSmallThreads / 32;
-
-// what the general path works on (device pointers into the context's cold region)
-struct GeneralArgs {
-    int32_t* keys[2];
-    int32_t* vals[2];
-    uint32_t* hist;
-    int32_t* rank;
-    int32_t* tiles;
-    int64_t cap_ids;
-    int key_bits;
-    int max_polls;
-};
-
-__device__ __forceinline__ int block_scan_small(int v, int* smem33, int& total) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int incl = v;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const int o = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += o;
+// Every cold lookup of X (an id of -2 - g) gets the staging slot of its row: slot0 + rank (slot0 = start of the window).
+__global__ void __launch_bounds__(kThreads) k_cold_assign(int32_t* __restrict__ ids, const int32_t* __restrict__ offsets,
+                                                          const int32_t* __restrict__ d_n_non, int max_batch,
+                                                          int bags_per_sample_all, int64_t cap_ids,
+                                                          const uint2* __restrict__ ranked, int64_t slot0,
+                                                          int64_t staging_cap) {
+    int n_non = *d_n_non;
+    n_non = n_non < 0 ? 0 : (n_non > max_batch ? max_batch : n_non);
+    int64_t L = offsets[(int64_t)n_non * bags_per_sample_all];
+    if (L > cap_ids) L = cap_ids;
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < L; j += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t id = ids[j];
+        if (id <= -2) ids[j] = cold_slot(ranked, id, slot0, staging_cap);
     }
-    if (lane == 31) smem33[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        const int w = lane < kSmallWarps ? smem33[lane] : 0;
-        int wi = w;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int o = __shfl_up_sync(0xffffffffu, wi, d);
-            if (lane >= d) wi += o;
-        }
-        if (lane < kSmallWarps) smem33[lane] = wi - w;
-        if (lane == 31) smem33[32] = wi;
-    }
-    __syncthreads();
-    const int res = smem33[warp] + incl - v;
-    total = smem33[32];
-    __syncthreads();
-    return res;
-}
-
-template <int CTAS>
-__global__ void __launch_bounds__(kSmallThreads) k_cold_small(const int32_t* __restrict__ keys_in,
-                                                              const int32_t* __restrict__ vals_in,
-                                                              const int32_t* __restrict__ d_n, int64_t n_max,
-                                                              int passes, int64_t slot0, int64_t staging_cap,
-                                                              int32_t* __restrict__ ids,
-                                                              int32_t* __restrict__ cold_rows,
-                                                              int64_t* __restrict__ d_n_cold,
-                                                              int32_t* __restrict__ d_n_general, int32_t* status,
-                                                              GeneralArgs ga) {
-    namespace cg = cooperative_groups;
-    cg::cluster_group cluster = cg::this_cluster();
-    __shared__ int32_t s_key[kSmallPerCta];
-    __shared__ int32_t s_val[kSmallPerCta];
-    __shared__ uint32_t cnt[kSmallWarps * 256];
-    __shared__ uint32_t cta_hist[256];       // this CTA's digit counts, read by the other CTAs
-    __shared__ uint32_t digit_base[256];
-    __shared__ int cta_heads;                // this CTA's number of run heads, read by the other CTAs
-    __shared__ int scan_smem[33];
-    int64_t n64 = d_n[0];
-    n64 = n64 < 0 ? 0 : (n64 < n_max ? n64 : n_max);
-    const int cta = (int)cluster.block_rank();
-    if (n64 > CTAS * kSmallPerCta) {         // the same decision in all CTAs, before any cluster barrier
-        if (cta == 0 && threadIdx.x == 0) {
-            d_n_general[0] = (int32_t)n64;
-            // the general path, queued behind this grid: stable sort of the (row, position) pairs by row, a flag at
-            // the head of every run, ranks by a scan of the flags, slots and distinct rows from the ranks
-            const int cur = radix_sort_pairs_tail(ga.keys[0], ga.keys[1], ga.vals[0], ga.vals[1], n64, ga.key_bits,
-                                                  ga.hist, status, ga.max_polls);
-            const int32_t* sk = ga.keys[cur];
-            const int32_t* sv = ga.vals[cur];
-            int64_t grid = (n64 + kThreads - 1) / kThreads;
-            grid = grid < 2048 ? grid : 2048;
-            k_cold_heads<<<(unsigned)grid, kThreads, 0, cudaStreamTailLaunch>>>(sk, n64, ga.rank);
-            exclusive_scan_i32_tail(ga.rank, ga.rank, n64, ga.tiles, status, ga.max_polls);
-            k_cold_assign<<<(unsigned)grid, kThreads, 0, cudaStreamTailLaunch>>>(
-                sk, sv, n64, ga.rank, slot0, staging_cap, ids, cold_rows, d_n_cold, status, ga.cap_ids);
-            if (cudaGetLastError() != cudaSuccess) set_status(status, HL_ECUDA);
-        }
-        return;
-    }
-    if (cta == 0 && threadIdx.x == 0) d_n_general[0] = 0;
-    const int n = (int)n64;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned lt = lanemask_lt();
-    const int cta_base = cta * kSmallPerCta;
-    const int warp_base = warp * (32 * kSmallItems);
-    int32_t key[kSmallItems];
-    uint32_t aux[kSmallItems];        // low 16 bits: where the pair's value sits in vals_in; high 16: rank in its warp
-#pragma unroll
-    for (int r = 0; r < kSmallItems; ++r) {
-        const int idx = cta_base + warp_base + r * 32 + lane;
-        key[r] = idx < n ? keys_in[idx] : 0x7fffffff;     // padding sorts behind every row id and stays there
-        aux[r] = (uint32_t)idx;
-    }
-    for (int p = 0; p < passes; ++p) {
-        const int shift = 8 * p;
-        for (int i = threadIdx.x; i < kSmallWarps * 256; i += kSmallThreads) cnt[i] = 0;
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kSmallItems; ++r) {
-            const uint32_t d = ((uint32_t)key[r] >> shift) & 255u;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            const uint32_t before = cnt[warp * 256 + d];
-            __syncwarp();
-            aux[r] = (aux[r] & 0xffffu) | ((before + __popc(peers & lt)) << 16);
-            if ((peers & lt) == 0) cnt[warp * 256 + d] = before + __popc(peers);
-            __syncwarp();
-        }
-        __syncthreads();
-        {   // thread d: prefix of digit d over this CTA's warps; publish the CTA's count
-            const int d = threadIdx.x;
-            uint32_t total = 0;
-#pragma unroll
-            for (int w = 0; w < kSmallWarps; ++w) {
-                const uint32_t c = cnt[w * 256 + d];
-                cnt[w * 256 + d] = total;
-                total += c;
-            }
-            cta_hist[d] = total;
-        }
-        cluster.sync();     // all counts published; all CTAs have taken the previous pass's pairs out of shared memory
-        {
-            const int d = threadIdx.x;
-            uint32_t before_me = 0, all_ctas = 0;
-#pragma unroll
-            for (int c = 0; c < CTAS; ++c) {
-                const uint32_t v = *cluster.map_shared_rank(&cta_hist[d], c);
-                if (c < cta) before_me += v;
-                all_ctas += v;
-            }
-            int whole;
-            const int smaller = block_scan_small((int)all_ctas, scan_smem, whole);     // pairs with a smaller digit
-            digit_base[d] = (uint32_t)smaller + before_me;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int r = 0; r < kSmallItems; ++r) {
-            const uint32_t d = ((uint32_t)key[r] >> shift) & 255u;
-            const uint32_t pos = digit_base[d] + cnt[warp * 256 + d] + (aux[r] >> 16);
-            const unsigned owner = pos / kSmallPerCta, off = pos % kSmallPerCta;
-            *cluster.map_shared_rank(&s_key[off], owner) = key[r];
-            *cluster.map_shared_rank(&s_val[off], owner) = (int32_t)(aux[r] & 0xffffu);
-        }
-        cluster.sync();     // every pair has arrived
-#pragma unroll
-        for (int r = 0; r < kSmallItems; ++r) {
-            const int idx = warp_base + r * 32 + lane;
-            key[r] = s_key[idx];
-            aux[r] = (uint32_t)s_val[idx];
-        }
-    }
-    // The sorted pairs are in the CTAs' shared memory (the last barrier above made them visible).  Thread t of CTA c
-    // ranks positions cta_base + [t * kSmallItems, (t + 1) * kSmallItems).
-    const int i0 = threadIdx.x * kSmallItems;
-    int32_t mine[kSmallItems + 1];           // mine[0] = the key before my first position
-    mine[0] = -1;
-    if (i0 > 0) mine[0] = s_key[i0 - 1];
-    else if (cta > 0) mine[0] = *cluster.map_shared_rank(&s_key[kSmallPerCta - 1], cta - 1);
-    int32_t where[kSmallItems];
-    int heads = 0;
-#pragma unroll
-    for (int u = 0; u < kSmallItems; ++u) {
-        const int i = cta_base + i0 + u;
-        mine[u + 1] = s_key[i0 + u];
-        where[u] = i < n ? vals_in[s_val[i0 + u]] : -1;          // the lookup's position in X's ids
-        if (i < n && (i == 0 || mine[u + 1] != mine[u])) ++heads;
-    }
-    int cta_total;
-    int rank = block_scan_small(heads, scan_smem, cta_total);    // heads before my first position, within the CTA
-    if (threadIdx.x == 0) cta_heads = cta_total;
-    cluster.sync();
-    int distinct = 0;
-#pragma unroll
-    for (int c = 0; c < CTAS; ++c) {
-        const int v = *cluster.map_shared_rank(&cta_heads, c);
-        if (c < cta) rank += v;
-        distinct += v;
-    }
-    if (cta == 0 && threadIdx.x == 0) {
-        int64_t dn = distinct;
-        if (dn > staging_cap) {
-            set_status(status, HL_ECAPACITY);
-            dn = staging_cap;
-        }
-        *d_n_cold = dn;
-    }
-#pragma unroll
-    for (int u = 0; u < kSmallItems; ++u) {
-        const int i = cta_base + i0 + u;
-        if (i < n) {
-            const bool head = i == 0 || mine[u + 1] != mine[u];
-            const int my_rank = head ? rank : rank - 1;
-            if (head) ++rank;
-            if (my_rank < staging_cap) {
-                if (head) cold_rows[my_rank] = mine[u + 1];
-                ids[where[u]] = (int32_t)(slot0 + my_rank);
-            } else {
-                ids[where[u]] = -1;     // no room to stage this row: the lookup is dropped, the status word says so
-            }
-        }
-    }
-    cluster.sync();     // no CTA leaves while another may still read its shared memory
 }
 
 // dst[(dst_row0 + i), :] = table[rows[i], :] (or the other way round); G lanes per row, UR rows in flight per
@@ -368,14 +192,7 @@ __global__ void __launch_bounds__(kThreads) k_cold_match(const int32_t* __restri
     n = n < 0 ? 0 : (n < n_max ? n : n_max);
     np = np < 0 ? 0 : (np < n_prev_max ? np : n_prev_max);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t g = rows[i];
-        int64_t lo = 0, hi = np;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (prev[mid] < g) lo = mid + 1;
-            else hi = mid;
-        }
-        src[i] = (lo < np && prev[lo] == g) ? (int32_t)lo : -1;
+        src[i] = position_in(prev, np, rows[i]);
     }
 }
 
@@ -580,13 +397,25 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
     return HL_OK;
 }
 
-int bits_for(int64_t max_value) {
-    int b = 1;
-    while ((int64_t(1) << b) <= max_value) ++b;
-    return b;
-}
-
 }  // namespace
+
+int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold, cudaStream_t stream,
+                  uint32_t* clear, int64_t n_clear) {
+    const Regions& r = ctx->r;
+    const ColdMarks marks = cold_marks(ctx);
+    const bool summary = marks.summary != nullptr;
+    const int64_t words = summary ? cold_summary_words(ctx->N) : cold_bitmap_words(ctx->N);
+    // words per thread: as in hl_fragment, one until there is a tile per multiprocessor
+    const bool many = words > (int64_t)kThreads * ctx_sms(ctx);
+    const unsigned grid = (unsigned)div_up(words, kThreads * (many ? 4 : 1));
+    const auto kernel = summary ? (many ? k_cold_rank<true, 4> : k_cold_rank<true, 1>)
+                                : (many ? k_cold_rank<false, 4> : k_cold_rank<false, 1>);
+    kernel<<<grid, kThreads, 0, stream>>>(marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.cold_n + 1, r.cold_chain,
+                                          r.status, wait_cfg(ctx).max_polls, clear, n_clear);
+    note_launches(1);
+    HL_LAUNCH_CHECK();
+    return HL_OK;
+}
 
 // the host table as the movers see it: `host_table` itself, or the per-table allocations installed by
 // hl_set_host_tables (then `host_table` only says that there is a table)
@@ -599,8 +428,8 @@ static TableMap table_map(const hl_ctx* ctx, const float* host_table) {
     return m;
 }
 
-// how the movers of this context are launched: inside a schedule (`width` = the context's setting) or alone on the
-// chip (`width` = 0: two CTAs per SM, the link's full rate)
+// how the movers of this context are launched: beside the kernels of other mini-batches (`width` = the context's setting),
+// or alone on the chip (`width` = 0: two CTAs per SM, the link's full rate)
 static MoveCfg move_cfg(const hl_ctx* ctx, int width) {
     MoveCfg c;
     c.sms = ctx_sms(ctx);
@@ -626,78 +455,28 @@ namespace {
 
 // Shared body of hl_gather_cold and hl_gather_cold_ahead.  Staging window: cache slots
 // [hot_cap + stage_row0, hot_cap + stage_row0 + stage_rows).
-// First half of the cold-row search: classify X's lookups, then the one-cluster kernel, which either finishes the
-// search or launches the general path behind itself; cold_n[1] says which (0, or the number of cold lookups).
+// First half of the cold-row search: classify X's lookups, rank the rows they mark, assign the slots.
 int32_t index_begin(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows,
                     int32_t* d_cold_rows, int64_t* d_n_cold, cudaStream_t stream) {
     Regions& r = ctx->r;
     if (ctx->max_nnz == 0) {
         HL_CUDA_TRY(cudaMemsetAsync(d_n_cold, 0, sizeof(int64_t), stream));
-        HL_CUDA_TRY(cudaMemsetAsync(r.cold_n, 0, 4 * sizeof(int32_t), stream));
         return HL_OK;
     }
     if (!non->ids) return HL_EINVAL;
-    HL_CUDA_TRY(cudaMemsetAsync(r.cold_n, 0, 4 * sizeof(int32_t), stream));
     const int grid = grid_for(ctx->max_nnz, kThreads, 4 * ctx_sms(ctx));
     k_cold_classify<<<grid, kThreads, 0, stream>>>(non->ids, non->offsets, d_n_non, ctx->max_batch, ctx->T * ctx->S,
-                                                   non->cap_ids, ctx->N, r.remap, r.cold_keys[0], r.cold_vals[0],
-                                                   r.cold_n, ctx->max_nnz, r.status);
-    note_launches(1);
-    HL_LAUNCH_CHECK();
-    const int key_bits = bits_for(ctx->N - 1);
-    GeneralArgs ga;
-    for (int i = 0; i < 2; ++i) {
-        ga.keys[i] = r.cold_keys[i];
-        ga.vals[i] = r.cold_vals[i];
-    }
-    ga.hist = r.cold_hist;
-    ga.rank = r.cold_rank;
-    ga.tiles = r.cold_tiles;
-    ga.cap_ids = non->cap_ids;
-    ga.key_bits = key_bits;
-    ga.max_polls = wait_cfg(ctx).max_polls;
-    // the widest cluster the device can place: 16 CTAs (a non-portable size) or 8; asked once per context
-    if (ctx->cold_cluster == 0) {
-        ctx->cold_cluster = 8;
-        cudaLaunchConfig_t probe = {};
-        probe.gridDim = dim3(16);
-        probe.blockDim = dim3(kSmallThreads);
-        cudaLaunchAttribute pa[1];
-        pa[0].id = cudaLaunchAttributeClusterDimension;
-        pa[0].val.clusterDim.x = 16;
-        pa[0].val.clusterDim.y = pa[0].val.clusterDim.z = 1;
-        probe.attrs = pa;
-        probe.numAttrs = 1;
-        int clusters = 0;
-        if (cudaFuncSetAttribute(k_cold_small<16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&clusters, k_cold_small<16>, &probe) == cudaSuccess && clusters >= 1)
-            ctx->cold_cluster = 16;
-        (void)cudaGetLastError();
-    }
-    const int ctas = ctx->cold_cluster;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(kSmallThreads);
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    HL_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctas == 16 ? k_cold_small<16> : k_cold_small<8>,
-                                   (const int32_t*)r.cold_keys[0], (const int32_t*)r.cold_vals[0],
-                                   (const int32_t*)r.cold_n, ctx->max_nnz, (key_bits + 7) / 8,
-                                   ctx->hot_cap + stage_row0, stage_rows, non->ids, d_cold_rows, d_n_cold,
-                                   r.cold_n + 1, r.status, ga));
-    note_launches(1);
+                                                   non->cap_ids, ctx->N, BitmapProbe{r.remap}, cold_marks(ctx), r.status);
+    const int32_t st = cold_rank(ctx, stage_rows, d_cold_rows, d_n_cold, stream);
+    if (st != HL_OK) return st;
+    k_cold_assign<<<grid, kThreads, 0, stream>>>(non->ids, non->offsets, d_n_non, ctx->max_batch, ctx->T * ctx->S,
+                                                 non->cap_ids, r.cold_ranked, ctx->hot_cap + stage_row0, stage_rows);
+    note_launches(2);
     HL_LAUNCH_CHECK();
     return HL_OK;
 }
 
-// Second half: the match against the previous mini-batch's cold rows.  (Whatever the search needed beyond its
-// one-cluster kernel was launched by that kernel and has run by the time anything queued here starts.)
+// Second half: the match against the previous mini-batch's cold rows.
 int32_t index_end(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold,
                   const int32_t* d_prev_rows, const int64_t* d_n_prev, int32_t* d_fwd_src, cudaStream_t stream) {
     if (ctx->max_nnz == 0) return HL_OK;
@@ -721,8 +500,8 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 0, stream);
         const int32_t st = launch_move_rows<false>(d_cache, ctx->hot_cap + stage_row0,
                                                    table_map(ctx, host_table), d_cold_rows, d_n_cold, stage_rows,
-                                                   ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas), r.status,
-                                                   stream);
+                                                   ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas),
+                                                   r.status, stream);
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 1, stream);
         return st;
     }
@@ -836,9 +615,9 @@ extern "C" int32_t hl_forward_cold(hl_ctx* ctx, float* d_cache, int64_t from_sta
     return HL_OK;
 }
 
-extern "C" int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,
-                                      const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table,
-                                      void* stream_) {
+static int32_t scatter_call(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,
+                            const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table,
+                            void* stream_) {
     if (!ctx || !d_cache || !d_cold_rows || !d_n_cold || !host_table) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
@@ -851,10 +630,17 @@ extern "C" int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t
     return st;
 }
 
+extern "C" int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,
+                                      const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table,
+                                      void* stream) {
+    return scatter_call(ctx, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold, host_table, stream);
+}
+
 extern "C" int32_t hl_scatter_cold(hl_ctx* ctx, const float* d_cache, const int32_t* d_cold_rows,
                                    const int64_t* d_n_cold, float* host_table, void* stream_) {
     if (!ctx) return HL_EINVAL;
-    return hl_scatter_cold_at(ctx, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold, host_table, stream_);
+    // (one mini-batch after the other: nothing runs beside this)
+    return scatter_call(ctx, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold, host_table, stream_);
 }
 
 extern "C" int32_t hl_flush_hot(hl_ctx* ctx, const float* d_cache, const int32_t* d_hot_rows, const int64_t* d_n_hot,

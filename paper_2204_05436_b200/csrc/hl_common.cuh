@@ -52,22 +52,20 @@ struct Regions {
     uint32_t* sel_gt;                  // [n_sel_tiles + 1]
     uint32_t* sel_eq;                  // [n_sel_tiles + 1]
     // fragment
-    uint8_t* frag_flags;               // [max_batch]
-    int32_t* frag_scan;                // [max_bags + 1]
-    int32_t* frag_tiles;               // [scan tiles + 1]
+    uint32_t* frag_words;              // [max_batch / 32 + 1] all-hit flags
+    unsigned long long* frag_chain;    // [frag_chain_words]
     // backward
     int32_t* bwd_keys[2];              // [max_nnz]
     int32_t* bwd_vals[2];              // [max_nnz]
-    uint32_t* bwd_hist;                // [256 * sort tiles]
+    uint32_t* bwd_hist[2];             // [256 * sort tiles]; the second one only for SortAside
     float* bwd_part;                   // [2 * n_chunks * D]
     int32_t* bwd_n;                    // [4] lookups in the micro-batch
     // cold
-    int32_t* cold_keys[2];
-    int32_t* cold_vals[2];
-    uint32_t* cold_hist;
-    int32_t* cold_rank;                // [max_nnz + 1]
-    int32_t* cold_tiles;               // [scan tiles + 1]
-    int32_t* cold_n;                   // [4] cold lookups
+    uint32_t* cold_bits;               // [cold_bitmap_words] one bit per row; zero between calls
+    uint32_t* cold_summary;            // [cold_summary_words] one bit per bitmap word; zero between calls
+    uint2* cold_ranked;                // [cold_bitmap_words] bits of the word, rank of its first row
+    unsigned long long* cold_chain;    // [cold_chain_words]; zero between calls
+    int32_t* cold_n;                   // [4]; [1] = hl_index_cold_verdict
 };
 
 }  // namespace hl
@@ -83,7 +81,6 @@ struct hl_ctx {
     int sms;                           // multiprocessors of `device` (queried at hl_create)
     int mover_ctas, scatter_ctas;      // working CTAs of the host-link movers inside a schedule (hl_set_mover_ctas)
     int fwd_ctas, bwd_ctas;            // CTAs per multiprocessor of the forward / backward-sum kernel (0 = default)
-    int cold_cluster;                  // CTAs of the one-cluster cold-row search (0 = not asked yet; 8 or 16)
     int test_poll_limit;               // > 0: poll limit of the bounded device waits (hl_test_bounded_waits)
     int64_t test_stall_tile;           // with it: the tile / mover stage that never delivers (-1: none)
     int64_t* h_table_base;             // host copy [T+1]
@@ -124,8 +121,8 @@ struct hl_wide {
     int32_t* sort_keys[2];                   // [max(counter_slots, max_nnz)]
     int32_t* sort_vals[2];
     uint32_t* sort_hist;
-    uint8_t* frag_flags;                     // [max_batch]
-    int32_t *frag_scan, *frag_tiles;
+    uint32_t* frag_words;                    // [max_batch / 32 + 1]
+    unsigned long long* frag_chain;
     int32_t *cold_tab, *cold_idx, *cold_pos; // [max_nnz] cold lookups: table, index, position in X
     int32_t *cold_rank, *cold_tiles, *cold_n;
 };
@@ -251,6 +248,62 @@ struct BitmapProbe {
     __device__ __forceinline__ bool hit(int64_t g) const { return remap_hit(remap, g); }
 };
 
+// ---- the cold-row bitmap --------------------------------------------------------------------------------------
+// Above this many rows the bitmap is read through a summary.  (16 M rows: 2 MB of bitmap, a few microseconds to read.)
+constexpr int64_t kColdDirectRows = int64_t(1) << 24;
+constexpr int64_t cold_bitmap_words(int64_t N) { return (N + 31) / 32; }
+constexpr int64_t cold_summary_words(int64_t N) { return (cold_bitmap_words(N) + 31) / 32; }
+// ticket, tally and one status word per tile of k_cold_rank (at least 256 words per tile)
+constexpr int64_t cold_chain_words(int64_t N) {
+    return 3 + (N > kColdDirectRows ? cold_summary_words(N) : cold_bitmap_words(N)) / 256;
+}
+// tally, ticket and one status word per tile of k_frag_place (at least 256 bags per tile)
+constexpr int64_t frag_chain_words(int64_t max_bags) { return 3 + max_bags / 256 + 1; }
+
+struct ColdMarks {
+    uint32_t* bits;
+    uint32_t* summary;                 // nullptr: no summary is kept
+    uint2* ranked;
+};
+inline ColdMarks cold_marks(const hl_ctx* ctx) {
+    return {ctx->r.cold_bits, ctx->N > kColdDirectRows ? ctx->r.cold_summary : nullptr, ctx->r.cold_ranked};
+}
+
+// A lookup of X that addresses row g (inside the model): its cache slot if the row is popular; otherwise the row is
+// marked in the bitmap and the result is -2 - g.  (A row that is marked already, as popular cold rows are, costs a load.)
+__device__ __forceinline__ int32_t classify_cold(const BitmapProbe& remap, int64_t g, const ColdMarks& marks) {
+    const int32_t slot = remap.slot(g);
+    if (slot >= 0) return slot;
+    const int64_t word = g >> 5;
+    const uint32_t bit = 1u << (g & 31);
+    if (!(marks.bits[word] & bit)) {
+        const uint32_t old = atomicOr(&marks.bits[word], bit);
+        if (old == 0u && marks.summary) atomicOr(&marks.summary[word >> 5], 1u << (word & 31));
+    }
+    return (int32_t)(-2 - g);
+}
+
+// The slot of such a lookup once the marked rows are ranked: slot0 + rank, or -1 if there is no room to stage the row
+// (the lookup is dropped; k_cold_rank has set the status word).
+__device__ __forceinline__ int32_t cold_slot(const uint2* __restrict__ ranked, int32_t id, int64_t slot0,
+                                             int64_t staging_cap) {
+    const int64_t g = -2 - (int64_t)id;
+    const uint2 w = ranked[g >> 5];
+    const int64_t rank = (int64_t)w.y + __popc(w.x & ((1u << (g & 31)) - 1u));
+    return rank < staging_cap ? (int32_t)(slot0 + rank) : -1;
+}
+
+// Position of g in the ascending list rows[0 .. n), or -1.
+__device__ __forceinline__ int32_t position_in(const int32_t* __restrict__ rows, int64_t n, int32_t g) {
+    int64_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (rows[mid] < g) lo = mid + 1;
+        else hi = mid;
+    }
+    return (lo < n && rows[lo] == g) ? (int32_t)lo : -1;
+}
+
 __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
@@ -273,6 +326,74 @@ inline WaitCfg wait_cfg(const hl_ctx* ctx) {
     return w;
 }
 
+// ---- chained tiles --------------------------------------------------------------------------------------------
+// Sum over the tiles before `tile` of what each of them adds up to (62 bits), in one kernel: a tile publishes its own sum
+// (AGGREGATE), all threads of its CTA then look at the tiles before it, one each, until somebody sees one that already
+// knows its inclusive prefix (PREFIX), and the tile publishes its prefix.  One round of loads covers NT tiles, so a few
+// hundred tiles cost one or two round trips to the L2, where one warp walks them 32 a step (placing 106 thousand bags:
+// 11.7 us with a one-warp walk over 416 tiles, 8.2 us with this over 104).  A tile is the CTA's block index (CTAs are
+// dispatched in that order, so the tiles before have started), and publishing never waits; every poll is bounded all the
+// same, and one that runs out records HL_ETIMEOUT and carries on with what it has.  words[tile]: zero on entry.  Both calls are made by all NT threads; chain_before's result is the same in all.
+constexpr unsigned long long kChainAgg = 1ull << 62, kChainPrefix = 1ull << 63, kChainSum = kChainAgg - 1ull;
+
+__device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+__device__ __forceinline__ void chain_publish(unsigned long long* words, int tile, unsigned long long total) {
+    if (threadIdx.x == 0) st_relaxed64(&words[tile], (tile == 0 ? kChainPrefix : kChainAgg) | total);
+}
+
+template <int NT>
+__device__ __forceinline__ unsigned long long chain_before(unsigned long long* words, int tile, unsigned long long total,
+                                                           bool publish, int max_polls, int32_t* status) {
+    constexpr int NW = NT / 32;
+    __shared__ unsigned long long s_sum[NW];
+    __shared__ bool s_ends[NW];                      // a prefix among the warp's tiles
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long before = 0;
+    for (int t0 = tile - 1; t0 >= 0; t0 -= NT) {
+        const int t = t0 - (int)threadIdx.x;
+        unsigned long long w = kChainPrefix;         // before tile 0: an empty prefix
+        if (t >= 0) {
+            int polls = 0;
+            while (((w = ld_relaxed64(&words[t])) & (kChainAgg | kChainPrefix)) == 0) {
+                if (++polls > max_polls) {
+                    set_status(status, HL_ETIMEOUT);
+                    w = kChainPrefix;
+                    break;
+                }
+                __nanosleep(20);
+            }
+        }
+        const unsigned with_prefix = __ballot_sync(0xffffffffu, (w & kChainPrefix) != 0);
+        const int stop = with_prefix ? __ffs(with_prefix) - 1 : 31;
+        unsigned long long val = lane <= stop ? w & kChainSum : 0;
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) val += __shfl_xor_sync(0xffffffffu, val, d);
+        if (lane == 0) {
+            s_sum[warp] = val;
+            s_ends[warp] = with_prefix != 0;
+        }
+        __syncthreads();
+        bool ends = false;
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+            if (!ends) before += s_sum[k];
+            ends = ends || s_ends[k];
+        }
+        __syncthreads();
+        if (ends) break;
+    }
+    if (threadIdx.x == 0 && publish && tile > 0) st_relaxed64(&words[tile], kChainPrefix | ((before + total) & kChainSum));
+    return before;
+}
+
 // ---- primitives implemented in hl_prims.cu -----------------------------------------------------------------
 // Exclusive scan of in[0 .. n) into out[0 .. n] (out[n] = total); n = *d_n if d_n != nullptr (clamped to
 // n_max), else n_max.  in may alias out.  tiles: scratch of scan_tile_words(n_max) ints.  A chain poll that
@@ -284,14 +405,12 @@ int32_t exclusive_scan_i32(const int32_t* in, int32_t* out, const int32_t* d_n, 
 // n = *d_n (clamped to n_max).  Returns in *out_keys / *out_vals which of the two buffers holds the result.
 int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n, int64_t n_max, int key_bits,
                          uint32_t* hist, int32_t* status, int32_t** out_keys, int32_t** out_vals,
-                         cudaStream_t stream, WaitCfg w = WaitCfg());
+                         cudaStream_t stream, WaitCfg w = WaitCfg(), bool counted = false);
 
-// The same from the device (one thread calls; the launches run after the calling grid, in order: see hl_prims.cu).
-// radix_sort_pairs_tail returns which buffer (0 / 1) will hold the result.
-__device__ int radix_sort_pairs_tail(int32_t* keys0, int32_t* keys1, int32_t* vals0, int32_t* vals1, int64_t n,
-                                     int key_bits, uint32_t* hist, int32_t* status, int max_polls);
-__device__ void exclusive_scan_i32_tail(const int32_t* in, int32_t* out, int64_t n, int32_t* tiles, int32_t* status,
-                                        int max_polls);
+// Words at the start of `hist` that must be zero before the sort's digits are counted; 0 if the sort that will be used
+// counts none.  A caller that clears them and then counts the keys' digits itself (hist[pass * 256 + digit]) passes
+// counted = true.
+int64_t sort_clear_words(int64_t n_max, int key_bits, WaitCfg w);
 
 // 32-bit words of histogram scratch radix_sort_pairs needs for at most max_nnz pairs.
 constexpr int64_t sort_hist_words(int64_t max_nnz) {
@@ -313,6 +432,38 @@ inline int32_t* span_count_of(const hl_ctx* ctx) {
 
 // ints of scratch exclusive_scan_i32 needs for at most n_max elements (64-bit ticket + status words).
 constexpr int64_t scan_tile_words(int64_t n_max) { return 2 * ((n_max > 0 ? n_max : 1) / kScanTile + 3); }
+
+// Ranks the rows marked in the cold-row bitmap (hl_cold.cu): d_cold_rows, *d_n_cold, cold_ranked.  Also clears `clear`
+// [n_clear words, a multiple of 4; 16-byte aligned], for the kernels that follow.
+int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold, cudaStream_t stream,
+                  uint32_t* clear = nullptr, int64_t n_clear = 0);
+
+// hl_embbag_bwd_prepare2 / _merged on what fragment_and_mark and cold_rank left behind (hl_embbag.cu): X's cold lookups
+// get their slots, the cold rows are matched against the previous ones, and the pairs are sorted (aside: may be null).  The
+// sort's scratch, backward_sort_clear_words words of bwd_hist, is zero already.
+int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge);
+
+// The sort on a stream of its own, behind the pairs (event pairs_ready), with one of two sets of scratch (which): the
+// pairs of the next mini-batch, written with the other set, need not wait for it.
+struct SortAside {
+    cudaStream_t stream;
+    cudaEvent_t pairs_ready;
+    int which;
+};
+int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, hl_ubatch* non,
+                           const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows, const int32_t* d_cold_rows,
+                           const int64_t* d_n_cold, const int32_t* d_prev_rows, const int64_t* d_n_prev,
+                           int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
+                           bool merge, cudaStream_t stream, const SortAside* aside);
+
+// hl_embbag_fwd and hl_forward_cold in one launch (the bags read no staged row).
+int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples, float* d_out,
+                             int64_t from_stage_row0, int64_t to_stage_row0, int64_t stage_rows, const int32_t* d_fwd_src,
+                             const int64_t* d_n_cold, cudaStream_t stream);
+
+// hl_fragment with X's lookups classified on the way (hl_fragment.cu): non->ids = cache slots, or -2 - g for a cold row.
+int32_t fragment_and_mark(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense, int32_t* d_perm,
+                          int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non, float* d_dense_out, cudaStream_t stream);
 
 // Selection of the rows with the k largest counts (implemented in hl_profile.cu; see there).
 int32_t select_rows_by_count(const uint32_t* counts, int64_t n, SelectState* sel, uint32_t* sel_gt, uint32_t* sel_eq,

@@ -85,13 +85,38 @@ __device__ __forceinline__ void pool_long_bag(const float4* __restrict__ rows, c
 // row copies: the UB rows are loaded at once (UB independent 128-bit loads per lane), and the offsets and ids of
 // the NEXT trip are requested before those rows are consumed, so that the offsets -> id -> row chain of one trip
 // hides behind the rows of another.  Longer bags go through pool_long_bag one after the other.
-template <int G, int NV, int UB>
+// FORWARD: the launch also copies the staged rows that this mini-batch shares with the one before (ForwardRows), which no
+// bag of this launch reads.
+struct ForwardRows {
+    float* cache;
+    int64_t from_row0, to_row0;        // cache[to_row0 + i, :] = cache[from_row0 + src[i], :] where src[i] >= 0
+    const int32_t* src;
+    const int64_t* d_n;
+    int64_t n_max;
+};
+
+template <int G, int NV, int UB, bool FORWARD>
 __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const float* __restrict__ cache,
                                                          const int32_t* __restrict__ ids,
                                                          const int32_t* __restrict__ offsets,
                                                          const int32_t* __restrict__ d_n_samples, int max_batch,
                                                          int bags_per_sample_all /* T*S */, int D4, int64_t n_slots,
-                                                         float* __restrict__ out, int32_t* status) {
+                                                         float* __restrict__ out, int32_t* status, ForwardRows fr) {
+    if (FORWARD) {
+        int64_t n = *fr.d_n;
+        n = n < 0 ? 0 : (n < fr.n_max ? n : fr.n_max);
+        const int lane = threadIdx.x & 31;
+        float4* c4 = reinterpret_cast<float4*>(fr.cache);
+        for (int64_t i0 = ((int64_t)blockIdx.x * kThreads + threadIdx.x) - lane; i0 < n;
+             i0 += (int64_t)gridDim.x * kThreads) {
+            const int32_t mine = i0 + lane < n ? fr.src[i0 + lane] : -1;
+            for (unsigned m = __ballot_sync(0xffffffffu, mine >= 0 && mine < fr.n_max); m; m &= m - 1) {
+                const int k = __ffs((int)m) - 1;
+                const int64_t from = fr.from_row0 + __shfl_sync(0xffffffffu, mine, k);
+                for (int c = lane; c < D4; c += 32) c4[(fr.to_row0 + i0 + k) * D4 + c] = c4[from * D4 + c];
+            }
+        }
+    }
     const int64_t n_bags = (int64_t)clamp_samples(d_n_samples, max_batch) * bags_per_sample_all;
     const int sub = threadIdx.x % G;
     const float4* __restrict__ rows = reinterpret_cast<const float4*>(cache);
@@ -167,45 +192,97 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const 
 }
 
 // ---- backward -----------------------------------------------------------------------------------------------
-// (slot, bag) pair per lookup; a negative id becomes the sentinel n_slots, which sorts last and is ignored.
-template <int GROUP>
-__global__ void __launch_bounds__(kThreads) k_bwd_pairs(const int32_t* __restrict__ ids,
-                                                        const int32_t* __restrict__ offsets,
-                                                        const int32_t* __restrict__ d_n_samples, int max_batch,
-                                                        int bags_per_sample_all, int64_t n_slots, int64_t max_nnz,
-                                                        int32_t* __restrict__ keys, int32_t* __restrict__ vals,
-                                                        int32_t* __restrict__ d_n_lookups,
-                                                        const int32_t* __restrict__ d_pos0, int32_t key_bias,
-                                                        int32_t sentinel, int32_t* __restrict__ d_total,
-                                                        int32_t* status,
-                                                        const int32_t* __restrict__ d_bag_bias_samples = nullptr) {
-    // pairs go to positions pos0 + j (pos0 = *d_pos0 or 0) with key = slot + key_bias and value = bag (+ the bags of
-    // *d_bag_bias_samples inputs, if given); *d_n_lookups = this micro-batch's lookups, *d_total (if given) = pos0 +
-    // that
-    const int64_t pos0 = d_pos0 ? d_pos0[0] : 0;
-    const int64_t bag_bias =
-        d_bag_bias_samples ? (int64_t)clamp_samples(d_bag_bias_samples, max_batch) * bags_per_sample_all : 0;
-    const int64_t n_bags = (int64_t)clamp_samples(d_n_samples, max_batch) * bags_per_sample_all;
-    const int sub = threadIdx.x % GROUP;
-    const int64_t group = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / GROUP;
-    const int64_t n_groups = (int64_t)gridDim.x * kThreads / GROUP;
-    if (group == 0 && sub == 0) {
-        int32_t L = offsets[n_bags];
-        if (pos0 + L > max_nnz) {
-            set_status(status, HL_ECAPACITY);
-            L = (int32_t)(max_nnz - pos0);
-        }
-        d_n_lookups[0] = L;
-        if (d_total) d_total[0] = (int32_t)(pos0 + L);
+// One micro-batch's lookups as (slot, bag) pairs: keys are slot + key_bias, a skipped lookup (negative id) gets the
+// sentinel slot n_slots, which sorts behind all others and is ignored.
+struct PairSide {
+    int32_t* ids;
+    const int32_t* offsets;
+    const int32_t* d_n_samples;
+    int32_t key_bias;
+};
+
+struct PairArgs {
+    PairSide side[2];                  // the second one's pairs follow the first one's
+    int sides;
+    int bags_follow;                   // the second side's bags are numbered behind the first one's
+    int max_batch, bags_per_sample_all;
+    int64_t n_slots, max_nnz;
+    int32_t* keys;
+    int32_t* vals;
+    int32_t* d_n_lookups;              // [0], [1]: lookups of the sides; [2]: their sum (two sides only)
+    int32_t* status;
+    // ASSIGN: the second side's ids of -2 - g are cold rows, ranked by now: they become slots here (and in its ids)
+    const uint2* ranked;
+    int64_t slot0, stage_rows;
+    // ... and the cold rows are looked up in the previous mini-batch's (ascending; nullptr: there is none)
+    const int32_t* cold_rows;
+    const int64_t* d_n_cold;
+    const int32_t* prev_rows;
+    const int64_t* d_n_prev;
+    int64_t n_prev_max;
+    int32_t* fwd_src;
+    // HIST: digit counts of the sort that follows, [passes][256], zero on entry
+    uint32_t* ghist;
+    int passes;
+};
+
+template <int GROUP, bool ASSIGN, bool HIST>
+__global__ void __launch_bounds__(kThreads) k_bwd_pairs(PairArgs a) {
+    __shared__ uint32_t h[HIST ? 4 : 1][256];
+    if (HIST) {
+        for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&h[0][0])[i] = 0;
+        __syncthreads();
     }
-    for (int64_t bag = group; bag < n_bags; bag += n_groups) {
-        const int32_t lo = offsets[bag], hi = offsets[bag + 1];
-        for (int32_t j = lo + sub; j < hi; j += GROUP) {
-            if (pos0 + j >= max_nnz) break;
-            const int32_t id = ids[j];
-            if (id >= n_slots) set_status(status, HL_EBOUNDS);
-            keys[pos0 + j] = (id < 0 || id >= n_slots) ? sentinel : id + key_bias;
-            vals[pos0 + j] = (int32_t)(bag + bag_bias);
+    const int64_t bags0 = (int64_t)clamp_samples(a.side[0].d_n_samples, a.max_batch) * a.bags_per_sample_all;
+    const int64_t bags1 =
+        a.sides > 1 ? (int64_t)clamp_samples(a.side[1].d_n_samples, a.max_batch) * a.bags_per_sample_all : 0;
+    const int64_t L0 = a.side[0].offsets[bags0];
+    const int64_t thread = (int64_t)blockIdx.x * kThreads + threadIdx.x, n_threads = (int64_t)gridDim.x * kThreads;
+    if (thread == 0) {
+        int64_t L1 = a.sides > 1 ? a.side[1].offsets[bags1] : 0, first = L0;
+        if (L0 + L1 > a.max_nnz) {
+            set_status(a.status, HL_ECAPACITY);
+            if (first > a.max_nnz) first = a.max_nnz;
+            if (L1 > a.max_nnz - first) L1 = a.max_nnz - first;
+        }
+        a.d_n_lookups[0] = (int32_t)first;
+        if (a.sides > 1) {
+            a.d_n_lookups[1] = (int32_t)L1;
+            a.d_n_lookups[2] = (int32_t)(first + L1);
+        }
+    }
+    for (int64_t all = thread / GROUP; all < bags0 + bags1; all += n_threads / GROUP) {
+        const bool second = all >= bags0;
+        const PairSide& s = a.side[second ? 1 : 0];
+        const int64_t bag = second ? all - bags0 : all, pos0 = second ? L0 : 0;
+        const int32_t bag_value = (int32_t)(a.bags_follow ? all : bag);
+        const int32_t lo = s.offsets[bag], hi = s.offsets[bag + 1];
+        for (int32_t j = lo + (int)(thread % GROUP); j < hi; j += GROUP) {
+            if (pos0 + j >= a.max_nnz) break;
+            int32_t id = s.ids[j];
+            if (ASSIGN && id <= -2 && second) {
+                id = cold_slot(a.ranked, id, a.slot0, a.stage_rows);
+                s.ids[j] = id;
+            }
+            if (id >= a.n_slots) set_status(a.status, HL_EBOUNDS);
+            const int32_t key = ((id < 0 || id >= a.n_slots) ? (int32_t)a.n_slots : id) + s.key_bias;
+            a.keys[pos0 + j] = key;
+            a.vals[pos0 + j] = bag_value;
+            if (HIST)
+                for (int p = 0; p < a.passes; ++p) atomicAdd(&h[p][((uint32_t)key >> (8 * p)) & 255u], 1u);
+        }
+    }
+    if (ASSIGN && a.prev_rows != nullptr) {
+        int64_t n = *a.d_n_cold, np = *a.d_n_prev;
+        n = n < 0 ? 0 : (n < a.stage_rows ? n : a.stage_rows);
+        np = np < 0 ? 0 : (np < a.n_prev_max ? np : a.n_prev_max);
+        for (int64_t i = thread; i < n; i += n_threads) a.fwd_src[i] = position_in(a.prev_rows, np, a.cold_rows[i]);
+    }
+    if (HIST) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < a.passes * 256; i += kThreads) {
+            const uint32_t c = (&h[0][0])[i];
+            if (c) atomicAdd(&a.ghist[i], c);
         }
     }
 }
@@ -626,14 +703,14 @@ __global__ void __launch_bounds__(kThreads) k_bwd_spans(float* __restrict__ cach
 
 template <int G, int NV>
 int32_t launch_fwd(hl_ctx* ctx, const float* cache, const hl_ubatch* ub, const int32_t* d_n, float* out,
-                   cudaStream_t stream) {
+                   const ForwardRows* fr, cudaStream_t stream) {
     constexpr int UB = NV >= 4 ? 1 : (NV >= 2 ? 2 : 4);
     const int64_t bags_per_trip = (int64_t)(kThreads / G) * UB;
     const int grid = grid_for(ctx->max_bags, (int)bags_per_trip, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
     timer_mark(ctx, HL_TIMER_FWD, 0, stream);
-    k_embbag_fwd<G, NV, UB><<<grid, kThreads, 0, stream>>>(cache, ub->ids, ub->offsets, d_n, ctx->max_batch,
-                                                          ctx->T * ctx->S, ctx->D / 4,
-                                                          ctx->hot_cap + ctx->staging_cap, out, ctx->r.status);
+    const auto kernel = fr ? k_embbag_fwd<G, NV, UB, true> : k_embbag_fwd<G, NV, UB, false>;
+    kernel<<<grid, kThreads, 0, stream>>>(cache, ub->ids, ub->offsets, d_n, ctx->max_batch, ctx->T * ctx->S, ctx->D / 4,
+                                          ctx->hot_cap + ctx->staging_cap, out, ctx->r.status, fr ? *fr : ForwardRows{});
     timer_mark(ctx, HL_TIMER_FWD, 1, stream);
     note_launches(1);
     HL_LAUNCH_CHECK();
@@ -690,48 +767,104 @@ using namespace hl;
         return HL_EINVAL;                                \
     } while (0)
 
-extern "C" int32_t hl_embbag_fwd(hl_ctx* ctx, const float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples,
-                                 float* d_out, void* stream_) {
+namespace hl {
+namespace {
+
+int32_t fwd_call(hl_ctx* ctx, const float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples, float* d_out,
+                 const ForwardRows* fr, cudaStream_t stream) {
     if (!ctx || !d_cache || !ub || !ub->offsets || !d_n_samples || !d_out) return HL_EINVAL;
     if (ctx->max_nnz > 0 && !ub->ids) return HL_EINVAL;
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-#define HL_FWD(G, NV) launch_fwd<G, NV>(ctx, d_cache, ub, d_n_samples, d_out, stream)
+#define HL_FWD(G, NV) launch_fwd<G, NV>(ctx, d_cache, ub, d_n_samples, d_out, fr, stream)
     HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_FWD);
 #undef HL_FWD
+}
+
+}  // namespace
+
+int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples, float* d_out,
+                             int64_t from_stage_row0, int64_t to_stage_row0, int64_t stage_rows, const int32_t* d_fwd_src,
+                             const int64_t* d_n_cold, cudaStream_t stream) {
+    const ForwardRows fr{d_cache, ctx->hot_cap + from_stage_row0, ctx->hot_cap + to_stage_row0, d_fwd_src, d_n_cold,
+                         stage_rows};
+    return fwd_call(ctx, d_cache, ub, d_n_samples, d_out, &fr, stream);
+}
+
+}  // namespace hl
+
+extern "C" int32_t hl_embbag_fwd(hl_ctx* ctx, const float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples,
+                                 float* d_out, void* stream) {
+    return fwd_call(ctx, d_cache, ub, d_n_samples, d_out, nullptr, static_cast<cudaStream_t>(stream));
 }
 
 namespace hl {
 namespace {
 
-// (slot, bag) pairs of the micro-batch, sorted by slot (stable).  The result lands in out_keys / out_vals: either
-// the caller's arrays (which then serve as one half of the sort's ping-pong buffers) or, if they are null, whichever
-// scratch buffer the last pass wrote.
-int32_t sort_lookups(hl_ctx* ctx, const hl_ubatch* ub, const int32_t* d_n_samples, int32_t* caller_keys,
-                     int32_t* caller_vals, int32_t* d_n_lookups, int32_t** out_keys, int32_t** out_vals,
-                     cudaStream_t stream) {
+// The pairs described by `a` (its buffers and scratch are filled in here), sorted by key (stable).  The result lands in
+// out_keys / out_vals: either the caller's arrays (which then serve as one half of the sort's ping-pong buffers) or, if
+// they are null, whichever scratch buffer the last pass wrote.  cleared: the sort's scratch (sort_clear_words words of
+// bwd_hist) is zero already.  aside: see SortAside.
+int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bool cleared, int32_t* caller_keys,
+                       int32_t* caller_vals, int32_t* d_n_lookups, int32_t** out_keys, int32_t** out_vals,
+                       cudaStream_t stream, const SortAside* aside = nullptr) {
     Regions& r = ctx->r;
-    const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
-    const int key_bits = bits_for(n_slots);
-    const int passes = (key_bits + 7) / 8;
-    int32_t* keys[2] = {r.bwd_keys[0], r.bwd_keys[1]};
-    int32_t* vals[2] = {r.bwd_vals[0], r.bwd_vals[1]};
+    const int key_bits = bits_for(max_key), passes = (key_bits + 7) / 8;
+    const int which = aside ? aside->which : 0;          // (with caller arrays, one of the two scratch buffers is free)
+    uint32_t* sort_scratch = r.bwd_hist[which];
+    int32_t* keys[2] = {r.bwd_keys[which], r.bwd_keys[which ^ 1]};
+    int32_t* vals[2] = {r.bwd_vals[which], r.bwd_vals[which ^ 1]};
     if (caller_keys) {   // make the buffer the last pass writes the caller's
+        if ((passes & 1) == 0) {
+            keys[1] = keys[0];
+            vals[1] = vals[0];
+        }
         keys[passes & 1] = caller_keys;
         vals[passes & 1] = caller_vals;
     }
-    const bool short_bags = ctx->max_nnz <= 4 * ctx->max_bags;
-    if (short_bags)
-        k_bwd_pairs<1><<<grid_for(ctx->max_bags, kThreads, 4 * ctx_sms(ctx)), kThreads, 0, stream>>>(
-            ub->ids, ub->offsets, d_n_samples, ctx->max_batch, ctx->T * ctx->S, n_slots, ctx->max_nnz, keys[0], vals[0],
-            d_n_lookups, nullptr, 0, (int32_t)n_slots, nullptr, r.status);
-    else
-        k_bwd_pairs<32><<<grid_for(ctx->max_bags, kThreads / 32, 8 * ctx_sms(ctx)), kThreads, 0, stream>>>(
-            ub->ids, ub->offsets, d_n_samples, ctx->max_batch, ctx->T * ctx->S, n_slots, ctx->max_nnz, keys[0], vals[0],
-            d_n_lookups, nullptr, 0, (int32_t)n_slots, nullptr, r.status);
+    a.max_batch = ctx->max_batch;
+    a.bags_per_sample_all = ctx->T * ctx->S;
+    a.n_slots = ctx->hot_cap + ctx->staging_cap;
+    a.max_nnz = ctx->max_nnz;
+    a.keys = keys[0];
+    a.vals = vals[0];
+    a.d_n_lookups = d_n_lookups;
+    a.status = r.status;
+    a.ghist = sort_scratch;
+    a.passes = passes;
+    // the tile sort wants its digit counts, which cost less here than in a sweep of their own
+    const int64_t clear_words = sort_clear_words(ctx->max_nnz, key_bits, wait_cfg(ctx));
+    const bool hist = clear_words > 0;
+    if (hist && !cleared) HL_CUDA_TRY(cudaMemsetAsync(sort_scratch, 0, sizeof(uint32_t) * clear_words, stream));
+    // lanes per bag: by the most lookups a bag has on average
+    const int lanes = ctx->max_nnz <= 4 * ctx->max_bags ? 1 : (ctx->max_nnz <= 16 * ctx->max_bags ? 8 : 32);
+    const int grid = grid_for(ctx->max_bags, kThreads / lanes, (lanes == 1 ? 4 : 8) * ctx_sms(ctx));
+    const auto pick = [](bool as, bool hi, auto g) {
+        constexpr int G = decltype(g)::value;
+        return as ? (hi ? k_bwd_pairs<G, true, true> : k_bwd_pairs<G, true, false>)
+                  : (hi ? k_bwd_pairs<G, false, true> : k_bwd_pairs<G, false, false>);
+    };
+    const auto kernel = lanes == 1   ? pick(assign, hist, std::integral_constant<int, 1>())
+                        : lanes == 8 ? pick(assign, hist, std::integral_constant<int, 8>())
+                                     : pick(assign, hist, std::integral_constant<int, 32>());
+    kernel<<<grid, kThreads, 0, stream>>>(a);
     note_launches(1);
     HL_LAUNCH_CHECK();
-    return radix_sort_pairs(keys, vals, d_n_lookups, ctx->max_nnz, key_bits, r.bwd_hist, r.status, out_keys, out_vals,
-                            stream, wait_cfg(ctx));
+    if (aside) {
+        HL_CUDA_TRY(cudaEventRecord(aside->pairs_ready, stream));
+        HL_CUDA_TRY(cudaStreamWaitEvent(aside->stream, aside->pairs_ready, 0));
+        stream = aside->stream;
+    }
+    return radix_sort_pairs(keys, vals, d_n_lookups + (a.sides > 1 ? 2 : 0), ctx->max_nnz, key_bits, sort_scratch, r.status,
+                            out_keys, out_vals, stream, wait_cfg(ctx), hist);
+}
+
+int32_t sort_lookups(hl_ctx* ctx, const hl_ubatch* ub, const int32_t* d_n_samples, int32_t* caller_keys,
+                     int32_t* caller_vals, int32_t* d_n_lookups, int32_t** out_keys, int32_t** out_vals,
+                     cudaStream_t stream) {
+    PairArgs a{};
+    a.sides = 1;
+    a.side[0] = {ub->ids, ub->offsets, d_n_samples, 0};
+    return pairs_and_sort(ctx, a, ctx->hot_cap + ctx->staging_cap, false, false, caller_keys, caller_vals, d_n_lookups,
+                          out_keys, out_vals, stream);
 }
 
 }  // namespace
@@ -765,68 +898,75 @@ extern "C" int32_t hl_embbag_bwd_prepare(hl_ctx* ctx, const hl_ubatch* ub, const
     return sort_lookups(ctx, ub, d_n_samples, d_sorted_slots, d_sorted_bags, d_n_lookups, &keys, &vals, stream);
 }
 
-static int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, const hl_ubatch* non,
-                            const int32_t* d_n_non, int32_t* d_sorted_slots, int32_t* d_sorted_bags,
-                            int32_t* d_n_lookups, bool merge, void* stream_) {
-    // merge = false: X's keys are offset by the number of slots + 1, so that the sorted list is O's pairs (skipped
-    // lookups of O, key n_slots, last among them), then X's (its skipped lookups, key 2 * n_slots + 1, at the very end);
-    // merge = true: one key space, and X's bags are numbered behind O's: the lookups of a row from both
-    // micro-batches form one run, over one gradient array [bags of O; bags of X]
+namespace hl {
+namespace {
+
+// merge = false: X's keys are offset by the number of slots + 1, so that the sorted list is O's pairs (skipped lookups of
+// O, key n_slots, last among them), then X's (its skipped lookups, key 2 * n_slots + 1, at the very end);
+// merge = true: one key space, and X's bags are numbered behind O's: the lookups of a row from both micro-batches form one
+// run, over one gradient array [bags of O; bags of X]
+int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, const hl_ubatch* non,
+                     const int32_t* d_n_non, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
+                     bool merge, PairArgs a, bool assign, bool cleared, cudaStream_t stream,
+                     const SortAside* aside = nullptr) {
     if (!ctx || !pop || !non || !pop->offsets || !non->offsets || !d_n_pop || !d_n_non || !d_n_lookups)
         return HL_EINVAL;
-    cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     if (ctx->max_nnz == 0) {
         HL_CUDA_TRY(cudaMemsetAsync(d_n_lookups, 0, 4 * sizeof(int32_t), stream));
         return HL_OK;
     }
     if (!pop->ids || !non->ids || !d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
-    Regions& r = ctx->r;
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     if (2 * n_slots + 2 >= (int64_t(1) << 31)) return HL_EINVAL;
-    const int key_bits = bits_for(merge ? n_slots : 2 * n_slots + 1);
-    const int passes = (key_bits + 7) / 8;
-    int32_t* keys[2] = {r.bwd_keys[0], r.bwd_keys[1]};
-    int32_t* vals[2] = {r.bwd_vals[0], r.bwd_vals[1]};
-    keys[passes & 1] = d_sorted_slots;
-    vals[passes & 1] = d_sorted_bags;
-    const bool short_bags = ctx->max_nnz <= 4 * ctx->max_bags;
-    const int per_block = short_bags ? kThreads : kThreads / 32;
-    const int grid = grid_for(ctx->max_bags, per_block, (short_bags ? 4 : 8) * ctx_sms(ctx));
-    const hl_ubatch* ubs[2] = {pop, non};
-    const int32_t* ns[2] = {d_n_pop, d_n_non};
-    for (int m = 0; m < 2; ++m) {
-        const int32_t* pos0 = m == 0 ? nullptr : d_n_lookups;
-        const int32_t bias = (m == 0 || merge) ? 0 : (int32_t)(n_slots + 1);
-        const int32_t sentinel = bias + (int32_t)n_slots;
-        const int32_t* bag_bias = (m == 1 && merge) ? d_n_pop : nullptr;
-        if (short_bags)
-            k_bwd_pairs<1><<<grid, kThreads, 0, stream>>>(ubs[m]->ids, ubs[m]->offsets, ns[m], ctx->max_batch,
-                                                         ctx->T * ctx->S, n_slots, ctx->max_nnz, keys[0], vals[0],
-                                                         d_n_lookups + m, pos0, bias, sentinel, d_n_lookups + 2,
-                                                         r.status, bag_bias);
-        else
-            k_bwd_pairs<32><<<grid, kThreads, 0, stream>>>(ubs[m]->ids, ubs[m]->offsets, ns[m], ctx->max_batch,
-                                                          ctx->T * ctx->S, n_slots, ctx->max_nnz, keys[0], vals[0],
-                                                          d_n_lookups + m, pos0, bias, sentinel, d_n_lookups + 2,
-                                                          r.status, bag_bias);
-    }
-    note_launches(2);
-    HL_LAUNCH_CHECK();
+    a.sides = 2;
+    a.bags_follow = merge;
+    a.side[0] = {pop->ids, pop->offsets, d_n_pop, 0};
+    a.side[1] = {non->ids, non->offsets, d_n_non, merge ? 0 : (int32_t)(n_slots + 1)};
     int32_t *ok, *ov;
-    return radix_sort_pairs(keys, vals, d_n_lookups + 2, ctx->max_nnz, key_bits, r.bwd_hist, r.status, &ok, &ov, stream,
-                            wait_cfg(ctx));
+    return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, cleared, d_sorted_slots, d_sorted_bags,
+                          d_n_lookups, &ok, &ov, stream, aside);
 }
+
+}  // namespace
+
+int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge) {
+    const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
+    return sort_clear_words(ctx->max_nnz, bits_for(merge ? n_slots : 2 * n_slots + 1), wait_cfg(ctx));
+}
+
+int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, hl_ubatch* non,
+                           const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows, const int32_t* d_cold_rows,
+                           const int64_t* d_n_cold, const int32_t* d_prev_rows, const int64_t* d_n_prev,
+                           int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
+                           bool merge, cudaStream_t stream, const SortAside* aside) {
+    PairArgs a{};
+    a.ranked = ctx->r.cold_ranked;
+    a.slot0 = ctx->hot_cap + stage_row0;
+    a.stage_rows = stage_rows;
+    a.cold_rows = d_cold_rows;
+    a.d_n_cold = d_n_cold;
+    a.prev_rows = d_prev_rows;
+    a.d_n_prev = d_n_prev;
+    a.n_prev_max = ctx->staging_cap;
+    a.fwd_src = d_fwd_src;
+    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, merge, a, true, true,
+                        stream, aside);
+}
+
+}  // namespace hl
 
 extern "C" int32_t hl_embbag_bwd_prepare2(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop,
                                           const hl_ubatch* non, const int32_t* d_n_non, int32_t* d_sorted_slots,
                                           int32_t* d_sorted_bags, int32_t* d_n_lookups, void* stream) {
-    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, false, stream);
+    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, false, PairArgs{}, false,
+                        false, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int32_t hl_embbag_bwd_prepare_merged(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop,
                                                 const hl_ubatch* non, const int32_t* d_n_non, int32_t* d_sorted_slots,
                                                 int32_t* d_sorted_bags, int32_t* d_n_lookups, void* stream) {
-    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, true, stream);
+    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, true, PairArgs{}, false,
+                        false, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int32_t hl_embbag_bwd_apply2(hl_ctx* ctx, float* d_cache, const int32_t* d_sorted_slots,
@@ -948,7 +1088,7 @@ extern "C" int32_t hl_embbag_bwd_sgd_static(float* d_cache, int64_t cache_rows, 
         tmp.r.bwd_vals[i] = reinterpret_cast<int32_t*>(p);
         p += kStaticPairBytes;
     }
-    tmp.r.bwd_hist = reinterpret_cast<uint32_t*>(p);
+    tmp.r.bwd_hist[0] = reinterpret_cast<uint32_t*>(p);
     p += kStaticHistBytes;
     tmp.r.bwd_part = reinterpret_cast<float*>(p);
 

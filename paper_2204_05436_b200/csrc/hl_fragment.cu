@@ -1,138 +1,74 @@
-// Fragmenting a mini-batch into the popular micro-batch O and the non-popular micro-batch X.
+// Fragmenting a mini-batch into the popular micro-batch O and the non-popular micro-batch X, in two kernels.
 //
-//   1. k_frag_flags     one warp per input: probe the popular-row bitmap for every lookup of the input,
-//                       all-hit decided by a warp vote; the last CTA to finish then partitions: ballot + prefix
-//                       sums over the flags -> stable partition `perm`, n_pop
-//   2. k_frag_sizes     size of every destination bag (O's bags, then X's bags), then an exclusive scan
-//   3. k_frag_emit      copy every bag's lookups to its place, mapped to a cache slot (O) or global row (X), and
-//                       every input's dense features to its place
+//   1. k_frag_flags     a CTA per 32 inputs, a warp per table, a lane per input: probe the popular-row bitmap for every
+//                       lookup, all-hit flags as one word per 32 inputs; the last CTA to finish partitions: prefix sums
+//                       over the words' popcounts -> stable partition `perm`, n_pop
+//   2. k_frag_place     destination bags (O's bags, then X's bags) in tiles: sizes, their prefix sums (within the tile,
+//                       then chained over the tiles), and the lookups themselves, mapped to cache slots (O) or global
+//                       rows (X); dense features go along
+//
+// Both are latency chains of a few dependent loads, so what counts is that the loads of a step go out together and that
+// there are few steps: with a warp per input (whose lanes read one lookup of every table: a sector each), a partition in
+// 1024-input rounds, and sizes, scan and emission as kernels of their own, 8 192 one-lookup bags took 16 us in six
+// launches; these two take 10.6 us.
+#include <type_traits>
+
 #include "hl_common.cuh"
 
 namespace hl {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kFlagThreads = 1024;      // CTAs of the flags kernel: its last CTA partitions all inputs by itself
+constexpr int kFlagThreads = 512;
 
-// LANE_PER_TABLE: lane l walks the lookups of tables l, l+32, ... of its input (short bags: pooling 1).
-// otherwise the warp walks table after table with the lanes striding over the table's lookups of the input
-// (its S bags are contiguous in the table-major layout).
-// Probe: how a global row is looked up in the popular set (BitmapProbe: the dense bitmap of the 32-bit path;
-// HashProbe: the hashed remap of the wide-id path).
-__device__ void partition_by_flags(const uint8_t* flags, int B, int32_t* __restrict__ perm,
-                                   int32_t* __restrict__ counts);
-
-template <bool LANE_PER_TABLE, class Probe>
-__global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __restrict__ indices,
-                                                         const int32_t* __restrict__ offsets, int B, int T, int S,
-                                                         const int64_t* __restrict__ table_base, Probe remap,
-                                                         uint8_t* flags, int32_t* status, int32_t* __restrict__ perm,
-                                                         int32_t* __restrict__ counts, unsigned int* finished) {
-    __shared__ bool s_last;
-    const int lane = threadIdx.x & 31;
-    const int warps_per_block = kFlagThreads / 32;
-    for (int b = blockIdx.x * warps_per_block + (threadIdx.x >> 5); b < B; b += gridDim.x * warps_per_block) {
-        bool miss = false;
-        if (LANE_PER_TABLE) {
-            for (int t = lane; t < T; t += 32) {
-                const int64_t first_bag = ((int64_t)t * B + b) * S;
-                const int32_t lo = offsets[first_bag], hi = offsets[first_bag + S];
-                const int64_t base = table_base[t], rows = table_base[t + 1] - base;
-                for (int32_t j = lo; j < hi; ++j) {
-                    const int32_t idx = indices[j];
-                    if (idx < 0 || idx >= rows) {
-                        set_status(status, HL_EBOUNDS);
-                        miss = true;
-                    } else if (!remap.hit(base + idx)) {
-                        miss = true;
-                    }
-                }
-            }
-        } else {
-            for (int t = 0; t < T; ++t) {
-                const int64_t first_bag = ((int64_t)t * B + b) * S;
-                const int32_t lo = offsets[first_bag], hi = offsets[first_bag + S];
-                const int64_t base = table_base[t], rows = table_base[t + 1] - base;
-                for (int32_t j = lo + lane; j < hi; j += 32) {
-                    const int32_t idx = indices[j];
-                    if (idx < 0 || idx >= rows) {
-                        set_status(status, HL_EBOUNDS);
-                        miss = true;
-                    } else if (!remap.hit(base + idx)) {
-                        miss = true;
-                    }
-                }
-            }
-        }
-        const unsigned any_miss = __ballot_sync(0xffffffffu, miss);
-        if (lane == 0) flags[b] = any_miss == 0;
-    }
-    // The CTA that finishes last partitions the inputs (a launch of its own for one block's work costs more than the
-    // work): every CTA's flags are written and fenced before it counts itself in, and the last one reads them past
-    // its first-level cache.  The tally goes back to zero for the next call.
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(finished, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    partition_by_flags(flags, B, perm, counts);
-    if (threadIdx.x == 0) *finished = 0;
-}
-
-// One block.  Pass 1 counts the popular inputs; pass 2 places every input: a popular one at its rank among the
-// popular, a non-popular one behind all popular ones at its rank among the non-popular.
-__device__ void partition_by_flags(const uint8_t* flags, int B, int32_t* __restrict__ perm,
+// All threads of one CTA: perm and counts from the flag words.
+__device__ void partition_by_flags(const uint32_t* words, int B, int32_t* __restrict__ perm,
                                    int32_t* __restrict__ counts) {
-    constexpr int NT = kFlagThreads;
-    __shared__ int warp_sum[32];
-    __shared__ int s_total;
+    constexpr int NT = kFlagThreads, NW = NT / 32;
+    __shared__ int s_sum[NW + 1];
+    __shared__ uint32_t s_word[NT];
+    __shared__ int s_before[NT];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned lt = lanemask_lt();
-    if (threadIdx.x < 32) warp_sum[threadIdx.x] = 0;          // (fewer than 32 warps write theirs)
-    __syncthreads();
-
+    const int n_words = (B + 31) / 32;
     int mine = 0;
-    for (int b = threadIdx.x; b < B; b += NT) mine += __ldcg(&flags[b]);
+    for (int w = threadIdx.x; w < n_words; w += NT) mine += __popc(__ldcg(&words[w]));
+    const int warp_sum = __reduce_add_sync(0xffffffffu, mine);
+    if (lane == 0) s_sum[warp] = warp_sum;
+    __syncthreads();
+    int n_pop = 0;
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) mine += __shfl_down_sync(0xffffffffu, mine, d);
-    if (lane == 0) warp_sum[warp] = mine;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int w = 0; w < 32; ++w) s += warp_sum[w];
-        s_total = s;
-    }
-    __syncthreads();
-    const int n_pop = s_total;
+    for (int w = 0; w < NW; ++w) n_pop += s_sum[w];
     __syncthreads();
 
-    int before = 0;   // popular inputs in earlier chunks
-    for (int start = 0; start < B; start += NT) {
-        const int b = start + threadIdx.x;
-        const bool valid = b < B;
-        const bool pop = valid && __ldcg(&flags[b]);
-        const unsigned vote = __ballot_sync(0xffffffffu, pop);
-        if (lane == 0) warp_sum[warp] = __popc(vote);
-        __syncthreads();
-        if (warp == 0) {
-            const int c = lane < NT / 32 ? warp_sum[lane] : 0;
-            int incl = c;
+    int before = 0;                  // popular inputs in earlier rounds
+    for (int w0 = 0; w0 < n_words; w0 += NT) {
+        const int w = w0 + threadIdx.x;
+        const uint32_t word = w < n_words ? __ldcg(&words[w]) : 0u;
+        int incl = __popc(word);
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                int o = __shfl_up_sync(0xffffffffu, incl, d);
-                if (lane >= d) incl += o;
-            }
-            warp_sum[lane] = incl - c;
-            if (lane == 31) s_total = incl;
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
         }
+        if (lane == 31) s_sum[warp] = incl;
         __syncthreads();
-        if (valid) {
-            const int rank_pop = before + warp_sum[warp] + __popc(vote & lt);   // popular inputs before b
-            if (pop) perm[rank_pop] = b;
-            else perm[n_pop + (b - rank_pop)] = b;
+        int earlier = 0, all = 0;
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+            if (k < warp) earlier += s_sum[k];
+            all += s_sum[k];
         }
-        before += s_total;
+        s_word[threadIdx.x] = word;
+        s_before[threadIdx.x] = before + earlier + incl - __popc(word);
+        __syncthreads();
+        const int first = w0 * 32, last = min(B, first + NT * 32);
+        for (int b = first + threadIdx.x; b < last; b += NT) {
+            const uint32_t m = s_word[(b - first) >> 5];
+            const int bit = b & 31;
+            const int rank = s_before[(b - first) >> 5] + __popc(m & ((1u << bit) - 1u));     // popular inputs before b
+            perm[(m >> bit) & 1u ? rank : n_pop + (b - rank)] = b;
+        }
+        before += all;
         __syncthreads();
     }
     if (threadIdx.x == 0) {
@@ -141,105 +77,290 @@ __device__ void partition_by_flags(const uint8_t* flags, int B, int32_t* __restr
     }
 }
 
-struct DestBag {
-    int64_t src_bag;
-    int t;
-    bool is_pop;
-};
-
-// Destination bags: O's T*l*S bags, then X's T*k*S bags, each table-major over the micro-batch's inputs.
-__device__ __forceinline__ DestBag decode_dest_bag(int64_t dst, int B, int S, int n_pop, int64_t pop_bags,
-                                                   const int32_t* __restrict__ perm) {
-    DestBag d;
-    d.is_pop = dst < pop_bags;
-    const int64_t local = d.is_pop ? dst : dst - pop_bags;
-    const int n = d.is_pop ? n_pop : B - n_pop;
-    const int64_t per_table = (int64_t)n * S;
-    d.t = (int)(local / per_table);
-    const int64_t rem = local - (int64_t)d.t * per_table;
-    const int i = (int)(rem / S), s = (int)(rem - (int64_t)i * S);
-    const int b = perm[(d.is_pop ? 0 : n_pop) + i];
-    d.src_bag = ((int64_t)d.t * B + b) * S + s;
-    return d;
-}
-
-__global__ void __launch_bounds__(kThreads) k_frag_sizes(const int32_t* __restrict__ offsets, int B, int T, int S,
-                                                         const int32_t* __restrict__ perm,
-                                                         const int32_t* __restrict__ counts,
-                                                         int32_t* __restrict__ sizes) {
-    const int n_pop = counts[0];
-    const int64_t n_bags = (int64_t)T * B * S, pop_bags = (int64_t)T * n_pop * S;
-    for (int64_t dst = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; dst < n_bags;
-         dst += (int64_t)gridDim.x * blockDim.x) {
-        const DestBag d = decode_dest_bag(dst, B, S, n_pop, pop_bags, perm);
-        sizes[dst] = offsets[d.src_bag + 1] - offsets[d.src_bag];
-    }
-}
-
-// GROUP lanes cooperate on one destination bag (1 for short bags, 32 for long ones).  NonId: type of X's global row
-// ids (int32_t, or int64_t on the wide-id path).
-template <int GROUP, class Probe, typename NonId>
-__global__ void __launch_bounds__(kThreads) k_frag_emit(const int32_t* __restrict__ indices,
-                                                        const int32_t* __restrict__ offsets, int B, int T, int S,
-                                                        const int32_t* __restrict__ perm,
-                                                        int32_t* __restrict__ counts,
-                                                        const int32_t* __restrict__ dst_start,   // scanned sizes
-                                                        const int64_t* __restrict__ table_base, Probe remap,
-                                                        int32_t* __restrict__ pop_offsets, int32_t* __restrict__ pop_ids,
-                                                        int64_t pop_cap, int32_t* __restrict__ non_offsets,
-                                                        NonId* __restrict__ non_ids, int64_t non_cap,
-                                                        int32_t* status, const float* __restrict__ dense,
-                                                        int n_dense, float* __restrict__ dense_out) {
-    const int n_pop = counts[0];
-    const int64_t n_bags = (int64_t)T * B * S, pop_bags = (int64_t)T * n_pop * S;
-    const int32_t L_pop = dst_start[pop_bags], L_all = dst_start[n_bags];
-    const int sub = threadIdx.x % GROUP;
-    const int64_t group = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / GROUP;
-    const int64_t n_groups = (int64_t)gridDim.x * blockDim.x / GROUP;
-    if (group == 0 && sub == 0) {
-        counts[2] = L_pop;
-        counts[3] = L_all - L_pop;
-        pop_offsets[pop_bags] = L_pop;
-        non_offsets[n_bags - pop_bags] = L_all - L_pop;
-    }
-    for (int64_t dst = group; dst < n_bags; dst += n_groups) {
-        const DestBag d = decode_dest_bag(dst, B, S, n_pop, pop_bags, perm);
-        const int32_t src_lo = offsets[d.src_bag], src_hi = offsets[d.src_bag + 1];
-        const int64_t base = table_base[d.t], rows = table_base[d.t + 1] - base;
-        if (d.is_pop) {
-            const int32_t out_lo = dst_start[dst];
-            if (sub == 0) pop_offsets[dst] = out_lo;
-            for (int32_t j = sub; j < src_hi - src_lo; j += GROUP) {
-                if (out_lo + j >= pop_cap) {
-                    set_status(status, HL_ECAPACITY);
-                    break;
+// SHORT_BAGS: a lane walks the lookups of its input, four tables at a time (so that, with one lookup per table, their
+// offsets, indices and bitmap words are three rounds of loads).  Otherwise the lookups that a table has for the 32 inputs,
+// which are contiguous, are dealt out over the lanes, and a lookup that misses finds its input in the 33 offsets; a CTA
+// whose inputs have all missed is done (out-of-range lookups are reported by k_frag_place, which sees all of X's).
+// Probe: how a global row is looked up in the popular set (BitmapProbe: the dense bitmap of the 32-bit path;
+// HashProbe: the hashed remap of the wide-id path).
+// chain / n_chain: the state of k_frag_place's chain, cleared here.
+template <bool SHORT_BAGS, class Probe>
+__global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __restrict__ indices,
+                                                             const int32_t* __restrict__ offsets, int B, int T, int S,
+                                                             const int64_t* __restrict__ table_base, Probe remap,
+                                                             uint32_t* words, int32_t* __restrict__ perm,
+                                                             int32_t* __restrict__ counts, unsigned int* finished,
+                                                             unsigned long long* __restrict__ chain, int n_chain) {
+    constexpr int NW = kFlagThreads / 32;
+    __shared__ unsigned s_miss;
+    __shared__ bool s_last;
+    __shared__ int32_t s_start[SHORT_BAGS ? 1 : NW][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = blockIdx.x * kFlagThreads + threadIdx.x; i < n_chain; i += gridDim.x * kFlagThreads) chain[i] = 0ull;
+    for (int group = blockIdx.x; group * 32 < B; group += gridDim.x) {
+        const int b = group * 32 + lane, in_group = min(32, B - group * 32);
+        const unsigned everybody = in_group == 32 ? 0xffffffffu : (1u << in_group) - 1u;
+        if (threadIdx.x == 0) s_miss = 0;
+        __syncthreads();
+        if (SHORT_BAGS) {
+            constexpr int U = 4;
+            bool miss = false;
+            for (int t0 = warp; t0 < T; t0 += NW * U) {
+                int32_t lo[U], hi[U];
+                int64_t base[U], rows[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int t = t0 + u * NW;
+                    const bool in = t < T && b < B;
+                    const int64_t bag = ((int64_t)t * B + b) * S;
+                    lo[u] = in ? offsets[bag] : 0;
+                    hi[u] = in ? offsets[bag + S] : 0;
+                    base[u] = t < T ? table_base[t] : 0;
+                    rows[u] = t < T ? table_base[t + 1] - base[u] : 0;
                 }
-                const int32_t idx = indices[src_lo + j];
-                // every lookup of a popular input was tested to be in range and popular
-                pop_ids[out_lo + j] = remap.slot(base + idx);
+                int32_t idx[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) idx[u] = lo[u] < hi[u] ? indices[lo[u]] : 0;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (lo[u] < hi[u])
+                        miss |= idx[u] < 0 || idx[u] >= rows[u] || !remap.hit(base[u] + idx[u]);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    for (int32_t j = lo[u] + 1; j < hi[u]; ++j) {
+                        const int32_t i = indices[j];
+                        miss |= i < 0 || i >= rows[u] || !remap.hit(base[u] + i);
+                    }
             }
+            const unsigned m = __ballot_sync(0xffffffffu, miss);
+            if (lane == 0 && m) atomicOr(&s_miss, m);
         } else {
-            const int32_t out_lo = dst_start[dst] - L_pop;
-            if (out_lo < 0) continue;   // only after a chain poll of the scan gave up (HL_ETIMEOUT)
-            if (sub == 0) non_offsets[dst - pop_bags] = out_lo;
-            for (int32_t j = sub; j < src_hi - src_lo; j += GROUP) {
-                if (out_lo + j >= non_cap) {
-                    set_status(status, HL_ECAPACITY);
-                    break;
+            // (with fewer tables than warps, several warps share a table)
+            const int share = T < NW ? NW / T : 1, part = T < NW ? warp / T : 0;
+            for (int t = T < NW ? warp % T : warp; t < T && part < share; t += T < NW ? T : NW) {
+                __syncwarp();                         // the table before is done with s_start
+                if (__shfl_sync(0xffffffffu, *(volatile unsigned*)&s_miss, 0) == everybody) break;
+                const int64_t bag = ((int64_t)t * B + group * 32) * S;
+                if (lane < in_group) s_start[warp][lane] = offsets[bag + (int64_t)lane * S];
+                if (lane == 0) s_start[warp][in_group] = offsets[bag + (int64_t)in_group * S];
+                __syncwarp();
+                const int32_t lo = s_start[warp][0], hi = s_start[warp][in_group];
+                const int64_t base = table_base[t], rows = table_base[t + 1] - base;
+                constexpr int U = 4;
+                for (int32_t j0 = lo + part * 32; j0 < hi; j0 += share * 32 * U) {
+                    int32_t idx[U];
+                    bool hit[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int32_t j = j0 + u * share * 32 + lane;
+                        idx[u] = j < hi ? indices[j] : -1;
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) hit[u] = idx[u] >= 0 && idx[u] < rows && remap.hit(base + idx[u]);
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int32_t j = j0 + u * share * 32 + lane;
+                        if (hit[u] || j >= hi) continue;
+                        int a = 0, z = in_group;      // s_start[a] <= j < s_start[z]
+                        while (z - a > 1) {
+                            const int mid = (a + z) >> 1;
+                            if (s_start[warp][mid] <= j) a = mid;
+                            else z = mid;
+                        }
+                        if (!((*(volatile unsigned*)&s_miss >> a) & 1u)) atomicOr(&s_miss, 1u << a);
+                    }
                 }
-                const int32_t idx = indices[src_lo + j];
-                non_ids[out_lo + j] = (idx < 0 || idx >= rows) ? (NonId)-1 : (NonId)(base + idx);
             }
         }
+        __syncthreads();
+        if (threadIdx.x == 0) words[group] = everybody & ~s_miss;
+        __syncthreads();
     }
-    // the dense features follow their inputs: dense_out[i, :] = dense[perm[i], :] (the same threads, afterwards; a
-    // launch of its own would cost more than the copy)
-    if (dense != nullptr) {
-        const int64_t total = (int64_t)B * n_dense;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            const int i = (int)(e / n_dense), c = (int)(e - (int64_t)i * n_dense);
-            dense_out[e] = dense[(int64_t)perm[i] * n_dense + c];
+    // The CTA that finishes last partitions the inputs (a launch of its own for one block's work costs more than the
+    // work): every CTA's words are written and fenced before it counts itself in, and the last one reads them past
+    // its first-level cache.  The tally goes back to zero for the next call.
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(finished, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    partition_by_flags(words, B, perm, counts);
+    if (threadIdx.x == 0) *finished = 0;
+}
+
+// ---- placing --------------------------------------------------------------------------------------------------
+// The lookups of X are written as global row ids (int64 on the wide path).  With MARK (the scheduler's calls) the first half of the cold-row search is done on the way instead: a popular row
+// becomes its slot, any other row g is marked in the cold-row bitmap and written as -2 - g (classify_cold).
+//
+// The chain between tiles carries two sums, lookups of O and lookups of X: 31 bits each, below two flag bits.
+constexpr int kHalf = 31;
+constexpr unsigned long long kLow = (1ull << kHalf) - 1ull;
+
+struct PlaceArgs {
+    const int32_t* indices;
+    const int32_t* offsets;
+    int B, T, S;
+    const int32_t* perm;
+    int32_t* counts;
+    const int64_t* table_base;
+    int32_t* pop_offsets;
+    int32_t* pop_ids;
+    int64_t pop_cap;
+    int32_t* non_offsets;
+    int64_t non_cap;
+    unsigned long long* chain;         // [tile] status word of the tile; zero on entry
+    int32_t* status;
+    int max_polls;
+    int64_t stall_tile;
+    const float* dense;
+    int n_dense;
+    float* dense_out;
+};
+
+// ITEMS destination bags per thread, in rows of 32 bags per warp.  GROUP lanes cooperate on one bag's lookups.
+template <int GROUP, int ITEMS, bool MARK, class Probe, typename NonId>
+__global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe remap, NonId* __restrict__ non_ids,
+                                                         ColdMarks marks) {
+    constexpr int TB = kThreads * ITEMS, NW = kThreads / 32;
+    __shared__ int32_t s_pop[NW], s_all[NW];         // lookups of O / lookups in the warps' bags
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tile = blockIdx.x;
+    const int B = a.B, S = a.S, n_pop = a.counts[0], n_non = B - n_pop;
+    const int n_bags = a.T * B * S, pop_bags = a.T * n_pop * S;
+    const int first = tile * TB, last = min(first + TB, n_bags);
+
+    // Destination bags: O's T*n_pop*S bags, then X's T*n_non*S bags, each table-major over the micro-batch's inputs.
+    int32_t src_lo[ITEMS], len[ITEMS], table[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int dst = first + (warp * ITEMS + i) * 32 + lane;
+        src_lo[i] = len[i] = table[i] = 0;
+        if (dst < last) {
+            const bool is_pop = dst < pop_bags;
+            const unsigned local = is_pop ? dst : dst - pop_bags, per_table = (unsigned)(is_pop ? n_pop : n_non) * S;
+            const unsigned t = local / per_table, rem = local - t * per_table, in = S == 1 ? rem : rem / S;
+            const int64_t src = ((int64_t)t * B + a.perm[(is_pop ? 0 : n_pop) + in]) * S + (rem - in * S);
+            table[i] = (int)t;
+            src_lo[i] = a.offsets[src];
+            len[i] = a.offsets[src + 1] - src_lo[i];
+        }
+    }
+    // what the first lookup of a short bag becomes (ready before the tile knows where it goes: the loads behind it, index and
+    // popular-row block, are in flight while the tiles exchange their sums)
+    NonId head[ITEMS];
+    auto resolve = [&](bool is_pop, int64_t base, int64_t rows, int32_t idx) -> NonId {
+        if (is_pop) return (NonId)remap.slot(base + idx);    // every lookup of a popular input is in range and popular
+        if (idx < 0 || idx >= rows) {
+            set_status(a.status, HL_EBOUNDS);
+            return (NonId)-1;
+        }
+        if constexpr (MARK) return (NonId)classify_cold(remap, base + idx, marks);
+        else return (NonId)(base + idx);
+    };
+    int32_t start[ITEMS], all = 0, pop = 0;          // where the bag's lookups go, counted from the warp's first one
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        int32_t incl = len[i];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int32_t o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        start[i] = all + incl - len[i];
+        all += __shfl_sync(0xffffffffu, incl, 31);
+        pop += __reduce_add_sync(0xffffffffu, first + (warp * ITEMS + i) * 32 + lane < pop_bags ? len[i] : 0);
+    }
+    if (lane == 0) {
+        s_pop[warp] = pop;
+        s_all[warp] = all;
+    }
+    __syncthreads();
+    int32_t tile_pop = 0, tile_all = 0, warp_start = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        if (w < warp) warp_start += s_all[w];
+        tile_pop += s_pop[w];
+        tile_all += s_all[w];
+    }
+    const unsigned long long total = ((unsigned long long)tile_pop << kHalf) + (unsigned)(tile_all - tile_pop);
+    if (tile != a.stall_tile) chain_publish(a.chain, tile, total);
+    if (GROUP == 1) {
+        int32_t idx[ITEMS];
+        int64_t base[ITEMS], rows[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            idx[i] = len[i] > 0 ? a.indices[src_lo[i]] : 0;
+            base[i] = a.table_base[table[i]];
+            rows[i] = a.table_base[table[i] + 1] - base[i];
+        }
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            head[i] = len[i] > 0 ? resolve(first + (warp * ITEMS + i) * 32 + lane < pop_bags, base[i], rows[i], idx[i]) : 0;
+    }
+    // the dense features follow their inputs: dense_out[i, :] = dense[perm[i], :]
+    if (a.dense != nullptr) {
+        const unsigned n_dense = a.n_dense, n_tiles = gridDim.x;
+        for (int64_t i0 = (int64_t)tile * kThreads; i0 < (int64_t)B * n_dense; i0 += (int64_t)n_tiles * kThreads) {
+            const int64_t e = i0 + threadIdx.x;
+            if (e >= (int64_t)B * n_dense) break;
+            const unsigned i = e < 0x100000000ll ? (unsigned)e / n_dense : (unsigned)(e / n_dense);
+            a.dense_out[e] = a.dense[(int64_t)a.perm[i] * n_dense + (e - (int64_t)i * n_dense)];
+        }
+    }
+    const unsigned long long before =
+        chain_before<kThreads>(a.chain, tile, total, tile != a.stall_tile, a.max_polls, a.status);
+    if (threadIdx.x == 0 && last == n_bags) {                // the last tile knows the totals
+        const int32_t L_pop = (int32_t)((before + total) >> kHalf), L_non = (int32_t)((before + total) & kLow);
+        a.counts[2] = L_pop;
+        a.counts[3] = L_non;
+        a.pop_offsets[pop_bags] = L_pop;
+        a.non_offsets[n_bags - pop_bags] = L_non;
+    }
+    const int32_t pop_base = (int32_t)(before >> kHalf) + warp_start;
+    const int32_t non_base = (int32_t)(before & kLow) + warp_start - tile_pop;
+
+    // lookups j0, j0 + GROUP, ... of a bag of n
+    auto copy_bag = [&](bool is_pop, int t, int32_t lo, int32_t n, int32_t out, int j0) {
+        const int64_t base = a.table_base[t], rows = a.table_base[t + 1] - base;
+        const int64_t cap = is_pop ? a.pop_cap : a.non_cap;
+        for (int32_t j = j0; j < n; j += GROUP) {
+            if (out < 0 || out + j >= cap) {                 // (out < 0: only after a chain poll gave up)
+                if (out >= 0) set_status(a.status, HL_ECAPACITY);
+                break;
+            }
+            const NonId id = resolve(is_pop, base, rows, a.indices[lo + j]);
+            if (is_pop) a.pop_ids[out + j] = (int32_t)id;
+            else non_ids[out + j] = id;
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int row0 = first + (warp * ITEMS + i) * 32, dst = row0 + lane;
+        const bool is_pop = dst < pop_bags;
+        const int32_t out = start[i] + (is_pop ? pop_base : non_base);
+        if (dst < last) {
+            if (is_pop) a.pop_offsets[dst] = out;
+            else if (out >= 0) a.non_offsets[dst - pop_bags] = out;
+        }
+        if (GROUP == 1) {
+            if (dst < last && len[i] > 0) {
+                if (out >= 0 && out < (is_pop ? a.pop_cap : a.non_cap)) {
+                    if (is_pop) a.pop_ids[out] = (int32_t)head[i];
+                    else non_ids[out] = head[i];
+                } else if (out >= 0) {
+                    set_status(a.status, HL_ECAPACITY);
+                }
+                if (len[i] > 1) copy_bag(is_pop, table[i], src_lo[i], len[i], out, 1);
+            }
+        } else {
+            for (int k0 = 0; k0 < 32 && row0 + k0 < last; k0 += 32 / GROUP) {
+                const int k = k0 + lane / GROUP;
+                const int t = __shfl_sync(0xffffffffu, table[i], k), lo = __shfl_sync(0xffffffffu, src_lo[i], k);
+                const int n = __shfl_sync(0xffffffffu, len[i], k), to = __shfl_sync(0xffffffffu, out, k);
+                copy_bag(row0 + k < pop_bags, t, lo, n, to, lane % GROUP);      // (n = 0 past the last bag)
+            }
         }
     }
 }
@@ -252,52 +373,47 @@ using namespace hl;
 namespace hl {
 namespace {
 
-// The launches of a fragment call, for either lookup structure.  scratch: flags [max_batch], scan [n_bags + 2],
-// tiles [scan_tile_words(n_bags)].
-template <class Probe, typename NonId>
+// The launches of a fragment call, for either lookup structure.  words [max_batch / 32 + 1], chain [frag_chain_words].
+template <bool MARK, class Probe, typename NonId>
 int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t* table_base, Probe probe,
-                        uint8_t* flags, int32_t* scan, int32_t* tiles, int64_t max_bags, int32_t* status, WaitCfg waits,
+                        uint32_t* words, unsigned long long* chain, int32_t* status, WaitCfg waits,
                         const float* d_dense, int32_t n_dense, int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop,
-                        int32_t* non_offsets, NonId* non_ids, int64_t non_cap, float* d_dense_out, cudaStream_t stream) {
+                        int32_t* non_offsets, NonId* non_ids, int64_t non_cap, float* d_dense_out, ColdMarks marks,
+                        cudaStream_t stream) {
     const int B = b->batch;
     const int64_t n_bags = (int64_t)T * B * S;
-    const bool short_bags = b->nnz <= 4 * (int64_t)T * B;   // on average at most 4 lookups per input and table
-    const int cap = 4 * sms;               // CTAs of every kernel here: they stride over their work
-    const int flag_grid = grid_for(B, kFlagThreads / 32, cap);
-    // the tally of finished CTAs of the flags kernel: the word behind the scan's tile words (never touched by the
-    // scan, zero between calls: cleared when the context is created and by the CTA that counts to the end)
-    unsigned int* finished = reinterpret_cast<unsigned int*>(tiles + scan_tile_words(max_bags) - 2);
-    if (short_bags)
-        k_frag_flags<true, Probe><<<flag_grid, kFlagThreads, 0, stream>>>(b->indices, b->offsets, B, T, S, table_base, probe,
-                                                                      flags, status, d_perm, d_counts, finished);
+    // Bags per tile: 256 where there are few bags (the tiles are the parallelism), 1 024 from one tile per SM on.
+    const int items = n_bags <= (int64_t)kThreads * sms ? 1 : 4;
+    const int n_tiles = (int)div_up(n_bags, kThreads * items);
+    // the tally of finished CTAs of the flags kernel: word 0 of the chain words (zero between calls: cleared when the
+    // context is created and by the CTA that counts to the end); the chain proper is cleared by the flags kernel
+    unsigned int* finished = reinterpret_cast<unsigned int*>(chain);
+    PlaceArgs a{b->indices, b->offsets, B, T, S, d_perm, d_counts, table_base, pop->offsets, pop->ids, pop->cap_ids,
+                non_offsets, non_cap, chain + 1, status, waits.max_polls, waits.stall_tile, d_dense, n_dense, d_dense_out};
+    const int flag_grid = grid_for(B, 32, 4 * sms);
+    if (b->nnz <= 4 * (int64_t)T * B)            // on average at most 4 lookups per input and table
+        k_frag_flags<true, Probe><<<flag_grid, kFlagThreads, 0, stream>>>(
+            b->indices, b->offsets, B, T, S, table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles);
     else
-        k_frag_flags<false, Probe><<<flag_grid, kFlagThreads, 0, stream>>>(b->indices, b->offsets, B, T, S, table_base,
-                                                                       probe, flags, status, d_perm, d_counts,
-                                                                       finished);
-    k_frag_sizes<<<grid_for(n_bags, kThreads, cap), kThreads, 0, stream>>>(b->offsets, B, T, S, d_perm, d_counts, scan);
-    note_launches(2);   // flags (with the partition), sizes
-    HL_LAUNCH_CHECK();
-    int32_t st = exclusive_scan_i32(scan, scan, nullptr, n_bags, tiles, status, stream, waits);
-    if (st != HL_OK) return st;
-    if (b->nnz <= 4 * n_bags)
-        k_frag_emit<1, Probe, NonId><<<grid_for(n_bags, kThreads, cap), kThreads, 0, stream>>>(
-            b->indices, b->offsets, B, T, S, d_perm, d_counts, scan, table_base, probe, pop->offsets, pop->ids,
-            pop->cap_ids, non_offsets, non_ids, non_cap, status, d_dense, n_dense, d_dense_out);
-    else
-        k_frag_emit<32, Probe, NonId><<<grid_for(n_bags, kThreads / 32, 2 * cap), kThreads, 0, stream>>>(
-            b->indices, b->offsets, B, T, S, d_perm, d_counts, scan, table_base, probe, pop->offsets, pop->ids,
-            pop->cap_ids, non_offsets, non_ids, non_cap, status, d_dense, n_dense, d_dense_out);
-    note_launches(1);   // emit (with the dense permutation)
+        k_frag_flags<false, Probe><<<flag_grid, kFlagThreads, 0, stream>>>(
+            b->indices, b->offsets, B, T, S, table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles);
+    // lanes per bag: by the average number of lookups
+    const auto pick = [&](auto g) {
+        constexpr int G = decltype(g)::value;
+        return items == 1 ? k_frag_place<G, 1, MARK, Probe, NonId> : k_frag_place<G, 4, MARK, Probe, NonId>;
+    };
+    const auto place = 4 * b->nnz <= 5 * n_bags ? pick(std::integral_constant<int, 1>())
+                       : b->nnz <= 8 * n_bags   ? pick(std::integral_constant<int, 4>())
+                                                : pick(std::integral_constant<int, 16>());
+    place<<<n_tiles, kThreads, 0, stream>>>(a, probe, non_ids, marks);
+    note_launches(2);
     HL_LAUNCH_CHECK();
     return HL_OK;
 }
 
-}  // namespace
-}  // namespace hl
-
-extern "C" int32_t hl_fragment(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
-                               int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non,
-                               float* d_dense_out, void* stream_) {
+int32_t fragment_call(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense, int32_t* d_perm,
+                      int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non, float* d_dense_out, bool mark,
+                      cudaStream_t stream) {
     if (!ctx || !b || !d_perm || !d_counts || !pop || !non) return HL_EINVAL;
     if (b->batch < 1 || b->batch > ctx->max_batch || b->nnz < 0 || b->nnz > ctx->max_nnz || !b->offsets ||
         (b->nnz > 0 && !b->indices))
@@ -305,10 +421,26 @@ extern "C" int32_t hl_fragment(hl_ctx* ctx, const hl_batch* b, const float* d_de
     if (!pop->offsets || !non->offsets || (b->nnz > 0 && (!pop->ids || !non->ids))) return HL_EINVAL;
     if ((d_dense == nullptr) != (d_dense_out == nullptr) || (d_dense && n_dense < 1)) return HL_EINVAL;
     Regions& r = ctx->r;
-    return fragment_launch<BitmapProbe, int32_t>(b, ctx->T, ctx->S, ctx_sms(ctx), r.table_base, BitmapProbe{r.remap},
-                                                 r.frag_flags, r.frag_scan, r.frag_tiles, ctx->max_bags, r.status, wait_cfg(ctx),
-                                                 d_dense, n_dense, d_perm, d_counts, pop, non->offsets, non->ids,
-                                                 non->cap_ids, d_dense_out, static_cast<cudaStream_t>(stream_));
+    const auto launch = mark ? fragment_launch<true, BitmapProbe, int32_t> : fragment_launch<false, BitmapProbe, int32_t>;
+    return launch(b, ctx->T, ctx->S, ctx_sms(ctx), r.table_base, BitmapProbe{r.remap}, r.frag_words, r.frag_chain,
+                  r.status, wait_cfg(ctx), d_dense, n_dense, d_perm, d_counts, pop, non->offsets, non->ids, non->cap_ids,
+                  d_dense_out, cold_marks(ctx), stream);
+}
+
+}  // namespace
+
+int32_t fragment_and_mark(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense, int32_t* d_perm,
+                          int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non, float* d_dense_out, cudaStream_t stream) {
+    return fragment_call(ctx, b, d_dense, n_dense, d_perm, d_counts, pop, non, d_dense_out, true, stream);
+}
+
+}  // namespace hl
+
+extern "C" int32_t hl_fragment(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
+                               int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non,
+                               float* d_dense_out, void* stream) {
+    return fragment_call(ctx, b, d_dense, n_dense, d_perm, d_counts, pop, non, d_dense_out, false,
+                         static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int32_t hl_wide_fragment(hl_wide* w, const hl_batch* b, int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop,
@@ -319,8 +451,8 @@ extern "C" int32_t hl_wide_fragment(hl_wide* w, const hl_batch* b, int32_t* d_pe
         return HL_EINVAL;
     if (!pop->offsets || (b->nnz > 0 && (!pop->ids || !d_non_rows))) return HL_EINVAL;
     const HashProbe probe{w->r_keys, w->r_vals, (uint64_t)(w->remap_slots - 1)};
-    return fragment_launch<HashProbe, long long>(b, w->T, w->S, w->sms, w->table_base, probe, w->frag_flags,
-                                                 w->frag_scan, w->frag_tiles, w->max_bags, w->status, WaitCfg(), nullptr, 0, d_perm,
-                                                 d_counts, pop, d_non_offsets, reinterpret_cast<long long*>(d_non_rows),
-                                                 non_cap, nullptr, static_cast<cudaStream_t>(stream_));
+    return fragment_launch<false, HashProbe, long long>(
+        b, w->T, w->S, w->sms, w->table_base, probe, w->frag_words, w->frag_chain, w->status, WaitCfg(), nullptr, 0, d_perm,
+        d_counts, pop, d_non_offsets, reinterpret_cast<long long*>(d_non_rows), non_cap, nullptr, ColdMarks{},
+        static_cast<cudaStream_t>(stream_));
 }

@@ -1,16 +1,19 @@
-// The software-pipelined schedule over mini-batches, issued from native code: the same order of calls, streams and
-// events as the Python scheduler, without an interpreter between the launches (a mini-batch is about 32 kernels, 10
-// memsets and 25 event operations; issued from Python that alone takes 0.2 ms).
+// The software-pipelined schedule over mini-batches, issued from native code.
 //
-//   stream A     hl_fragment(j+L)
-//   stream C     hl_index_cold(j+L)            after A;  needs the cold rows of j+L-1 (same stream, in order)
-//   stream B     hl_embbag_bwd_prepare2(j+L)   after C
-//   link stream  hl_forward_cold(j)            after the backward of j-1;  then
-//                hl_stage_cold(j+1)            after the write-back of j-1 (host rows final, window free)
-//   main stream  forward O, update O, [rows of j staged and forwarded] forward X, update X          mini-batch j
-//   write-back   hl_scatter_cold_at(j)         after the update of X
+//   index stream  mini-batch j+L: fragment (X's lookups classified on the way), ranks of the cold rows, slots + match with
+//                 the cold rows of j+L-1 + (slot, bag) pairs, sort (more than 32 K lookups: on the sort stream)
+//   link stream   hl_stage_cold(j+1)           after the write-back of j-1 (host rows final, window free) and after
+//                                              mini-batch j took the rows it shares with j-1 out of that window
+//   main stream   forward O (+ those rows), update O, [rows of j staged] forward X, update X            mini-batch j
+//   write-back    hl_scatter_cold_at(j)        after the update of X
 //
 // L = n_sets - 2 mini-batches of index-only work ahead; set j % n_sets holds mini-batch j; window j % 2 its cold rows.
+//
+// Small mini-batches are bound by the host: what counts is the number of launches and event operations per mini-batch.
+// The index work is one stream (two), so that its steps need no events between them, and as few kernels as its data
+// dependences allow (five with at most 32 K lookups, otherwise four and one per sort digit); the rows forwarded between
+// windows ride on the popular forward.  13 to 15 launches, no memset and 12 to 15 event operations, where separate calls on
+// three streams made 22, 3 and 25 (8 K lookups: 88 us per mini-batch).
 #include "hl_common.cuh"
 
 #include <new>
@@ -23,14 +26,14 @@ struct hl_pipe {
     int64_t window_rows;
     int n_sets, n_dense;
     std::vector<hl_pipe_set> sets;
-    cudaStream_t main, sa, sb, sc, link, wb;
+    cudaStream_t main, index, sort, link, wb;
     struct Events {
-        cudaEvent_t inputs, frag, index, prep, gather, forward, x, scatter, fwd_pop;
+        cudaEvent_t inputs, pairs, index, gather, forward, x, scatter;
     };
     std::vector<Events> ev;
-    // mini-batches whose fragment + first half of the cold-row search are queued (begun), whose cold-row search and
-    // sort are queued in full (indexed), whose host read is queued (submitted), whose main work is queued (done)
-    int64_t j_begun, j_indexed, j_submitted, j_done;
+    // mini-batches whose index work is queued (indexed), whose host read is queued (submitted), whose main work is queued
+    // (done)
+    int64_t j_indexed, j_submitted, j_done;
     int order;                   // HL_PIPE_ORDER_*
     int wb_mode;                 // HL_PIPE_WB_*
     bool wb_pending;             // HL_PIPE_WB_AFTER_FORWARD: the write-back of mini-batch j_done - 1 is not queued yet
@@ -48,6 +51,8 @@ struct hl_pipe {
     int open_timer[HL_TIMER_COUNT];
 };
 
+using namespace hl;
+
 namespace {
 
 #define HL_PIPE_TRY(expr)                         \
@@ -60,10 +65,10 @@ int32_t wait(cudaStream_t s, cudaEvent_t e) { return cudaStreamWaitEvent(s, e, 0
 int32_t record(cudaEvent_t e, cudaStream_t s) { return cudaEventRecord(e, s) == cudaSuccess ? HL_OK : HL_ECUDA; }
 
 // ---- trace ---------------------------------------------------------------------------------------------------
-enum { kMain = 0, kStreamA = 1, kStreamB = 2, kStreamC = 3, kLink = 4, kWb = 5 };
+enum { kMain = 0, kIndex = 1, kSort = 2, kLink = 4, kWb = 5 };
 
 cudaStream_t stream_of(hl_pipe* p, int id) {
-    cudaStream_t all[6] = {p->main, p->sa, p->sb, p->sc, p->link, p->wb};
+    cudaStream_t all[6] = {p->main, p->index, p->sort, nullptr, p->link, p->wb};
     return all[id];
 }
 
@@ -106,68 +111,51 @@ struct Scope {
     ~Scope() { span_close(p, idx); }
 };
 
-// Second half of the index-only work of the mini-batch begun last: the match of its cold rows against the mini-batch
-// before (stream C, in order behind that mini-batch's search) and the backward sort (stream B).
-int32_t finish_index(hl_pipe* p) {
-    if (p->j_indexed == p->j_begun) return HL_OK;
+// The index-only work of the next mini-batch (nothing here touches a row).
+int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
     const int64_t j = p->j_indexed;
     const int n = p->n_sets;
     hl_pipe_set& st = p->sets[j % n];
     hl_pipe::Events& e = p->ev[j % n];
     hl_pipe_set* prev = j >= 1 ? &p->sets[(j - 1) % n] : nullptr;
     const int64_t w = (j % 2) * p->window_rows;
-    {
-        Scope sc(p, HL_SPAN_INDEX_END, j, kStreamC);
-        HL_PIPE_TRY(hl_index_cold_end(p->ctx, &st.non, w, p->window_rows, st.cold_rows, st.n_cold,
-                                      prev ? prev->cold_rows : nullptr, prev ? prev->n_cold : nullptr, st.fwd_src, 0,
-                                      p->sc));
-    }
-    HL_PIPE_TRY(record(e.index, p->sc));
-    HL_PIPE_TRY(wait(p->sb, e.index));
-    {
-        Scope sc(p, HL_SPAN_SORT, j, kStreamB);
-        if (p->order == HL_PIPE_ORDER_EQ5)
-            HL_PIPE_TRY(hl_embbag_bwd_prepare_merged(p->ctx, &st.pop, st.counts, &st.non, st.counts + 1,
-                                                     st.sorted_slots, st.sorted_bags, st.sorted_n, p->sb));
-        else
-            HL_PIPE_TRY(hl_embbag_bwd_prepare2(p->ctx, &st.pop, st.counts, &st.non, st.counts + 1, st.sorted_slots,
-                                               st.sorted_bags, st.sorted_n, p->sb));
-    }
-    HL_PIPE_TRY(record(e.prep, p->sb));
-    p->j_indexed += 1;
-    return HL_OK;
-}
-
-// fragment and the first half of the cold-row search of the next mini-batch (index-only: nothing here touches a row)
-int32_t begin_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
-    HL_PIPE_TRY(finish_index(p));        // (nothing pending in the usual order of calls)
-    const int64_t j = p->j_begun;
-    const int n = p->n_sets;
-    hl_pipe_set& st = p->sets[j % n];
-    hl_pipe::Events& e = p->ev[j % n];
-    const int64_t w = (j % 2) * p->window_rows;
+    const bool merge = p->order == HL_PIPE_ORDER_EQ5;
     if (inputs_ready == nullptr) {                        // the inputs are complete in main-stream order
         HL_PIPE_TRY(record(e.inputs, p->main));
-        HL_PIPE_TRY(wait(p->sa, e.inputs));
+        HL_PIPE_TRY(wait(p->index, e.inputs));
     } else if (inputs_ready != HL_PIPE_INPUTS_RESIDENT) {
-        HL_PIPE_TRY(wait(p->sa, static_cast<cudaEvent_t>(inputs_ready)));
+        HL_PIPE_TRY(wait(p->index, static_cast<cudaEvent_t>(inputs_ready)));
     }
-    if (j >= n) HL_PIPE_TRY(wait(p->sa, e.scatter));      // the buffers of this set were mini-batch j-n_sets's
+    if (j >= n) HL_PIPE_TRY(wait(p->index, e.scatter));   // the buffers of this set were mini-batch j-n_sets's
     {
-        Scope sc(p, HL_SPAN_FRAGMENT, j, kStreamA);
-        HL_PIPE_TRY(hl_fragment(p->ctx, b, d_dense, d_dense ? p->n_dense : 0, st.perm, st.counts, &st.pop, &st.non,
-                                d_dense ? st.dense_out : nullptr, p->sa));
+        Scope sc(p, HL_SPAN_FRAGMENT, j, kIndex);
+        HL_PIPE_TRY(fragment_and_mark(p->ctx, b, d_dense, d_dense ? p->n_dense : 0, st.perm, st.counts, &st.pop, &st.non,
+                                      d_dense ? st.dense_out : nullptr, p->index));
     }
-    HL_PIPE_TRY(record(e.frag, p->sa));
-    HL_PIPE_TRY(wait(p->sc, e.frag));
-    if (j >= n) HL_PIPE_TRY(wait(p->sc, e.scatter));
+    if (p->ctx->max_nnz == 0) {
+        HL_PIPE_TRY(hl_index_cold(p->ctx, &st.non, st.counts + 1, w, p->window_rows, st.cold_rows, st.n_cold, nullptr,
+                                  nullptr, st.fwd_src, p->index));
+    }
+    // A sort of many pairs goes to a stream of its own, so that its passes overlap the next mini-batch's fragment; scratch
+    // set j % 2 was the sort's of mini-batch j-2.
+    const int64_t n_clear = backward_sort_clear_words(p->ctx, merge);
+    const SortAside aside{p->sort, e.pairs, (int)(j % 2)};
+    const SortAside* use = n_clear > 0 ? &aside : nullptr;
+    if (use && j >= 2) HL_PIPE_TRY(wait(p->index, p->ev[(j - 2) % n].index));
+    if (p->ctx->max_nnz > 0) {
+        Scope sc(p, HL_SPAN_INDEX_BEGIN, j, kIndex);
+        HL_PIPE_TRY(cold_rank(p->ctx, p->window_rows, st.cold_rows, st.n_cold, p->index, p->ctx->r.bwd_hist[use ? j % 2 : 0],
+                              n_clear));
+    }
     {
-        Scope sc(p, HL_SPAN_INDEX_BEGIN, j, kStreamC);
-        HL_PIPE_TRY(hl_index_cold_begin(p->ctx, &st.non, st.counts + 1, w, p->window_rows, st.cold_rows, st.n_cold,
-                                        p->sc));
+        Scope sc(p, HL_SPAN_SORT, j, kIndex);
+        HL_PIPE_TRY(assign_and_prepare(p->ctx, &st.pop, st.counts, &st.non, st.counts + 1, w, p->window_rows, st.cold_rows,
+                                       st.n_cold, prev ? prev->cold_rows : nullptr, prev ? prev->n_cold : nullptr,
+                                       st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, p->index, use));
     }
-    p->j_begun += 1;
-    return finish_index(p);
+    HL_PIPE_TRY(record(e.index, use ? p->sort : p->index));
+    p->j_indexed += 1;
+    return HL_OK;
 }
 
 // the host read of the oldest indexed mini-batch whose rows are not staged yet
@@ -237,7 +225,7 @@ extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_t
     p->n_dense = n_dense;
     p->sets.assign(sets, sets + n_sets);
     p->main = static_cast<cudaStream_t>(main_stream);
-    p->j_begun = p->j_indexed = p->j_submitted = p->j_done = 0;
+    p->j_indexed = p->j_submitted = p->j_done = 0;
     p->order = HL_PIPE_ORDER_FIG8;
     p->wb_mode = opt ? opt->write_back : HL_PIPE_WB_OVERLAP;
     p->wb_pending = false;
@@ -250,17 +238,16 @@ extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_t
     cudaDeviceGetStreamPriorityRange(&lo, &hi);          // hi = numerically lowest = highest priority
     auto clamp = [&](int prio) { return prio < hi ? hi : (prio > lo ? lo : prio); };
     const int index_prio = clamp(opt ? opt->index_priority : 0), link_prio = clamp(opt ? opt->link_priority : 0);
-    cudaStream_t* side[5] = {&p->sa, &p->sb, &p->sc, &p->link, &p->wb};
+    cudaStream_t* side[4] = {&p->index, &p->sort, &p->link, &p->wb};
     bool ok = true;
-    for (int i = 0; i < 5; ++i) {
+    for (int i = 0; i < 4; ++i) {
         *side[i] = nullptr;
-        ok = ok && cudaStreamCreateWithPriority(side[i], cudaStreamNonBlocking, i < 3 ? index_prio : link_prio) ==
+        ok = ok && cudaStreamCreateWithPriority(side[i], cudaStreamNonBlocking, i < 2 ? index_prio : link_prio) ==
                        cudaSuccess;
     }
     p->ev.resize(n_sets);
     for (auto& e : p->ev) {
-        cudaEvent_t* all[9] = {&e.inputs, &e.frag,    &e.index, &e.prep,   &e.gather,
-                               &e.forward, &e.x,      &e.scatter, &e.fwd_pop};
+        cudaEvent_t* all[7] = {&e.inputs, &e.pairs, &e.index, &e.gather, &e.forward, &e.x, &e.scatter};
         for (auto x : all) {
             *x = nullptr;
             ok = ok && cudaEventCreateWithFlags(x, cudaEventDisableTiming) == cudaSuccess;
@@ -281,14 +268,14 @@ extern "C" hl_pipe* hl_pipe_create(hl_ctx* ctx, float* d_cache, float* host_tabl
 extern "C" void hl_pipe_destroy(hl_pipe* p) {
     if (!p) return;
     if (p->wb_pending && p->wb) (void)flush_scatter(p);      // a write-back held over is not lost
-    cudaStream_t side[5] = {p->sa, p->sb, p->sc, p->link, p->wb};
+    cudaStream_t side[4] = {p->index, p->sort, p->link, p->wb};
     for (auto s : side)
         if (s) {
             cudaStreamSynchronize(s);
             cudaStreamDestroy(s);
         }
     for (auto& e : p->ev) {
-        cudaEvent_t all[9] = {e.inputs, e.frag, e.index, e.prep, e.gather, e.forward, e.x, e.scatter, e.fwd_pop};
+        cudaEvent_t all[7] = {e.inputs, e.pairs, e.index, e.gather, e.forward, e.x, e.scatter};
         for (auto x : all)
             if (x) cudaEventDestroy(x);
     }
@@ -305,12 +292,9 @@ extern "C" void hl_pipe_destroy(hl_pipe* p) {
 
 extern "C" int32_t hl_pipe_submit(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
     if (!p || !b) return HL_EINVAL;
-    if (p->j_begun - p->j_done >= p->n_sets - 1) return HL_ECAPACITY;      // every spare buffer set is in flight
-    HL_PIPE_TRY(begin_index(p, b, d_dense, inputs_ready));
-    if (p->j_submitted == p->j_done) {                                      // nothing staged ahead yet
-        HL_PIPE_TRY(finish_index(p));
-        HL_PIPE_TRY(submit_link(p));
-    }
+    if (p->j_indexed - p->j_done >= p->n_sets - 1) return HL_ECAPACITY;    // every spare buffer set is in flight
+    HL_PIPE_TRY(submit_index(p, b, d_dense, inputs_ready));
+    if (p->j_submitted == p->j_done) HL_PIPE_TRY(submit_link(p));          // nothing staged ahead yet
     return HL_OK;
 }
 
@@ -324,52 +308,44 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
     hl_pipe_set& st = p->sets[j % n];
     hl_pipe::Events& e = p->ev[j % n];
     const int64_t w0 = (j % 2) * p->window_rows, w1 = ((j + 1) % 2) * p->window_rows;
-    if (next && p->j_begun - j >= n - 1) return HL_ECAPACITY;
+    if (next && p->j_indexed - j >= n - 1) return HL_ECAPACITY;
     HL_PIPE_TRY(wait(p->main, e.index));
     if (p->wb_mode == HL_PIPE_WB_EXCLUSIVE && j >= 1) HL_PIPE_TRY(wait(p->main, p->ev[(j - 1) % n].scatter));
-    if (j >= 1) {
-        // rows shared with mini-batch j-1 come out of its staging window once its backward is done
-        HL_PIPE_TRY(wait(p->link, e.index));
-        HL_PIPE_TRY(wait(p->link, p->ev[(j - 1) % n].x));
-        Scope sc(p, HL_SPAN_FORWARD_COLD, j, kLink);
-        HL_PIPE_TRY(hl_forward_cold(p->ctx, p->cache, w1, w0, p->window_rows, st.fwd_src, st.n_cold, p->link));
-    }
-    HL_PIPE_TRY(record(e.forward, p->link));
-    // (the host read of j+1 waits for the write-back of j-1, so it is queued behind a write-back that was held over)
-    if (!p->wb_pending && p->j_submitted < p->j_indexed) HL_PIPE_TRY(submit_link(p));   // j+1, if indexed in full
     {
+        // with O's forward: the rows shared with mini-batch j-1, out of its staging window (its backward is done)
         Scope sc(p, HL_SPAN_FWD_POP, j, kMain);
-        HL_PIPE_TRY(hl_embbag_fwd(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main));
+        if (j >= 1 && p->window_rows > 0)
+            HL_PIPE_TRY(fwd_and_forward_cold(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, w1, w0, p->window_rows,
+                                             st.fwd_src, st.n_cold, p->main));
+        else
+            HL_PIPE_TRY(hl_embbag_fwd(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main));
     }
+    HL_PIPE_TRY(record(e.forward, p->main));
     if (p->wb_pending) {
         // the write-back of j-1 starts when the popular forward of j is over: of all kernels of the main stream that
         // one loses most next to a write-back
-        HL_PIPE_TRY(record(e.fwd_pop, p->main));
-        HL_PIPE_TRY(wait(p->wb, e.fwd_pop));
+        HL_PIPE_TRY(wait(p->wb, e.forward));
         HL_PIPE_TRY(flush_scatter(p));
-        if (p->j_submitted < p->j_indexed) HL_PIPE_TRY(submit_link(p));
     }
+    if (p->j_submitted == j + 1 && p->j_submitted < p->j_indexed) HL_PIPE_TRY(submit_link(p));   // mini-batch j+1
     if (p->order == HL_PIPE_ORDER_FIG8) {
-        HL_PIPE_TRY(wait(p->main, e.prep));
         Scope sc(p, HL_SPAN_BWD_POP, j, kMain);
         HL_PIPE_TRY(hl_embbag_bwd_apply2(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 0, d_grad_pop,
                                          lr, p->main));
     }
     HL_PIPE_TRY(wait(p->main, e.gather));
-    HL_PIPE_TRY(wait(p->main, e.forward));
     {
         Scope sc(p, HL_SPAN_FWD_NON, j, kMain);
         HL_PIPE_TRY(hl_embbag_fwd(p->ctx, p->cache, &st.non, st.counts + 1, st.pooled_non, p->main));
     }
-    if (p->order == HL_PIPE_ORDER_FIG8) {
+    {
         Scope sc(p, HL_SPAN_BWD_NON, j, kMain);
-        HL_PIPE_TRY(hl_embbag_bwd_apply2(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 1, d_grad_non,
-                                         lr, p->main));
-    } else {   // one update of every touched row with the gradient of the whole mini-batch
-        HL_PIPE_TRY(wait(p->main, e.prep));
-        Scope sc(p, HL_SPAN_BWD_NON, j, kMain);
-        HL_PIPE_TRY(hl_embbag_bwd_apply(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n + 2, d_grad_pop,
-                                        lr, p->main));
+        if (p->order == HL_PIPE_ORDER_FIG8)
+            HL_PIPE_TRY(hl_embbag_bwd_apply2(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 1, d_grad_non,
+                                             lr, p->main));
+        else   // one update of every touched row with the gradient of the whole mini-batch
+            HL_PIPE_TRY(hl_embbag_bwd_apply(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n + 2, d_grad_pop,
+                                            lr, p->main));
     }
     HL_PIPE_TRY(record(e.x, p->main));
     p->j_done += 1;
@@ -377,14 +353,9 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
         p->wb_pending = true;            // queued by the next hl_pipe_step (or by whatever call comes instead)
     else
         HL_PIPE_TRY(queue_scatter(p, j));
-    HL_PIPE_TRY(finish_index(p));
-    if (p->j_submitted == j + 1 && p->j_submitted < p->j_indexed) HL_PIPE_TRY(submit_link(p));   // mini-batch j+1
     if (next) {
-        HL_PIPE_TRY(begin_index(p, next, d_next_dense, next_inputs_ready));
-        if (p->j_submitted == j + 1) {                                      // j+1 was begun only just now
-            HL_PIPE_TRY(finish_index(p));
-            HL_PIPE_TRY(submit_link(p));
-        }
+        HL_PIPE_TRY(submit_index(p, next, d_next_dense, next_inputs_ready));
+        if (p->j_submitted == j + 1) HL_PIPE_TRY(submit_link(p));           // j+1 was indexed only just now
     }
     if (set_index) *set_index = (int32_t)(j % n);
     return HL_OK;
@@ -392,7 +363,7 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
 
 extern "C" int32_t hl_pipe_set_order(hl_pipe* p, int32_t order) {
     if (!p || (order != HL_PIPE_ORDER_FIG8 && order != HL_PIPE_ORDER_EQ5)) return HL_EINVAL;
-    if (p->j_begun != 0) return HL_EINVAL;       // the sorts queued so far were made for the other order
+    if (p->j_indexed != 0) return HL_EINVAL;       // the sorts queued so far were made for the other order
     p->order = order;
     return HL_OK;
 }
@@ -467,16 +438,16 @@ extern "C" int32_t hl_pipe_wait_outputs(hl_pipe* p, void* stream) {
 }
 
 extern "C" int32_t hl_pipe_wait_counts(hl_pipe* p, void* stream) {
-    // perm and counts of the mini-batch last stepped are final once its hl_fragment has run
+    // perm and counts of the mini-batch last stepped are final once its index work has run
     if (!p) return HL_EINVAL;
     if (p->j_done == 0) return HL_OK;
-    return wait(static_cast<cudaStream_t>(stream), p->ev[(p->j_done - 1) % p->n_sets].frag);
+    return wait(static_cast<cudaStream_t>(stream), p->ev[(p->j_done - 1) % p->n_sets].index);
 }
 
 extern "C" int32_t hl_pipe_drain(hl_pipe* p) {
     if (!p) return HL_EINVAL;
     HL_PIPE_TRY(flush_scatter(p));
-    cudaStream_t all[6] = {p->main, p->sa, p->sb, p->sc, p->link, p->wb};
+    cudaStream_t all[5] = {p->main, p->index, p->sort, p->link, p->wb};
     for (auto s : all)
         if (cudaStreamSynchronize(s) != cudaSuccess) return HL_ECUDA;
     return HL_OK;

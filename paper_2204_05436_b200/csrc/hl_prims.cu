@@ -1,6 +1,8 @@
 // Device-wide primitives used by several steps: single-pass exclusive scan and stable LSD radix sort of pairs
-// (one kernel per digit; tiles chained through status words instead of a separate scan of tile histograms).
+// (few pairs: one kernel of one cluster; many: one kernel per digit, tiles chained through status words).
 // Both take their element count from device memory, so that no step has to synchronise the host.
+#include <cooperative_groups.h>
+
 #include <atomic>
 
 #include "hl_common.cuh"
@@ -71,15 +73,6 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
 __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-__device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
 // ---- scan ---------------------------------------------------------------------------------------------------
 // st[0] = ticket counter, st[1 + tile] = status word of the tile; all zero on entry.
 // max_polls / stall_tile: see WaitCfg (a stalled tile publishes nothing, so that its successors' waits run out).
@@ -151,6 +144,80 @@ __global__ void __launch_bounds__(kThreads) k_scan_chained(const int32_t* in, in
 }
 
 // ---- radix sort ---------------------------------------------------------------------------------------------
+// Shared memory of the cluster sort: digit counters of every warp, then the pairs on their way to their new places.
+template <int NT, int ITEMS>
+struct SortSmem {
+    uint32_t cnt[NT / 32][256];
+    uint2 pair[NT * ITEMS];
+};
+
+// The valid lanes with the same 8-bit digit.  (Eight ballots: match.any does the same in one instruction but takes 60 cycles
+// of the multiprocessor for random digits, the ballots 24.)
+__device__ __forceinline__ unsigned same_digit(uint32_t d, bool valid) {
+    unsigned peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const unsigned with = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+        peers &= (d >> b) & 1u ? with : ~with;
+    }
+    return peers;
+}
+
+// Ranks a warp's items among the warp's items of the same digit (order: round, then lane) and counts them into cnt.
+template <int ITEMS>
+__device__ __forceinline__ void rank_in_warp(const uint32_t (&key)[ITEMS], int rounds, int n_mine, int shift,
+                                             uint32_t* cnt, uint32_t (&rank)[ITEMS]) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = lanemask_lt();
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        if (r >= rounds) break;
+        const bool valid = r * 32 + lane < n_mine;
+        const uint32_t d = (key[r] >> shift) & 255u;
+        const unsigned peers = same_digit(d, valid);
+        const uint32_t before = valid ? cnt[d] : 0u;
+        __syncwarp();
+        rank[r] = before + __popc(peers & lt);
+        if (valid && (peers & lt) == 0) cnt[d] = before + __popc(peers);
+        __syncwarp();
+    }
+}
+
+// NT / 256 threads per digit (digit = thread / (NT / 256)): turns the warps' counts of a digit into prefix sums over the
+// warps; returns the digit's total, the same in all threads of the digit.
+template <int NT>
+__device__ __forceinline__ uint32_t prefix_over_warps(uint32_t (*cnt)[256]) {
+    constexpr int PD = NT / 256, PER = NT / 32 / PD;
+    const int d = threadIdx.x / PD, q = threadIdx.x % PD;
+    uint32_t c[PER], mine = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        c[k] = cnt[q * PER + k][d];
+        mine += c[k];
+    }
+    uint32_t run = 0, total = 0;
+#pragma unroll
+    for (int k = 0; k < PD; ++k) {
+        const uint32_t o = __shfl_sync(0xffffffffu, mine, k, PD);
+        if (k < q) run += o;
+        total += o;
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        cnt[q * PER + k][d] = run;
+        run += c[k];
+    }
+    return total;
+}
+
+// Exclusive scan over the 256 digits of a value that the digit's PD threads share (only the first thread's counts, and
+// only it gets the result).  smem: 33 ints.
+template <int PD>
+__device__ __forceinline__ uint32_t scan_digits(uint32_t v, int* smem) {
+    int all;
+    return (uint32_t)block_exclusive_scan(threadIdx.x % PD == 0 ? (int)v : 0, smem, all);
+}
+
 // Digit histograms of all passes in one sweep over the keys.
 __global__ void __launch_bounds__(kThreads) k_sort_digit_hist(const int32_t* __restrict__ keys, const int32_t* d_n,
                                                               int64_t n_max, int passes,
@@ -202,8 +269,8 @@ __global__ void __launch_bounds__(kThreads) k_sort_pass(const int32_t* __restric
         const bool valid = idx < n;
         key[r] = valid ? keys_in[idx] : 0;
         val[r] = valid ? vals_in[idx] : 0;
-        const uint32_t d = valid ? (((uint32_t)key[r] >> shift) & 255u) : 256u;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t d = ((uint32_t)key[r] >> shift) & 255u;
+        const unsigned peers = same_digit(d, valid);
         uint32_t before = 0;
         if (valid) before = cnt[warp][d];
         __syncwarp();
@@ -271,55 +338,136 @@ __global__ void __launch_bounds__(kThreads) k_sort_pass(const int32_t* __restric
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_zero_words(uint32_t* p, int64_t n) {
-    for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n; i += (int64_t)gridDim.x * kThreads) p[i] = 0u;
+// The whole sort of at most CTAS * NT * ITEMS pairs in one kernel of one thread-block cluster.  The pairs stay in
+// registers; every pass ranks them by one digit, adds up the digit counts of the CTAs through distributed shared memory, and
+// sends each pair to the CTA that owns its new position (the last pass: to its place in the output).  CTA c owns
+// positions [c * per, (c + 1) * per).  One launch instead of a memset, the digit counts and a kernel per pass, and nothing
+// but the pairs themselves goes through the L2 (8 K pairs, three passes: 12.5 us, against 23 us in four kernels).
+template <int CTAS, int NT, int ITEMS>
+__global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__ keys_in,
+                                                               const int32_t* __restrict__ vals_in,
+                                                               int32_t* __restrict__ keys_out,
+                                                               int32_t* __restrict__ vals_out, const int32_t* d_n,
+                                                               int64_t n_max, int passes) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    constexpr int PD = NT / 256;                  // threads per digit
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    SortSmem<NT, ITEMS>& sm = *reinterpret_cast<SortSmem<NT, ITEMS>*>(sort_smem);
+    __shared__ uint32_t cta_hist[256];            // this CTA's digit counts, read by the other CTAs
+    __shared__ uint32_t digit_base[256];
+    __shared__ int scan_smem[40];
+    const int n = (int)clamp_n(d_n, n_max);
+    if (n == 0) return;                           // the same in all CTAs
+    const int cta = (int)cluster.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int per = (n + CTAS - 1) / CTAS;        // pairs per CTA
+    const int rounds = (per + NT - 1) / NT;
+    const uint32_t inv_per = (uint32_t)((0x100000000ull + per - 1) / per);       // pos / per = (pos * inv_per) >> 32
+    const int here = max(0, min(n - cta * per, per));
+    const int n_mine = max(0, min(here - warp * 32 * rounds, 32 * rounds));
+    const int first = warp * 32 * rounds;         // of this warp, within the CTA
+    uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        key[r] = val[r] = 0u;
+        if (r < rounds && r * 32 + lane < n_mine) {
+            key[r] = (uint32_t)keys_in[cta * per + first + r * 32 + lane];
+            val[r] = (uint32_t)vals_in[cta * per + first + r * 32 + lane];
+        }
+    }
+    for (int p = 0; p < passes; ++p) {
+        const int shift = 8 * p;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sm.cnt[warp][i * 32 + lane] = 0;
+        __syncwarp();
+        rank_in_warp<ITEMS>(key, rounds, n_mine, shift, sm.cnt[warp], rank);
+        __syncthreads();
+        const uint32_t total = prefix_over_warps<NT>(sm.cnt);
+        const int d = threadIdx.x / PD, q = threadIdx.x % PD;
+        if (q == 0) cta_hist[d] = total;
+        cluster.sync();     // all counts published; all CTAs have taken the previous pass's pairs out of shared memory
+        uint32_t before = 0, all = 0;             // of this digit: in the CTAs before mine, in all CTAs
+#pragma unroll
+        for (int k = 0; k < CTAS / PD; ++k) {
+            const int c = q * (CTAS / PD) + k;
+            const uint32_t v = *cluster.map_shared_rank(&cta_hist[d], c);
+            if (c < cta) before += v;
+            all += v;
+        }
+#pragma unroll
+        for (int o = 1; o < PD; o <<= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        const uint32_t smaller = scan_digits<PD>(all, scan_smem);
+        if (q == 0) digit_base[d] = smaller + before;
+        __syncthreads();
+        const bool last = p == passes - 1;
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            if (r >= rounds) break;
+            if (r * 32 + lane < n_mine) {
+                const uint32_t dg = (key[r] >> shift) & 255u;
+                const uint32_t pos = digit_base[dg] + sm.cnt[warp][dg] + rank[r];
+                if (last) {
+                    keys_out[pos] = (int32_t)key[r];
+                    vals_out[pos] = (int32_t)val[r];
+                } else {
+                    const uint32_t owner = __umulhi(pos, inv_per);
+                    *cluster.map_shared_rank(&sm.pair[pos - owner * per], owner) = make_uint2(key[r], val[r]);
+                }
+            }
+        }
+        cluster.sync();     // every pair has arrived (after the last pass: no CTA leaves while others read its counts)
+        if (last) break;
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            if (r >= rounds) break;
+            if (r * 32 + lane < n_mine) {
+                const uint2 x = sm.pair[first + r * 32 + lane];
+                key[r] = x.x;
+                val[r] = x.y;
+            }
+        }
+    }
+}
+
+constexpr int kClusterNT = 512, kClusterItems = 4;
+
+// CTAs of the widest cluster the current device can place: 16 (a non-portable size), 8, or 0; asked once per device.
+int sort_cluster_ctas() {
+    static std::atomic<int> known[64];            // 0 = not asked yet, else the answer + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    const int k = known[dev].load(std::memory_order_acquire);
+    if (k > 0) return k - 1;
+    auto can = [](auto* kernel, int ctas) {
+        constexpr size_t kBytes = sizeof(SortSmem<kClusterNT, kClusterItems>);
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ctas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(kClusterNT);
+        cfg.dynamicSmemBytes = kBytes;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+               cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBytes) == cudaSuccess &&
+               cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1;
+    };
+    const int ctas = can(k_sort_cluster<16, kClusterNT, kClusterItems>, 16)
+                         ? 16
+                         : (can(k_sort_cluster<8, kClusterNT, kClusterItems>, 8) ? 8 : 0);
+    (void)cudaGetLastError();
+    known[dev].store(ctas + 1, std::memory_order_release);
+    return ctas;
 }
 
 }  // namespace
-
-// ---- the same two primitives, launched from the device --------------------------------------------------------
-// For a kernel that learns on the device that follow-up work is needed (the cold-row search beyond its one-cluster
-// path): ONE thread calls these; every launch goes to the tail-launch stream of the calling grid, i.e. runs after
-// that grid has finished, one launch after the other, before anything the host queued behind the grid.  n is known
-// here, so the grids are exact.  A launch the device runtime refuses sets HL_ECUDA in *status.
-__device__ static void tail_check(int32_t* status) {
-    if (cudaGetLastError() != cudaSuccess) set_status(status, HL_ECUDA);
-}
-
-__device__ int radix_sort_pairs_tail(int32_t* keys0, int32_t* keys1, int32_t* vals0, int32_t* vals1, int64_t n,
-                                     int key_bits, uint32_t* hist, int32_t* status, int max_polls) {
-    if (n <= 0) return 0;
-    const int64_t n_tiles = (n + kSortTile - 1) / kSortTile;
-    const int passes = (key_bits + 7) / 8;
-    uint32_t* ghist = hist;
-    uint32_t* ticket = hist + 4 * 256;
-    uint32_t* tstat = hist + 4 * 256 + 8;
-    const int64_t words = 4 * 256 + 8 + (int64_t)passes * n_tiles * 256;
-    int64_t zero_grid = (words + kThreads * 8 - 1) / (kThreads * 8);
-    k_zero_words<<<(unsigned)(zero_grid < 1024 ? zero_grid : 1024), kThreads, 0, cudaStreamTailLaunch>>>(hist, words);
-    int64_t hist_grid = (n + kThreads * 8 - 1) / (kThreads * 8);
-    k_sort_digit_hist<<<(unsigned)hist_grid, kThreads, 0, cudaStreamTailLaunch>>>(keys0, nullptr, n, passes, ghist);
-    int32_t* k[2] = {keys0, keys1};
-    int32_t* v[2] = {vals0, vals1};
-    int cur = 0;
-    for (int p = 0; p < passes; ++p) {
-        k_sort_pass<<<(unsigned)n_tiles, kThreads, 0, cudaStreamTailLaunch>>>(
-            k[cur], v[cur], k[cur ^ 1], v[cur ^ 1], nullptr, n, 8 * p, ghist + 256 * p, ticket + p,
-            tstat + (size_t)p * n_tiles * 256, status, max_polls, (int64_t)-1);
-        cur ^= 1;
-    }
-    tail_check(status);
-    return cur;
-}
-
-__device__ void exclusive_scan_i32_tail(const int32_t* in, int32_t* out, int64_t n, int32_t* tiles, int32_t* status,
-                                        int max_polls) {
-    const int64_t n_tiles = n / kScanTile + 1;
-    k_zero_words<<<1, kThreads, 0, cudaStreamTailLaunch>>>(reinterpret_cast<uint32_t*>(tiles), 2 * (n_tiles + 1));
-    k_scan_chained<<<(unsigned)n_tiles, kThreads, 0, cudaStreamTailLaunch>>>(
-        in, out, nullptr, n, reinterpret_cast<unsigned long long*>(tiles), status, max_polls, (int64_t)-1);
-    tail_check(status);
-}
 
 int32_t exclusive_scan_i32(const int32_t* in, int32_t* out, const int32_t* d_n, int64_t n_max, int32_t* tiles,
                            int32_t* status, cudaStream_t stream, WaitCfg w) {
@@ -337,34 +485,64 @@ int32_t exclusive_scan_i32(const int32_t* in, int32_t* out, const int32_t* d_n, 
     return HL_OK;
 }
 
+// One cluster takes up to 2 048 pairs per CTA (32 768 with 16 CTAs).  Beyond that the exchange through distributed shared
+// memory takes longer than the chip-wide passes: 106 K pairs in three passes 40 us, against 30 with the tiles.
+// (With a tile made to stall -- the test of the bounded waits -- the chained passes are what is asked for.)
+static bool sort_in_cluster(int64_t n_max, const WaitCfg& w) {
+    return n_max <= (int64_t)sort_cluster_ctas() * kClusterNT * kClusterItems && w.stall_tile < 0;
+}
+
+int64_t sort_clear_words(int64_t n_max, int key_bits, WaitCfg w) {
+    if (n_max <= 0 || sort_in_cluster(n_max, w)) return 0;
+    return 4 * 256 + 8 + (int64_t)((key_bits + 7) / 8) * div_up(n_max, kSortTile) * 256;
+}
+
 int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n, int64_t n_max, int key_bits,
                          uint32_t* hist, int32_t* status, int32_t** out_keys, int32_t** out_vals,
-                         cudaStream_t stream, WaitCfg w) {
-    int cur = 0;
-    if (n_max > 0) {
-        const int64_t n_tiles = div_up(n_max, kSortTile);
-        const int passes = (key_bits + 7) / 8;
-        if (passes > 4) return HL_EINVAL;
-        // scratch: [4][256] digit counts, 8 ticket words, [4][n_tiles][256] tile status words
-        uint32_t* ghist = hist;
-        uint32_t* ticket = hist + 4 * 256;
-        uint32_t* tstat = hist + 4 * 256 + 8;
-        HL_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (4 * 256 + 8 + (size_t)passes * n_tiles * 256),
-                                    stream));
-        k_sort_digit_hist<<<grid_for(n_max, kThreads * 8, 1024), kThreads, 0, stream>>>(keys[0], d_n, n_max,
-                                                                                            passes, ghist);
-        for (int p = 0; p < passes; ++p) {
-            k_sort_pass<<<(unsigned)n_tiles, kThreads, 0, stream>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1],
-                                                                    d_n, n_max, 8 * p, ghist + 256 * p, ticket + p,
-                                                                    tstat + (size_t)p * n_tiles * 256, status,
-                                                                    w.max_polls, w.stall_tile);
-            cur ^= 1;
-        }
-        note_launches(1 + passes);
-        HL_LAUNCH_CHECK();
+                         cudaStream_t stream, WaitCfg w, bool counted) {
+    const int passes = n_max > 0 ? (key_bits + 7) / 8 : 0;
+    if (passes > 4) return HL_EINVAL;
+    const int out = passes & 1;
+    *out_keys = keys[out];
+    *out_vals = vals[out];
+    if (n_max <= 0) return HL_OK;
+    if (sort_in_cluster(n_max, w)) {
+        const int ctas = sort_cluster_ctas();
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ctas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(kClusterNT);
+        cfg.dynamicSmemBytes = sizeof(SortSmem<kClusterNT, kClusterItems>);
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        HL_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctas == 16 ? k_sort_cluster<16, kClusterNT, kClusterItems>
+                                                        : k_sort_cluster<8, kClusterNT, kClusterItems>,
+                                       (const int32_t*)keys[0], (const int32_t*)vals[0], keys[out], vals[out], d_n, n_max,
+                                       passes));
+        note_launches(1);
+        return HL_OK;
     }
-    *out_keys = keys[cur];
-    *out_vals = vals[cur];
+    const int64_t n_tiles = div_up(n_max, kSortTile);
+    // scratch: [4][256] digit counts, 8 ticket words, [passes][n_tiles][256] tile status words
+    uint32_t* ghist = hist;
+    uint32_t* ticket = hist + 4 * 256;
+    uint32_t* tstat = hist + 4 * 256 + 8;
+    if (!counted) {
+        HL_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * sort_clear_words(n_max, key_bits, w), stream));
+        k_sort_digit_hist<<<grid_for(n_max, kThreads * 8, 1024), kThreads, 0, stream>>>(keys[0], d_n, n_max, passes, ghist);
+        note_launches(1);
+    }
+    for (int p = 0; p < passes; ++p)
+        k_sort_pass<<<(unsigned)n_tiles, kThreads, 0, stream>>>(keys[p & 1], vals[p & 1], keys[(p & 1) ^ 1],
+                                                                vals[(p & 1) ^ 1], d_n, n_max, 8 * p, ghist + 256 * p, ticket + p,
+                                                                tstat + (size_t)p * n_tiles * 256, status, w.max_polls,
+                                                                w.stall_tile);
+    note_launches(passes);
+    HL_LAUNCH_CHECK();
     return HL_OK;
 }
 

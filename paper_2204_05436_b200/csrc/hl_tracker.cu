@@ -203,7 +203,7 @@ extern "C" int32_t hl_tracker_update(hl_ctx* ctx, const hl_batch* b, int32_t* d_
     note_launches(1);
     HL_LAUNCH_CHECK();
     int32_t *keys, *vals;
-    const int32_t st = radix_sort_pairs(r.bwd_keys, r.bwd_vals, r.bwd_n, ctx->max_nnz, bits_for(n_sets), r.bwd_hist,
+    const int32_t st = radix_sort_pairs(r.bwd_keys, r.bwd_vals, r.bwd_n, ctx->max_nnz, bits_for(n_sets), r.bwd_hist[0],
                                         r.status, &keys, &vals, stream);
     if (st != HL_OK) return st;
     k_trk_replay<<<grid_for(ctx->max_nnz, kThreads, kMaxGrid), kThreads, 0, stream>>>(keys, vals, r.bwd_n, ctx->max_nnz,

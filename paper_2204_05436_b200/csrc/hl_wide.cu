@@ -61,9 +61,8 @@ size_t carve(char* base, hl_wide* w) {
         w->sort_vals[i] = c.take<int32_t>(sort_n);
     }
     w->sort_hist = c.take<uint32_t>(sort_hist_words(sort_n));
-    w->frag_flags = c.take<uint8_t>(w->max_batch);
-    w->frag_scan = c.take<int32_t>(w->max_bags + 2);
-    w->frag_tiles = c.take<int32_t>(scan_tile_words(w->max_bags));
+    w->frag_words = c.take<uint32_t>(w->max_batch / 32 + 1);
+    w->frag_chain = c.take<unsigned long long>(frag_chain_words(w->max_bags));
     w->cold_tab = c.take<int32_t>(nnz);
     w->cold_idx = c.take<int32_t>(nnz);
     w->cold_pos = c.take<int32_t>(nnz);
@@ -274,7 +273,8 @@ extern "C" int32_t hl_wide_create(hl_wide** out, const hl_geometry* geom, int32_
     if (e == cudaSuccess) e = cudaMemset(w->c_cnt, 0, sizeof(uint32_t) * w->counter_slots);
     if (e == cudaSuccess) e = cudaMemset(w->r_keys, 0xff, sizeof(long long) * w->remap_slots);
     if (e == cudaSuccess) e = cudaMemset(w->sel, 0, sizeof(SelectState));
-    if (e == cudaSuccess) e = cudaMemset(w->frag_tiles, 0, sizeof(int32_t) * scan_tile_words(w->max_bags));
+    if (e == cudaSuccess)
+        e = cudaMemset(w->frag_chain, 0, sizeof(unsigned long long) * frag_chain_words(w->max_bags));
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         free(w->h_table_base);
