@@ -171,6 +171,7 @@ extern "C" int32_t hl_set_host_tables(hl_ctx* ctx, float* const* h_table_bases) 
 extern "C" int32_t hl_set_mover_ctas(hl_ctx* ctx, int32_t read_ctas, int32_t write_ctas) {
     if (!ctx || read_ctas < 0 || write_ctas < 0) return HL_EINVAL;
     const int most = 2 * ctx_sms(ctx);
+    ctx->mover_width_set = read_ctas != 0 || write_ctas != 0;
     ctx->mover_ctas = read_ctas == 0 ? kReadCtasDefault : (read_ctas < most ? read_ctas : most);
     ctx->scatter_ctas = write_ctas == 0 ? kMoverCtasDefault : (write_ctas < most ? write_ctas : most);
     return HL_OK;

@@ -236,27 +236,39 @@ __device__ __forceinline__ void bulk_store(void* gmem_dst, const void* smem_src,
 }
 
 constexpr int kBulkThreads = 128;
-constexpr int kBulkStages = 2;
-constexpr int kBulkStageBytes = 16384;
+constexpr int kBulkStages = 3;
+constexpr int kBulkStageBytes = 12288;
 constexpr int kBulkMaxPolls = 1 << 22;
-constexpr int kBulkStagesPerCta = 16;     // stages of rows per working CTA before another CTA joins in
-// Working CTAs of the mover inside a schedule (hl_set_mover_ctas changes it per context).  16 CTAs x 2 stages x
-// 16 KB keep 512 KB of rows in flight: 16 K rows of 256 bytes take about 150 us to read and 120 us to write back
-// next to the other streams' kernels.  More CTAs move the rows faster (about 100 us with 2 per SM, alone), fewer
-// slower (one CTA writes back 64 rows every 3.4 us); what a transfer costs the kernels that run next to it hardly
-// depends on that, so the host read, which nothing else of its mini-batch waits for at once, runs on 24 CTAs (about
-// 135 us) and the write-back on 16.  (The hot-cache load of hl_build_remap and hl_flush_hot, which run alone, use
-// 2 CTAs per SM and reach 90 % of the memcpy rate.)  The defaults, kReadCtasDefault and kMoverCtasDefault, are set at
-// hl_create.
+constexpr int kBulkStagesPerCta = 200;    // stages of rows per working CTA before another CTA joins in
+// How many rows are on the link at a time decides what the transfer costs everything else on the chip.  The link takes
+// some 300 M requests a second (a request: a row's 128-byte line, or what there is of it) and answers in about 1.5 us, so
+// 400 to 500 outstanding requests fill it; any more queue up in front of it, and the memory system behind the queue comes
+// to a near standstill.  Measured beside write-backs of random rows of 64 bytes (256 bytes): 16 CTAs that put up to 32 KB
+// each on the way move 288 M (302 M) requests a second, a streaming read of 256 MB takes 217 us (104) instead of 62, and a
+// kernel that does next to nothing takes 24 us (12) instead of 4; 8 CTAs with 48 requests each move 210 M (193 M), and
+// the read takes 65 us (66), the small kernel 6.8 us (6.4).  Reads of host rows are milder: 8 CTAs with 16 KB each reach
+// 226 M (259 M) requests a second, and the streaming read takes 67 us (68).  So inside a schedule a transfer that is short
+// all the same is paced: writes with kPacedRequests requests per CTA and every store completed before the next ones start,
+// reads with two stages of kPacedReadBytes on the way.  16 CTAs of these move the 7.4 thousand rows of 64 bytes of a
+// click-log mini-batch in 34 us (in) and 29 us (out), the 8.7 thousand rows of 256 bytes of a DLRM-sized one in 75 us and
+// 70 us: what the full-rate mover takes while nothing else runs, and one pass of the schedule went from 174 to 157 us
+// (DLRM-sized) and from 86 to 76 us (click log).  Above kPacedMost requests the link is what the mini-batch waits for, and
+// the mover takes it all.
+constexpr int kPacedRequests = 40;
+constexpr int kPacedReadBytes = 8192;
+constexpr int64_t kPacedMost = 1 << 16;
 
 // What a launch of the mover needs to know about its context.
 struct MoveCfg {
     int sms;            // multiprocessors of the device: the launch has at most 2 CTAs per SM
-    int min_ctas;       // CTAs that work however few rows there are
+    int min_ctas;       // CTAs that work however few rows there are (at full rate)
+    int paced_ctas;     // CTAs of a paced transfer; 0: never paced
     int max_polls;      // poll limit of the wait for a stage to fill
     int stall;          // tests only: CTA 0 issues no loads for its first stage, whose wait then runs out
 };
 
+// One row per thread and stage.  While the rows of one stage travel, the next stage's are requested (and the row ids of
+// the one after that are read): the loop waits for one thing at a time.
 template <bool TO_TABLE>
 __global__ void __launch_bounds__(kBulkThreads) k_move_rows_bulk(float* dense_side, int64_t dense_row0, TableMap table,
                                                                  const int32_t* __restrict__ rows,
@@ -264,66 +276,72 @@ __global__ void __launch_bounds__(kBulkThreads) k_move_rows_bulk(float* dense_si
                                                                  int64_t table_rows, int row_bytes,
                                                                  int rows_per_stage,
                                                                  const int32_t* __restrict__ skip, int32_t* status,
-                                                                 int min_ctas, int max_polls, int stall) {
+                                                                 int min_ctas, int paced_ctas, int64_t paced_most,
+                                                                 int paced_rows, int max_polls, int stall) {
     __shared__ __align__(128) unsigned char stage[kBulkStages][kBulkStageBytes];
     __shared__ __align__(8) uint64_t mbar[kBulkStages];
-    __shared__ unsigned int stage_bytes[kBulkStages];
     __shared__ int s_gave_up;
     int64_t n = *d_n;
     n = n < 0 ? 0 : (n < n_max ? n : n_max);
     const int tid = threadIdx.x;
     if (tid == 0) {
-        for (int s = 0; s < kBulkStages; ++s) {
+        for (int s = 0; s < kBulkStages; ++s)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&mbar[s])), "r"(1) : "memory");
-            stage_bytes[s] = 0;
-        }
         s_gave_up = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     unsigned char* dense = reinterpret_cast<unsigned char*>(dense_side) + dense_row0 * row_bytes;
+    const bool paced = paced_ctas > 0 && n <= paced_most;
+    if (paced) rows_per_stage = paced_rows;
     const int64_t n_batches = (n + rows_per_stage - 1) / rows_per_stage;
     // The launch has as many CTAs as the largest transfer could use; how many of them work is decided here, from the
-    // number of rows there really are: min_ctas for a mini-batch's worth of a DLRM-sized model (more would only slow
+    // number of rows there really are: few for a mini-batch's worth of a DLRM-sized model (more would only slow
     // the kernels that run beside the mover), up to all of them when a mini-batch moves hundreds of thousands of rows
     // (the link is then all that matters): one more CTA for every kBulkStagesPerCta stages of rows.
     int64_t active = n_batches / kBulkStagesPerCta;
     active = active < min_ctas ? min_ctas : active;
+    if (paced) active = paced_ctas;
     active = active < (int64_t)gridDim.x ? active : (int64_t)gridDim.x;
     if ((int64_t)blockIdx.x >= active) return;
-    int it = 0;
-    for (int64_t b = blockIdx.x; b < n_batches; b += active, ++it) {
+
+    // this thread's row of a batch, -1 if it has none or the row does not move
+    auto row_of = [&](int64_t batch) -> int64_t {
+        const int64_t i = batch * rows_per_stage + tid;
+        if (tid >= rows_per_stage || i >= n) return -1;
+        const int64_t g = rows[i];
+        if (g >= table_rows) {
+            set_status(status, HL_EBOUNDS);
+            return -1;
+        }
+        return skip != nullptr && skip[i] >= 0 ? -1 : g;
+    };
+    auto dense_row = [&](int64_t batch) { return dense + (batch * rows_per_stage + tid) * row_bytes; };
+    // all threads: requests the rows of a batch into stage s
+    auto request = [&](int s, int64_t batch, int64_t g, bool withhold) {
+        const int moving = __syncthreads_count(g >= 0);
+        if (tid == 0)
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&mbar[s])),
+                         "r"((unsigned)moving * (unsigned)row_bytes)
+                         : "memory");
+        if (g >= 0 && !withhold)
+            bulk_load(&stage[s][tid * row_bytes], TO_TABLE ? dense_row(batch) : row_address(table, g, row_bytes),
+                      (uint32_t)row_bytes, &mbar[s]);
+    };
+
+    int64_t batch = blockIdx.x;
+    if (batch >= n_batches) return;
+    int64_t g = row_of(batch), g1 = batch + active < n_batches ? row_of(batch + active) : -1;
+    request(0, batch, g, stall && blockIdx.x == 0);          // (stall: tests; the expected bytes never arrive)
+    for (int it = 0; batch < n_batches; batch += active, ++it) {
         const int s = it % kBulkStages;
         const uint32_t parity = (uint32_t)(it / kBulkStages) & 1u;
-        const int64_t i0 = b * rows_per_stage;
-        const int cnt = (int)min((int64_t)rows_per_stage, n - i0);
-        // this thread's earlier stores out of stage s have finished reading shared memory
-        asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBulkStages - 1) : "memory");
-        __syncthreads();
-        // which of my rows move, and how many bytes the stage expects
-        unsigned int my_bytes = 0;
-        for (int r = tid; r < cnt; r += kBulkThreads) {
-            const int64_t g = rows[i0 + r];
-            const bool ok = g >= 0 && g < table_rows && !(skip != nullptr && skip[i0 + r] >= 0);
-            if (g >= table_rows) set_status(status, HL_EBOUNDS);
-            if (ok) my_bytes += (unsigned int)row_bytes;
+        if (batch + active < n_batches) {
+            // the stores that last left from the next stage's place have finished reading shared memory
+            asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kBulkStages - 2) : "memory");
+            request((it + 1) % kBulkStages, batch + active, g1, false);
         }
-        if (my_bytes) atomicAdd(&stage_bytes[s], my_bytes);
-        __syncthreads();
-        if (tid == 0) {
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(&mbar[s])),
-                         "r"(stage_bytes[s])
-                         : "memory");
-            stage_bytes[s] = 0;
-        }
-        const bool stalled = stall && blockIdx.x == 0 && it == 0;     // tests: the expected bytes never arrive
-        for (int r = tid; r < cnt && !stalled; r += kBulkThreads) {
-            const int64_t g = rows[i0 + r];
-            const bool ok = g >= 0 && g < table_rows && !(skip != nullptr && skip[i0 + r] >= 0);
-            if (!ok) continue;
-            const unsigned char* src = TO_TABLE ? dense + (i0 + r) * row_bytes : row_address(table, g, row_bytes);
-            bulk_load(&stage[s][r * row_bytes], src, (uint32_t)row_bytes, &mbar[s]);
-        }
+        const int64_t g2 = batch + 2 * active < n_batches ? row_of(batch + 2 * active) : -1;
         // wait for the stage to fill (bounded)
         uint32_t done = 0;
         for (int polls = 0; !done; ++polls) {
@@ -343,18 +361,18 @@ __global__ void __launch_bounds__(kBulkThreads) k_move_rows_bulk(float* dense_si
         // it was responsible for stay unmoved; the status word says so.
         __syncthreads();
         if (s_gave_up) break;
-        for (int r = tid; r < cnt; r += kBulkThreads) {
-            const int64_t g = rows[i0 + r];
-            const bool ok = g >= 0 && g < table_rows && !(skip != nullptr && skip[i0 + r] >= 0);
-            if (!ok) continue;
-            unsigned char* dst = TO_TABLE ? row_address(table, g, row_bytes) : dense + (i0 + r) * row_bytes;
-            bulk_store(dst, &stage[s][r * row_bytes], (uint32_t)row_bytes);
-        }
+        // (paced: this thread's earlier store has arrived)
+        if (TO_TABLE && paced) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if (g >= 0)
+            bulk_store(TO_TABLE ? row_address(table, g, row_bytes) : dense_row(batch), &stage[s][tid * row_bytes],
+                       (uint32_t)row_bytes);
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        g = g1;
+        g1 = g2;
     }
     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (s_gave_up) {
-        // loads of the abandoned stage that are still on their way get a bounded grace period to land before the
+        // loads of the abandoned stages that are still on their way get a bounded grace period to land before the
         // shared memory goes back to the SM
         for (int i = 0; i < 64; ++i) __nanosleep(1000);
     }
@@ -368,16 +386,20 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
     const int D4 = D / 4;
     const int row_bytes = D * 4;
     if (row_bytes <= kBulkStageBytes) {
-        const int rows_per_stage = kBulkStageBytes / row_bytes;
+        const int rows_per_stage = kBulkStageBytes / row_bytes < kBulkThreads ? kBulkStageBytes / row_bytes : kBulkThreads;
         const int grid = grid_for(n_max, rows_per_stage, 2 * cfg.sms);
+        const int requests = (row_bytes + 127) / 128;        // of one row
+        const int paced_fit = TO_TABLE ? kPacedRequests / requests : kPacedReadBytes / row_bytes;
+        const int paced_rows = paced_fit > 1 ? paced_fit : 1;
         k_move_rows_bulk<TO_TABLE><<<grid, kBulkThreads, 0, stream>>>(
             dense_side, dense_row0, table, rows, d_n, n_max, table_rows, row_bytes, rows_per_stage, skip, status,
-            cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.max_polls, cfg.stall);
+            cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, kPacedMost / requests,
+            paced_rows < rows_per_stage ? paced_rows : rows_per_stage, cfg.max_polls, cfg.stall);
         note_launches(1);
         HL_LAUNCH_CHECK();
         return HL_OK;
     }
-    // Rows wider than a stage of the bulk mover (16 KB): plain 128-bit loads and stores, 48 CTAs x 16 groups x 16 rows
+    // Rows wider than a stage of the bulk mover (12 KB): plain 128-bit loads and stores, 48 CTAs x 16 groups x 16 rows
     // in flight on a third of the SMs, so that the kernels of the other streams keep CTA slots.
     const int grid = 48;
     if (D4 <= 4)
@@ -430,10 +452,11 @@ static TableMap table_map(const hl_ctx* ctx, const float* host_table) {
 
 // how the movers of this context are launched: beside the kernels of other mini-batches (`width` = the context's setting),
 // or alone on the chip (`width` = 0: two CTAs per SM, the link's full rate)
-static MoveCfg move_cfg(const hl_ctx* ctx, int width) {
+static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false) {
     MoveCfg c;
     c.sms = ctx_sms(ctx);
     c.min_ctas = width > 0 ? width : 2 * c.sms;
+    c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : kPacedCtas) : 0;
     c.max_polls = ctx->test_poll_limit > 0 ? ctx->test_poll_limit : kBulkMaxPolls;
     c.stall = ctx->test_poll_limit > 0 && ctx->test_stall_tile >= 0;
     return c;
@@ -500,7 +523,7 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 0, stream);
         const int32_t st = launch_move_rows<false>(d_cache, ctx->hot_cap + stage_row0,
                                                    table_map(ctx, host_table), d_cold_rows, d_n_cold, stage_rows,
-                                                   ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas),
+                                                   ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas, true),
                                                    r.status, stream);
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 1, stream);
         return st;
@@ -616,7 +639,7 @@ extern "C" int32_t hl_forward_cold(hl_ctx* ctx, float* d_cache, int64_t from_sta
 }
 
 static int32_t scatter_call(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,
-                            const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table,
+                            const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table, bool in_schedule,
                             void* stream_) {
     if (!ctx || !d_cache || !d_cold_rows || !d_n_cold || !host_table) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
@@ -625,7 +648,7 @@ static int32_t scatter_call(hl_ctx* ctx, const float* d_cache, int64_t stage_row
     const int32_t st = launch_move_rows<true>(const_cast<float*>(d_cache), ctx->hot_cap + stage_row0,
                                               table_map(ctx, host_table),
                                               d_cold_rows, d_n_cold, stage_rows, ctx->N, ctx->D, nullptr,
-                                              move_cfg(ctx, ctx->scatter_ctas), ctx->r.status, stream);
+                                              move_cfg(ctx, ctx->scatter_ctas, in_schedule), ctx->r.status, stream);
     timer_mark(ctx, HL_TIMER_SCATTER_MOVE, 1, stream);
     return st;
 }
@@ -633,14 +656,14 @@ static int32_t scatter_call(hl_ctx* ctx, const float* d_cache, int64_t stage_row
 extern "C" int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,
                                       const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table,
                                       void* stream) {
-    return scatter_call(ctx, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold, host_table, stream);
+    return scatter_call(ctx, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold, host_table, true, stream);
 }
 
 extern "C" int32_t hl_scatter_cold(hl_ctx* ctx, const float* d_cache, const int32_t* d_cold_rows,
                                    const int64_t* d_n_cold, float* host_table, void* stream_) {
     if (!ctx) return HL_EINVAL;
     // (one mini-batch after the other: nothing runs beside this)
-    return scatter_call(ctx, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold, host_table, stream_);
+    return scatter_call(ctx, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold, host_table, false, stream_);
 }
 
 extern "C" int32_t hl_flush_hot(hl_ctx* ctx, const float* d_cache, const int32_t* d_hot_rows, const int64_t* d_n_hot,

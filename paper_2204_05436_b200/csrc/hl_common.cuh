@@ -17,6 +17,7 @@ constexpr int kSelTile = 4096;             // rows per hot-set selection tile (2
 constexpr int kBwdChunk = 32;              // sorted lookups per backward chunk
 constexpr int kMoverCtasDefault = 16;      // working CTAs of a host-link mover inside a schedule: write-backs
 constexpr int kReadCtasDefault = 24;       // ... and host reads (a wider read finishes sooner and costs the step nothing)
+constexpr int kPacedCtas = 16;             // ... of either, when the transfer is short and therefore paced (hl_cold.cu)
 // Per-mini-batch kernels are launched with one CTA per tile of work rather than as chip-filling persistent grids:
 // they run next to the host-link movers of another micro-batch, which slow down the SMs they sit on, and the
 // hardware block scheduler then simply hands those SMs fewer CTAs.
@@ -80,6 +81,7 @@ struct hl_ctx {
     int device;
     int sms;                           // multiprocessors of `device` (queried at hl_create)
     int mover_ctas, scatter_ctas;      // working CTAs of the host-link movers inside a schedule (hl_set_mover_ctas)
+    int mover_width_set;               // 1: chosen by the caller
     int fwd_ctas, bwd_ctas;            // CTAs per multiprocessor of the forward / backward-sum kernel (0 = default)
     int test_poll_limit;               // > 0: poll limit of the bounded device waits (hl_test_bounded_waits)
     int64_t test_stall_tile;           // with it: the tile / mover stage that never delivers (-1: none)
