@@ -81,10 +81,74 @@ __device__ __forceinline__ void pool_long_bag(const float4* __restrict__ rows, c
     }
 }
 
+// The bags [bag0, bag1), one after the other, by one warp (rows wider than 64 fp32).  A warp reads 32 lookups with one load
+// and checks them with one vote, so that a row costs its load, its additions, a shuffle and an address; and the next 32 (of
+// the next bag, if this one ends) are on their way meanwhile, so that a bag starts without waiting for its ids.  2.6 M
+// lookups of 512-byte rows in bags of 20 on average: 154 us (8.9 TB/s out of the L2, which is what bounds it: neither 6 or 8
+// rows at a time nor a fifth CTA per multiprocessor gains anything, they lose 5-25 %); with every lane reading and
+// checking every id, four at a time and bag by bag (pool_long_bag), 183 us.
+template <int NV>
+__device__ __forceinline__ void pool_bags(const float4* __restrict__ rows, const int32_t* __restrict__ ids,
+                                          const int32_t* __restrict__ offsets, int64_t bag0, int64_t bag1, int lane, int D4,
+                                          int64_t n_slots, float4* __restrict__ out4, int32_t* status) {
+    constexpr int U = NV >= 4 ? 1 : 4 / NV;
+    int col[NV];                                   // (lanes past the row's end read its last column and store nothing)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) col[v] = min(lane + v * 32, D4 - 1);
+    int32_t lo = __ldg(&offsets[bag0]), end = __ldg(&offsets[bag0 + 1]);
+    const int32_t all_end = __ldg(&offsets[bag1]);
+    auto ids_at = [&](int32_t q) { return q + lane < all_end ? __ldg(&ids[q + lane]) : -1; };
+    int32_t mine = ids_at(lo);
+    for (int64_t bag = bag0; bag < bag1; ++bag) {
+        const int32_t next_end = bag + 1 < bag1 ? __ldg(&offsets[bag + 2]) : end;
+        double acc[NV][4] = {};
+        while (lo < end) {
+            const int n = min(32, end - lo);
+            const int32_t next = ids_at(lo + n);
+            if (lane < n && mine >= n_slots) set_status(status, HL_EBOUNDS);
+            const unsigned good = __ballot_sync(0xffffffffu, lane < n && (uint32_t)mine < (uint32_t)n_slots);
+            const int rows_n = __popc(good);
+            if (rows_n < n) {                      // skipped lookups (negative ids) among them: close the gaps
+                const int from = lane < rows_n ? (int)__fns(good, 0, lane + 1) : 0;
+                mine = __shfl_sync(0xffffffffu, mine, from);
+            }
+            auto some = [&](int k0, int most) {    // rows k0 .. of the chunk; most = U unless they are the last
+                float4 r[U][NV];
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    const int64_t id = __shfl_sync(0xffffffffu, mine, k0 + k);
+#pragma unroll
+                    for (int v = 0; v < NV; ++v)
+                        if (k < most) r[k][v] = __ldg(&rows[id * D4 + col[v]]);
+                }
+#pragma unroll
+                for (int k = 0; k < U; ++k)
+                    if (k < most) {
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) add_row(acc[v], r[k][v]);
+                    }
+            };
+            int k0 = 0;
+#pragma unroll 1
+            for (; k0 + U <= rows_n; k0 += U) some(k0, U);
+            if (k0 < rows_n) some(k0, rows_n - k0);
+            lo += n;
+            mine = next;
+        }
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+            if (lane + v * 32 < D4)
+                __stcs(&out4[bag * D4 + (lane + v * 32)],
+                       make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]));
+        end = next_end;
+    }
+}
+
 // A group of G lanes takes UB consecutive bags per trip.  Bags of at most one lookup (the one-hot case) are plain
 // row copies: the UB rows are loaded at once (UB independent 128-bit loads per lane), and the offsets and ids of
 // the NEXT trip are requested before those rows are consumed, so that the offsets -> id -> row chain of one trip
 // hides behind the rows of another.  Longer bags go through pool_long_bag one after the other.
+// MANY: bags of several lookups are the rule; every warp takes an equal share of consecutive bags through pool_bags.
 // FORWARD: the launch also copies the staged rows that this mini-batch shares with the one before (ForwardRows), which no
 // bag of this launch reads.
 struct ForwardRows {
@@ -95,7 +159,7 @@ struct ForwardRows {
     int64_t n_max;
 };
 
-template <int G, int NV, int UB, bool FORWARD>
+template <int G, int NV, int UB, bool MANY, bool FORWARD>
 __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const float* __restrict__ cache,
                                                          const int32_t* __restrict__ ids,
                                                          const int32_t* __restrict__ offsets,
@@ -121,6 +185,13 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const 
     const int sub = threadIdx.x % G;
     const float4* __restrict__ rows = reinterpret_cast<const float4*>(cache);
     float4* __restrict__ out4 = reinterpret_cast<float4*>(out);
+
+    if (MANY) {
+        const int64_t warps = (int64_t)gridDim.x * (kThreads / 32), me = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
+        const int64_t first = n_bags * me / warps, last = n_bags * (me + 1) / warps;
+        if (first < last) pool_bags<NV>(rows, ids, offsets, first, last, threadIdx.x & 31, D4, n_slots, out4, status);
+        return;
+    }
 
     // lo/len of the UB bags of a trip, and the id of every bag that has exactly one lookup (-1 otherwise)
     auto load_index = [&](int64_t bag0, int32_t (&lo)[UB], int32_t (&len)[UB], int32_t (&id1)[UB]) {
@@ -706,9 +777,12 @@ int32_t launch_fwd(hl_ctx* ctx, const float* cache, const hl_ubatch* ub, const i
                    const ForwardRows* fr, cudaStream_t stream) {
     constexpr int UB = NV >= 4 ? 1 : (NV >= 2 ? 2 : 4);
     const int64_t bags_per_trip = (int64_t)(kThreads / G) * UB;
-    const int grid = grid_for(ctx->max_bags, (int)bags_per_trip, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
     timer_mark(ctx, HL_TIMER_FWD, 0, stream);
-    const auto kernel = fr ? k_embbag_fwd<G, NV, UB, true> : k_embbag_fwd<G, NV, UB, false>;
+    // more than 1.5 lookups per bag at most: the one-hot loop is not worth trying first
+    const bool many = G == 32 && 2 * ctx->max_nnz > 3 * (int64_t)ctx->max_bags;
+    const int grid = grid_for(ctx->max_bags, many ? kThreads / 32 : (int)bags_per_trip, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
+    const auto kernel = many ? (fr ? k_embbag_fwd<G, NV, UB, G == 32, true> : k_embbag_fwd<G, NV, UB, G == 32, false>)
+                             : (fr ? k_embbag_fwd<G, NV, UB, false, true> : k_embbag_fwd<G, NV, UB, false, false>);
     kernel<<<grid, kThreads, 0, stream>>>(cache, ub->ids, ub->offsets, d_n, ctx->max_batch, ctx->T * ctx->S, ctx->D / 4,
                                           ctx->hot_cap + ctx->staging_cap, out, ctx->r.status, fr ? *fr : ForwardRows{});
     timer_mark(ctx, HL_TIMER_FWD, 1, stream);
