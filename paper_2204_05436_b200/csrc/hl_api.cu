@@ -2,6 +2,8 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <new>
+
 #include "hl_common.cuh"
 
 namespace hl {
@@ -127,6 +129,7 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
         free(ctx);
         return HL_EINVAL;
     }
+    ctx->launches = new (std::nothrow) LaunchCache(4);
     ctx->h_table_base[0] = 0;
     for (int t = 0; t < ctx->T; ++t) ctx->h_table_base[t + 1] = ctx->h_table_base[t] + geom->table_rows[t];
 
@@ -146,6 +149,7 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
     if (e == cudaSuccess) e = cudaMemset(span_count_of(ctx), 0, 8 * sizeof(int32_t));   // kept zero between backward calls
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
+        delete ctx->launches;
         free(ctx->h_table_base);
         free(ctx);
         return HL_ECUDA;
@@ -216,6 +220,7 @@ extern "C" int32_t hl_destroy(hl_ctx* ctx) {
     for (int w = 0; w < HL_TIMER_COUNT; ++w)
         for (int e = 0; e < 2; ++e)
             if (ctx->timer[w][e]) cudaEventDestroy(ctx->timer[w][e]);
+    delete ctx->launches;
     free(ctx->h_table_base);
     free(ctx);
     return HL_OK;

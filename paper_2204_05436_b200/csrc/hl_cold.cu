@@ -391,10 +391,9 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
         const int requests = (row_bytes + 127) / 128;        // of one row
         const int paced_fit = TO_TABLE ? kPacedRequests / requests : kPacedReadBytes / row_bytes;
         const int paced_rows = paced_fit > 1 ? paced_fit : 1;
-        k_move_rows_bulk<TO_TABLE><<<grid, kBulkThreads, 0, stream>>>(
-            dense_side, dense_row0, table, rows, d_n, n_max, table_rows, row_bytes, rows_per_stage, skip, status,
-            cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, kPacedMost / requests,
-            paced_rows < rows_per_stage ? paced_rows : rows_per_stage, cfg.max_polls, cfg.stall);
+        HL_CUDA_TRY(launch(k_move_rows_bulk<TO_TABLE>, grid, kBulkThreads, stream, dense_side, dense_row0, table, rows, d_n,
+                           n_max, table_rows, row_bytes, rows_per_stage, skip, status,
+                           cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, kPacedMost / requests, paced_rows < rows_per_stage ? paced_rows : rows_per_stage, cfg.max_polls, cfg.stall));
         note_launches(1);
         HL_LAUNCH_CHECK();
         return HL_OK;
@@ -403,17 +402,17 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
     // in flight on a third of the SMs, so that the kernels of the other streams keep CTA slots.
     const int grid = 48;
     if (D4 <= 4)
-        k_move_rows<4, TO_TABLE><<<grid, kThreads, 0, stream>>>(dense_side, dense_row0, table, rows, d_n, n_max,
-                                                               table_rows, D4, skip, status);
+        HL_CUDA_TRY(launch(k_move_rows<4, TO_TABLE>, grid, kThreads, stream, dense_side, dense_row0, table, rows, d_n,
+                           n_max, table_rows, D4, skip, status));
     else if (D4 <= 8)
-        k_move_rows<8, TO_TABLE><<<grid, kThreads, 0, stream>>>(dense_side, dense_row0, table, rows, d_n, n_max,
-                                                               table_rows, D4, skip, status);
+        HL_CUDA_TRY(launch(k_move_rows<8, TO_TABLE>, grid, kThreads, stream, dense_side, dense_row0, table, rows, d_n,
+                           n_max, table_rows, D4, skip, status));
     else if (D4 <= 16)
-        k_move_rows<16, TO_TABLE><<<grid, kThreads, 0, stream>>>(dense_side, dense_row0, table, rows, d_n, n_max,
-                                                                table_rows, D4, skip, status);
+        HL_CUDA_TRY(launch(k_move_rows<16, TO_TABLE>, grid, kThreads, stream, dense_side, dense_row0, table, rows, d_n,
+                           n_max, table_rows, D4, skip, status));
     else
-        k_move_rows<32, TO_TABLE><<<grid, kThreads, 0, stream>>>(dense_side, dense_row0, table, rows, d_n, n_max,
-                                                                table_rows, D4, skip, status);
+        HL_CUDA_TRY(launch(k_move_rows<32, TO_TABLE>, grid, kThreads, stream, dense_side, dense_row0, table, rows, d_n,
+                           n_max, table_rows, D4, skip, status));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -432,8 +431,8 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
     const unsigned grid = (unsigned)div_up(words, kThreads * (many ? 4 : 1));
     const auto kernel = summary ? (many ? k_cold_rank<true, 4> : k_cold_rank<true, 1>)
                                 : (many ? k_cold_rank<false, 4> : k_cold_rank<false, 1>);
-    kernel<<<grid, kThreads, 0, stream>>>(marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.cold_n + 1, r.cold_chain,
-                                          r.status, wait_cfg(ctx).max_polls, clear, n_clear);
+    HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.cold_n + 1,
+                       r.cold_chain, r.status, wait_cfg(ctx).max_polls, clear, n_clear));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -483,17 +482,17 @@ int32_t index_begin(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, int64_t
                     int32_t* d_cold_rows, int64_t* d_n_cold, cudaStream_t stream) {
     Regions& r = ctx->r;
     if (ctx->max_nnz == 0) {
-        HL_CUDA_TRY(cudaMemsetAsync(d_n_cold, 0, sizeof(int64_t), stream));
+        HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(d_n_cold), 2, stream));
         return HL_OK;
     }
     if (!non->ids) return HL_EINVAL;
     const int grid = grid_for(ctx->max_nnz, kThreads, 4 * ctx_sms(ctx));
-    k_cold_classify<<<grid, kThreads, 0, stream>>>(non->ids, non->offsets, d_n_non, ctx->max_batch, ctx->T * ctx->S,
-                                                   non->cap_ids, ctx->N, BitmapProbe{r.remap}, cold_marks(ctx), r.status);
+    HL_CUDA_TRY(launch(k_cold_classify, grid, kThreads, stream, non->ids, non->offsets, d_n_non, ctx->max_batch,
+                       ctx->T * ctx->S, non->cap_ids, ctx->N, BitmapProbe{r.remap}, cold_marks(ctx), r.status));
     const int32_t st = cold_rank(ctx, stage_rows, d_cold_rows, d_n_cold, stream);
     if (st != HL_OK) return st;
-    k_cold_assign<<<grid, kThreads, 0, stream>>>(non->ids, non->offsets, d_n_non, ctx->max_batch, ctx->T * ctx->S,
-                                                 non->cap_ids, r.cold_ranked, ctx->hot_cap + stage_row0, stage_rows);
+    HL_CUDA_TRY(launch(k_cold_assign, grid, kThreads, stream, non->ids, non->offsets, d_n_non, ctx->max_batch,
+                       ctx->T * ctx->S, non->cap_ids, r.cold_ranked, ctx->hot_cap + stage_row0, stage_rows));
     note_launches(2);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -504,8 +503,8 @@ int32_t index_end(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
                   const int32_t* d_prev_rows, const int64_t* d_n_prev, int32_t* d_fwd_src, cudaStream_t stream) {
     if (ctx->max_nnz == 0) return HL_OK;
     if (d_prev_rows) {
-        k_cold_match<<<grid_for(stage_rows, kThreads, 2 * ctx_sms(ctx)), kThreads, 0, stream>>>(
-            d_cold_rows, d_n_cold, stage_rows, d_prev_rows, d_n_prev, ctx->staging_cap, d_fwd_src);
+        HL_CUDA_TRY(launch(k_cold_match, grid_for(stage_rows, kThreads, 2 * ctx_sms(ctx)), kThreads, stream, d_cold_rows,
+                           d_n_cold, stage_rows, d_prev_rows, d_n_prev, ctx->staging_cap, d_fwd_src));
         note_launches(1);
         HL_LAUNCH_CHECK();
     }
@@ -518,6 +517,7 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
                     cudaEvent_t record_after_index, cudaEvent_t wait_a, cudaEvent_t wait_b, bool do_index,
                     bool do_move, cudaStream_t stream) {
     Regions& r = ctx->r;
+    LaunchBatch batch(ctx->launches);
     if (!do_index) {
         if (ctx->max_nnz == 0) return HL_OK;
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 0, stream);
@@ -526,14 +526,15 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
                                                    ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas, true),
                                                    r.status, stream);
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 1, stream);
-        return st;
+        return batch.end(st);
     }
     int32_t st = index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold, stream);
     if (st != HL_OK) return st;
     st = index_end(ctx, stage_rows, d_cold_rows, d_n_cold, d_prev_rows, d_n_prev, d_fwd_src, stream);
     if (st != HL_OK) return st;
+    if (record_after_index || wait_a || wait_b) HL_CUDA_TRY(launch_flush());
     if (record_after_index) HL_CUDA_TRY(cudaEventRecord(record_after_index, stream));
-    if (!do_move) return HL_OK;
+    if (!do_move) return batch.end();
     if (wait_a) HL_CUDA_TRY(cudaStreamWaitEvent(stream, wait_a, 0));
     if (wait_b) HL_CUDA_TRY(cudaStreamWaitEvent(stream, wait_b, 0));
     timer_mark(ctx, HL_TIMER_GATHER_MOVE, 0, stream);
@@ -541,7 +542,7 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
                                  d_n_cold, stage_rows, ctx->N, ctx->D, d_prev_rows ? d_fwd_src : nullptr,
                                  move_cfg(ctx, ctx->mover_ctas), r.status, stream);
     timer_mark(ctx, HL_TIMER_GATHER_MOVE, 1, stream);
-    return st;
+    return batch.end(st);
 }
 
 bool window_ok(const hl_ctx* ctx, int64_t row0, int64_t rows) {
@@ -590,8 +591,9 @@ extern "C" int32_t hl_index_cold_begin(hl_ctx* ctx, hl_ubatch* non, const int32_
                                        int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold, void* stream_) {
     if (!ctx || !non || !non->offsets || !d_n_non || !d_cold_rows || !d_n_cold) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
-    return index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
-                       static_cast<cudaStream_t>(stream_));
+    LaunchBatch batch(ctx->launches);
+    return batch.end(index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+                                 static_cast<cudaStream_t>(stream_)));
 }
 
 extern "C" const int32_t* hl_index_cold_verdict(hl_ctx* ctx) { return ctx ? ctx->r.cold_n + 1 : nullptr; }
@@ -629,10 +631,14 @@ extern "C" int32_t hl_forward_cold(hl_ctx* ctx, float* d_cache, int64_t from_sta
     const int D4 = ctx->D / 4;
     const int grid = 2 * ctx_sms(ctx);
     const int64_t from = ctx->hot_cap + from_stage_row0, to = ctx->hot_cap + to_stage_row0;
-    if (D4 <= 4) k_forward_rows<4><<<grid, kThreads, 0, stream>>>(d_cache, from, to, d_fwd_src, d_n_cold, stage_rows, D4);
-    else if (D4 <= 8) k_forward_rows<8><<<grid, kThreads, 0, stream>>>(d_cache, from, to, d_fwd_src, d_n_cold, stage_rows, D4);
-    else if (D4 <= 16) k_forward_rows<16><<<grid, kThreads, 0, stream>>>(d_cache, from, to, d_fwd_src, d_n_cold, stage_rows, D4);
-    else k_forward_rows<32><<<grid, kThreads, 0, stream>>>(d_cache, from, to, d_fwd_src, d_n_cold, stage_rows, D4);
+    if (D4 <= 4) HL_CUDA_TRY(launch(k_forward_rows<4>, grid, kThreads, stream, d_cache, from, to, d_fwd_src, d_n_cold,
+                                    stage_rows, D4));
+    else if (D4 <= 8) HL_CUDA_TRY(launch(k_forward_rows<8>, grid, kThreads, stream, d_cache, from, to, d_fwd_src, d_n_cold,
+                                         stage_rows, D4));
+    else if (D4 <= 16) HL_CUDA_TRY(launch(k_forward_rows<16>, grid, kThreads, stream, d_cache, from, to, d_fwd_src,
+                                          d_n_cold, stage_rows, D4));
+    else HL_CUDA_TRY(launch(k_forward_rows<32>, grid, kThreads, stream, d_cache, from, to, d_fwd_src, d_n_cold, stage_rows,
+                            D4));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -644,13 +650,14 @@ static int32_t scatter_call(hl_ctx* ctx, const float* d_cache, int64_t stage_row
     if (!ctx || !d_cache || !d_cold_rows || !d_n_cold || !host_table) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    LaunchBatch batch(ctx->launches);
     timer_mark(ctx, HL_TIMER_SCATTER_MOVE, 0, stream);
     const int32_t st = launch_move_rows<true>(const_cast<float*>(d_cache), ctx->hot_cap + stage_row0,
                                               table_map(ctx, host_table),
                                               d_cold_rows, d_n_cold, stage_rows, ctx->N, ctx->D, nullptr,
                                               move_cfg(ctx, ctx->scatter_ctas, in_schedule), ctx->r.status, stream);
     timer_mark(ctx, HL_TIMER_SCATTER_MOVE, 1, stream);
-    return st;
+    return batch.end(st);
 }
 
 extern "C" int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,

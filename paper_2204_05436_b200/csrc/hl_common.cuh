@@ -5,6 +5,11 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <mutex>
+#include <tuple>
+#include <utility>
+#include <vector>
+
 #include "hotline.h"
 
 namespace hl {
@@ -69,6 +74,8 @@ struct Regions {
     int32_t* cold_n;                   // [4]; [1] = hl_index_cold_verdict
 };
 
+class LaunchCache;
+
 }  // namespace hl
 
 struct hl_ctx {
@@ -93,6 +100,8 @@ struct hl_ctx {
     // optional observer of the kernel timers' marks (the pipeline's trace): called with (user, which, end, stream)
     void (*mark_hook)(void*, int, int, cudaStream_t);
     void* mark_user;
+    // graphs of the calls that make several kernels, or one in a run of calls (nullptr: plain launches)
+    hl::LaunchCache* launches;
 };
 
 // Context of the wide-id index path (hl_wide_*): global row ids are 64-bit, every table still has fewer than 2^31
@@ -131,9 +140,9 @@ struct hl_wide {
 
 namespace hl {
 
-#define HL_CUDA_TRY(expr)                         \
+#define HL_CUDA_TRY(...)                          \
     do {                                          \
-        cudaError_t e__ = (expr);                 \
+        cudaError_t e__ = (__VA_ARGS__);          \
         if (e__ != cudaSuccess) return HL_ECUDA;  \
     } while (0)
 
@@ -142,8 +151,72 @@ namespace hl {
         if (cudaGetLastError() != cudaSuccess) return HL_ECUDA; \
     } while (0)
 
+// ---- launches (hl_graph.cu) -----------------------------------------------------------------------------------
+// Kernels are launched through `launch`.  Inside a LaunchBatch they are collected instead, per stream, and go out as one
+// graph at its end, when the stream changes, or at launch_flush(), which has to come before anything else is put on the
+// stream (an event, a memset).
+class LaunchCache {
+public:
+    explicit LaunchCache(int variants);              // graphs of the same kernels, with different arguments, worth keeping
+    ~LaunchCache();
+    LaunchCache(const LaunchCache&) = delete;
+    LaunchCache& operator=(const LaunchCache&) = delete;
+    cudaError_t launch(const void* recording, cudaStream_t stream);
+
+private:
+    static constexpr int kMaxEntries = 24;
+    struct Entry;
+    std::vector<Entry*> entries_;
+    std::mutex mutex_;
+    int variants_;
+    uint64_t tick_ = 0;
+};
+
+class LaunchBatch {
+public:
+    explicit LaunchBatch(LaunchCache* cache);        // nullptr, or inside another batch: nothing of its own
+    ~LaunchBatch();
+    int32_t end(int32_t st = HL_OK);                 // `st`, or HL_ECUDA if that is HL_OK and a launch failed
+
+private:
+    bool mine_;
+};
+
+cudaError_t launch_flush();
+cudaError_t clear_words(uint32_t* p, int64_t n_words, cudaStream_t stream);      // p[0 .. n_words) = 0
+cudaError_t launch_kernel(const void* func, dim3 grid, dim3 block, size_t smem, int cluster, void** args,
+                          const uint32_t* sizes, int n_args, cudaStream_t stream);
+
+template <typename... P, typename... A>
+cudaError_t launch_cluster(void (*kernel)(P...), int64_t grid, int block, size_t smem, int cluster, cudaStream_t stream,
+                           A&&... a) {
+    static_assert(sizeof...(P) == sizeof...(A), "one argument per parameter");
+    std::tuple<P...> args(static_cast<P>(a)...);
+    const uint32_t sizes[] = {(uint32_t)sizeof(P)...};
+    return std::apply(
+        [&](auto&... x) {
+            void* ptrs[] = {const_cast<void*>(static_cast<const void*>(&x))...};
+            return launch_kernel(reinterpret_cast<const void*>(kernel), dim3((unsigned)grid), dim3((unsigned)block), smem,
+                                 cluster, ptrs, sizes, (int)sizeof...(P), stream);
+        },
+        args);
+}
+template <typename... P, typename... A>
+cudaError_t launch(void (*kernel)(P...), int64_t grid, int block, cudaStream_t stream, A&&... a) {
+    return launch_cluster(kernel, grid, block, 0, 0, stream, std::forward<A>(a)...);
+}
+
+// f() with its launches collected in `cache` (nullptr: not)
+template <typename F>
+int32_t as_graph(LaunchCache* cache, F f) {
+    LaunchBatch batch(cache);
+    return batch.end(f());
+}
+
 // Records the start/end event of one of the optional kernel timers on `stream` (no-op unless enabled).
 inline void timer_mark(hl_ctx* ctx, int which, int end, cudaStream_t stream) {
+    if (!ctx->timing_on && !ctx->mark_hook) return;
+    launch_flush();
     if (ctx->timing_on && ctx->timer[which][end]) cudaEventRecord(ctx->timer[which][end], stream);
     if (ctx->mark_hook) ctx->mark_hook(ctx->mark_user, which, end, stream);
 }

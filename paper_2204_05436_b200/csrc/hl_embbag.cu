@@ -783,8 +783,8 @@ int32_t launch_fwd(hl_ctx* ctx, const float* cache, const hl_ubatch* ub, const i
     const int grid = grid_for(ctx->max_bags, many ? kThreads / 32 : (int)bags_per_trip, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
     const auto kernel = many ? (fr ? k_embbag_fwd<G, NV, UB, G == 32, true> : k_embbag_fwd<G, NV, UB, G == 32, false>)
                              : (fr ? k_embbag_fwd<G, NV, UB, false, true> : k_embbag_fwd<G, NV, UB, false, false>);
-    kernel<<<grid, kThreads, 0, stream>>>(cache, ub->ids, ub->offsets, d_n, ctx->max_batch, ctx->T * ctx->S, ctx->D / 4,
-                                          ctx->hot_cap + ctx->staging_cap, out, ctx->r.status, fr ? *fr : ForwardRows{});
+    HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, cache, ub->ids, ub->offsets, d_n, ctx->max_batch, ctx->T * ctx->S,
+                       ctx->D / 4, ctx->hot_cap + ctx->staging_cap, out, ctx->r.status, fr ? *fr : ForwardRows{}));
     timer_mark(ctx, HL_TIMER_FWD, 1, stream);
     note_launches(1);
     HL_LAUNCH_CHECK();
@@ -805,14 +805,13 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
     // The count is zero between calls: hl_create clears it and k_bwd_spans clears it again when it is done.
     int32_t* span_count = span_count_of(ctx);
     int32_t* span_list = span_count + 8;
-    k_bwd_chunks<G, NV><<<grid, kThreads, 0, stream>>>(cache, keys, vals, d_n_lookups, grad, ctx->D / 4, n_slots,
-                                                      lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list,
-                                                      ctx->max_bags, max_chunks, ctx->r.status);
+    HL_CUDA_TRY(launch(k_bwd_chunks<G, NV>, grid, kThreads, stream, cache, keys, vals, d_n_lookups, grad, ctx->D / 4,
+                       n_slots, lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list, ctx->max_bags, max_chunks,
+                       ctx->r.status));
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 1, stream);
     const int span_grid = grid_for(max_chunks * 32, kThreads, 4 * ctx_sms(ctx));   // the warps stride over the listed runs
-    k_bwd_spans<G, NV><<<span_grid, kThreads, 0, stream>>>(cache, keys, d_n_lookups, ctx->D / 4, n_slots, lr,
-                                                          ctx->r.bwd_part, d_first, key_bias, span_count,
-                                                          (const int32_t*)span_list, max_chunks);
+    HL_CUDA_TRY(launch(k_bwd_spans<G, NV>, span_grid, kThreads, stream, cache, keys, d_n_lookups, ctx->D / 4, n_slots, lr,
+                       ctx->r.bwd_part, d_first, key_bias, span_count, (const int32_t*)span_list, max_chunks));
     note_launches(2);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -867,7 +866,9 @@ int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, c
 
 extern "C" int32_t hl_embbag_fwd(hl_ctx* ctx, const float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples,
                                  float* d_out, void* stream) {
-    return fwd_call(ctx, d_cache, ub, d_n_samples, d_out, nullptr, static_cast<cudaStream_t>(stream));
+    return as_graph(ctx ? ctx->launches : nullptr, [&] {
+        return fwd_call(ctx, d_cache, ub, d_n_samples, d_out, nullptr, static_cast<cudaStream_t>(stream));
+    });
 }
 
 namespace hl {
@@ -907,7 +908,7 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
     // the tile sort wants its digit counts, which cost less here than in a sweep of their own
     const int64_t clear_words = sort_clear_words(ctx->max_nnz, key_bits, wait_cfg(ctx));
     const bool hist = clear_words > 0;
-    if (hist && !cleared) HL_CUDA_TRY(cudaMemsetAsync(sort_scratch, 0, sizeof(uint32_t) * clear_words, stream));
+    if (hist && !cleared) HL_CUDA_TRY(hl::clear_words(sort_scratch, clear_words, stream));
     // lanes per bag: by the most lookups a bag has on average
     const int lanes = ctx->max_nnz <= 4 * ctx->max_bags ? 1 : (ctx->max_nnz <= 16 * ctx->max_bags ? 8 : 32);
     const int grid = grid_for(ctx->max_bags, kThreads / lanes, (lanes == 1 ? 4 : 8) * ctx_sms(ctx));
@@ -919,10 +920,11 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
     const auto kernel = lanes == 1   ? pick(assign, hist, std::integral_constant<int, 1>())
                         : lanes == 8 ? pick(assign, hist, std::integral_constant<int, 8>())
                                      : pick(assign, hist, std::integral_constant<int, 32>());
-    kernel<<<grid, kThreads, 0, stream>>>(a);
+    HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, a));
     note_launches(1);
     HL_LAUNCH_CHECK();
     if (aside) {
+        HL_CUDA_TRY(launch_flush());
         HL_CUDA_TRY(cudaEventRecord(aside->pairs_ready, stream));
         HL_CUDA_TRY(cudaStreamWaitEvent(aside->stream, aside->pairs_ready, 0));
         stream = aside->stream;
@@ -950,12 +952,14 @@ extern "C" int32_t hl_embbag_bwd_sgd(hl_ctx* ctx, float* d_cache, const hl_ubatc
     if (ctx->max_nnz == 0) return HL_OK;
     if (!ub->ids) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    int32_t *keys, *vals;
-    int32_t st = sort_lookups(ctx, ub, d_n_samples, nullptr, nullptr, ctx->r.bwd_n, &keys, &vals, stream);
-    if (st != HL_OK) return st;
+    return as_graph(ctx->launches, [&]() -> int32_t {
+        int32_t *keys, *vals;
+        const int32_t st = sort_lookups(ctx, ub, d_n_samples, nullptr, nullptr, ctx->r.bwd_n, &keys, &vals, stream);
+        if (st != HL_OK) return st;
 #define HL_BWD(G, NV) launch_bwd<G, NV>(ctx, d_cache, keys, vals, ctx->r.bwd_n, d_grad_out, lr, stream)
-    HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
+        HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD
+    });
 }
 
 extern "C" int32_t hl_embbag_bwd_prepare(hl_ctx* ctx, const hl_ubatch* ub, const int32_t* d_n_samples,
@@ -968,8 +972,10 @@ extern "C" int32_t hl_embbag_bwd_prepare(hl_ctx* ctx, const hl_ubatch* ub, const
         return HL_OK;
     }
     if (!ub->ids || !d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
-    int32_t *keys, *vals;
-    return sort_lookups(ctx, ub, d_n_samples, d_sorted_slots, d_sorted_bags, d_n_lookups, &keys, &vals, stream);
+    return as_graph(ctx->launches, [&] {
+        int32_t *keys, *vals;
+        return sort_lookups(ctx, ub, d_n_samples, d_sorted_slots, d_sorted_bags, d_n_lookups, &keys, &vals, stream);
+    });
 }
 
 namespace hl {
@@ -996,9 +1002,11 @@ int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, 
     a.bags_follow = merge;
     a.side[0] = {pop->ids, pop->offsets, d_n_pop, 0};
     a.side[1] = {non->ids, non->offsets, d_n_non, merge ? 0 : (int32_t)(n_slots + 1)};
-    int32_t *ok, *ov;
-    return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, cleared, d_sorted_slots, d_sorted_bags,
-                          d_n_lookups, &ok, &ov, stream, aside);
+    return as_graph(ctx->launches, [&] {
+        int32_t *ok, *ov;
+        return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, cleared, d_sorted_slots, d_sorted_bags,
+                              d_n_lookups, &ok, &ov, stream, aside);
+    });
 }
 
 }  // namespace
@@ -1052,10 +1060,12 @@ extern "C" int32_t hl_embbag_bwd_apply2(hl_ctx* ctx, float* d_cache, const int32
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const int32_t* d_first = which == 0 ? nullptr : d_n_lookups;             // X's block starts behind O's
     const int32_t bias = which == 0 ? 0 : (int32_t)(ctx->hot_cap + ctx->staging_cap + 1);
+    return as_graph(ctx->launches, [&]() -> int32_t {
 #define HL_BWD(G, NV) \
     launch_bwd<G, NV>(ctx, d_cache, d_sorted_slots, d_sorted_bags, d_n_lookups + which, d_grad_out, lr, stream, d_first, bias)
-    HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
+        HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD
+    });
 }
 
 extern "C" int32_t hl_embbag_bwd_apply(hl_ctx* ctx, float* d_cache, const int32_t* d_sorted_slots,
@@ -1065,9 +1075,11 @@ extern "C" int32_t hl_embbag_bwd_apply(hl_ctx* ctx, float* d_cache, const int32_
     if (ctx->max_nnz == 0) return HL_OK;
     if (!d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
+    return as_graph(ctx->launches, [&]() -> int32_t {
 #define HL_BWD(G, NV) launch_bwd<G, NV>(ctx, d_cache, d_sorted_slots, d_sorted_bags, d_n_lookups, d_grad_out, lr, stream)
-    HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
+        HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD
+    });
 }
 
 // ---------------------------------------------------------------------------------------------------------------
@@ -1166,14 +1178,14 @@ extern "C" int32_t hl_embbag_bwd_sgd_static(float* d_cache, int64_t cache_rows, 
     p += kStaticHistBytes;
     tmp.r.bwd_part = reinterpret_cast<float*>(p);
 
-    k_static_begin<<<1, 1, 0, stream>>>(header, n_bags, span_count_of(&tmp));
+    HL_CUDA_TRY(launch(k_static_begin, 1, 1, stream, header, n_bags, span_count_of(&tmp)));
     note_launches(1);
     HL_LAUNCH_CHECK();
     hl_ubatch ub{const_cast<int32_t*>(d_offsets), const_cast<int32_t*>(d_ids), nnz};
     const int32_t st = hl_embbag_bwd_sgd(&tmp, d_cache, &ub, header + 8, d_grad_out, lr, stream_);
     if (st != HL_OK) return st;
     if (d_status) {
-        k_static_end<<<1, 1, 0, stream>>>(header, d_status);
+        HL_CUDA_TRY(launch(k_static_end, 1, 1, stream, header, d_status));
         note_launches(1);
         HL_LAUNCH_CHECK();
     }

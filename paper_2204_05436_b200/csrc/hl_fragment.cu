@@ -392,11 +392,11 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
                 non_offsets, non_cap, chain + 1, status, waits.max_polls, waits.stall_tile, d_dense, n_dense, d_dense_out};
     const int flag_grid = grid_for(B, 32, 4 * sms);
     if (b->nnz <= 4 * (int64_t)T * B)            // on average at most 4 lookups per input and table
-        k_frag_flags<true, Probe><<<flag_grid, kFlagThreads, 0, stream>>>(
-            b->indices, b->offsets, B, T, S, table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles);
+        HL_CUDA_TRY(launch(k_frag_flags<true, Probe>, flag_grid, kFlagThreads, stream, b->indices, b->offsets, B, T, S,
+                           table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles));
     else
-        k_frag_flags<false, Probe><<<flag_grid, kFlagThreads, 0, stream>>>(
-            b->indices, b->offsets, B, T, S, table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles);
+        HL_CUDA_TRY(launch(k_frag_flags<false, Probe>, flag_grid, kFlagThreads, stream, b->indices, b->offsets, B, T, S,
+                           table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles));
     // lanes per bag: by the average number of lookups
     const auto pick = [&](auto g) {
         constexpr int G = decltype(g)::value;
@@ -405,7 +405,7 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
     const auto place = 4 * b->nnz <= 5 * n_bags ? pick(std::integral_constant<int, 1>())
                        : b->nnz <= 8 * n_bags   ? pick(std::integral_constant<int, 4>())
                                                 : pick(std::integral_constant<int, 16>());
-    place<<<n_tiles, kThreads, 0, stream>>>(a, probe, non_ids, marks);
+    HL_CUDA_TRY(launch(place, n_tiles, kThreads, stream, a, probe, non_ids, marks));
     note_launches(2);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -439,8 +439,10 @@ int32_t fragment_and_mark(hl_ctx* ctx, const hl_batch* b, const float* d_dense, 
 extern "C" int32_t hl_fragment(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
                                int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non,
                                float* d_dense_out, void* stream) {
-    return fragment_call(ctx, b, d_dense, n_dense, d_perm, d_counts, pop, non, d_dense_out, false,
-                         static_cast<cudaStream_t>(stream));
+    return as_graph(ctx ? ctx->launches : nullptr, [&] {
+        return fragment_call(ctx, b, d_dense, n_dense, d_perm, d_counts, pop, non, d_dense_out, false,
+                             static_cast<cudaStream_t>(stream));
+    });
 }
 
 extern "C" int32_t hl_wide_fragment(hl_wide* w, const hl_batch* b, int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop,

@@ -16,6 +16,7 @@
 // three streams made 22, 3 and 25 (8 K lookups: 88 us per mini-batch).
 #include "hl_common.cuh"
 
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -31,6 +32,9 @@ struct hl_pipe {
         cudaEvent_t inputs, pairs, index, gather, forward, x, scatter;
     };
     std::vector<Events> ev;
+    // the graphs of mini-batch j's kernels: slot j % slots, so that set and window, and with them nearly all arguments, are
+    // the same whenever a slot is used
+    std::vector<std::unique_ptr<hl::LaunchCache>> launches;
     // mini-batches whose index work is queued (indexed), whose host read is queued (submitted), whose main work is queued
     // (done)
     int64_t j_indexed, j_submitted, j_done;
@@ -111,6 +115,11 @@ struct Scope {
     ~Scope() { span_close(p, idx); }
 };
 
+// where the launches made for mini-batch j are collected (traced spans bracket single calls: then nowhere)
+hl::LaunchCache* launches_of(hl_pipe* p, int64_t j) {
+    return p->trace_mask ? nullptr : p->launches[j % p->launches.size()].get();
+}
+
 // The index-only work of the next mini-batch (nothing here touches a row).
 int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
     const int64_t j = p->j_indexed;
@@ -127,6 +136,7 @@ int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* 
         HL_PIPE_TRY(wait(p->index, static_cast<cudaEvent_t>(inputs_ready)));
     }
     if (j >= n) HL_PIPE_TRY(wait(p->index, e.scatter));   // the buffers of this set were mini-batch j-n_sets's
+    LaunchBatch batch(launches_of(p, j));
     {
         Scope sc(p, HL_SPAN_FRAGMENT, j, kIndex);
         HL_PIPE_TRY(fragment_and_mark(p->ctx, b, d_dense, d_dense ? p->n_dense : 0, st.perm, st.counts, &st.pop, &st.non,
@@ -141,7 +151,10 @@ int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* 
     const int64_t n_clear = backward_sort_clear_words(p->ctx, merge);
     const SortAside aside{p->sort, e.pairs, (int)(j % 2)};
     const SortAside* use = n_clear > 0 ? &aside : nullptr;
-    if (use && j >= 2) HL_PIPE_TRY(wait(p->index, p->ev[(j - 2) % n].index));
+    if (use && j >= 2) {
+        HL_PIPE_TRY(launch_flush() == cudaSuccess ? HL_OK : HL_ECUDA);
+        HL_PIPE_TRY(wait(p->index, p->ev[(j - 2) % n].index));
+    }
     if (p->ctx->max_nnz > 0) {
         Scope sc(p, HL_SPAN_INDEX_BEGIN, j, kIndex);
         HL_PIPE_TRY(cold_rank(p->ctx, p->window_rows, st.cold_rows, st.n_cold, p->index, p->ctx->r.bwd_hist[use ? j % 2 : 0],
@@ -153,6 +166,7 @@ int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* 
                                        st.n_cold, prev ? prev->cold_rows : nullptr, prev ? prev->n_cold : nullptr,
                                        st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, p->index, use));
     }
+    HL_PIPE_TRY(batch.end());
     HL_PIPE_TRY(record(e.index, use ? p->sort : p->index));
     p->j_indexed += 1;
     return HL_OK;
@@ -169,8 +183,10 @@ int32_t submit_link(hl_pipe* p) {
     if (j >= 1) HL_PIPE_TRY(wait(p->link, p->ev[(j - 1) % n].forward));   // j-1 took what it needs out of the window
     {
         Scope sc(p, HL_SPAN_STAGE, j, kLink);
+        LaunchBatch batch(launches_of(p, j));
         HL_PIPE_TRY(hl_stage_cold(p->ctx, p->host_table, p->cache, w, p->window_rows, st.cold_rows, st.n_cold,
                                   j >= 1 ? st.fwd_src : nullptr, p->link));
+        HL_PIPE_TRY(batch.end());
     }
     HL_PIPE_TRY(record(p->ev[j % n].gather, p->link));
     p->j_submitted += 1;
@@ -186,8 +202,10 @@ int32_t queue_scatter(hl_pipe* p, int64_t j) {
     HL_PIPE_TRY(wait(p->wb, e.x));
     {
         Scope sc(p, HL_SPAN_SCATTER, j, kWb);
+        LaunchBatch batch(launches_of(p, j));
         HL_PIPE_TRY(hl_scatter_cold_at(p->ctx, p->cache, w0, p->window_rows, st.cold_rows, st.n_cold, p->host_table,
                                        p->wb));
+        HL_PIPE_TRY(batch.end());
     }
     return record(e.scatter, p->wb);
 }
@@ -244,6 +262,11 @@ extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_t
         *side[i] = nullptr;
         ok = ok && cudaStreamCreateWithPriority(side[i], cudaStreamNonBlocking, i < 2 ? index_prio : link_prio) ==
                        cudaSuccess;
+    }
+    p->launches.resize(n_sets % 2 ? 2 * n_sets : n_sets);
+    for (auto& l : p->launches) {
+        l.reset(new (std::nothrow) LaunchCache(1));
+        ok = ok && l;
     }
     p->ev.resize(n_sets);
     for (auto& e : p->ev) {
@@ -314,11 +337,13 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
     {
         // with O's forward: the rows shared with mini-batch j-1, out of its staging window (its backward is done)
         Scope sc(p, HL_SPAN_FWD_POP, j, kMain);
+        LaunchBatch batch(launches_of(p, j));
         if (j >= 1 && p->window_rows > 0)
             HL_PIPE_TRY(fwd_and_forward_cold(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, w1, w0, p->window_rows,
                                              st.fwd_src, st.n_cold, p->main));
         else
             HL_PIPE_TRY(hl_embbag_fwd(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main));
+        HL_PIPE_TRY(batch.end());
     }
     HL_PIPE_TRY(record(e.forward, p->main));
     if (p->wb_pending) {
@@ -330,10 +355,13 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
     if (p->j_submitted == j + 1 && p->j_submitted < p->j_indexed) HL_PIPE_TRY(submit_link(p));   // mini-batch j+1
     if (p->order == HL_PIPE_ORDER_FIG8) {
         Scope sc(p, HL_SPAN_BWD_POP, j, kMain);
+        LaunchBatch batch(launches_of(p, j));
         HL_PIPE_TRY(hl_embbag_bwd_apply2(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 0, d_grad_pop,
                                          lr, p->main));
+        HL_PIPE_TRY(batch.end());
     }
     HL_PIPE_TRY(wait(p->main, e.gather));
+    LaunchBatch batch(launches_of(p, j));
     {
         Scope sc(p, HL_SPAN_FWD_NON, j, kMain);
         HL_PIPE_TRY(hl_embbag_fwd(p->ctx, p->cache, &st.non, st.counts + 1, st.pooled_non, p->main));
@@ -347,6 +375,7 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
             HL_PIPE_TRY(hl_embbag_bwd_apply(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n + 2, d_grad_pop,
                                             lr, p->main));
     }
+    HL_PIPE_TRY(batch.end());
     HL_PIPE_TRY(record(e.x, p->main));
     p->j_done += 1;
     if (p->wb_mode == HL_PIPE_WB_AFTER_FORWARD && next)

@@ -472,14 +472,14 @@ int sort_cluster_ctas() {
 int32_t exclusive_scan_i32(const int32_t* in, int32_t* out, const int32_t* d_n, int64_t n_max, int32_t* tiles,
                            int32_t* status, cudaStream_t stream, WaitCfg w) {
     if (n_max <= 0) {
-        HL_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(int32_t), stream));
+        HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(out), 1, stream));
         return HL_OK;
     }
     const int64_t n_tiles = n_max / kScanTile + 1;   // one more than needed when n is a multiple of the tile
     unsigned long long* st = reinterpret_cast<unsigned long long*>(tiles);
-    HL_CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(unsigned long long) * (n_tiles + 1), stream));
-    k_scan_chained<<<(unsigned)n_tiles, kThreads, 0, stream>>>(in, out, d_n, n_max, st, status, w.max_polls,
-                                                               w.stall_tile);
+    HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(st), 2 * (n_tiles + 1), stream));
+    HL_CUDA_TRY(launch(k_scan_chained, (unsigned)n_tiles, kThreads, stream, in, out, d_n, n_max, st, status, w.max_polls,
+                       w.stall_tile));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -508,21 +508,10 @@ int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n,
     if (n_max <= 0) return HL_OK;
     if (sort_in_cluster(n_max, w)) {
         const int ctas = sort_cluster_ctas();
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = ctas;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3(ctas);
-        cfg.blockDim = dim3(kClusterNT);
-        cfg.dynamicSmemBytes = sizeof(SortSmem<kClusterNT, kClusterItems>);
-        cfg.stream = stream;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        HL_CUDA_TRY(cudaLaunchKernelEx(&cfg, ctas == 16 ? k_sort_cluster<16, kClusterNT, kClusterItems>
-                                                        : k_sort_cluster<8, kClusterNT, kClusterItems>,
-                                       (const int32_t*)keys[0], (const int32_t*)vals[0], keys[out], vals[out], d_n, n_max,
-                                       passes));
+        HL_CUDA_TRY(launch_cluster(ctas == 16 ? k_sort_cluster<16, kClusterNT, kClusterItems>
+                                              : k_sort_cluster<8, kClusterNT, kClusterItems>,
+                                   ctas, kClusterNT, sizeof(SortSmem<kClusterNT, kClusterItems>), ctas, stream, keys[0],
+                                   vals[0], keys[out], vals[out], d_n, n_max, passes));
         note_launches(1);
         return HL_OK;
     }
@@ -532,15 +521,15 @@ int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n,
     uint32_t* ticket = hist + 4 * 256;
     uint32_t* tstat = hist + 4 * 256 + 8;
     if (!counted) {
-        HL_CUDA_TRY(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * sort_clear_words(n_max, key_bits, w), stream));
-        k_sort_digit_hist<<<grid_for(n_max, kThreads * 8, 1024), kThreads, 0, stream>>>(keys[0], d_n, n_max, passes, ghist);
+        HL_CUDA_TRY(clear_words(hist, sort_clear_words(n_max, key_bits, w), stream));
+        HL_CUDA_TRY(launch(k_sort_digit_hist, grid_for(n_max, kThreads * 8, 1024), kThreads, stream, keys[0], d_n, n_max,
+                           passes, ghist));
         note_launches(1);
     }
     for (int p = 0; p < passes; ++p)
-        k_sort_pass<<<(unsigned)n_tiles, kThreads, 0, stream>>>(keys[p & 1], vals[p & 1], keys[(p & 1) ^ 1],
-                                                                vals[(p & 1) ^ 1], d_n, n_max, 8 * p, ghist + 256 * p, ticket + p,
-                                                                tstat + (size_t)p * n_tiles * 256, status, w.max_polls,
-                                                                w.stall_tile);
+        HL_CUDA_TRY(launch(k_sort_pass, (unsigned)n_tiles, kThreads, stream, keys[p & 1], vals[p & 1], keys[(p & 1) ^ 1],
+                           vals[(p & 1) ^ 1], d_n, n_max, 8 * p, ghist + 256 * p, ticket + p,
+                           tstat + (size_t)p * n_tiles * 256, status, w.max_polls, w.stall_tile));
     note_launches(passes);
     HL_LAUNCH_CHECK();
     return HL_OK;

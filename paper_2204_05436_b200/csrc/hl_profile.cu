@@ -322,16 +322,16 @@ int32_t select_rows_by_count(const uint32_t* counts, int64_t n, SelectState* sel
                              long long k, long long share_num, long long share_den, int64_t cap, int32_t* out_idx,
                              int64_t* d_n_out, int32_t* status, int sms, cudaStream_t stream) {
     const int64_t n_tiles = div_up(n, kSelTile);
-    k_select_begin<<<1, 256, 0, stream>>>(sel, (unsigned long long)k, share_num, share_den);
+    HL_CUDA_TRY(launch(k_select_begin, 1, 256, stream, sel, (unsigned long long)k, share_num, share_den));
     const int grid = grid_for(n, kThreads * 16, sms * 8);
     for (int shift = 24; shift >= 0; shift -= 8) {
-        k_select_hist<<<grid, kThreads, 0, stream>>>(counts, n, shift, sel);
-        k_select_pick<<<1, 256, 0, stream>>>(sel, shift);
+        HL_CUDA_TRY(launch(k_select_hist, grid, kThreads, stream, counts, n, shift, sel));
+        HL_CUDA_TRY(launch(k_select_pick, 1, 256, stream, sel, shift));
     }
-    k_select_tile_counts<<<(unsigned)n_tiles, kThreads, 0, stream>>>(counts, n, sel, sel_gt, sel_eq);
-    k_select_spine<<<1, 1024, 0, stream>>>(sel_gt, sel_eq, n_tiles);
-    k_select_emit<<<(unsigned)n_tiles, kThreads, 0, stream>>>(counts, n, sel, sel_gt, sel_eq, n_tiles, cap, out_idx,
-                                                             d_n_out, status);
+    HL_CUDA_TRY(launch(k_select_tile_counts, (unsigned)n_tiles, kThreads, stream, counts, n, sel, sel_gt, sel_eq));
+    HL_CUDA_TRY(launch(k_select_spine, 1, 1024, stream, sel_gt, sel_eq, n_tiles));
+    HL_CUDA_TRY(launch(k_select_emit, (unsigned)n_tiles, kThreads, stream, counts, n, sel, sel_gt, sel_eq, n_tiles, cap,
+                       out_idx, d_n_out, status));
     note_launches(12);   // begin, 4 x (histogram, pick), tile counts, spine, emit
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -357,8 +357,8 @@ extern "C" int32_t hl_profile_hot(hl_ctx* ctx, const hl_batch* b, int32_t reset,
             return HL_EINVAL;
         const int64_t bags_per_table = (int64_t)b->batch * ctx->S;
         const int64_t n_bags = bags_per_table * ctx->T;
-        k_count<<<grid_for(n_bags, kThreads, ctx_sms(ctx) * 8), kThreads, 0, stream>>>(
-            b->indices, b->offsets, n_bags, bags_per_table, r.table_base, r.counts, r.sel, r.status);
+        HL_CUDA_TRY(launch(k_count, grid_for(n_bags, kThreads, ctx_sms(ctx) * 8), kThreads, stream, b->indices, b->offsets,
+                           n_bags, bags_per_table, r.table_base, r.counts, r.sel, r.status));
         note_launches(1);
         HL_LAUNCH_CHECK();
     }
@@ -396,16 +396,16 @@ extern "C" int32_t hl_build_remap(hl_ctx* ctx, const int32_t* d_hot_rows, const 
     Regions& r = ctx->r;
     HL_CUDA_TRY(cudaMemsetAsync(r.remap, 0, sizeof(RemapBlock) * ctx->n_remap_blocks, stream));
     if (ctx->hot_cap > 0) {
-        k_remap_bits<<<grid_for(ctx->hot_cap, kThreads, ctx_sms(ctx) * 8), kThreads, 0, stream>>>(
-            d_hot_rows, d_n_hot, ctx->hot_cap, ctx->N, r.remap, r.status);
+        HL_CUDA_TRY(launch(k_remap_bits, grid_for(ctx->hot_cap, kThreads, ctx_sms(ctx) * 8), kThreads, stream, d_hot_rows,
+                           d_n_hot, ctx->hot_cap, ctx->N, r.remap, r.status));
         note_launches(1);
     }
-    k_remap_prefix<<<grid_for(ctx->n_remap_blocks, kThreads, ctx_sms(ctx) * 8), kThreads, 0, stream>>>(
-        d_hot_rows, d_n_hot, ctx->hot_cap, ctx->n_remap_blocks, r.remap);
+    HL_CUDA_TRY(launch(k_remap_prefix, grid_for(ctx->n_remap_blocks, kThreads, ctx_sms(ctx) * 8), kThreads, stream,
+                       d_hot_rows, d_n_hot, ctx->hot_cap, ctx->n_remap_blocks, r.remap));
     note_launches(d_remap_out ? 2 : 1);
     if (d_remap_out)
-        k_remap_dense<<<grid_for(ctx->N, kThreads * 4, ctx_sms(ctx) * 16), kThreads, 0, stream>>>(r.remap, ctx->N,
-                                                                                         d_remap_out);
+        HL_CUDA_TRY(launch(k_remap_dense, grid_for(ctx->N, kThreads * 4, ctx_sms(ctx) * 16), kThreads, stream, r.remap,
+                           ctx->N, d_remap_out));
     HL_LAUNCH_CHECK();
     if (host_table && ctx->hot_cap > 0)
         return launch_gather_rows(ctx, d_cache, 0, host_table, d_hot_rows, d_n_hot, ctx->hot_cap, r.status, stream);

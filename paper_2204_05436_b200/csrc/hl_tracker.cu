@@ -197,18 +197,17 @@ extern "C" int32_t hl_tracker_update(hl_ctx* ctx, const hl_batch* b, int32_t* d_
     Regions& r = ctx->r;
     const int64_t bags_per_table = (int64_t)b->batch * ctx->S;
     const int64_t n_bags = bags_per_table * ctx->T;
-    k_trk_keys<<<grid_for(n_bags, kThreads, kMaxGrid), kThreads, 0, stream>>>(
-        b->indices, b->offsets, n_bags, bags_per_table, r.table_base, ctx->max_nnz, (uint32_t)n_sets, r.bwd_keys[0],
-        r.bwd_vals[0], r.bwd_n, r.status);
+    HL_CUDA_TRY(launch(k_trk_keys, grid_for(n_bags, kThreads, kMaxGrid), kThreads, stream, b->indices, b->offsets, n_bags,
+                       bags_per_table, r.table_base, ctx->max_nnz, (uint32_t)n_sets, r.bwd_keys[0], r.bwd_vals[0], r.bwd_n,
+                       r.status));
     note_launches(1);
     HL_LAUNCH_CHECK();
     int32_t *keys, *vals;
     const int32_t st = radix_sort_pairs(r.bwd_keys, r.bwd_vals, r.bwd_n, ctx->max_nnz, bits_for(n_sets), r.bwd_hist[0],
                                         r.status, &keys, &vals, stream);
     if (st != HL_OK) return st;
-    k_trk_replay<<<grid_for(ctx->max_nnz, kThreads, kMaxGrid), kThreads, 0, stream>>>(keys, vals, r.bwd_n, ctx->max_nnz,
-                                                                                    d_tags, d_rrpv, n_sets, ways,
-                                                                                    d_hits);
+    HL_CUDA_TRY(launch(k_trk_replay, grid_for(ctx->max_nnz, kThreads, kMaxGrid), kThreads, stream, keys, vals, r.bwd_n,
+                       ctx->max_nnz, d_tags, d_rrpv, n_sets, ways, d_hits));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -222,8 +221,8 @@ extern "C" int32_t hl_tracker_export(hl_ctx* ctx, const int32_t* d_tags, const u
     HL_CUDA_TRY(cudaMemsetAsync(r.counts, 0, sizeof(uint32_t) * ctx->N, stream));
     HL_CUDA_TRY(cudaMemsetAsync(r.sel, 0, sizeof(SelectState), stream));
     const int64_t n_blocks = n_sets * ways;
-    k_trk_export<<<grid_for(n_blocks, kThreads, kMaxGrid), kThreads, 0, stream>>>(d_tags, d_rrpv, n_blocks, ctx->N,
-                                                                                 r.counts, r.sel, r.status);
+    HL_CUDA_TRY(launch(k_trk_export, grid_for(n_blocks, kThreads, kMaxGrid), kThreads, stream, d_tags, d_rrpv, n_blocks,
+                       ctx->N, r.counts, r.sel, r.status));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;

@@ -318,8 +318,8 @@ int32_t sort_by_row(hl_wide* w, const int32_t* table_of_entry, const int32_t* d_
         HL_CUDA_TRY(cudaMemcpyAsync(w->sort_vals[0], w->sort_vals[1], sizeof(int32_t) * n_max, cudaMemcpyDeviceToDevice,
                                     stream));
     }
-    k_wide_gather_key<<<grid_for(n_max, kThreads, 8 * w->sms), kThreads, 0, stream>>>(w->sort_vals[0], table_of_entry,
-                                                                                      d_n, n_max, w->sort_keys[0]);
+    HL_CUDA_TRY(launch(k_wide_gather_key, grid_for(n_max, kThreads, 8 * w->sms), kThreads, stream, w->sort_vals[0],
+                       table_of_entry, d_n, n_max, w->sort_keys[0]));
     note_launches(1);
     HL_LAUNCH_CHECK();
     int32_t* k2;
@@ -436,9 +436,9 @@ extern "C" int32_t hl_wide_profile_hot(hl_wide* w, const hl_batch* b, int32_t re
             return HL_EINVAL;
         const int64_t bags_per_table = (int64_t)b->batch * w->S;
         const int64_t n_bags = bags_per_table * w->T;
-        k_wide_count<<<grid_for(n_bags, kThreads, w->sms * 8), kThreads, 0, stream>>>(
-            b->indices, b->offsets, n_bags, bags_per_table, w->table_base, w->c_keys, w->c_cnt, (uint64_t)(E - 1),
-            w->sel, w->status);
+        HL_CUDA_TRY(launch(k_wide_count, grid_for(n_bags, kThreads, w->sms * 8), kThreads, stream, b->indices, b->offsets,
+                           n_bags, bags_per_table, w->table_base, w->c_keys, w->c_cnt, (uint64_t)(E - 1), w->sel,
+                           w->status));
         note_launches(1);
         HL_LAUNCH_CHECK();
     }
@@ -468,24 +468,22 @@ extern "C" int32_t hl_wide_profile_hot(hl_wide* w, const hl_batch* b, int32_t re
     // the counted rows in ascending order of their global id, with their counts: then the selection is the one of the
     // dense counter, over positions instead of rows (ties at the threshold go to the smaller position = smaller id)
     HL_CUDA_TRY(cudaMemsetAsync(w->n_seen, 0, 4 * sizeof(int32_t), stream));
-    k_wide_entries<<<grid_for(E, kThreads, w->sms * 8), kThreads, 0, stream>>>(
-        w->c_keys, w->c_cnt, E, w->table_base, w->T, w->n_seen, w->e_tab, w->e_idx, w->e_cnt, w->sort_keys[0],
-        w->sort_vals[0]);
+    HL_CUDA_TRY(launch(k_wide_entries, grid_for(E, kThreads, w->sms * 8), kThreads, stream, w->c_keys, w->c_cnt, E,
+                       w->table_base, w->T, w->n_seen, w->e_tab, w->e_idx, w->e_cnt, w->sort_keys[0], w->sort_vals[0]));
     note_launches(1);
     HL_LAUNCH_CHECK();
     int32_t* order;
     int32_t st = sort_by_row(w, w->e_tab, w->n_seen, E, &order, stream);
     if (st != HL_OK) return st;
-    k_wide_row_order<<<grid_for(E, kThreads, w->sms * 8), kThreads, 0, stream>>>(order, w->e_cnt, w->n_seen, E, w->s_cnt,
-                                                                               w->s_ent);
+    HL_CUDA_TRY(launch(k_wide_row_order, grid_for(E, kThreads, w->sms * 8), kThreads, stream, order, w->e_cnt, w->n_seen, E,
+                       w->s_cnt, w->s_ent));
     note_launches(1);
     HL_LAUNCH_CHECK();
     st = select_rows_by_count(w->s_cnt, E, w->sel, w->sel_gt, w->sel_eq, k, share_num, share_den, w->hot_cap,
                               w->sel_idx, d_n_hot, w->status, w->sms, stream);
     if (st != HL_OK) return st;
-    k_wide_hot_rows<<<grid_for(w->hot_cap, kThreads, w->sms * 8), kThreads, 0, stream>>>(
-        w->sel_idx, d_n_hot, w->hot_cap, w->s_ent, w->e_tab, w->e_idx, w->table_base,
-        reinterpret_cast<long long*>(d_hot_rows));
+    HL_CUDA_TRY(launch(k_wide_hot_rows, grid_for(w->hot_cap, kThreads, w->sms * 8), kThreads, stream, w->sel_idx, d_n_hot,
+                       w->hot_cap, w->s_ent, w->e_tab, w->e_idx, w->table_base, reinterpret_cast<long long*>(d_hot_rows)));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -496,9 +494,9 @@ extern "C" int32_t hl_wide_build_remap(hl_wide* w, const int64_t* d_hot_rows, co
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     HL_CUDA_TRY(cudaMemsetAsync(w->r_keys, 0xff, sizeof(long long) * w->remap_slots, stream));
     if (w->hot_cap > 0) {
-        k_wide_remap<<<grid_for(w->hot_cap, kThreads, w->sms * 8), kThreads, 0, stream>>>(
-            reinterpret_cast<const long long*>(d_hot_rows), d_n_hot, w->hot_cap, w->N, w->r_keys, w->r_vals,
-            (uint64_t)(w->remap_slots - 1), w->status);
+        HL_CUDA_TRY(launch(k_wide_remap, grid_for(w->hot_cap, kThreads, w->sms * 8), kThreads, stream,
+                           reinterpret_cast<const long long*>(d_hot_rows), d_n_hot, w->hot_cap, w->N, w->r_keys, w->r_vals,
+                           (uint64_t)(w->remap_slots - 1), w->status));
         note_launches(1);
         HL_LAUNCH_CHECK();
     }
@@ -518,24 +516,24 @@ extern "C" int32_t hl_wide_index_cold(hl_wide* w, const int32_t* d_non_offsets, 
     HL_CUDA_TRY(cudaMemsetAsync(w->cold_n, 0, 4 * sizeof(int32_t), stream));
     const HashProbe probe{w->r_keys, w->r_vals, (uint64_t)(w->remap_slots - 1)};
     const int grid = grid_for(w->max_nnz, kThreads, 8 * w->sms);
-    k_wide_classify<<<grid, kThreads, 0, stream>>>(reinterpret_cast<const long long*>(d_non_rows), d_non_offsets, d_n_non,
-                                                   w->max_batch, w->T * w->S, non_cap, w->N, probe, w->table_base, w->T,
-                                                   d_non_slots, w->cold_tab, w->cold_idx, w->cold_pos, w->sort_keys[0],
-                                                   w->sort_vals[0], w->cold_n, w->max_nnz, w->status);
+    HL_CUDA_TRY(launch(k_wide_classify, grid, kThreads, stream, reinterpret_cast<const long long*>(d_non_rows),
+                       d_non_offsets, d_n_non, w->max_batch, w->T * w->S, non_cap, w->N, probe, w->table_base, w->T,
+                       d_non_slots, w->cold_tab, w->cold_idx, w->cold_pos, w->sort_keys[0], w->sort_vals[0], w->cold_n,
+                       w->max_nnz, w->status));
     note_launches(1);
     HL_LAUNCH_CHECK();
     int32_t* order;
     int32_t st = sort_by_row(w, w->cold_tab, w->cold_n, w->max_nnz, &order, stream);
     if (st != HL_OK) return st;
-    k_wide_heads<<<grid, kThreads, 0, stream>>>(order, w->cold_tab, w->cold_idx, w->cold_n, w->max_nnz, w->cold_rank);
+    HL_CUDA_TRY(launch(k_wide_heads, grid, kThreads, stream, order, w->cold_tab, w->cold_idx, w->cold_n, w->max_nnz,
+                       w->cold_rank));
     note_launches(1);
     HL_LAUNCH_CHECK();
     st = exclusive_scan_i32(w->cold_rank, w->cold_rank, w->cold_n, w->max_nnz, w->cold_tiles, w->status, stream);
     if (st != HL_OK) return st;
-    k_wide_assign<<<grid, kThreads, 0, stream>>>(order, w->cold_tab, w->cold_idx, w->cold_pos, w->cold_n, w->max_nnz,
-                                                 w->cold_rank, w->table_base, w->hot_cap, w->staging_cap, non_cap,
-                                                 d_non_slots, reinterpret_cast<long long*>(d_cold_rows), d_n_cold,
-                                                 w->status);
+    HL_CUDA_TRY(launch(k_wide_assign, grid, kThreads, stream, order, w->cold_tab, w->cold_idx, w->cold_pos, w->cold_n,
+                       w->max_nnz, w->cold_rank, w->table_base, w->hot_cap, w->staging_cap, non_cap, d_non_slots,
+                       reinterpret_cast<long long*>(d_cold_rows), d_n_cold, w->status));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
