@@ -29,12 +29,19 @@ __device__ __forceinline__ uint32_t randomizer(uint32_t g) {
 }
 
 // (set, row) of every lookup, at the lookup's own position; lookups outside their table get the sentinel set n_sets.
+// HIST: also the digit counts of the sort that follows (ghist [passes][256], zero on entry).
+template <bool HIST>
 __global__ void __launch_bounds__(kThreads) k_trk_keys(const int32_t* __restrict__ indices,
                                                        const int32_t* __restrict__ offsets, int64_t n_bags,
                                                        int64_t bags_per_table, const int64_t* __restrict__ table_base,
                                                        int64_t max_nnz, uint32_t n_sets, int32_t* __restrict__ keys,
                                                        int32_t* __restrict__ vals, int32_t* __restrict__ d_n,
-                                                       int32_t* status) {
+                                                       uint32_t* ghist, int passes, int32_t* status) {
+    __shared__ uint32_t h[HIST ? 4 : 1][256];
+    if (HIST) {
+        for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&h[0][0])[i] = 0;
+        __syncthreads();
+    }
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         int64_t L = offsets[n_bags];
         if (L > max_nnz) {
@@ -50,15 +57,26 @@ __global__ void __launch_bounds__(kThreads) k_trk_keys(const int32_t* __restrict
         const int64_t lo = offsets[bag], hi = offsets[bag + 1];
         for (int64_t j = lo; j < hi && j < max_nnz; ++j) {
             const int32_t idx = indices[j];
+            uint32_t key = n_sets;
+            int32_t val = -1;
             if (idx < 0 || idx >= rows) {
                 set_status(status, HL_EBOUNDS);
-                keys[j] = (int32_t)n_sets;
-                vals[j] = -1;
             } else {
                 const uint32_t g = (uint32_t)(base + idx);
-                keys[j] = (int32_t)(randomizer(g) % n_sets);
-                vals[j] = (int32_t)g;
+                key = randomizer(g) % n_sets;
+                val = (int32_t)g;
             }
+            keys[j] = (int32_t)key;
+            vals[j] = val;
+            if (HIST)
+                for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 255u], 1u);
+        }
+    }
+    if (HIST) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < passes * 256; i += kThreads) {
+            const uint32_t c = (&h[0][0])[i];
+            if (c) atomicAdd(&ghist[i], c);
         }
     }
 }
@@ -66,72 +84,116 @@ __global__ void __launch_bounds__(kThreads) k_trk_keys(const int32_t* __restrict
 // One warp per 32 positions of the sorted list: every position where a new set's run begins is a head, and the warp
 // replays, head after head, the accesses of that set (the run may reach far beyond the warp's own 32 positions; the
 // warps there find no head in it and leave it alone).  While a set is replayed lane w holds its way w.
+//
+// What bounds it is latency: of a set's blocks, which come from DRAM, and, in the set of a popular row (thousands of
+// lookups of a mini-batch), of the lookups themselves.  So the blocks of the next two heads are on their way while one is
+// replayed, the 64 lookups behind the warp's first stay in registers, and beyond them four groups of 32 are read at once.
+// 426 K lookups, 131 072 sets of 16: the whole update, with its sort, takes 78 us; with every load waited for where it is
+// needed, and the digits counted in a kernel of their own, 112 us.
 __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ vals,
                                                          const int32_t* __restrict__ d_n, int64_t n_max,
                                                          int32_t* __restrict__ tags, uint8_t* __restrict__ rrpv,
                                                          int64_t n_sets, int ways,
                                                          unsigned long long* __restrict__ d_hits) {
+    constexpr unsigned kAll = 0xffffffffu;
+    constexpr int kAhead = 4;                                    // groups of 32 lookups read at once
     int64_t n = d_n[0];
     n = n < 0 ? 0 : (n < n_max ? n : n_max);
     const int lane = threadIdx.x & 31;
     const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     unsigned long long hits = 0;
+    struct Blocks {
+        int64_t s;
+        int tag, rr;
+    };
     for (int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; w0 < n; w0 += n_warps * 32) {
+        auto key_at = [&](int64_t i) { return i < n ? keys[i] : -1; };
+        auto val_at = [&](int64_t i) { return i < n ? vals[i] : -1; };
         const int64_t p = w0 + lane;
-        const int32_t kp = p < n ? keys[p] : -1;
-        const int32_t kprev = (p > 0 && p < n) ? keys[p - 1] : -1;
-        unsigned heads = __ballot_sync(0xffffffffu, p < n && kp >= 0 && kp < n_sets && kp != kprev);
+        const int32_t k0 = key_at(p), k1 = key_at(p + 32), g0 = val_at(p), g1 = val_at(p + 32);
+        const int32_t before = w0 > 0 ? keys[w0 - 1] : -1;
+        const int32_t up = __shfl_up_sync(kAll, k0, 1);
+        unsigned heads = __ballot_sync(kAll, k0 >= 0 && k0 < n_sets && k0 != (lane ? up : before));
+        // a head's set and its blocks: -2 matches no row; RRPV -1 is never a victim and never aged
+        auto load = [&](unsigned hs) {
+            Blocks b{-1, -2, -1};
+            if (hs) {
+                b.s = __shfl_sync(kAll, k0, __ffs((int)hs) - 1);
+                if (lane < ways) {
+                    b.tag = tags[b.s * ways + lane];
+                    b.rr = (int)rrpv[b.s * ways + lane];
+                }
+            }
+            return b;
+        };
+        Blocks next = load(heads), after = load(heads & (heads - 1));
         while (heads) {
-            const int h = __ffs(heads) - 1;
+            const int h = __ffs((int)heads) - 1;
             heads &= heads - 1;
-            const int64_t s = __shfl_sync(0xffffffffu, kp, h);
-            int32_t tag = lane < ways ? tags[s * ways + lane] : -2;          // -2: matches no row
-            int rr = lane < ways ? (int)rrpv[s * ways + lane] : -1;          // -1: never a victim, never aged
+            const Blocks now = next;
+            next = after;
+            const unsigned behind = heads & (heads - 1);
+            after = load(behind);
+            int32_t tag = now.tag;
+            int rr = now.rr;
             int32_t last = -1;            // the row of the previous access
             bool last_zero = false;       // ... which left that row at RRPV 0, so that repeating it changes nothing
-            for (int64_t i = w0 + h;; i += 32) {
-                const bool in = i + lane < n;
-                const int32_t k = in ? keys[i + lane] : -1;
-                const int32_t g = in ? vals[i + lane] : -1;
-                const int cnt = __ffs(~__ballot_sync(0xffffffffu, k == (int32_t)s)) - 1;   // leading lanes of the run
-                const int c = cnt < 0 ? 32 : cnt;
-                if (last_zero && __all_sync(0xffffffffu, lane >= c || g == last)) {
+            // replays one group of up to 32 lookups; false: the run ended in it
+            auto replay = [&](int32_t k, int32_t g) {
+                const unsigned mine = __ballot_sync(kAll, k == (int32_t)now.s);
+                const int c = mine == kAll ? 32 : __ffs((int)~mine) - 1;                       // leading lanes of the run
+                if (last_zero && __all_sync(kAll, lane >= c || g == last)) {
                     hits += c;                                                    // a burst of one popular row
-                } else {
-                    for (int t = 0; t < c; ++t) {
-                        const int32_t gg = __shfl_sync(0xffffffffu, g, t);
-                        if (gg == last && last_zero) {
-                            ++hits;
-                            continue;
-                        }
-                        const unsigned hit = __ballot_sync(0xffffffffu, tag == gg);
-                        if (hit) {
-                            if (lane == __ffs(hit) - 1) rr = 0;
-                            last_zero = true;
-                            ++hits;
-                        } else {
-                            unsigned vm = __ballot_sync(0xffffffffu, rr == kRrpvMax);
-                            if (!vm) {   // age the whole set until its oldest block reaches the maximum
-                                const int add = __ballot_sync(0xffffffffu, rr == 2) ? 1
-                                                : __ballot_sync(0xffffffffu, rr == 1) ? 2 : 3;
-                                if (lane < ways) rr += add;
-                                vm = __ballot_sync(0xffffffffu, rr == kRrpvMax);
-                            }
-                            if (lane == __ffs(vm) - 1) {
-                                tag = gg;
-                                rr = kRrpvInsert;
-                            }
-                            last_zero = false;
-                        }
-                        last = gg;
-                    }
+                    return c == 32;
                 }
-                if (c < 32) break;
+                for (int t = 0; t < c; ++t) {
+                    const int32_t gg = __shfl_sync(kAll, g, t);
+                    if (gg == last && last_zero) {
+                        ++hits;
+                        continue;
+                    }
+                    const unsigned hit = __ballot_sync(kAll, tag == gg);
+                    if (hit) {
+                        if (lane == __ffs((int)hit) - 1) rr = 0;
+                        last_zero = true;
+                        ++hits;
+                    } else {
+                        unsigned vm = __ballot_sync(kAll, rr == kRrpvMax);
+                        if (!vm) {   // age the whole set until its oldest block reaches the maximum
+                            const int add = __ballot_sync(kAll, rr == 2) ? 1 : __ballot_sync(kAll, rr == 1) ? 2 : 3;
+                            if (lane < ways) rr += add;
+                            vm = __ballot_sync(kAll, rr == kRrpvMax);
+                        }
+                        if (lane == __ffs((int)vm) - 1) {
+                            tag = gg;
+                            rr = kRrpvInsert;
+                        }
+                        last_zero = false;
+                    }
+                    last = gg;
+                }
+                return c == 32;
+            };
+            // the first 32 lookups of the run, out of the 64 at hand
+            const int from = (h + lane) & 31;
+            const int32_t ka = __shfl_sync(kAll, k0, from), kb = __shfl_sync(kAll, k1, from);
+            const int32_t ga = __shfl_sync(kAll, g0, from), gb = __shfl_sync(kAll, g1, from);
+            bool more = replay(h + lane < 32 ? ka : kb, h + lane < 32 ? ga : gb);
+            for (int64_t i = w0 + h + 32; more; i += 32 * kAhead) {
+                int32_t k[kAhead], g[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    k[u] = key_at(i + 32 * u + lane);
+                    g[u] = val_at(i + 32 * u + lane);
+                }
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u)
+                    if (more) more = replay(k[u], g[u]);
             }
             if (lane < ways) {
-                tags[s * ways + lane] = tag;
-                rrpv[s * ways + lane] = (uint8_t)rr;
+                tags[now.s * ways + lane] = tag;
+                rrpv[now.s * ways + lane] = (uint8_t)rr;
             }
         }
     }
@@ -197,20 +259,25 @@ extern "C" int32_t hl_tracker_update(hl_ctx* ctx, const hl_batch* b, int32_t* d_
     Regions& r = ctx->r;
     const int64_t bags_per_table = (int64_t)b->batch * ctx->S;
     const int64_t n_bags = bags_per_table * ctx->T;
-    HL_CUDA_TRY(launch(k_trk_keys, grid_for(n_bags, kThreads, kMaxGrid), kThreads, stream, b->indices, b->offsets, n_bags,
-                       bags_per_table, r.table_base, ctx->max_nnz, (uint32_t)n_sets, r.bwd_keys[0], r.bwd_vals[0], r.bwd_n,
+    LaunchBatch batch(ctx->launches);
+    const int key_bits = bits_for(n_sets);
+    const int64_t n_clear = sort_clear_words(ctx->max_nnz, key_bits, WaitCfg());
+    if (n_clear > 0) HL_CUDA_TRY(clear_words(r.bwd_hist[0], n_clear, stream));
+    HL_CUDA_TRY(launch(n_clear > 0 ? k_trk_keys<true> : k_trk_keys<false>, grid_for(n_bags, kThreads, 4 * ctx_sms(ctx)),
+                       kThreads, stream, b->indices, b->offsets, n_bags, bags_per_table, r.table_base, ctx->max_nnz,
+                       (uint32_t)n_sets, r.bwd_keys[0], r.bwd_vals[0], r.bwd_n, r.bwd_hist[0], (key_bits + 7) / 8,
                        r.status));
     note_launches(1);
     HL_LAUNCH_CHECK();
     int32_t *keys, *vals;
-    const int32_t st = radix_sort_pairs(r.bwd_keys, r.bwd_vals, r.bwd_n, ctx->max_nnz, bits_for(n_sets), r.bwd_hist[0],
-                                        r.status, &keys, &vals, stream);
+    const int32_t st = radix_sort_pairs(r.bwd_keys, r.bwd_vals, r.bwd_n, ctx->max_nnz, key_bits, r.bwd_hist[0], r.status,
+                                        &keys, &vals, stream, WaitCfg(), true);
     if (st != HL_OK) return st;
     HL_CUDA_TRY(launch(k_trk_replay, grid_for(ctx->max_nnz, kThreads, kMaxGrid), kThreads, stream, keys, vals, r.bwd_n,
                        ctx->max_nnz, d_tags, d_rrpv, n_sets, ways, d_hits));
     note_launches(1);
     HL_LAUNCH_CHECK();
-    return HL_OK;
+    return batch.end();
 }
 
 extern "C" int32_t hl_tracker_export(hl_ctx* ctx, const int32_t* d_tags, const uint8_t* d_rrpv, int64_t n_sets,
