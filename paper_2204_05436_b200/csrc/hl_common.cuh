@@ -17,7 +17,6 @@ namespace hl {
 constexpr int kSMsFallback = 148;          // used only if the device's SM count cannot be queried (B200: 2 x 74)
 constexpr int kRemapRowsPerBlock = 224;    // 7 bitmap words per 32-byte remap block
 constexpr int kSortTile = 2048;            // keys per radix-sort tile (256 threads x 8)
-constexpr int kScanTile = 2048;            // elements per scan tile (256 threads x 8)
 constexpr int kSelTile = 4096;             // rows per hot-set selection tile (256 threads x 16)
 constexpr int kBwdChunk = 32;              // sorted lookups per backward chunk
 constexpr int kMoverCtasDefault = 16;      // working CTAs of a host-link mover inside a schedule: write-backs
@@ -134,8 +133,10 @@ struct hl_wide {
     uint32_t* sort_hist;
     uint32_t* frag_words;                    // [max_batch / 32 + 1]
     unsigned long long* frag_chain;
-    int32_t *cold_tab, *cold_idx, *cold_pos; // [max_nnz] cold lookups: table, index, position in X
-    int32_t *cold_rank, *cold_tiles, *cold_n;
+    uint32_t* cold_clear;                    // cold_n, cold_chain and sort_hist, one behind the other
+    int32_t* cold_n;                         // cold lookups of X
+    unsigned long long* cold_chain;          // [max_nnz / 1024 + 1]
+    hl::LaunchCache* launches;
 };
 
 namespace hl {
@@ -470,13 +471,7 @@ __device__ __forceinline__ unsigned long long chain_before(unsigned long long* w
 }
 
 // ---- primitives implemented in hl_prims.cu -----------------------------------------------------------------
-// Exclusive scan of in[0 .. n) into out[0 .. n] (out[n] = total); n = *d_n if d_n != nullptr (clamped to
-// n_max), else n_max.  in may alias out.  tiles: scratch of scan_tile_words(n_max) ints.  A chain poll that
-// gives up records HL_ETIMEOUT in *status.
-int32_t exclusive_scan_i32(const int32_t* in, int32_t* out, const int32_t* d_n, int64_t n_max, int32_t* tiles,
-                           int32_t* status, cudaStream_t stream, WaitCfg w = WaitCfg());
-
-// Stable LSD radix sort of (key, value) pairs by the low key_bits bits of the non-negative keys.
+// Stable LSD radix sort of (key, value) pairs by the low key_bits bits of the keys (as unsigned numbers).
 // n = *d_n (clamped to n_max).  Returns in *out_keys / *out_vals which of the two buffers holds the result.
 int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n, int64_t n_max, int key_bits,
                          uint32_t* hist, int32_t* status, int32_t** out_keys, int32_t** out_vals,
@@ -504,9 +499,6 @@ inline int32_t* span_count_of(const hl_ctx* ctx) {
     const int64_t max_chunks = ((ctx->max_nnz > 0 ? ctx->max_nnz : 1) + kBwdChunk - 1) / kBwdChunk;
     return reinterpret_cast<int32_t*>(ctx->r.bwd_part + 2 * max_chunks * ctx->D);
 }
-
-// ints of scratch exclusive_scan_i32 needs for at most n_max elements (64-bit ticket + status words).
-constexpr int64_t scan_tile_words(int64_t n_max) { return 2 * ((n_max > 0 ? n_max : 1) / kScanTile + 3); }
 
 // Ranks the rows marked in the cold-row bitmap (hl_cold.cu): d_cold_rows, *d_n_cold, cold_ranked.  Also clears `clear`
 // [n_clear words, a multiple of 4; 16-byte aligned], for the kernels that follow.

@@ -16,8 +16,8 @@ unsigned long long launches_so_far() { return g_launches.load(std::memory_order_
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kItems = 8;   // kThreads * kItems == kScanTile == kSortTile
-static_assert(kThreads * kItems == kScanTile && kThreads * kItems == kSortTile, "tile shape");
+constexpr int kItems = 8;
+static_assert(kThreads * kItems == kSortTile, "tile shape");
 
 __device__ __forceinline__ int warp_inclusive_scan(int v) {
     const int lane = threadIdx.x & 31;
@@ -63,7 +63,6 @@ __device__ __forceinline__ int64_t clamp_n(const int32_t* d_n, int64_t n_max) {
 // prefix.  Publishing never waits on anything, so the walk always terminates; every poll is bounded all the same,
 // and a poll that runs out records HL_ETIMEOUT and carries on with what it has (positions are range-checked).
 constexpr uint32_t kFlagAgg = 1u << 30, kFlagPrefix = 1u << 31, kValueMask = kFlagAgg - 1u;
-constexpr unsigned long long kFlagAgg64 = 1ull << 62, kFlagPrefix64 = 1ull << 63, kValueMask64 = kFlagAgg64 - 1ull;
 
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
     uint32_t v;
@@ -73,76 +72,6 @@ __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
 __device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-// ---- scan ---------------------------------------------------------------------------------------------------
-// st[0] = ticket counter, st[1 + tile] = status word of the tile; all zero on entry.
-// max_polls / stall_tile: see WaitCfg (a stalled tile publishes nothing, so that its successors' waits run out).
-__global__ void __launch_bounds__(kThreads) k_scan_chained(const int32_t* in, int32_t* out, const int32_t* d_n,
-                                                           int64_t n_max, unsigned long long* st, int32_t* status,
-                                                           int max_polls, int64_t stall_tile) {
-    __shared__ int smem[40];
-    __shared__ long long s_tile, s_excl;
-    if (threadIdx.x == 0) s_tile = (long long)atomicAdd(&st[0], 1ull);
-    __syncthreads();
-    const int64_t tile = s_tile;
-    const int64_t n = clamp_n(d_n, n_max);
-    const int64_t tile_base = tile * kScanTile;
-    if (tile_base > n) return;   // the tile at tile_base == n has no element but still writes out[n]
-    const int64_t base = tile_base + (int64_t)threadIdx.x * kItems;
-    int v[kItems];
-    int s = 0;
-#pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-        v[i] = base + i < n ? in[base + i] : 0;
-        s += v[i];
-    }
-    int total;
-    int excl = block_exclusive_scan(s, smem, total);
-    if (threadIdx.x < 32) {
-        // warp 0 walks back over the predecessors 32 tiles at a time: lane l looks at tile t0 - l; the sums up to
-        // and including the nearest tile that already knows its inclusive prefix are added
-        const int lane = threadIdx.x;
-        long long before = 0;
-        if (tile > 0) {
-            if (lane == 0 && tile != stall_tile) st_relaxed64(&st[1 + tile], kFlagAgg64 | (unsigned long long)total);
-            bool done = false;
-            for (int64_t t0 = tile - 1; t0 >= 0 && !done; t0 -= 32) {
-                const int64_t t = t0 - lane;
-                unsigned long long w = kFlagPrefix64;            // before tile 0: an empty prefix
-                if (t >= 0) {
-                    int polls = 0;
-                    while (((w = ld_relaxed64(&st[1 + t])) & (kFlagAgg64 | kFlagPrefix64)) == 0) {
-                        if (++polls > max_polls) {               // give up: carry on with what there is
-                            set_status(status, HL_ETIMEOUT);
-                            w = kFlagPrefix64;
-                            break;
-                        }
-                        __nanosleep(20);
-                    }
-                }
-                const unsigned with_prefix = __ballot_sync(0xffffffffu, (w & kFlagPrefix64) != 0);
-                const int stop = with_prefix ? __ffs(with_prefix) - 1 : 31;
-                long long val = lane <= stop ? (long long)(w & kValueMask64) : 0;
-#pragma unroll
-                for (int d = 16; d > 0; d >>= 1) val += __shfl_down_sync(0xffffffffu, val, d);
-                before += __shfl_sync(0xffffffffu, val, 0);
-                done = with_prefix != 0;
-            }
-        }
-        if (lane == 0) {
-            if (tile != stall_tile) st_relaxed64(&st[1 + tile], kFlagPrefix64 | (unsigned long long)(before + total));
-            s_excl = before;
-            if (n < tile_base + kScanTile) out[n] = (int32_t)(before + total);
-        }
-    }
-    __syncthreads();
-    excl += (int)s_excl;
-#pragma unroll
-    for (int i = 0; i < kItems; ++i) {
-        if (base + i < n) out[base + i] = excl;
-        excl += v[i];
-    }
-}
-
 // ---- radix sort ---------------------------------------------------------------------------------------------
 // Shared memory of the cluster sort: digit counters of every warp, then the pairs on their way to their new places.
 template <int NT, int ITEMS>
@@ -468,22 +397,6 @@ int sort_cluster_ctas() {
 }
 
 }  // namespace
-
-int32_t exclusive_scan_i32(const int32_t* in, int32_t* out, const int32_t* d_n, int64_t n_max, int32_t* tiles,
-                           int32_t* status, cudaStream_t stream, WaitCfg w) {
-    if (n_max <= 0) {
-        HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(out), 1, stream));
-        return HL_OK;
-    }
-    const int64_t n_tiles = n_max / kScanTile + 1;   // one more than needed when n is a multiple of the tile
-    unsigned long long* st = reinterpret_cast<unsigned long long*>(tiles);
-    HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(st), 2 * (n_tiles + 1), stream));
-    HL_CUDA_TRY(launch(k_scan_chained, (unsigned)n_tiles, kThreads, stream, in, out, d_n, n_max, st, status, w.max_polls,
-                       w.stall_tile));
-    note_launches(1);
-    HL_LAUNCH_CHECK();
-    return HL_OK;
-}
 
 // One cluster takes up to 2 048 pairs per CTA (32 768 with 16 CTAs).  Beyond that the exchange through distributed shared
 // memory takes longer than the chip-wide passes: 106 K pairs in three passes 40 us, against 30 with the tiles.

@@ -1,8 +1,10 @@
 // The index-only calls of the path for models with 2^31 rows and more (the paper's SYN-M1/M2 sizes): global row ids
 // are 64-bit, counted in a hashed counter and looked up in a hashed remap whose hash is the randomizer of Section
-// V-C.  Every table still has fewer than 2^31 rows, so a row is the pair (table, table-local index): the order of
-// global ids is the order of those pairs, which two stable 32-bit sorts give (index, then table).
+// V-C.  Every table still has fewer than 2^31 rows, so a row is the pair (table, table-local index), and the profile sorts
+// its rows by those (by index, then, stable, by table).
 #include <stdlib.h>
+
+#include <new>
 
 #include "hl_common.cuh"
 
@@ -60,15 +62,14 @@ size_t carve(char* base, hl_wide* w) {
         w->sort_keys[i] = c.take<int32_t>(sort_n);
         w->sort_vals[i] = c.take<int32_t>(sort_n);
     }
-    w->sort_hist = c.take<uint32_t>(sort_hist_words(sort_n));
+    // the cold-row search clears, in one go: its count, the chain words of its ranks, the scratch of its sort
+    const int64_t chain_words = div_up(nnz, 1024) * 2;
+    w->cold_clear = c.take<uint32_t>(8 + chain_words + sort_hist_words(sort_n));
+    w->cold_n = reinterpret_cast<int32_t*>(w->cold_clear);
+    w->cold_chain = reinterpret_cast<unsigned long long*>(w->cold_clear + 8);
+    w->sort_hist = w->cold_clear + 8 + chain_words;
     w->frag_words = c.take<uint32_t>(w->max_batch / 32 + 1);
     w->frag_chain = c.take<unsigned long long>(frag_chain_words(w->max_bags));
-    w->cold_tab = c.take<int32_t>(nnz);
-    w->cold_idx = c.take<int32_t>(nnz);
-    w->cold_pos = c.take<int32_t>(nnz);
-    w->cold_rank = c.take<int32_t>(nnz + 2);
-    w->cold_tiles = c.take<int32_t>(scan_tile_words(nnz));
-    w->cold_n = c.take<int32_t>(4);
     return (c.off + 255) & ~size_t(255);
 }
 
@@ -281,12 +282,14 @@ extern "C" int32_t hl_wide_create(hl_wide** out, const hl_geometry* geom, int32_
         free(w);
         return HL_ECUDA;
     }
+    w->launches = new (std::nothrow) LaunchCache(4);
     *out = w;
     return HL_OK;
 }
 
 extern "C" int32_t hl_wide_destroy(hl_wide* w) {
     if (!w) return HL_EINVAL;
+    delete w->launches;
     free(w->h_table_base);
     free(w);
     return HL_OK;
@@ -327,92 +330,149 @@ int32_t sort_by_row(hl_wide* w, const int32_t* table_of_entry, const int32_t* d_
                             out_vals, stream);
 }
 
-// cold lookups of X as (table, index, position): a lookup whose row is popular gets its slot at once
+// ---- cold rows of X -----------------------------------------------------------------------------------------------
+// What bounds the search is the chain of sort passes and small kernels: a clear, this kernel, one pass per 8 bits of the
+// rows, the ranks.  426 K lookups, 2.6 billion rows: fragment and search 105 us; with a sort by index, one by table, and
+// heads, scan and assignment as kernels of their own, 149 us.
+// X's lookups: a popular row gets its slot at once; a cold one goes on the list of pairs to sort (lower 32 bits of the
+// row, position).  The list is in any order.  HIST: also the digit counts of the sort (ghist [4][256], zero on entry).
+template <bool HIST>
 __global__ void __launch_bounds__(kThreads) k_wide_classify(const long long* __restrict__ rows,
                                                             const int32_t* __restrict__ offsets,
                                                             const int32_t* __restrict__ d_n_non, int max_batch,
                                                             int bags_per_sample_all, int64_t cap, int64_t N,
-                                                            HashProbe probe, const int64_t* __restrict__ table_base,
-                                                            int T, int32_t* __restrict__ slots, int32_t* c_tab,
-                                                            int32_t* c_idx, int32_t* c_pos, int32_t* sort_key,
-                                                            int32_t* sort_val, int32_t* d_n_cold_lookups,
-                                                            int64_t max_nnz, int32_t* status) {
+                                                            HashProbe probe, int32_t* __restrict__ slots,
+                                                            int32_t* __restrict__ sort_key, int32_t* __restrict__ sort_val,
+                                                            int32_t* d_n_cold_lookups, int64_t max_nnz, uint32_t* ghist,
+                                                            int passes, int32_t* status) {
+    __shared__ uint32_t h[HIST ? 4 : 1][256];
+    if (HIST) {
+        for (int i = threadIdx.x; i < 4 * 256; i += kThreads) (&h[0][0])[i] = 0;
+        __syncthreads();
+    }
     int n_non = *d_n_non;
     n_non = n_non < 0 ? 0 : (n_non > max_batch ? max_batch : n_non);
     int64_t L = offsets[(int64_t)n_non * bags_per_sample_all];
     if (L > cap) L = cap;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < L; j += (int64_t)gridDim.x * blockDim.x) {
-        const long long g = rows[j];
-        if (g < 0 || g >= N) {
-            if (g >= N) set_status(status, HL_EBOUNDS);
-            slots[j] = -1;
-            continue;
+    const int lane = threadIdx.x & 31;
+    for (int64_t j0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x - lane; j0 < L; j0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = j0 + lane;
+        const long long g = j < L ? rows[j] : -1;
+        int32_t s = -1;
+        const bool valid = g >= 0 && g < N;
+        if (g >= N) set_status(status, HL_EBOUNDS);
+        if (valid) s = probe.slot(g);
+        const bool cold = valid && s < 0;
+        if (j < L && !cold) slots[j] = s;
+        const unsigned m = __ballot_sync(0xffffffffu, cold);
+        int32_t first = 0;
+        if (lane == 0 && m) first = atomicAdd(d_n_cold_lookups, __popc(m));
+        const int64_t i = __shfl_sync(0xffffffffu, first, 0) + __popc(m & ((1u << lane) - 1u));
+        if (cold && i < max_nnz) {
+            const uint32_t key = (uint32_t)g;
+            sort_key[i] = (int32_t)key;
+            sort_val[i] = (int32_t)j;
+            if (HIST)
+                for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 255u], 1u);
         }
-        const int32_t s = probe.slot(g);
-        if (s >= 0) {
-            slots[j] = s;
-            continue;
+    }
+    if (HIST) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < passes * 256; i += kThreads) {
+            const uint32_t c = (&h[0][0])[i];
+            if (c) atomicAdd(&ghist[i], c);
         }
-        int lo = 0, hi = T;
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (table_base[mid] <= g) lo = mid;
-            else hi = mid;
-        }
-        const int32_t i = atomicAdd(d_n_cold_lookups, 1);
-        if (i >= max_nnz) continue;
-        c_tab[i] = lo;
-        c_idx[i] = (int32_t)(g - table_base[lo]);
-        c_pos[i] = (int32_t)j;
-        sort_key[i] = c_idx[i];
-        sort_val[i] = i;
     }
 }
 
-// head[j] = 1 where the j-th cold lookup in row order addresses another row than the one before
-__global__ void __launch_bounds__(kThreads) k_wide_heads(const int32_t* __restrict__ ent,
-                                                         const int32_t* __restrict__ c_tab,
-                                                         const int32_t* __restrict__ c_idx, const int32_t* d_n,
-                                                         int64_t n_max, int32_t* __restrict__ heads) {
+// the upper bits of the rows, in the order of their lower bits
+__global__ void __launch_bounds__(kThreads) k_wide_upper_key(const int32_t* __restrict__ pos,
+                                                             const long long* __restrict__ rows, const int32_t* d_n,
+                                                             int64_t n_max, int32_t* __restrict__ key,
+                                                             int32_t* __restrict__ val) {
     int64_t n = *d_n;
     n = n < n_max ? n : n_max;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t e = ent[j], p = j > 0 ? ent[j - 1] : -1;
-        heads[j] = (j == 0 || c_tab[e] != c_tab[p] || c_idx[e] != c_idx[p]) ? 1 : 0;
+        const int32_t p = pos[j];
+        key[j] = (int32_t)(rows[p] >> 32);
+        val[j] = p;
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_wide_assign(const int32_t* __restrict__ ent,
-                                                          const int32_t* __restrict__ c_tab,
-                                                          const int32_t* __restrict__ c_idx,
-                                                          const int32_t* __restrict__ c_pos, const int32_t* d_n,
-                                                          int64_t n_max, const int32_t* __restrict__ rank_excl,
-                                                          const int64_t* __restrict__ table_base, int64_t slot0,
-                                                          int64_t staging_cap, int64_t cap_ids,
-                                                          int32_t* __restrict__ slots, long long* __restrict__ cold_rows,
-                                                          int64_t* __restrict__ d_n_cold, int32_t* status) {
+// Ranks of the distinct rows among the sorted cold lookups, and the slot of every lookup: heads, their prefix sums
+// (within the tile, then chained over the tiles) and the assignment in one kernel.  UPPER: the rows have more than 32
+// bits, the sorted keys are not the rows.
+constexpr int kRankItems = 4, kRankTile = kThreads * kRankItems;
+template <bool UPPER>
+__global__ void __launch_bounds__(kThreads) k_wide_ranks(const int32_t* __restrict__ keys, const int32_t* __restrict__ pos,
+                                                         const long long* __restrict__ rows, const int32_t* d_n,
+                                                         int64_t n_max, unsigned long long* chain, int64_t slot0,
+                                                         int64_t staging_cap, int64_t cap_ids,
+                                                         int32_t* __restrict__ slots, long long* __restrict__ cold_rows,
+                                                         int64_t* __restrict__ d_n_cold, int max_polls, int32_t* status) {
+    __shared__ int s_warp[kThreads / 32];
     int64_t n = *d_n;
     n = n < n_max ? n : n_max;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        int64_t distinct = n > 0 ? rank_excl[n] : 0;
+    const int64_t tile0 = (int64_t)blockIdx.x * kRankTile;
+    if (tile0 >= n) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) *d_n_cold = 0;
+        return;
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t j0 = tile0 + threadIdx.x * kRankItems;
+    auto row_at = [&](int64_t j) -> long long { return UPPER ? rows[pos[j]] : (long long)(uint32_t)keys[j]; };
+    long long g[kRankItems];
+    int32_t at[kRankItems];
+    long long prev = j0 > 0 && j0 < n ? row_at(j0 - 1) : -1;
+    int mine = 0;
+    unsigned heads = 0;
+#pragma unroll
+    for (int k = 0; k < kRankItems; ++k) {
+        const bool in = j0 + k < n;
+        g[k] = in ? row_at(j0 + k) : -1;
+        at[k] = in ? pos[j0 + k] : -1;
+        if (in && g[k] != prev) {
+            heads |= 1u << k;
+            ++mine;
+        }
+        prev = g[k];
+    }
+    int incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += o;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    int before = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kThreads / 32; ++w) {
+        if (w < warp) before += s_warp[w];
+        total += s_warp[w];
+    }
+    chain_publish(chain, blockIdx.x, (unsigned long long)total);
+    const int64_t base = (int64_t)chain_before<kThreads>(chain, blockIdx.x, (unsigned long long)total, true, max_polls, status);
+    int64_t rank = base + before + (incl - mine) - 1;
+#pragma unroll
+    for (int k = 0; k < kRankItems; ++k) {
+        const bool head = heads >> k & 1u;
+        rank += head;
+        if (at[k] < 0 || at[k] >= cap_ids || rank < 0) continue;
+        if (rank < staging_cap) {
+            if (head) cold_rows[rank] = g[k];
+            slots[at[k]] = (int32_t)(slot0 + rank);
+        } else {
+            slots[at[k]] = -1;      // no room to stage this row: the lookup is dropped, the status word says so
+        }
+    }
+    if (threadIdx.x == 0 && tile0 + kRankTile >= n) {
+        int64_t distinct = base + total;
         if (distinct > staging_cap) {
             set_status(status, HL_ECAPACITY);
             distinct = staging_cap;
         }
         *d_n_cold = distinct;
-    }
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t e = ent[j], p = j > 0 ? ent[j - 1] : -1;
-        const bool head = j == 0 || c_tab[e] != c_tab[p] || c_idx[e] != c_idx[p];
-        const int64_t rank = head ? rank_excl[j] : rank_excl[j] - 1;
-        const int64_t where = c_pos[e];
-        if (where < 0 || where >= cap_ids || rank < 0) continue;
-        if (rank < staging_cap) {
-            if (head) cold_rows[rank] = table_base[c_tab[e]] + c_idx[e];
-            slots[where] = (int32_t)(slot0 + rank);
-        } else {
-            slots[where] = -1;      // no room to stage this row: the lookup is dropped, the status word says so
-        }
     }
 }
 
@@ -513,28 +573,37 @@ extern "C" int32_t hl_wide_index_cold(hl_wide* w, const int32_t* d_non_offsets, 
         return HL_OK;
     }
     if (!d_non_rows || !d_non_slots) return HL_EINVAL;
-    HL_CUDA_TRY(cudaMemsetAsync(w->cold_n, 0, 4 * sizeof(int32_t), stream));
+    LaunchBatch batch(w->launches);
     const HashProbe probe{w->r_keys, w->r_vals, (uint64_t)(w->remap_slots - 1)};
-    const int grid = grid_for(w->max_nnz, kThreads, 8 * w->sms);
-    HL_CUDA_TRY(launch(k_wide_classify, grid, kThreads, stream, reinterpret_cast<const long long*>(d_non_rows),
-                       d_non_offsets, d_n_non, w->max_batch, w->T * w->S, non_cap, w->N, probe, w->table_base, w->T,
-                       d_non_slots, w->cold_tab, w->cold_idx, w->cold_pos, w->sort_keys[0], w->sort_vals[0], w->cold_n,
-                       w->max_nnz, w->status));
+    // Rows of up to 32 bits are sorted as they are; others by their lower 32 bits, then (stable) by the rest.
+    const int upper_bits = (w->N - 1) >> 32 ? bits_for((w->N - 1) >> 32) : 0;
+    const int lower_bits = upper_bits ? 32 : bits_for(w->N - 1);
+    const int64_t sort_words = sort_clear_words(w->max_nnz, lower_bits, WaitCfg());
+    HL_CUDA_TRY(clear_words(w->cold_clear, (int64_t)(w->sort_hist - w->cold_clear) + sort_words, stream));
+    HL_CUDA_TRY(launch(sort_words ? k_wide_classify<true> : k_wide_classify<false>,
+                       grid_for(w->max_nnz, kThreads, 8 * w->sms), kThreads, stream,
+                       reinterpret_cast<const long long*>(d_non_rows), d_non_offsets, d_n_non, w->max_batch, w->T * w->S,
+                       non_cap, w->N, probe, d_non_slots, w->sort_keys[0], w->sort_vals[0], w->cold_n, w->max_nnz,
+                       w->sort_hist, (lower_bits + 7) / 8, w->status));
     note_launches(1);
-    HL_LAUNCH_CHECK();
-    int32_t* order;
-    int32_t st = sort_by_row(w, w->cold_tab, w->cold_n, w->max_nnz, &order, stream);
+    int32_t *keys, *pos;
+    int32_t st = radix_sort_pairs(w->sort_keys, w->sort_vals, w->cold_n, w->max_nnz, lower_bits, w->sort_hist, w->status,
+                                  &keys, &pos, stream, WaitCfg(), true);
     if (st != HL_OK) return st;
-    HL_CUDA_TRY(launch(k_wide_heads, grid, kThreads, stream, order, w->cold_tab, w->cold_idx, w->cold_n, w->max_nnz,
-                       w->cold_rank));
+    if (upper_bits) {
+        const int other = pos == w->sort_vals[0] ? 1 : 0;
+        int32_t* k2[2] = {w->sort_keys[other], w->sort_keys[other ^ 1]};
+        int32_t* v2[2] = {w->sort_vals[other], w->sort_vals[other ^ 1]};
+        HL_CUDA_TRY(launch(k_wide_upper_key, grid_for(w->max_nnz, kThreads, 8 * w->sms), kThreads, stream, pos,
+                           reinterpret_cast<const long long*>(d_non_rows), w->cold_n, w->max_nnz, k2[0], v2[0]));
+        note_launches(1);
+        st = radix_sort_pairs(k2, v2, w->cold_n, w->max_nnz, upper_bits, w->sort_hist, w->status, &keys, &pos, stream);
+        if (st != HL_OK) return st;
+    }
+    HL_CUDA_TRY(launch(upper_bits ? k_wide_ranks<true> : k_wide_ranks<false>, div_up(w->max_nnz, kRankTile), kThreads,
+                       stream, keys, pos, reinterpret_cast<const long long*>(d_non_rows), w->cold_n, w->max_nnz,
+                       w->cold_chain, w->hot_cap, w->staging_cap, non_cap, d_non_slots,
+                       reinterpret_cast<long long*>(d_cold_rows), d_n_cold, WaitCfg().max_polls, w->status));
     note_launches(1);
-    HL_LAUNCH_CHECK();
-    st = exclusive_scan_i32(w->cold_rank, w->cold_rank, w->cold_n, w->max_nnz, w->cold_tiles, w->status, stream);
-    if (st != HL_OK) return st;
-    HL_CUDA_TRY(launch(k_wide_assign, grid, kThreads, stream, order, w->cold_tab, w->cold_idx, w->cold_pos, w->cold_n,
-                       w->max_nnz, w->cold_rank, w->table_base, w->hot_cap, w->staging_cap, non_cap, d_non_slots,
-                       reinterpret_cast<long long*>(d_cold_rows), d_n_cold, w->status));
-    note_launches(1);
-    HL_LAUNCH_CHECK();
-    return HL_OK;
+    return batch.end();
 }
