@@ -372,6 +372,26 @@ HL_API int32_t hl_stage_cold(hl_ctx* ctx, const float* host_table, float* d_cach
 HL_API int32_t hl_forward_cold(hl_ctx* ctx, float* d_cache, int64_t from_stage_row0, int64_t to_stage_row0,
                                int64_t stage_rows, const int32_t* d_fwd_src, const int64_t* d_n_cold, void* stream);
 
+/* One mini-batch through fragment, cold-row gather, both forwards, both updates and write-back: the results of hl_fragment,
+ * hl_gather_cold, hl_embbag_fwd (O), hl_embbag_bwd_sgd (O), hl_embbag_fwd (X), hl_embbag_bwd_sgd (X), hl_scatter_cold in
+ * this order, with one sort for both updates.  Host rows are read on `side_stream` (may be main_stream) while the sort and
+ * O's part run on `main_stream`; everything is complete in main_stream's order.  flags: HL_STEP_DEFERRED = both forwards
+ * before both updates. */
+typedef struct {
+    int32_t*  perm;                /* as for hl_fragment ... */
+    int32_t*  counts;
+    hl_ubatch pop, non;
+    float*    dense_out;           /* (NULL without dense features) */
+    int32_t*  cold_rows;           /* ... hl_gather_cold ... */
+    int64_t*  n_cold;
+    float*    pooled_pop;          /* ... and hl_embbag_fwd */
+    float*    pooled_non;
+} hl_step_buffers;
+#define HL_STEP_DEFERRED 1
+HL_API int32_t hl_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense, const hl_step_buffers* buffers,
+                       float* d_cache, float* host_table, const float* d_grad_pop, const float* d_grad_non, float lr,
+                       int32_t flags, void* main_stream, void* side_stream);
+
 /* hl_scatter_cold from the window [stage_row0, stage_row0 + stage_rows) of the staging area. */
 HL_API int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t stage_row0, int64_t stage_rows,
                                   const int32_t* d_cold_rows, const int64_t* d_n_cold, float* host_table,

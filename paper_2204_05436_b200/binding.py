@@ -27,7 +27,7 @@ EXPORTS = (
     "hl_wide_workspace_bytes", "hl_wide_create", "hl_wide_destroy", "hl_wide_status", "hl_wide_profile_hot",
     "hl_wide_build_remap", "hl_wide_fragment", "hl_wide_index_cold",
     "hl_index_cold_begin", "hl_index_cold_end", "hl_index_cold_verdict",
-    "hl_embbag_bwd_prepare_merged", "hl_pipe_set_order",
+    "hl_embbag_bwd_prepare_merged", "hl_pipe_set_order", "hl_step",
 )
 
 
@@ -49,6 +49,12 @@ class hl_batch(ctypes.Structure):
 
 class hl_ubatch(ctypes.Structure):
     _fields_ = [("offsets", ctypes.c_void_p), ("ids", ctypes.c_void_p), ("cap_ids", ctypes.c_int64)]
+
+
+class hl_step_buffers(ctypes.Structure):
+    _fields_ = [("perm", ctypes.c_void_p), ("counts", ctypes.c_void_p), ("pop", hl_ubatch), ("non", hl_ubatch),
+                ("dense_out", ctypes.c_void_p), ("cold_rows", ctypes.c_void_p), ("n_cold", ctypes.c_void_p),
+                ("pooled_pop", ctypes.c_void_p), ("pooled_non", ctypes.c_void_p)]
 
 
 class hl_pipe_set(ctypes.Structure):
@@ -191,6 +197,9 @@ def _load() -> ctypes.CDLL:
     lib.hl_set_host_tables.argtypes = [vp, ctypes.POINTER(vp)]
     lib.hl_test_bounded_waits.restype = i32
     lib.hl_test_bounded_waits.argtypes = [vp, i32, i64]
+    lib.hl_step.restype = i32
+    lib.hl_step.argtypes = [vp, ctypes.POINTER(hl_batch), vp, i32, ctypes.POINTER(hl_step_buffers), vp, vp, vp, vp,
+                            ctypes.c_float, i32, vp, vp]
     lib.hl_flush_hot.restype = i32
     lib.hl_flush_hot.argtypes = [vp, vp, vp, vp, vp, vp]
     lib.hl_embbag_bwd_sgd_static.restype = i32
@@ -385,6 +394,19 @@ def hl_scatter_cold_at(ctx: int, d_cache, stage_row0: int, stage_rows: int, d_co
                        stream: int) -> None:
     _check("hl_scatter_cold_at", _lib.hl_scatter_cold_at(ctx, _ptr(d_cache), int(stage_row0), int(stage_rows),
                                                          _ptr(d_cold_rows), _ptr(d_n_cold), _ptr(host_table), stream))
+
+
+def make_step_buffers(perm, counts, pop: hl_ubatch, non: hl_ubatch, dense_out, cold_rows, n_cold, pooled_pop,
+                      pooled_non) -> hl_step_buffers:
+    return hl_step_buffers(_ptr(perm), _ptr(counts), pop, non, _ptr(dense_out), _ptr(cold_rows), _ptr(n_cold),
+                           _ptr(pooled_pop), _ptr(pooled_non))
+
+
+def hl_step(ctx: int, batch: hl_batch, d_dense, n_dense: int, buffers: hl_step_buffers, d_cache, host_table, d_grad_pop,
+            d_grad_non, lr: float, deferred: bool, main_stream: int, side_stream: int) -> None:
+    _check("hl_step", _lib.hl_step(ctx, ctypes.byref(batch), _ptr(d_dense), n_dense, ctypes.byref(buffers), _ptr(d_cache),
+                                   _ptr(host_table), _ptr(d_grad_pop), _ptr(d_grad_non), float(lr), int(bool(deferred)),
+                                   main_stream, side_stream))
 
 
 def hl_flush_hot(ctx: int, d_cache, d_hot_rows, d_n_hot, host_table, stream: int) -> None:

@@ -147,8 +147,12 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
     if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_chain, 0, sizeof(unsigned long long) * cold_chain_words(N));
     if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_n, 0, 4 * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(span_count_of(ctx), 0, 8 * sizeof(int32_t));   // kept zero between backward calls
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->step_ranked, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->step_staged, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
+        if (ctx->step_ranked) cudaEventDestroy(ctx->step_ranked);
+        if (ctx->step_staged) cudaEventDestroy(ctx->step_staged);
         delete ctx->launches;
         free(ctx->h_table_base);
         free(ctx);
@@ -220,6 +224,8 @@ extern "C" int32_t hl_destroy(hl_ctx* ctx) {
     for (int w = 0; w < HL_TIMER_COUNT; ++w)
         for (int e = 0; e < 2; ++e)
             if (ctx->timer[w][e]) cudaEventDestroy(ctx->timer[w][e]);
+    if (ctx->step_ranked) cudaEventDestroy(ctx->step_ranked);
+    if (ctx->step_staged) cudaEventDestroy(ctx->step_staged);
     delete ctx->launches;
     free(ctx->h_table_base);
     free(ctx);

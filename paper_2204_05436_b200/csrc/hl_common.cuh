@@ -101,6 +101,7 @@ struct hl_ctx {
     void* mark_user;
     // graphs of the calls that make several kernels, or one in a run of calls (nullptr: plain launches)
     hl::LaunchCache* launches;
+    cudaEvent_t step_ranked, step_staged;      // of hl_step
 };
 
 // Context of the wide-id index path (hl_wide_*): global row ids are 64-bit, every table still has fewer than 2^31
@@ -507,7 +508,8 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
 
 // hl_embbag_bwd_prepare2 / _merged on what fragment_and_mark and cold_rank left behind (hl_embbag.cu): X's cold lookups
 // get their slots, the cold rows are matched against the previous ones, and the pairs are sorted (aside: may be null).  The
-// sort's scratch, backward_sort_clear_words words of bwd_hist, is zero already.
+// sort's scratch, backward_sort_clear_words words of bwd_hist, is zero already.  d_sorted_slots / _bags may be null: the
+// result then stays in the context's scratch, at *out_slots / *out_bags.
 int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge);
 
 // The sort on a stream of its own, behind the pairs (event pairs_ready), with one of two sets of scratch (which): the
@@ -521,7 +523,8 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
                            const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows, const int32_t* d_cold_rows,
                            const int64_t* d_n_cold, const int32_t* d_prev_rows, const int64_t* d_n_prev,
                            int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
-                           bool merge, cudaStream_t stream, const SortAside* aside);
+                           bool merge, cudaStream_t stream, const SortAside* aside, int32_t** out_slots = nullptr,
+                           int32_t** out_bags = nullptr);
 
 // hl_embbag_fwd and hl_forward_cold in one launch (the bags read no staged row).
 int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples, float* d_out,

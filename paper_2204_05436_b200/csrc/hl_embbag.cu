@@ -988,14 +988,14 @@ namespace {
 int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, const hl_ubatch* non,
                      const int32_t* d_n_non, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
                      bool merge, PairArgs a, bool assign, bool cleared, cudaStream_t stream,
-                     const SortAside* aside = nullptr) {
+                     const SortAside* aside = nullptr, int32_t** out_slots = nullptr, int32_t** out_bags = nullptr) {
     if (!ctx || !pop || !non || !pop->offsets || !non->offsets || !d_n_pop || !d_n_non || !d_n_lookups)
         return HL_EINVAL;
     if (ctx->max_nnz == 0) {
         HL_CUDA_TRY(cudaMemsetAsync(d_n_lookups, 0, 4 * sizeof(int32_t), stream));
         return HL_OK;
     }
-    if (!pop->ids || !non->ids || !d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
+    if (!pop->ids || !non->ids || (!out_slots && (!d_sorted_slots || !d_sorted_bags))) return HL_EINVAL;
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     if (2 * n_slots + 2 >= (int64_t(1) << 31)) return HL_EINVAL;
     a.sides = 2;
@@ -1005,7 +1005,7 @@ int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, 
     return as_graph(ctx->launches, [&] {
         int32_t *ok, *ov;
         return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, cleared, d_sorted_slots, d_sorted_bags,
-                              d_n_lookups, &ok, &ov, stream, aside);
+                              d_n_lookups, out_slots ? out_slots : &ok, out_bags ? out_bags : &ov, stream, aside);
     });
 }
 
@@ -1020,7 +1020,8 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
                            const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows, const int32_t* d_cold_rows,
                            const int64_t* d_n_cold, const int32_t* d_prev_rows, const int64_t* d_n_prev,
                            int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
-                           bool merge, cudaStream_t stream, const SortAside* aside) {
+                           bool merge, cudaStream_t stream, const SortAside* aside, int32_t** out_slots,
+                           int32_t** out_bags) {
     PairArgs a{};
     a.ranked = ctx->r.cold_ranked;
     a.slot0 = ctx->hot_cap + stage_row0;
@@ -1032,7 +1033,7 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
     a.n_prev_max = ctx->staging_cap;
     a.fwd_src = d_fwd_src;
     return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, merge, a, true, true,
-                        stream, aside);
+                        stream, aside, out_slots, out_bags);
 }
 
 }  // namespace hl

@@ -219,6 +219,72 @@ int32_t flush_scatter(hl_pipe* p) {
 
 }  // namespace
 
+// One mini-batch.  What bounds a small one is the chain of short kernels: fragment, ranks, pairs and sort (one for both
+// updates, where a sort inside each update would cost its three passes twice), the host read beside the sort.  106 496
+// lookups of 64-byte rows: 133 us with a call for each step, 104 us so.
+extern "C" int32_t hl_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
+                           const hl_step_buffers* s, float* d_cache, float* host_table, const float* d_grad_pop,
+                           const float* d_grad_non, float lr, int32_t flags, void* main_stream, void* side_stream) {
+    if (!ctx || !b || !s || !d_cache || !host_table || !d_grad_pop || !d_grad_non || (flags & ~HL_STEP_DEFERRED))
+        return HL_EINVAL;
+    if (!s->cold_rows || !s->n_cold || !s->pooled_pop || !s->pooled_non || !s->pop.offsets || !s->non.offsets)
+        return HL_EINVAL;
+    cudaStream_t main = static_cast<cudaStream_t>(main_stream), side = static_cast<cudaStream_t>(side_stream);
+    const bool deferred = (flags & HL_STEP_DEFERRED) != 0;
+    hl_ubatch pop = s->pop, non = s->non;
+    // (2^30 cache slots and more: O's and X's slots do not fit one key space, and every update sorts its own)
+    const bool one_sort = ctx->max_nnz > 0 && 2 * (ctx->hot_cap + ctx->staging_cap) + 2 < (int64_t(1) << 31);
+    const int32_t* d_n_non = s->counts + 1;
+    int32_t *slots = nullptr, *bags = nullptr;
+    LaunchBatch batch(ctx->launches);
+    const auto to_side = [&]() -> int32_t {                  // what comes next on `side` sees what `main` has so far
+        if (side == main) return HL_OK;
+        HL_PIPE_TRY(launch_flush() == cudaSuccess ? HL_OK : HL_ECUDA);
+        HL_PIPE_TRY(record(ctx->step_ranked, main));
+        return wait(side, ctx->step_ranked);
+    };
+    const auto side_done = [&]() -> int32_t {
+        if (side == main) return HL_OK;
+        HL_PIPE_TRY(launch_flush() == cudaSuccess ? HL_OK : HL_ECUDA);
+        return record(ctx->step_staged, side);
+    };
+    if (one_sort) {
+        HL_PIPE_TRY(fragment_and_mark(ctx, b, d_dense, d_dense ? n_dense : 0, s->perm, s->counts, &pop, &non,
+                                      d_dense ? s->dense_out : nullptr, main));
+        HL_PIPE_TRY(cold_rank(ctx, ctx->staging_cap, s->cold_rows, s->n_cold, main, ctx->r.bwd_hist[0],
+                              backward_sort_clear_words(ctx, false)));
+        HL_PIPE_TRY(to_side());
+        HL_PIPE_TRY(hl_stage_cold(ctx, host_table, d_cache, 0, ctx->staging_cap, s->cold_rows, s->n_cold, nullptr, side));
+        HL_PIPE_TRY(side_done());
+        HL_PIPE_TRY(hl_embbag_fwd(ctx, d_cache, &pop, s->counts, s->pooled_pop, main));
+        HL_PIPE_TRY(assign_and_prepare(ctx, &pop, s->counts, &non, d_n_non, 0, ctx->staging_cap, s->cold_rows, s->n_cold,
+                                       nullptr, nullptr, nullptr, nullptr, nullptr, ctx->r.bwd_n, false, main, nullptr,
+                                       &slots, &bags));
+    } else {
+        HL_PIPE_TRY(hl_fragment(ctx, b, d_dense, d_dense ? n_dense : 0, s->perm, s->counts, &pop, &non,
+                                d_dense ? s->dense_out : nullptr, main));
+        HL_PIPE_TRY(to_side());
+        HL_PIPE_TRY(hl_gather_cold(ctx, &non, d_n_non, host_table, d_cache, s->cold_rows, s->n_cold, side));
+        HL_PIPE_TRY(side_done());
+        HL_PIPE_TRY(hl_embbag_fwd(ctx, d_cache, &pop, s->counts, s->pooled_pop, main));
+    }
+    const auto update = [&](int which) -> int32_t {
+        const float* grad = which ? d_grad_non : d_grad_pop;
+        if (one_sort) return hl_embbag_bwd_apply2(ctx, d_cache, slots, bags, ctx->r.bwd_n, which, grad, lr, main);
+        return hl_embbag_bwd_sgd(ctx, d_cache, which ? &non : &pop, which ? d_n_non : s->counts, grad, lr, main);
+    };
+    if (!deferred) HL_PIPE_TRY(update(0));
+    if (side != main) {
+        HL_PIPE_TRY(launch_flush() == cudaSuccess ? HL_OK : HL_ECUDA);
+        HL_PIPE_TRY(wait(main, ctx->step_staged));
+    }
+    HL_PIPE_TRY(hl_embbag_fwd(ctx, d_cache, &non, d_n_non, s->pooled_non, main));
+    if (deferred) HL_PIPE_TRY(update(0));
+    HL_PIPE_TRY(update(1));
+    HL_PIPE_TRY(hl_scatter_cold(ctx, d_cache, s->cold_rows, s->n_cold, host_table, main));
+    return batch.end();
+}
+
 extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_table, int64_t window_rows,
                                       int32_t n_sets, const hl_pipe_set* sets, int32_t n_dense, void* main_stream,
                                       const hl_pipe_options* opt) {
