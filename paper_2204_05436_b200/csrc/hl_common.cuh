@@ -486,7 +486,7 @@ int64_t sort_clear_words(int64_t n_max, int key_bits, WaitCfg w);
 // 32-bit words of histogram scratch radix_sort_pairs needs for at most max_nnz pairs.
 constexpr int64_t sort_hist_words(int64_t max_nnz) {
     const int64_t n_tiles = ((max_nnz > 0 ? max_nnz : 1) + kSortTile - 1) / kSortTile;
-    return 4 * 256 + 8 + 4 * n_tiles * 256;   // digit counts, tickets, tile status words for up to 4 passes
+    return 4 * 256 + 4 * n_tiles * 256;   // digit counts, tile status words for up to 4 passes
 }
 
 // ints behind the backward's partial sums: count words + (chunk, key, last chunk of the run or -1, unused) per chunk

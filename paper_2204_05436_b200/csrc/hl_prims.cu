@@ -57,8 +57,8 @@ __device__ __forceinline__ int64_t clamp_n(const int32_t* d_n, int64_t n_max) {
 }
 
 // ---- single-pass chaining between tiles --------------------------------------------------------------------
-// Tiles are handed out by a ticket counter, so a tile's predecessors are always held by blocks that have
-// started.  A tile first publishes its own sum (AGGREGATE), then walks back over its predecessors adding their
+// A tile is a CTA's block index, and CTAs are dispatched in that order, so a tile's predecessors are always held by blocks
+// that have started.  A tile first publishes its own sum (AGGREGATE), then walks back over its predecessors adding their
 // sums until it meets one that already knows its inclusive prefix (PREFIX), and finally publishes its own
 // prefix.  Publishing never waits on anything, so the walk always terminates; every poll is bounded all the same,
 // and a poll that runs out records HL_ETIMEOUT and carries on with what it has (positions are range-checked).
@@ -167,37 +167,42 @@ __global__ void __launch_bounds__(kThreads) k_sort_digit_hist(const int32_t* __r
 }
 
 // One pass: stable scatter by one digit.  Order of the items of a tile: warp-major, then round, then lane.
-// ghist: this pass's 256 digit counts; ticket: tile counter; tstat[tile][256]: status words, zero on entry.
+// ghist: this pass's 256 digit counts; tstat[tile][256]: status words, zero on entry.  A tile is the CTA's block index: CTAs
+// are dispatched in that order, so those of the tiles before have started.  With few tiles a pass is a chain of latencies:
+// everything that does not depend on another load is requested first.
 __global__ void __launch_bounds__(kThreads) k_sort_pass(const int32_t* __restrict__ keys_in,
                                                         const int32_t* __restrict__ vals_in,
                                                         int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out,
                                                         const int32_t* d_n, int64_t n_max, int shift,
-                                                        const uint32_t* __restrict__ ghist, uint32_t* ticket,
+                                                        const uint32_t* __restrict__ ghist,
                                                         uint32_t* tstat, int32_t* status, int max_polls,
                                                         int64_t stall_tile) {
     constexpr int kWarps = kThreads / 32;
     __shared__ uint32_t cnt[kWarps][256];
     __shared__ uint32_t digit_base[256];
     __shared__ int scan_smem[40];
-    __shared__ uint32_t s_tile;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
-    for (int i = threadIdx.x; i < kWarps * 256; i += kThreads) (&cnt[0][0])[i] = 0;
-    __syncthreads();
-    const int64_t tile = s_tile;
+    const int64_t tile = blockIdx.x;
+    const int64_t warp_base = tile * kSortTile + (int64_t)warp * (32 * kItems);
     const int64_t n = clamp_n(d_n, n_max);
     if (tile * kSortTile >= n) return;
-
-    const int64_t warp_base = tile * kSortTile + (int64_t)warp * (32 * kItems);
     int32_t key[kItems], val[kItems];
     uint32_t rank[kItems];
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const int64_t idx = warp_base + r * 32 + lane;
+        key[r] = idx < n ? keys_in[idx] : 0;
+        val[r] = idx < n ? vals_in[idx] : 0;
+    }
+    const int32_t of_digit = (int32_t)ghist[threadIdx.x];
+    for (int i = threadIdx.x; i < kWarps * 256; i += kThreads) (&cnt[0][0])[i] = 0;
+    __syncthreads();
+
     const unsigned lt = lanemask_lt();
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const int64_t idx = warp_base + r * 32 + lane;
         const bool valid = idx < n;
-        key[r] = valid ? keys_in[idx] : 0;
-        val[r] = valid ? vals_in[idx] : 0;
         const uint32_t d = ((uint32_t)key[r] >> shift) & 255u;
         const unsigned peers = same_digit(d, valid);
         uint32_t before = 0;
@@ -219,8 +224,10 @@ __global__ void __launch_bounds__(kThreads) k_sort_pass(const int32_t* __restric
     }
     uint32_t before = 0;
     uint32_t* my = tstat + tile * 256 + d;
+    if (tile > 0 && tile != stall_tile) st_relaxed(my, kFlagAgg | total);
+    int all;
+    const int gbase = block_exclusive_scan(of_digit, scan_smem, all);   // keys with a smaller digit
     if (tile > 0) {
-        if (tile != stall_tile) st_relaxed(my, kFlagAgg | total);
         // walk back kLook tiles at a time (32 at a time was no faster and cost 16 registers): the kLook status
         // words are requested together, then consumed from the
         // nearest tile outwards until one of them already carries an inclusive prefix
@@ -249,8 +256,6 @@ __global__ void __launch_bounds__(kThreads) k_sort_pass(const int32_t* __restric
         }
     }
     if (tile != stall_tile) st_relaxed(my, kFlagPrefix | ((before + total) & kValueMask));
-    int all;
-    const int gbase = block_exclusive_scan((int)ghist[d], scan_smem, all);   // keys with a smaller digit
     digit_base[d] = (uint32_t)gbase + before;
     __syncthreads();
 #pragma unroll
@@ -407,7 +412,7 @@ static bool sort_in_cluster(int64_t n_max, const WaitCfg& w) {
 
 int64_t sort_clear_words(int64_t n_max, int key_bits, WaitCfg w) {
     if (n_max <= 0 || sort_in_cluster(n_max, w)) return 0;
-    return 4 * 256 + 8 + (int64_t)((key_bits + 7) / 8) * div_up(n_max, kSortTile) * 256;
+    return 4 * 256 + (int64_t)((key_bits + 7) / 8) * div_up(n_max, kSortTile) * 256;
 }
 
 int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n, int64_t n_max, int key_bits,
@@ -429,10 +434,9 @@ int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n,
         return HL_OK;
     }
     const int64_t n_tiles = div_up(n_max, kSortTile);
-    // scratch: [4][256] digit counts, 8 ticket words, [passes][n_tiles][256] tile status words
+    // scratch: [4][256] digit counts, [passes][n_tiles][256] tile status words
     uint32_t* ghist = hist;
-    uint32_t* ticket = hist + 4 * 256;
-    uint32_t* tstat = hist + 4 * 256 + 8;
+    uint32_t* tstat = hist + 4 * 256;
     if (!counted) {
         HL_CUDA_TRY(clear_words(hist, sort_clear_words(n_max, key_bits, w), stream));
         HL_CUDA_TRY(launch(k_sort_digit_hist, grid_for(n_max, kThreads * 8, 1024), kThreads, stream, keys[0], d_n, n_max,
@@ -441,7 +445,7 @@ int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n,
     }
     for (int p = 0; p < passes; ++p)
         HL_CUDA_TRY(launch(k_sort_pass, (unsigned)n_tiles, kThreads, stream, keys[p & 1], vals[p & 1], keys[(p & 1) ^ 1],
-                           vals[(p & 1) ^ 1], d_n, n_max, 8 * p, ghist + 256 * p, ticket + p,
+                           vals[(p & 1) ^ 1], d_n, n_max, 8 * p, ghist + 256 * p,
                            tstat + (size_t)p * n_tiles * 256, status, w.max_polls, w.stall_tile));
     note_launches(passes);
     HL_LAUNCH_CHECK();
