@@ -326,8 +326,10 @@ struct BitmapProbe {
 };
 
 // ---- the cold-row bitmap --------------------------------------------------------------------------------------
-// Above this many rows the bitmap is read through a summary.  (16 M rows: 2 MB of bitmap, a few microseconds to read.)
-constexpr int64_t kColdDirectRows = int64_t(1) << 24;
+// Above this many rows the bitmap is read through a summary.  Reading all of it costs little (64 M rows: 8 MB, 20 us), and
+// its words are dealt out evenly; behind a summary word the lookups of a table's first rows pile up on a few lanes (150 K
+// cold rows out of 18, 26 and 50 million: 36, 34 and 73 us through the summary, 15, 15 and 20 us without).
+constexpr int64_t kColdDirectRows = int64_t(1) << 26;
 constexpr int64_t cold_bitmap_words(int64_t N) { return (N + 31) / 32; }
 constexpr int64_t cold_summary_words(int64_t N) { return (cold_bitmap_words(N) + 31) / 32; }
 // ticket, tally and one status word per tile of k_cold_rank (at least 256 words per tile)

@@ -24,8 +24,8 @@ CASES = {
     "sort_32768": ([5000] * 8, 4096, 1, 1, 1, 0.9),
     "sort_32776": ([5000] * 8, 4097, 1, 1, 1, 0.9),
     "rank_four_words": ([1_300_000] * 4, 700, 1, 0, 4, 0.3),
-    "rank_16777216_rows": ([1 << 23] * 2, 500, 1, 1, 2, 0.02),
-    "rank_summary": ([1 << 23, (1 << 23) + 1], 500, 1, 1, 2, 0.02),
+    "rank_67108864_rows": ([1 << 25] * 2, 500, 1, 1, 2, 0.005),
+    "rank_summary": ([1 << 25, (1 << 25) + 1], 500, 1, 1, 2, 0.005),
     "rank_summary_four_words": ([60_000_001] * 2, 3000, 1, 0, 3, 0.001),
 }
 
