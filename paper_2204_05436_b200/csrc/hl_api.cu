@@ -51,8 +51,7 @@ size_t carve(char* base, const hl_geometry* g, int64_t N, int32_t max_batch, int
     r->remap = c.take<RemapBlock>(*n_remap_blocks);
     r->counts = c.take<uint32_t>(N);
     r->sel = c.take<SelectState>(1);
-    r->sel_gt = c.take<uint32_t>(*n_sel_tiles + 2);
-    r->sel_eq = c.take<uint32_t>(*n_sel_tiles + 2);
+    r->sel_chain = c.take<unsigned long long>(*n_sel_tiles + 1);
     r->frag_words = c.take<uint32_t>(max_batch / 32 + 1);
     r->frag_chain = c.take<unsigned long long>(frag_chain_words(max_bags));
     for (int i = 0; i < 2; ++i) {

@@ -42,6 +42,7 @@ struct SelectState {
     unsigned int mask;                 // bits of `prefix` that are fixed
     unsigned int c_min;                // smallest admissible count (>= 1)
     unsigned int threshold;            // final: k-th largest admissible count
+    unsigned int finished;             // CTAs done with the current digit
     int take_all;                      // fewer admissible rows than wanted: keep them all
 };
 
@@ -54,8 +55,7 @@ struct Regions {
     // profile
     uint32_t* counts;                  // [N]
     SelectState* sel;
-    uint32_t* sel_gt;                  // [n_sel_tiles + 1]
-    uint32_t* sel_eq;                  // [n_sel_tiles + 1]
+    unsigned long long* sel_chain;     // [n_sel_tiles + 1]
     // fragment
     uint32_t* frag_words;              // [max_batch / 32 + 1] all-hit flags
     unsigned long long* frag_chain;    // [frag_chain_words]
@@ -121,7 +121,7 @@ struct hl_wide {
     long long* c_keys;                       // [counter_slots] row id or -1
     uint32_t* c_cnt;                         // [counter_slots]
     hl::SelectState* sel;
-    uint32_t *sel_gt, *sel_eq;               // [counter_slots / kSelTile + 2]
+    unsigned long long* sel_chain;           // [counter_slots / kSelTile + 1]
     int32_t* n_seen;                         // [4]
     int32_t *e_tab, *e_idx;                  // [counter_slots] table and table-local index of every counted row
     uint32_t *e_cnt, *s_cnt;                 // [counter_slots] its count; the counts in row order
@@ -538,9 +538,9 @@ int32_t fragment_and_mark(hl_ctx* ctx, const hl_batch* b, const float* d_dense, 
                           int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non, float* d_dense_out, cudaStream_t stream);
 
 // Selection of the rows with the k largest counts (implemented in hl_profile.cu; see there).
-int32_t select_rows_by_count(const uint32_t* counts, int64_t n, SelectState* sel, uint32_t* sel_gt, uint32_t* sel_eq,
-                             long long k, long long share_num, long long share_den, int64_t cap, int32_t* out_idx,
-                             int64_t* d_n_out, int32_t* status, int sms, cudaStream_t stream);
+int32_t select_rows_by_count(const uint32_t* counts, int64_t n, SelectState* sel, unsigned long long* chain, long long k,
+                             long long share_num, long long share_den, int64_t cap, int32_t* out_idx, int64_t* d_n_out,
+                             int32_t* status, int sms, cudaStream_t stream);
 
 // Process-wide count of kernels this library has launched (read by hl_launch_count).
 void note_launches(int n);

@@ -47,8 +47,7 @@ size_t carve(char* base, hl_wide* w) {
     w->c_keys = c.take<long long>(E);
     w->c_cnt = c.take<uint32_t>(E);
     w->sel = c.take<SelectState>(1);
-    w->sel_gt = c.take<uint32_t>(div_up(E, kSelTile) + 2);
-    w->sel_eq = c.take<uint32_t>(div_up(E, kSelTile) + 2);
+    w->sel_chain = c.take<unsigned long long>(div_up(E, kSelTile) + 1);
     w->n_seen = c.take<int32_t>(4);
     w->e_tab = c.take<int32_t>(E);
     w->e_idx = c.take<int32_t>(E);
@@ -539,7 +538,7 @@ extern "C" int32_t hl_wide_profile_hot(hl_wide* w, const hl_batch* b, int32_t re
                        w->s_cnt, w->s_ent));
     note_launches(1);
     HL_LAUNCH_CHECK();
-    st = select_rows_by_count(w->s_cnt, E, w->sel, w->sel_gt, w->sel_eq, k, share_num, share_den, w->hot_cap,
+    st = select_rows_by_count(w->s_cnt, E, w->sel, w->sel_chain, k, share_num, share_den, w->hot_cap,
                               w->sel_idx, d_n_hot, w->status, w->sms, stream);
     if (st != HL_OK) return st;
     HL_CUDA_TRY(launch(k_wide_hot_rows, grid_for(w->hot_cap, kThreads, w->sms * 8), kThreads, stream, w->sel_idx, d_n_hot,
