@@ -17,7 +17,7 @@ namespace hl {
 constexpr int kSMsFallback = 148;          // used only if the device's SM count cannot be queried (B200: 2 x 74)
 constexpr int kRemapRowsPerBlock = 224;    // 7 bitmap words per 32-byte remap block
 constexpr int kSortTile = 2048;            // keys per radix-sort tile (256 threads x 8)
-constexpr int kSelTile = 4096;             // rows per hot-set selection tile (256 threads x 16)
+constexpr int kSelTile = 8192;             // rows per hot-set selection tile (256 threads x 32)
 constexpr int kBwdChunk = 32;              // sorted lookups per backward chunk
 constexpr int kMoverCtasDefault = 16;      // working CTAs of a host-link mover inside a schedule: write-backs
 constexpr int kReadCtasDefault = 24;       // ... and host reads (a wider read finishes sooner and costs the step nothing)

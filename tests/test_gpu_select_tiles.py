@@ -1,4 +1,4 @@
-"""The hot-set selection at the edges of its tiles (4 096 rows, four counts per load) and digits (8 bits of the count; digits
+"""The hot-set selection at the edges of its tiles (8 192 rows, four counts per load) and digits (8 bits of the count; digits
 that no count reaches are not looked at): ties cut by the quota, more rows wanted than were counted, none wanted."""
 import numpy as np
 import pytest
@@ -11,7 +11,7 @@ DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("top", [1, 255, 256, 70_000])
-@pytest.mark.parametrize("rows", [1, 3, 511, 4095, 4096, 4097, 8190, 1_300_001])
+@pytest.mark.parametrize("rows", [1, 3, 511, 1023, 1025, 8191, 8192, 8193, 16_382, 1_300_001])
 def test_selected_rows(rows, top):
     import paper_2204_05436_b200 as hl
     rng = np.random.default_rng(rows + top)
