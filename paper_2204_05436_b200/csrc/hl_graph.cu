@@ -103,7 +103,7 @@ cudaError_t launch_now(const void* func, dim3 grid, dim3 block, size_t smem, int
 
 }  // namespace
 
-// One kept graph: the recording it was last launched with, and its executable form.
+// One kept graph: the recording it was last launched with, and its executable form (none yet if it came only once).
 struct LaunchCache::Entry {
     Recording rec;
     cudaGraph_t graph = nullptr;
@@ -134,6 +134,8 @@ struct LaunchCache::Entry {
         if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
         return e;
     }
+
+    cudaError_t prepare(const Recording& r) { return exec ? update(r) : build(r); }
 
     // the arguments that differ from the last launch's (future launches only: one in flight keeps its own)
     cudaError_t update(const Recording& r) {
@@ -179,9 +181,10 @@ thread_local Collecting t_now;
 
 }  // namespace
 
-// Launches a recording: as the kept graph that had these kernels and arguments, as one with these kernels whose arguments
-// are brought up to date (the one not used for longest, once there are `variants_` of them), or as a new graph.  At most
-// kMaxEntries are kept.
+// Launches a recording: as the kept graph that had these kernels and arguments, or as one with these kernels whose arguments
+// are brought up to date (the one not used for longest, once there are `variants_` of them).  Building a graph costs some
+// 50 us, so kernels that come for the first time are launched one by one and only remembered; the graph is built when they
+// come again.  At most kMaxEntries are kept.
 cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
     Recording& r = *const_cast<Recording*>(static_cast<const Recording*>(recording));
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -204,27 +207,34 @@ cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
             break;
         }
     }
-    Entry* e = exact;
-    if (!e && alike >= variants_ && oldest->update(r) == cudaSuccess) e = oldest;
-    if (!e) {
+    Entry* e = exact ? exact : alike >= variants_ ? oldest : nullptr;
+    if (e && e->prepare(r) != cudaSuccess) {
+        for (auto& x : entries_)
+            if (x == e) {
+                x = entries_.back();
+                break;
+            }
+        entries_.pop_back();
+        delete e;
         cudaGetLastError();
-        if ((int)entries_.size() >= kMaxEntries || alike >= variants_) {
-            Entry* out = alike >= variants_ ? oldest : any_oldest;
+        return launch_one_by_one(r, stream);                 // (no memory for it: the plain launches still work)
+    }
+    if (!e) {
+        if ((int)entries_.size() >= kMaxEntries) {
             for (auto& x : entries_)
-                if (x == out) {
+                if (x == any_oldest) {
                     x = entries_.back();
                     break;
                 }
             entries_.pop_back();
-            delete out;
+            delete any_oldest;
         }
-        e = new (std::nothrow) Entry();
-        if (!e || e->build(r) != cudaSuccess) {              // (no memory for it: the plain launches still work)
-            delete e;
-            cudaGetLastError();
-            return launch_one_by_one(r, stream);
+        if (Entry* seen = new (std::nothrow) Entry()) {
+            seen->rec = r;
+            seen->used = ++tick_;
+            entries_.push_back(seen);
         }
-        entries_.push_back(e);
+        return launch_one_by_one(r, stream);
     }
     e->used = ++tick_;
     return cudaGraphLaunch(e->exec, stream);
