@@ -257,6 +257,7 @@ constexpr int kBulkStagesPerCta = 200;    // stages of rows per working CTA befo
 constexpr int kPacedRequests = 40;
 constexpr int kPacedReadBytes = 8192;
 constexpr int64_t kPacedMost = 1 << 16;
+constexpr int64_t kFarTableBytes = int64_t(32) << 30;     // between the two sizes measured (move_cfg)
 
 // What a launch of the mover needs to know about its context.
 struct MoveCfg {
@@ -451,11 +452,15 @@ static TableMap table_map(const hl_ctx* ctx, const float* host_table) {
 
 // how the movers of this context are launched: beside the kernels of other mini-batches (`width` = the context's setting),
 // or alone on the chip (`width` = 0: two CTAs per SM, the link's full rate)
-static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false) {
+static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false, bool reads = false) {
     MoveCfg c;
     c.sms = ctx_sms(ctx);
     c.min_ctas = width > 0 ? width : 2 * c.sms;
-    c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : kPacedCtas) : 0;
+    // Reads out of a large host table answer later (their address translations miss), so more of them have to be on the way:
+    // 16 K rows of 256 bytes out of 61 GiB take 159 us with 16 CTAs and 135 us with 24 (a pass of the schedule 0.241 and
+    // 0.231 ms); out of 6 GiB 24 CTAs only disturb the others (three pipelines in turn: 159 and 167 us a pass).
+    const bool far = reads && ctx->N * ctx->D * 4 > kFarTableBytes;
+    c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : far ? kReadCtasDefault : kPacedCtas) : 0;
     c.max_polls = ctx->test_poll_limit > 0 ? ctx->test_poll_limit : kBulkMaxPolls;
     c.stall = ctx->test_poll_limit > 0 && ctx->test_stall_tile >= 0;
     return c;
@@ -523,7 +528,7 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 0, stream);
         const int32_t st = launch_move_rows<false>(d_cache, ctx->hot_cap + stage_row0,
                                                    table_map(ctx, host_table), d_cold_rows, d_n_cold, stage_rows,
-                                                   ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas, true),
+                                                   ctx->N, ctx->D, d_fwd_src, move_cfg(ctx, ctx->mover_ctas, true, true),
                                                    r.status, stream);
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 1, stream);
         return batch.end(st);
