@@ -431,7 +431,7 @@ def timeline_text(spans, mini_batches):
     if not rows:
         return ""
     t0 = rows[0]["begin_ms"]
-    names = {0: "main", 1: "frag", 2: "sort", 3: "cold", 4: "read", 5: "wb"}
+    names = {0: "main", 1: "index", 2: "sort", 4: "read", 5: "wb"}
     out = ["   begin_us      end_us   dur_us  stream  mini-batch  what"]
     for sp in rows:
         out.append(f"{(sp['begin_ms'] - t0) * 1e3:10.1f}  {(sp['end_ms'] - t0) * 1e3:10.1f}  "

@@ -164,8 +164,8 @@ HL_API int32_t hl_set_mover_ctas(hl_ctx* ctx, int32_t read_ctas, int32_t write_c
 HL_API int32_t hl_set_kernel_width(hl_ctx* ctx, int32_t fwd_ctas_per_sm, int32_t bwd_ctas_per_sm);
 
 /* Test aid for the bounded device-side waits (the tile chaining of the prefix sums inside hl_fragment and
- * hl_gather_cold and of the sorts inside hl_embbag_bwd_*, the wait of a row mover for a stage of bulk copies).  In production these
- * waits poll for about a second before they give up, which never happens.  poll_limit > 0 makes them give up after
+ * hl_gather_cold and of the sorts inside hl_embbag_bwd_*, the wait of a row mover for a stage of bulk copies).  In
+ * production these waits poll for about a second before they give up, which never happens.  poll_limit > 0 makes them give up after
  * that many polls, and makes ONE participant withhold what the others wait for: tile `stall_tile` of every chained scan
  * and sort pass publishes nothing, and (stall_tile >= 0) the first stage of the movers' first CTA issues no copies.
  * The waits behind it then run out: the kernels return, the status word reads HL_ETIMEOUT, every position computed

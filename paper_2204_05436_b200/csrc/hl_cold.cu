@@ -394,7 +394,8 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
         const int paced_rows = paced_fit > 1 ? paced_fit : 1;
         HL_CUDA_TRY(launch(k_move_rows_bulk<TO_TABLE>, grid, kBulkThreads, stream, dense_side, dense_row0, table, rows, d_n,
                            n_max, table_rows, row_bytes, rows_per_stage, skip, status,
-                           cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, kPacedMost / requests, paced_rows < rows_per_stage ? paced_rows : rows_per_stage, cfg.max_polls, cfg.stall));
+                           cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, kPacedMost / requests,
+                           paced_rows < rows_per_stage ? paced_rows : rows_per_stage, cfg.max_polls, cfg.stall));
         note_launches(1);
         HL_LAUNCH_CHECK();
         return HL_OK;

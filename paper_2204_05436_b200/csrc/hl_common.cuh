@@ -412,7 +412,8 @@ inline WaitCfg wait_cfg(const hl_ctx* ctx) {
 // hundred tiles cost one or two round trips to the L2, where one warp walks them 32 a step (placing 106 thousand bags:
 // 11.7 us with a one-warp walk over 416 tiles, 8.2 us with this over 104).  A tile is the CTA's block index (CTAs are
 // dispatched in that order, so the tiles before have started), and publishing never waits; every poll is bounded all the
-// same, and one that runs out records HL_ETIMEOUT and carries on with what it has.  words[tile]: zero on entry.  Both calls are made by all NT threads; chain_before's result is the same in all.
+// same, and one that runs out records HL_ETIMEOUT and carries on with what it has.  words[tile]: zero on entry.
+// Both calls are made by all NT threads; chain_before's result is the same in all.
 constexpr unsigned long long kChainAgg = 1ull << 62, kChainPrefix = 1ull << 63, kChainSum = kChainAgg - 1ull;
 
 __device__ __forceinline__ unsigned long long ld_relaxed64(const unsigned long long* p) {

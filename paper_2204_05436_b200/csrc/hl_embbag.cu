@@ -187,7 +187,8 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const 
     float4* __restrict__ out4 = reinterpret_cast<float4*>(out);
 
     if (MANY) {
-        const int64_t warps = (int64_t)gridDim.x * (kThreads / 32), me = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
+        const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
+        const int64_t me = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
         const int64_t first = n_bags * me / warps, last = n_bags * (me + 1) / warps;
         if (first < last) pool_bags<NV>(rows, ids, offsets, first, last, threadIdx.x & 31, D4, n_slots, out4, status);
         return;

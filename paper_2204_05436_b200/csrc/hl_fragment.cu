@@ -190,8 +190,9 @@ __global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __re
 }
 
 // ---- placing --------------------------------------------------------------------------------------------------
-// The lookups of X are written as global row ids (int64 on the wide path).  With MARK (the scheduler's calls) the first half of the cold-row search is done on the way instead: a popular row
-// becomes its slot, any other row g is marked in the cold-row bitmap and written as -2 - g (classify_cold).
+// The lookups of X are written as global row ids (int64 on the wide path).  With MARK (the scheduler's calls) the first half
+// of the cold-row search is done on the way instead: a popular row becomes its slot, any other row g is marked in the
+// cold-row bitmap and written as -2 - g (classify_cold).
 //
 // The chain between tiles carries two sums, lookups of O and lookups of X: 31 bits each, below two flag bits.
 constexpr int kHalf = 31;

@@ -82,7 +82,8 @@ bool same_kernels(const Recording& a, const Recording& b) {
 
 bool same_node(const Recording& a, const Recording& b, int i) {
     const Node &x = a.node[i], &y = b.node[i];
-    return same_shape(x, y) && x.n_bytes == y.n_bytes && std::memcmp(a.arg + x.first_byte, b.arg + y.first_byte, x.n_bytes) == 0;
+    return same_shape(x, y) && x.n_bytes == y.n_bytes &&
+           std::memcmp(a.arg + x.first_byte, b.arg + y.first_byte, x.n_bytes) == 0;
 }
 
 cudaError_t launch_now(const void* func, dim3 grid, dim3 block, size_t smem, int cluster, void** args, cudaStream_t stream) {

@@ -13,7 +13,8 @@
 // The index work is one stream (two), so that its steps need no events between them, and as few kernels as its data
 // dependences allow (five with at most 32 K lookups, otherwise four and one per sort digit); the rows forwarded between
 // windows ride on the popular forward.  13 to 15 launches, no memset and 12 to 15 event operations, where separate calls on
-// three streams made 22, 3 and 25 (8 K lookups: 88 us per mini-batch).
+// three streams made 22, 3 and 25 (8 K lookups: 88 us per mini-batch).  The kernels between two event operations go out as one
+// graph (hl_graph.cu): 17 us on the host instead of 41, 35 us per mini-batch instead of 54.
 #include "hl_common.cuh"
 
 #include <memory>

@@ -136,8 +136,8 @@ __global__ void __launch_bounds__(kThreads) k_select_digit(const uint32_t* __res
 // Ordered compaction: a row is popular if its count beats the threshold, or equals it and fewer than quota_eq
 // equal rows precede it.  Its position = popular rows with a smaller id.  A warp takes an eighth of the tile, in rows of
 // 32 lanes x 4 counts; the sums of the tiles before (rows above the threshold, rows at it) come through chained tiles, so
-// that the counts are read once.  9.3 M rows: 42 us for the whole selection (tiles of 4 096 rows: 52); with the counts of the tiles, their prefix
-// sums and the emission as kernels of their own, and a kernel per picked digit, 110 us.
+// that the counts are read once.  9.3 M rows: 42 us for the whole selection (tiles of 4 096 rows: 52); with the counts of
+// the tiles, their prefix sums and the emission as kernels of their own, and a kernel per picked digit, 110 us.
 __global__ void __launch_bounds__(kThreads) k_select_emit(const uint32_t* __restrict__ counts, int64_t N,
                                                           const SelectState* __restrict__ sel, unsigned long long* chain,
                                                           int64_t hot_cap, int32_t* __restrict__ hot_rows,
