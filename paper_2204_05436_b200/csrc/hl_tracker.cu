@@ -263,7 +263,9 @@ extern "C" int32_t hl_tracker_update(hl_ctx* ctx, const hl_batch* b, int32_t* d_
     const int key_bits = bits_for(n_sets);
     const int64_t n_clear = sort_clear_words(ctx->max_nnz, key_bits, WaitCfg());
     if (n_clear > 0) HL_CUDA_TRY(clear_words(r.bwd_hist[0], n_clear, stream));
-    HL_CUDA_TRY(launch(n_clear > 0 ? k_trk_keys<true> : k_trk_keys<false>, grid_for(n_bags, kThreads, 4 * ctx_sms(ctx)),
+    // (every CTA adds its digit counts to the same words in the end: 426 K lookups 8.4 us with 3 CTAs per SM, 9.3 with 4,
+    // 18 with 16, 11.5 with 1)
+    HL_CUDA_TRY(launch(n_clear > 0 ? k_trk_keys<true> : k_trk_keys<false>, grid_for(n_bags, kThreads, 3 * ctx_sms(ctx)),
                        kThreads, stream, b->indices, b->offsets, n_bags, bags_per_table, r.table_base, ctx->max_nnz,
                        (uint32_t)n_sets, r.bwd_keys[0], r.bwd_vals[0], r.bwd_n, r.bwd_hist[0], (key_bits + 7) / 8,
                        r.status));

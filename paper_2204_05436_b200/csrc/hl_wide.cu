@@ -580,7 +580,7 @@ extern "C" int32_t hl_wide_index_cold(hl_wide* w, const int32_t* d_non_offsets, 
     const int64_t sort_words = sort_clear_words(w->max_nnz, lower_bits, WaitCfg());
     HL_CUDA_TRY(clear_words(w->cold_clear, (int64_t)(w->sort_hist - w->cold_clear) + sort_words, stream));
     HL_CUDA_TRY(launch(sort_words ? k_wide_classify<true> : k_wide_classify<false>,
-                       grid_for(w->max_nnz, kThreads, 8 * w->sms), kThreads, stream,
+                       grid_for(w->max_nnz, kThreads, 3 * w->sms), kThreads, stream,
                        reinterpret_cast<const long long*>(d_non_rows), d_non_offsets, d_n_non, w->max_batch, w->T * w->S,
                        non_cap, w->N, probe, d_non_slots, w->sort_keys[0], w->sort_vals[0], w->cold_n, w->max_nnz,
                        w->sort_hist, (lower_bits + 7) / 8, w->status));
