@@ -166,11 +166,15 @@ public:
     cudaError_t launch(const void* recording, cudaStream_t stream);
 
 private:
-    static constexpr int kMaxEntries = 24;
+    // (A context's calls make some 40 different runs of kernels, over all sizes of mini-batches; a program that had more than
+    // these in use would see the longest unused one's graphs built again.)
+    static constexpr int kMaxLists = 64, kMaxVariants = 4;
     struct Entry;
-    std::vector<Entry*> entries_;
+    struct List;
+    List* list_of(const void* recording);
+    List* lists_ = nullptr;
     std::mutex mutex_;
-    int variants_;
+    const int variants_;
     uint64_t tick_ = 0;
 };
 

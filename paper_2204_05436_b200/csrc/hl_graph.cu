@@ -73,13 +73,6 @@ bool same_shape(const Node& a, const Node& b) {
            a.block.y == b.block.y && a.block.z == b.block.z && a.smem == b.smem;
 }
 
-bool same_kernels(const Recording& a, const Recording& b) {
-    if (a.n != b.n) return false;
-    for (int i = 0; i < a.n; ++i)
-        if (a.node[i].func != b.node[i].func || a.node[i].cluster != b.node[i].cluster) return false;
-    return true;
-}
-
 bool same_node(const Recording& a, const Recording& b, int i) {
     const Node &x = a.node[i], &y = b.node[i];
     return same_shape(x, y) && x.n_bytes == y.n_bytes &&
@@ -104,7 +97,7 @@ cudaError_t launch_now(const void* func, dim3 grid, dim3 block, size_t smem, int
 
 }  // namespace
 
-// One kept graph: the recording it was last launched with, and its executable form (none yet if it came only once).
+// One kept graph: the recording it was last launched with, and its executable form.
 struct LaunchCache::Entry {
     Recording rec;
     cudaGraph_t graph = nullptr;
@@ -115,6 +108,12 @@ struct LaunchCache::Entry {
     ~Entry() {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
+    }
+
+    bool same_arguments(const Recording& r) const {
+        for (int i = 0; i < r.n; ++i)
+            if (!same_node(rec, r, i)) return false;
+        return true;
     }
 
     cudaError_t build(const Recording& r) {
@@ -136,8 +135,6 @@ struct LaunchCache::Entry {
         return e;
     }
 
-    cudaError_t prepare(const Recording& r) { return exec ? update(r) : build(r); }
-
     // the arguments that differ from the last launch's (future launches only: one in flight keeps its own)
     cudaError_t update(const Recording& r) {
         for (int i = 0; i < r.n; ++i) {
@@ -153,9 +150,67 @@ struct LaunchCache::Entry {
     }
 };
 
-LaunchCache::LaunchCache(int variants) : variants_(variants) {}
+// The kernels of one run, and the graphs of them that there are.
+struct LaunchCache::List {
+    List* next = nullptr;
+    uint64_t used = 0;
+    int n = 0, graphs = 0;
+    const void* func[kMaxNodes];
+    int cluster[kMaxNodes];
+    Entry* graph[kMaxVariants] = {};
+
+    ~List() {
+        for (int i = 0; i < graphs; ++i) delete graph[i];
+    }
+    bool has(const Recording& r) const {
+        if (n != r.n) return false;
+        for (int i = 0; i < n; ++i)
+            if (func[i] != r.node[i].func || cluster[i] != r.node[i].cluster) return false;
+        return true;
+    }
+    void drop(Entry* e) {
+        for (int i = 0; i < graphs; ++i)
+            if (graph[i] == e) {
+                graph[i] = graph[--graphs];
+                delete e;
+                return;
+            }
+    }
+};
+
+LaunchCache::LaunchCache(int variants) : variants_(variants < kMaxVariants ? variants : kMaxVariants) {}
 LaunchCache::~LaunchCache() {
-    for (Entry* e : entries_) delete e;
+    while (lists_) {
+        List* l = lists_;
+        lists_ = l->next;
+        delete l;
+    }
+}
+
+// the list of these kernels; a new one if they come for the first time (nullptr: no memory for it)
+LaunchCache::List* LaunchCache::list_of(const void* recording) {
+    const Recording& r = *static_cast<const Recording*>(recording);
+    int n = 0;
+    List** oldest = nullptr;
+    for (List** l = &lists_; *l; l = &(*l)->next, ++n) {
+        if ((*l)->has(r)) return *l;
+        if (!oldest || (*l)->used < (*oldest)->used) oldest = l;
+    }
+    if (n >= kMaxLists) {
+        List* gone = *oldest;
+        *oldest = gone->next;
+        delete gone;
+    }
+    List* l = new (std::nothrow) List();
+    if (!l) return nullptr;
+    l->n = r.n;
+    for (int i = 0; i < r.n; ++i) {
+        l->func[i] = r.node[i].func;
+        l->cluster[i] = r.node[i].cluster;
+    }
+    l->next = lists_;
+    lists_ = l;
+    return l;
 }
 
 namespace {
@@ -185,7 +240,7 @@ thread_local Collecting t_now;
 // Launches a recording: as the kept graph that had these kernels and arguments, or as one with these kernels whose arguments
 // are brought up to date (the one not used for longest, once there are `variants_` of them).  Building a graph costs some
 // 50 us, so kernels that come for the first time are launched one by one and only remembered; the graph is built when they
-// come again.  At most kMaxEntries are kept.
+// come again.
 cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
     Recording& r = *const_cast<Recording*>(static_cast<const Recording*>(recording));
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -194,49 +249,34 @@ cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
         return launch_one_by_one(r, stream);
     }
     std::lock_guard<std::mutex> lock(mutex_);
-    Entry *exact = nullptr, *oldest = nullptr, *any_oldest = nullptr;
-    int alike = 0;
-    for (Entry* e : entries_) {
-        if (!any_oldest || e->used < any_oldest->used) any_oldest = e;
-        if (!same_kernels(e->rec, r)) continue;
-        ++alike;
-        if (!oldest || e->used < oldest->used) oldest = e;
-        bool same = true;
-        for (int i = 0; i < r.n && same; ++i) same = same_node(e->rec, r, i);
-        if (same) {
-            exact = e;
-            break;
+    List* l = list_of(recording);
+    if (!l) return launch_one_by_one(r, stream);
+    const bool again = l->used != 0;
+    l->used = ++tick_;
+    Entry *e = nullptr, *oldest = nullptr;
+    for (int i = 0; i < l->graphs && !e; ++i) {
+        if (l->graph[i]->same_arguments(r)) e = l->graph[i];
+        if (!oldest || l->graph[i]->used < oldest->used) oldest = l->graph[i];
+    }
+    if (!e && l->graphs < variants_ && again) {
+        e = new (std::nothrow) Entry();
+        if (e && e->build(r) == cudaSuccess) {
+            l->graph[l->graphs++] = e;
+        } else {                                             // (no memory for it: there are other ways)
+            delete e;
+            e = nullptr;
+            cudaGetLastError();
         }
     }
-    Entry* e = exact ? exact : alike >= variants_ ? oldest : nullptr;
-    if (e && e->prepare(r) != cudaSuccess) {
-        for (auto& x : entries_)
-            if (x == e) {
-                x = entries_.back();
-                break;
-            }
-        entries_.pop_back();
-        delete e;
-        cudaGetLastError();
-        return launch_one_by_one(r, stream);                 // (no memory for it: the plain launches still work)
-    }
-    if (!e) {
-        if ((int)entries_.size() >= kMaxEntries) {
-            for (auto& x : entries_)
-                if (x == any_oldest) {
-                    x = entries_.back();
-                    break;
-                }
-            entries_.pop_back();
-            delete any_oldest;
+    if (!e && oldest) {
+        e = oldest;
+        if (e->update(r) != cudaSuccess) {
+            l->drop(e);
+            e = nullptr;
+            cudaGetLastError();
         }
-        if (Entry* seen = new (std::nothrow) Entry()) {
-            seen->rec = r;
-            seen->used = ++tick_;
-            entries_.push_back(seen);
-        }
-        return launch_one_by_one(r, stream);
     }
+    if (!e) return launch_one_by_one(r, stream);
     e->used = ++tick_;
     return cudaGraphLaunch(e->exec, stream);
 }
