@@ -176,6 +176,7 @@ private:
     std::mutex mutex_;
     const int variants_;
     uint64_t tick_ = 0;
+    int64_t lost_ns_ = 0;                            // what plain launches have cost, up to the price of a graph
 };
 
 class LaunchBatch {

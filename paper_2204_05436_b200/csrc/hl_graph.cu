@@ -1,8 +1,9 @@
-// Runs of kernels launched as one graph.  On the bench platform a kernel launch costs the host 2.1 us, a graph launch 0.9 us
-// however many kernels it holds, and changing the arguments of one of its kernels 0.25 us; on the device, a kernel of a
-// graph starts 0.8 us after the one before it.  The calls whose mini-batches are bound by the host collect their kernels
-// (LaunchBatch) and launch them together; the graphs are kept (LaunchCache) and launched again as they are, or with the
-// arguments that differ, as long as the call makes the same kernels.
+// Runs of kernels launched as one graph.  On the bench platform a kernel launch costs the host 2.1 us, a graph launch 1.0 us
+// however many kernels it holds, and changing the arguments of one of its kernels 0.28 us; building a graph of 1 to 12
+// kernels costs 65 to 90 us (cudaGraphInstantiate 60 to 70, the first launch 2 to 20 more than a later one).  On the device,
+// a kernel of a graph starts 0.8 us after the one before it.  The calls whose mini-batches are bound by the host collect
+// their kernels (LaunchBatch) and launch them together; the graphs are kept (LaunchCache) and launched again as they are, or
+// with the arguments that differ, as long as the call makes the same kernels.
 #include <cstring>
 #include <new>
 
@@ -13,6 +14,7 @@ namespace hl {
 namespace {
 
 constexpr int kMaxNodes = 12, kMaxArgBytes = 4096, kMaxParams = 160;
+constexpr int64_t kPlainNs = 2100, kGraphNs = 1000, kUpdateNs = 280, kBuildNs = 75000;
 
 struct Node {
     const void* func;
@@ -136,9 +138,10 @@ struct LaunchCache::Entry {
     }
 
     // the arguments that differ from the last launch's (future launches only: one in flight keeps its own)
-    cudaError_t update(const Recording& r) {
+    cudaError_t update(const Recording& r, int* changed) {
         for (int i = 0; i < r.n; ++i) {
             if (same_node(rec, r, i)) continue;
+            ++*changed;
             cudaKernelNodeParams p;
             void* ptrs[kMaxParams];
             const_cast<Recording&>(r).kernel_params(i, &p, ptrs);
@@ -238,9 +241,12 @@ thread_local Collecting t_now;
 }  // namespace
 
 // Launches a recording: as the kept graph that had these kernels and arguments, or as one with these kernels whose arguments
-// are brought up to date (the one not used for longest, once there are `variants_` of them).  Building a graph costs some
-// 50 us, so kernels that come for the first time are launched one by one and only remembered; the graph is built when they
-// come again.
+// are brought up to date (the one not used for longest), or kernel by kernel.
+//
+// Building a graph costs as much as some 30 plain launches, in the call that does it.  So none is built before the plain
+// launches of this cache (and, for one more graph of kernels that have one, the arguments changed) have cost that much more
+// than graphs would have: a program that makes a call a few times never pays for a graph, one that makes it for ever pays for
+// plain launches twice at most, and graphs come one at a time, however many runs of kernels a call makes.
 cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
     Recording& r = *const_cast<Recording*>(static_cast<const Recording*>(recording));
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -251,14 +257,14 @@ cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
     std::lock_guard<std::mutex> lock(mutex_);
     List* l = list_of(recording);
     if (!l) return launch_one_by_one(r, stream);
-    const bool again = l->used != 0;
     l->used = ++tick_;
     Entry *e = nullptr, *oldest = nullptr;
     for (int i = 0; i < l->graphs && !e; ++i) {
         if (l->graph[i]->same_arguments(r)) e = l->graph[i];
         if (!oldest || l->graph[i]->used < oldest->used) oldest = l->graph[i];
     }
-    if (!e && l->graphs < variants_ && again) {
+    if (!e && l->graphs < variants_ && lost_ns_ >= kBuildNs) {
+        lost_ns_ = 0;
         e = new (std::nothrow) Entry();
         if (e && e->build(r) == cudaSuccess) {
             l->graph[l->graphs++] = e;
@@ -268,14 +274,19 @@ cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
             cudaGetLastError();
         }
     }
+    int64_t lost = 0;
     if (!e && oldest) {
+        int changed = 0;
         e = oldest;
-        if (e->update(r) != cudaSuccess) {
+        if (e->update(r, &changed) != cudaSuccess) {
             l->drop(e);
             e = nullptr;
             cudaGetLastError();
         }
+        if (l->graphs < variants_) lost = kUpdateNs * changed;
     }
+    if (!e) lost = (kPlainNs - kUpdateNs) * r.n - kGraphNs;
+    lost_ns_ = lost_ns_ + lost < kBuildNs ? lost_ns_ + lost : kBuildNs;
     if (!e) return launch_one_by_one(r, stream);
     e->used = ++tick_;
     return cudaGraphLaunch(e->exec, stream);

@@ -178,6 +178,23 @@ def test_many_runs_of_kernels_with_many_argument_sets_all_become_graphs(B, lib):
     c.close()
 
 
+def test_graphs_are_built_when_plain_launches_have_cost_as_much(B, lib):
+    """A graph costs as much as some 30 plain launches: the first repeats of a call pay for none, and a new pipeline's
+    mini-batches, of seven runs of kernels in each of four slots, pay for one now and then, never for several at once."""
+    c = _Context(B)
+    s, tags, rrpv, hits = c.mem(), c.mem(), c.mem(), c.mem()
+    for k in range(5):
+        B.hl_tracker_update(c.ctx, c.inputs(), tags, rrpv, 64, 16, hits, s)
+    assert lib.fake_calls(b"cudaGraphInstantiate") == 0
+    for k in range(100):
+        B.hl_tracker_update(c.ctx, c.inputs(), tags, rrpv, 64, 16, hits, s)
+    assert lib.fake_calls(b"cudaGraphInstantiate") >= 1
+    c.close()
+    lib.fake_reset()
+    log, marks = _pipe_run(B, lib, 40)
+    assert lib.fake_calls(b"cudaGraphInstantiate") <= len([x for x in log if x.startswith("plain")]) / 30
+
+
 def test_a_graph_that_cannot_be_changed_or_built_gives_way_to_plain_launches(B, lib):
     c = _Context(B)
     s, grads = c.mem(), [c.mem() for _ in range(40)]
