@@ -422,6 +422,15 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
 
 }  // namespace
 
+int32_t marks_fresh(hl_ctx* ctx, cudaStream_t stream) {
+    if (!ctx->marks_suspect) return HL_OK;
+    const ColdMarks marks = cold_marks(ctx);
+    HL_CUDA_TRY(clear_words(marks.bits, cold_bitmap_words(ctx->N), stream));
+    if (marks.summary) HL_CUDA_TRY(clear_words(marks.summary, cold_summary_words(ctx->N), stream));
+    ctx->marks_suspect = 0;
+    return HL_OK;
+}
+
 int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold, cudaStream_t stream,
                   uint32_t* clear, int64_t n_clear) {
     const Regions& r = ctx->r;
@@ -492,6 +501,8 @@ int32_t index_begin(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, int64_t
         return HL_OK;
     }
     if (!non->ids) return HL_EINVAL;
+    const int32_t fresh = marks_fresh(ctx, stream);
+    if (fresh != HL_OK) return fresh;
     const int grid = grid_for(ctx->max_nnz, kThreads, 4 * ctx_sms(ctx));
     HL_CUDA_TRY(launch(k_cold_classify, grid, kThreads, stream, non->ids, non->offsets, d_n_non, ctx->max_batch,
                        ctx->T * ctx->S, non->cap_ids, ctx->N, BitmapProbe{r.remap}, cold_marks(ctx), r.status));
@@ -562,8 +573,9 @@ extern "C" int32_t hl_gather_cold(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_
                                   float* d_cache, int32_t* d_cold_rows, int64_t* d_n_cold, void* stream_) {
     if (!ctx || !non || !non->offsets || !d_n_non || !host_table || !d_cache || !d_cold_rows || !d_n_cold)
         return HL_EINVAL;
-    return gather_impl(ctx, non, d_n_non, host_table, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold, nullptr,
-                       nullptr, nullptr, nullptr, nullptr, nullptr, true, true, static_cast<cudaStream_t>(stream_));
+    return marks_kept(ctx, gather_impl(ctx, non, d_n_non, host_table, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold,
+                                       nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, true, true,
+                                       static_cast<cudaStream_t>(stream_)));
 }
 
 extern "C" int32_t hl_gather_cold_ahead(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const float* host_table,
@@ -575,10 +587,12 @@ extern "C" int32_t hl_gather_cold_ahead(hl_ctx* ctx, hl_ubatch* non, const int32
         return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     if ((d_prev_cold_rows != nullptr) != (d_n_prev != nullptr) || (d_prev_cold_rows && !d_fwd_src)) return HL_EINVAL;
-    return gather_impl(ctx, non, d_n_non, host_table, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold,
-                       d_prev_cold_rows, d_n_prev, d_fwd_src, static_cast<cudaEvent_t>(record_after_index),
-                       static_cast<cudaEvent_t>(wait_before_move_a), static_cast<cudaEvent_t>(wait_before_move_b), true,
-                       true, static_cast<cudaStream_t>(stream_));
+    return marks_kept(ctx, gather_impl(ctx, non, d_n_non, host_table, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+                                       d_prev_cold_rows, d_n_prev, d_fwd_src,
+                                       static_cast<cudaEvent_t>(record_after_index),
+                                       static_cast<cudaEvent_t>(wait_before_move_a),
+                                       static_cast<cudaEvent_t>(wait_before_move_b), true, true,
+                                       static_cast<cudaStream_t>(stream_)));
 }
 
 extern "C" int32_t hl_index_cold(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, int64_t stage_row0,
@@ -588,9 +602,9 @@ extern "C" int32_t hl_index_cold(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n
     if (!ctx || !non || !non->offsets || !d_n_non || !d_cold_rows || !d_n_cold) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     if ((d_prev_cold_rows != nullptr) != (d_n_prev != nullptr) || (d_prev_cold_rows && !d_fwd_src)) return HL_EINVAL;
-    return gather_impl(ctx, non, d_n_non, nullptr, nullptr, stage_row0, stage_rows, d_cold_rows, d_n_cold,
-                       d_prev_cold_rows, d_n_prev, d_fwd_src, nullptr, nullptr, nullptr, true, false,
-                       static_cast<cudaStream_t>(stream_));
+    return marks_kept(ctx, gather_impl(ctx, non, d_n_non, nullptr, nullptr, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+                                       d_prev_cold_rows, d_n_prev, d_fwd_src, nullptr, nullptr, nullptr, true, false,
+                                       static_cast<cudaStream_t>(stream_)));
 }
 
 extern "C" int32_t hl_index_cold_begin(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, int64_t stage_row0,
@@ -598,8 +612,8 @@ extern "C" int32_t hl_index_cold_begin(hl_ctx* ctx, hl_ubatch* non, const int32_
     if (!ctx || !non || !non->offsets || !d_n_non || !d_cold_rows || !d_n_cold) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     LaunchBatch batch(ctx->launches);
-    return batch.end(index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
-                                 static_cast<cudaStream_t>(stream_)));
+    return marks_kept(ctx, batch.end(index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+                                                 static_cast<cudaStream_t>(stream_))));
 }
 
 extern "C" const int32_t* hl_index_cold_verdict(hl_ctx* ctx) { return ctx ? ctx->r.cold_n + 1 : nullptr; }

@@ -102,6 +102,8 @@ struct hl_ctx {
     // graphs of the calls that make several kernels, or one in a run of calls (nullptr: plain launches)
     hl::LaunchCache* launches;
     cudaEvent_t step_ranked, step_staged;      // of hl_step
+    // a call that marks cold rows has failed since the marks were last known to be ranked and cleared
+    int marks_suspect;
 };
 
 // Context of the wide-id index path (hl_wide_*): global row ids are 64-bit, every table still has fewer than 2^31
@@ -366,6 +368,16 @@ __device__ __forceinline__ int32_t classify_cold(const BitmapProbe& remap, int64
     }
     return (int32_t)(-2 - g);
 }
+
+// Rows are marked and ranked in two kernels or two calls, and the marks must be gone when the next mini-batch's are set: a
+// call that ends in between, because a launch or an event failed, would leave its rows to be staged as the next one's.  So
+// every call that marks rows passes its result through marks_kept, and the next one starts with marks_fresh, which clears
+// the bitmap if the last one failed.
+inline int32_t marks_kept(hl_ctx* ctx, int32_t st) {
+    if (st != HL_OK && ctx) ctx->marks_suspect = 1;
+    return st;
+}
+int32_t marks_fresh(hl_ctx* ctx, cudaStream_t stream);
 
 // The slot of such a lookup once the marked rows are ranked: slot0 + rank, or -1 if there is no room to stage the row
 // (the lookup is dropped; k_cold_rank has set the status word).

@@ -454,6 +454,10 @@ int32_t fragment_call(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int3
     if (!pop->offsets || !non->offsets || (b->nnz > 0 && (!pop->ids || !non->ids))) return HL_EINVAL;
     if ((d_dense == nullptr) != (d_dense_out == nullptr) || (d_dense && n_dense < 1)) return HL_EINVAL;
     Regions& r = ctx->r;
+    if (mark) {
+        const int32_t fresh = marks_fresh(ctx, stream);
+        if (fresh != HL_OK) return fresh;
+    }
     const auto launch = mark ? fragment_launch<true, BitmapProbe, int32_t> : fragment_launch<false, BitmapProbe, int32_t>;
     return launch(b, ctx->T, ctx->S, ctx_sms(ctx), r.table_base, BitmapProbe{r.remap}, r.frag_words, r.frag_chain,
                   r.status, wait_cfg(ctx), d_dense, n_dense, d_perm, d_counts, pop, non->offsets, non->ids, non->cap_ids,

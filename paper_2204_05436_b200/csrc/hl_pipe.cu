@@ -122,7 +122,7 @@ hl::LaunchCache* launches_of(hl_pipe* p, int64_t j) {
 }
 
 // The index-only work of the next mini-batch (nothing here touches a row).
-int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
+int32_t queue_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
     const int64_t j = p->j_indexed;
     const int n = p->n_sets;
     hl_pipe_set& st = p->sets[j % n];
@@ -173,6 +173,10 @@ int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* 
     return HL_OK;
 }
 
+int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
+    return marks_kept(p->ctx, queue_index(p, b, d_dense, inputs_ready));
+}
+
 // the host read of the oldest indexed mini-batch whose rows are not staged yet
 int32_t submit_link(hl_pipe* p) {
     const int64_t j = p->j_submitted;
@@ -220,17 +224,18 @@ int32_t flush_scatter(hl_pipe* p) {
 
 }  // namespace
 
+namespace {
+
 // One mini-batch.  What bounds a small one is the chain of short kernels: fragment, ranks, pairs and sort (one for both
 // updates, where a sort inside each update would cost its three passes twice), the host read beside the sort.  106 496
 // lookups of 64-byte rows: 133 us with a call for each step, 104 us so.
-extern "C" int32_t hl_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
-                           const hl_step_buffers* s, float* d_cache, float* host_table, const float* d_grad_pop,
-                           const float* d_grad_non, float lr, int32_t flags, void* main_stream, void* side_stream) {
+int32_t queue_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense, const hl_step_buffers* s,
+                   float* d_cache, float* host_table, const float* d_grad_pop, const float* d_grad_non, float lr,
+                   int32_t flags, cudaStream_t main, cudaStream_t side) {
     if (!ctx || !b || !s || !d_cache || !host_table || !d_grad_pop || !d_grad_non || (flags & ~HL_STEP_DEFERRED))
         return HL_EINVAL;
     if (!s->cold_rows || !s->n_cold || !s->pooled_pop || !s->pooled_non || !s->pop.offsets || !s->non.offsets)
         return HL_EINVAL;
-    cudaStream_t main = static_cast<cudaStream_t>(main_stream), side = static_cast<cudaStream_t>(side_stream);
     const bool deferred = (flags & HL_STEP_DEFERRED) != 0;
     hl_ubatch pop = s->pop, non = s->non;
     // (2^30 cache slots and more: O's and X's slots do not fit one key space, and every update sorts its own)
@@ -284,6 +289,15 @@ extern "C" int32_t hl_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense,
     HL_PIPE_TRY(update(1));
     HL_PIPE_TRY(hl_scatter_cold(ctx, d_cache, s->cold_rows, s->n_cold, host_table, main));
     return batch.end();
+}
+
+}  // namespace
+
+extern "C" int32_t hl_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
+                           const hl_step_buffers* s, float* d_cache, float* host_table, const float* d_grad_pop,
+                           const float* d_grad_non, float lr, int32_t flags, void* main_stream, void* side_stream) {
+    return marks_kept(ctx, queue_step(ctx, b, d_dense, n_dense, s, d_cache, host_table, d_grad_pop, d_grad_non, lr, flags,
+                                      static_cast<cudaStream_t>(main_stream), static_cast<cudaStream_t>(side_stream)));
 }
 
 extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_table, int64_t window_rows,

@@ -252,3 +252,56 @@ def test_a_captured_stream_gets_plain_launches_only(B, lib):
         assert (lib.fake_calls(b"cudaGraphInstantiate"), lib.fake_calls(b"cudaGraphLaunch")) == (built, launched)
     assert launched > 100
     c.close()
+
+
+@pytest.mark.parametrize("which", ["hl_index_cold", "hl_gather_cold", "hl_index_cold_begin", "hl_step", "hl_pipe_submit"])
+def test_marks_left_by_a_call_that_failed_are_cleared_before_the_next_ones(B, lib, which):
+    """Cold rows are marked in the bitmap by one kernel and ranked (and the marks cleared) by another.  The launch of the
+    second one fails: the call says so, and the next call on the context first clears the bitmap; the one after that
+    does not."""
+    c = _Context(B)
+    s, side, st, b = c.mem(), c.mem(), c.one_set(), c.inputs()
+    pipe = None
+    if which == "hl_pipe_submit":
+        sets = [B.hl_pipe_set(x["perm"], x["counts"], x["pop"], x["non"], x["cold_rows"], x["n_cold"], x["fwd_src"],
+                              x["pooled_pop"], x["pooled_non"], None, x["slots"], x["bags"], x["n"])
+                for x in (c.one_set() for _ in range(6))]
+        pipe = B.hl_pipe_create(c.ctx, c.cache, c.table, c.staging // 2, sets, 0, s)
+    step_buffers = B.make_step_buffers(st["perm"], st["counts"], st["pop"], st["non"], None, st["cold_rows"], st["n_cold"],
+                                       st["pooled_pop"], st["pooled_non"])
+
+    def call():
+        at = lib.fake_lines()
+        if which == "hl_index_cold":
+            B.hl_index_cold(c.ctx, st["non"], st["counts"] + 4, 0, c.staging, st["cold_rows"], st["n_cold"], None, None, None, s)
+        elif which == "hl_gather_cold":
+            B.hl_gather_cold(c.ctx, st["non"], st["counts"] + 4, c.table, c.cache, st["cold_rows"], st["n_cold"], s)
+        elif which == "hl_index_cold_begin":
+            B.hl_index_cold_begin(c.ctx, st["non"], st["counts"] + 4, 0, c.staging, st["cold_rows"], st["n_cold"], s)
+        elif which == "hl_step":
+            B.hl_step(c.ctx, b, None, 0, step_buffers, c.cache, c.table, c.mem(), c.mem(), 0.1, False, s, side)
+        else:
+            B.hl_pipe_submit(pipe, b, None, "resident")
+        return _log(lib, at)
+
+    def clears(lines):
+        """Positions of clears of the bitmap and of the kernel that marks."""
+        rank = [x for x in lines if _name(x).startswith("k_cold_rank")][0]
+        bits, words = rank.split(" ")[7][:16], (3000 + 31) // 32
+        cleared = [i for i, x in enumerate(lines) if _name(x) == "k_clear_words" and
+                   x.split(" ")[7:9] == [bits, words.to_bytes(8, "little").hex()]]
+        marked = [i for i, x in enumerate(lines) if _name(x).startswith(("k_cold_classify", "k_frag_place"))]
+        return cleared, marked[0]
+
+    assert clears(call())[0] == []
+    lib.fake_fail_kernel(b"k_cold_rank")
+    with pytest.raises(B.HotlineError) as e:
+        call()
+    assert e.value.status == B.HL_ECUDA
+    lib.fake_fail_kernel(None)
+    cleared, marked = clears(call())
+    assert len(cleared) == 1 and cleared[0] < marked
+    assert clears(call())[0] == []
+    if pipe:
+        B.hl_pipe_destroy(pipe)
+    c.close()
