@@ -573,7 +573,7 @@ extern "C" int32_t hl_gather_cold(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_
                                   float* d_cache, int32_t* d_cold_rows, int64_t* d_n_cold, void* stream_) {
     if (!ctx || !non || !non->offsets || !d_n_non || !host_table || !d_cache || !d_cold_rows || !d_n_cold)
         return HL_EINVAL;
-    return marks_kept(ctx, gather_impl(ctx, non, d_n_non, host_table, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold,
+    return scratch_kept(ctx, gather_impl(ctx, non, d_n_non, host_table, d_cache, 0, ctx->staging_cap, d_cold_rows, d_n_cold,
                                        nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, true, true,
                                        static_cast<cudaStream_t>(stream_)));
 }
@@ -587,7 +587,7 @@ extern "C" int32_t hl_gather_cold_ahead(hl_ctx* ctx, hl_ubatch* non, const int32
         return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     if ((d_prev_cold_rows != nullptr) != (d_n_prev != nullptr) || (d_prev_cold_rows && !d_fwd_src)) return HL_EINVAL;
-    return marks_kept(ctx, gather_impl(ctx, non, d_n_non, host_table, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+    return scratch_kept(ctx, gather_impl(ctx, non, d_n_non, host_table, d_cache, stage_row0, stage_rows, d_cold_rows, d_n_cold,
                                        d_prev_cold_rows, d_n_prev, d_fwd_src,
                                        static_cast<cudaEvent_t>(record_after_index),
                                        static_cast<cudaEvent_t>(wait_before_move_a),
@@ -602,7 +602,7 @@ extern "C" int32_t hl_index_cold(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n
     if (!ctx || !non || !non->offsets || !d_n_non || !d_cold_rows || !d_n_cold) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     if ((d_prev_cold_rows != nullptr) != (d_n_prev != nullptr) || (d_prev_cold_rows && !d_fwd_src)) return HL_EINVAL;
-    return marks_kept(ctx, gather_impl(ctx, non, d_n_non, nullptr, nullptr, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+    return scratch_kept(ctx, gather_impl(ctx, non, d_n_non, nullptr, nullptr, stage_row0, stage_rows, d_cold_rows, d_n_cold,
                                        d_prev_cold_rows, d_n_prev, d_fwd_src, nullptr, nullptr, nullptr, true, false,
                                        static_cast<cudaStream_t>(stream_)));
 }
@@ -612,7 +612,7 @@ extern "C" int32_t hl_index_cold_begin(hl_ctx* ctx, hl_ubatch* non, const int32_
     if (!ctx || !non || !non->offsets || !d_n_non || !d_cold_rows || !d_n_cold) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     LaunchBatch batch(ctx->launches);
-    return marks_kept(ctx, batch.end(index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
+    return scratch_kept(ctx, batch.end(index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
                                                  static_cast<cudaStream_t>(stream_))));
 }
 

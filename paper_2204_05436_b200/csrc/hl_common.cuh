@@ -102,8 +102,8 @@ struct hl_ctx {
     // graphs of the calls that make several kernels, or one in a run of calls (nullptr: plain launches)
     hl::LaunchCache* launches;
     cudaEvent_t step_ranked, step_staged;      // of hl_step
-    // a call that marks cold rows has failed since the marks were last known to be ranked and cleared
-    int marks_suspect;
+    // a call has failed that may have left cold rows marked, or runs on the backward's list (scratch_kept)
+    int marks_suspect, spans_suspect;
 };
 
 // Context of the wide-id index path (hl_wide_*): global row ids are 64-bit, every table still has fewer than 2^31
@@ -370,11 +370,12 @@ __device__ __forceinline__ int32_t classify_cold(const BitmapProbe& remap, int64
 }
 
 // Rows are marked and ranked in two kernels or two calls, and the marks must be gone when the next mini-batch's are set: a
-// call that ends in between, because a launch or an event failed, would leave its rows to be staged as the next one's.  So
-// every call that marks rows passes its result through marks_kept, and the next one starts with marks_fresh, which clears
-// the bitmap if the last one failed.
-inline int32_t marks_kept(hl_ctx* ctx, int32_t st) {
-    if (st != HL_OK && ctx) ctx->marks_suspect = 1;
+// call that ends in between, because a launch or an event failed, would leave its rows to be staged as the next one's.  The
+// same goes for the runs that the backward's sum kernel lists and the next kernel finishes and takes off the list.  So every
+// call that marks rows or lists runs passes its result through scratch_kept, and the next one clears the bitmap
+// (marks_fresh) or the list's counts (launch_bwd) first if one has failed.
+inline int32_t scratch_kept(hl_ctx* ctx, int32_t st) {
+    if (st != HL_OK && ctx) ctx->marks_suspect = ctx->spans_suspect = 1;
     return st;
 }
 int32_t marks_fresh(hl_ctx* ctx, cudaStream_t stream);

@@ -803,9 +803,14 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 0, stream);
     // the list of runs that cross a chunk border sits behind the partial sums: [count words (8 ints)] [entries].
-    // The count is zero between calls: hl_create clears it and k_bwd_spans clears it again when it is done.
+    // The count is zero between calls: hl_create clears it and k_bwd_spans clears it again when it is done (a call that
+    // failed may have left it otherwise: scratch_kept).
     int32_t* span_count = span_count_of(ctx);
     int32_t* span_list = span_count + 8;
+    if (ctx->spans_suspect) {
+        HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(span_count), 8, stream));
+        ctx->spans_suspect = 0;
+    }
     HL_CUDA_TRY(launch(k_bwd_chunks<G, NV>, grid, kThreads, stream, cache, keys, vals, d_n_lookups, grad, ctx->D / 4,
                        n_slots, lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list, ctx->max_bags, max_chunks,
                        ctx->r.status));
@@ -954,14 +959,14 @@ extern "C" int32_t hl_embbag_bwd_sgd(hl_ctx* ctx, float* d_cache, const hl_ubatc
     if (ctx->max_nnz == 0) return HL_OK;
     if (!ub->ids) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    return as_graph(ctx->launches, [&]() -> int32_t {
+    return scratch_kept(ctx, as_graph(ctx->launches, [&]() -> int32_t {
         int32_t *keys, *vals;
         const int32_t st = sort_lookups(ctx, ub, d_n_samples, nullptr, nullptr, ctx->r.bwd_n, &keys, &vals, stream);
         if (st != HL_OK) return st;
 #define HL_BWD(G, NV) launch_bwd<G, NV>(ctx, d_cache, keys, vals, ctx->r.bwd_n, d_grad_out, lr, stream)
         HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD
-    });
+    }));
 }
 
 extern "C" int32_t hl_embbag_bwd_prepare(hl_ctx* ctx, const hl_ubatch* ub, const int32_t* d_n_samples,
@@ -1063,12 +1068,12 @@ extern "C" int32_t hl_embbag_bwd_apply2(hl_ctx* ctx, float* d_cache, const int32
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const int32_t* d_first = which == 0 ? nullptr : d_n_lookups;             // X's block starts behind O's
     const int32_t bias = which == 0 ? 0 : (int32_t)(ctx->hot_cap + ctx->staging_cap + 1);
-    return as_graph(ctx->launches, [&]() -> int32_t {
+    return scratch_kept(ctx, as_graph(ctx->launches, [&]() -> int32_t {
 #define HL_BWD(G, NV) \
     launch_bwd<G, NV>(ctx, d_cache, d_sorted_slots, d_sorted_bags, d_n_lookups + which, d_grad_out, lr, stream, d_first, bias)
         HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD
-    });
+    }));
 }
 
 extern "C" int32_t hl_embbag_bwd_apply(hl_ctx* ctx, float* d_cache, const int32_t* d_sorted_slots,
@@ -1078,11 +1083,11 @@ extern "C" int32_t hl_embbag_bwd_apply(hl_ctx* ctx, float* d_cache, const int32_
     if (ctx->max_nnz == 0) return HL_OK;
     if (!d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    return as_graph(ctx->launches, [&]() -> int32_t {
+    return scratch_kept(ctx, as_graph(ctx->launches, [&]() -> int32_t {
 #define HL_BWD(G, NV) launch_bwd<G, NV>(ctx, d_cache, d_sorted_slots, d_sorted_bags, d_n_lookups, d_grad_out, lr, stream)
         HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD
-    });
+    }));
 }
 
 // ---------------------------------------------------------------------------------------------------------------

@@ -174,7 +174,7 @@ int32_t queue_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* i
 }
 
 int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
-    return marks_kept(p->ctx, queue_index(p, b, d_dense, inputs_ready));
+    return scratch_kept(p->ctx, queue_index(p, b, d_dense, inputs_ready));
 }
 
 // the host read of the oldest indexed mini-batch whose rows are not staged yet
@@ -296,7 +296,7 @@ int32_t queue_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t
 extern "C" int32_t hl_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
                            const hl_step_buffers* s, float* d_cache, float* host_table, const float* d_grad_pop,
                            const float* d_grad_non, float lr, int32_t flags, void* main_stream, void* side_stream) {
-    return marks_kept(ctx, queue_step(ctx, b, d_dense, n_dense, s, d_cache, host_table, d_grad_pop, d_grad_non, lr, flags,
+    return scratch_kept(ctx, queue_step(ctx, b, d_dense, n_dense, s, d_cache, host_table, d_grad_pop, d_grad_non, lr, flags,
                                       static_cast<cudaStream_t>(main_stream), static_cast<cudaStream_t>(side_stream)));
 }
 
@@ -402,9 +402,8 @@ extern "C" int32_t hl_pipe_submit(hl_pipe* p, const hl_batch* b, const float* d_
     return HL_OK;
 }
 
-extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float* d_grad_non, float lr,
-                                const hl_batch* next, const float* d_next_dense, void* next_inputs_ready,
-                                int32_t* set_index) {
+static int32_t queue_mini_batch(hl_pipe* p, const float* d_grad_pop, const float* d_grad_non, float lr, const hl_batch* next,
+                                const float* d_next_dense, void* next_inputs_ready, int32_t* set_index) {
     if (!p || !d_grad_pop || (!d_grad_non && p->order != HL_PIPE_ORDER_EQ5)) return HL_EINVAL;
     const int64_t j = p->j_done;
     if (p->j_submitted < j + 1) return HL_EINVAL;          // hl_pipe_submit first
@@ -469,6 +468,13 @@ extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float
     }
     if (set_index) *set_index = (int32_t)(j % n);
     return HL_OK;
+}
+
+extern "C" int32_t hl_pipe_step(hl_pipe* p, const float* d_grad_pop, const float* d_grad_non, float lr,
+                                const hl_batch* next, const float* d_next_dense, void* next_inputs_ready,
+                                int32_t* set_index) {
+    return scratch_kept(p ? p->ctx : nullptr, queue_mini_batch(p, d_grad_pop, d_grad_non, lr, next, d_next_dense,
+                                                               next_inputs_ready, set_index));
 }
 
 extern "C" int32_t hl_pipe_set_order(hl_pipe* p, int32_t order) {

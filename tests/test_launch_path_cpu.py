@@ -305,3 +305,52 @@ def test_marks_left_by_a_call_that_failed_are_cleared_before_the_next_ones(B, li
     if pipe:
         B.hl_pipe_destroy(pipe)
     c.close()
+
+
+@pytest.mark.parametrize("which", ["hl_embbag_bwd_sgd", "hl_embbag_bwd_apply", "hl_embbag_bwd_apply2", "hl_step", "hl_pipe_step"])
+def test_runs_listed_by_a_call_that_failed_are_taken_off_the_list(B, lib, which):
+    """The sum kernel lists the runs that the span kernel finishes.  The span kernel's launch fails: the call says so, and
+    the next update on the context starts with an empty list; the one after that clears nothing."""
+    c = _Context(B)
+    s, side, st, b, grad = c.mem(), c.mem(), c.one_set(), c.inputs(), c.mem()
+    step_buffers = B.make_step_buffers(st["perm"], st["counts"], st["pop"], st["non"], None, st["cold_rows"], st["n_cold"],
+                                       st["pooled_pop"], st["pooled_non"])
+    sets = [B.hl_pipe_set(x["perm"], x["counts"], x["pop"], x["non"], x["cold_rows"], x["n_cold"], x["fwd_src"],
+                          x["pooled_pop"], x["pooled_non"], None, x["slots"], x["bags"], x["n"])
+            for x in (c.one_set() for _ in range(4))]
+    pipe = B.hl_pipe_create(c.ctx, c.cache, c.table, c.staging // 2, sets, 0, s)
+    if which == "hl_pipe_step":
+        for _ in range(3):
+            B.hl_pipe_submit(pipe, b, None, "resident")
+
+    def call():
+        at = lib.fake_lines()
+        if which == "hl_embbag_bwd_sgd":
+            B.hl_embbag_bwd_sgd(c.ctx, c.cache, st["pop"], st["counts"], grad, 0.1, s)
+        elif which == "hl_embbag_bwd_apply":
+            B.hl_embbag_bwd_apply(c.ctx, c.cache, st["slots"], st["bags"], st["n"], grad, 0.1, s)
+        elif which == "hl_embbag_bwd_apply2":
+            B.hl_embbag_bwd_apply2(c.ctx, c.cache, st["slots"], st["bags"], st["n"], 1, grad, 0.1, s)
+        elif which == "hl_step":
+            B.hl_step(c.ctx, b, None, 0, step_buffers, c.cache, c.table, grad, grad, 0.1, False, s, side)
+        else:
+            B.hl_pipe_step(pipe, grad, grad, 0.1, None, None)
+        return _log(lib, at)
+
+    def clears(lines):
+        sums = [i for i, x in enumerate(lines) if _name(x).startswith("k_bwd_chunks")]
+        count = lines[sums[0]].split(" ")[7 + 11]
+        return [i for i, x in enumerate(lines) if _name(x) == "k_clear_words" and x.split(" ")[7] == count], sums[0]
+
+    assert clears(call())[0] == []
+    lib.fake_fail_kernel(b"k_bwd_spans")
+    with pytest.raises(B.HotlineError) as e:
+        call()
+    assert e.value.status == B.HL_ECUDA
+    lib.fake_fail_kernel(None)
+    cleared, first = clears(call())
+    assert len(cleared) == 1 and cleared[0] < first
+    if which != "hl_pipe_step":
+        assert clears(call())[0] == []
+    B.hl_pipe_destroy(pipe)
+    c.close()
