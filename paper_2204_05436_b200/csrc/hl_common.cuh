@@ -7,6 +7,7 @@
 
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -200,6 +201,8 @@ template <typename... P, typename... A>
 cudaError_t launch_cluster(void (*kernel)(P...), int64_t grid, int block, size_t smem, int cluster, cudaStream_t stream,
                            A&&... a) {
     static_assert(sizeof...(P) == sizeof...(A), "one argument per parameter");
+    // (arguments are compared byte by byte: LaunchCache)
+    static_assert(((std::has_unique_object_representations_v<P> || std::is_floating_point_v<P>) && ...), "no padding");
     std::tuple<P...> args(static_cast<P>(a)...);
     const uint32_t sizes[] = {(uint32_t)sizeof(P)...};
     return std::apply(
@@ -275,12 +278,12 @@ struct TableMap {
     unsigned char* single;
     unsigned char* const* ptrs;
     const int64_t* base;               // [T+1]
-    int T;
+    int64_t T;
 };
 
 __device__ __forceinline__ unsigned char* row_address(const TableMap& m, int64_t g, int row_bytes) {
     if (m.ptrs == nullptr) return m.single + g * row_bytes;
-    int lo = 0, hi = m.T;              // base[lo] <= g < base[hi]
+    int lo = 0, hi = (int)m.T;         // base[lo] <= g < base[hi]
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (__ldg(&m.base[mid]) <= g) lo = mid;

@@ -270,7 +270,7 @@ struct PairSide {
     int32_t* ids;
     const int32_t* offsets;
     const int32_t* d_n_samples;
-    int32_t key_bias;
+    int32_t key_bias, unused;          // (no padding in launch arguments)
 };
 
 struct PairArgs {
@@ -295,7 +295,7 @@ struct PairArgs {
     int32_t* fwd_src;
     // HIST: digit counts of the sort that follows, [passes][256], zero on entry
     uint32_t* ghist;
-    int passes;
+    int passes, unused;
 };
 
 template <int GROUP, bool ASSIGN, bool HIST>

@@ -201,7 +201,7 @@ constexpr unsigned long long kLow = (1ull << kHalf) - 1ull;
 struct PlaceArgs {
     const int32_t* indices;
     const int32_t* offsets;
-    int B, T, S;
+    int B, T, S, n_dense;
     const int32_t* perm;
     int32_t* counts;
     const int64_t* table_base;
@@ -212,10 +212,9 @@ struct PlaceArgs {
     int64_t non_cap;
     unsigned long long* chain;         // [tile] status word of the tile; zero on entry
     int32_t* status;
-    int max_polls;
+    int64_t max_polls;
     int64_t stall_tile;
     const float* dense;
-    int n_dense;
     float* dense_out;
 };
 
@@ -313,7 +312,7 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
         }
     }
     const unsigned long long before =
-        chain_before<kThreads>(a.chain, tile, total, tile != a.stall_tile, a.max_polls, a.status);
+        chain_before<kThreads>(a.chain, tile, total, tile != a.stall_tile, (int)a.max_polls, a.status);
     if (threadIdx.x == 0 && last == n_bags) {                // the last tile knows the totals
         const int32_t L_pop = (int32_t)((before + total) >> kHalf), L_non = (int32_t)((before + total) & kLow);
         a.counts[2] = L_pop;
@@ -426,8 +425,9 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
     // the tally of finished CTAs of the flags kernel: word 0 of the chain words (zero between calls: cleared when the
     // context is created and by the CTA that counts to the end); the chain proper is cleared by the flags kernel
     unsigned int* finished = reinterpret_cast<unsigned int*>(chain);
-    PlaceArgs a{b->indices, b->offsets, B, T, S, d_perm, d_counts, table_base, pop->offsets, pop->ids, pop->cap_ids,
-                non_offsets, non_cap, chain + 1, status, waits.max_polls, waits.stall_tile, d_dense, n_dense, d_dense_out};
+    PlaceArgs a{b->indices, b->offsets, B, T, S, n_dense, d_perm, d_counts, table_base, pop->offsets, pop->ids,
+                pop->cap_ids, non_offsets, non_cap, chain + 1, status, waits.max_polls, waits.stall_tile, d_dense,
+                d_dense_out};
     const int flag_grid = grid_for(B, 32, 4 * sms);
     if (b->nnz <= 4 * (int64_t)T * B)            // on average at most 4 lookups per input and table
         HL_CUDA_TRY(launch(k_frag_flags<true, Probe>, flag_grid, kFlagThreads, stream, b->indices, b->offsets, B, T, S,

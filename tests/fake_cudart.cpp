@@ -49,12 +49,12 @@ bool fails(const char* name) {
 }
 cudaError_t result(const char* name) { return fails(name) ? cudaErrorUnknown : cudaSuccess; }
 
-// "int const*" -> 8, "hl::PairArgs" -> 64 (its leading bytes, none of them padding)
+// "int const*" -> 8, "hl::PairArgs" -> 64 (its leading bytes)
 size_t size_of(std::string t) {
     while (!t.empty() && t.front() == ' ') t.erase(0, 1);
     if (t.find('*') != std::string::npos) return 8;
     const std::pair<const char*, size_t> known[] = {
-        {"PairArgs", 28}, {"PlaceArgs", 28}, {"ForwardRows", 48}, {"TableMap", 28}, {"ColdMarks", 24}, {"BitmapProbe", 8},
+        {"PairArgs", 64}, {"PlaceArgs", 64}, {"ForwardRows", 48}, {"TableMap", 32}, {"ColdMarks", 24}, {"BitmapProbe", 8},
         {"HashProbe", 24}};
     for (const auto& k : known)
         if (t.find(k.first) != std::string::npos) return k.second;
