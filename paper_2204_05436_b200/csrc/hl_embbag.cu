@@ -647,8 +647,14 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
 // kernel's length depends on: its warps close in on the end with a 32-way search over the sorted keys, every group takes
 // every (8 * 32/G)-th piece, and one group combines the group sums in a fixed order.  (With both kinds in one list a CTA
 // met up to eight long runs one after the other: 2.6 M lookups of 512 bytes took 36.6 us.)
+//
+// A long run is a chain of round trips to the L2, so what helps is to have the pieces of the next trip on their way: two
+// CTAs per multiprocessor (the grid is no more than that) leave the compiler 120 registers for it; left alone it keeps to
+// 64 and asks for one trip at a time.  Zipf over 26 tables, alone, L2 flushed: 106 K / 426 K lookups of 256 bytes 9.6 / 15.7
+// us -> 6.3 / 11.0; 426 K of 64 bytes 11.5 -> 10.3, of 512 bytes 16.6 -> 13.8, of 2 KB 71.9 -> 33.9; 32 K of 256 bytes 5.9 ->
+// 4.8; no such run 3.2 either way.
 template <int G, int NV>
-__global__ void __launch_bounds__(kThreads) k_bwd_spans(float* __restrict__ cache, const int32_t* __restrict__ keys,
+__global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ cache, const int32_t* __restrict__ keys,
                                                         const int32_t* __restrict__ d_n_lookups, int D4,
                                                         int64_t n_slots, float lr, const float* __restrict__ part,
                                                         const int32_t* __restrict__ d_first, int32_t key_bias,
@@ -815,7 +821,7 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
                        n_slots, lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list, ctx->max_bags, max_chunks,
                        ctx->r.status));
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 1, stream);
-    const int span_grid = grid_for(max_chunks * 32, kThreads, 4 * ctx_sms(ctx));   // the warps stride over the listed runs
+    const int span_grid = grid_for(max_chunks * 32, kThreads, 2 * ctx_sms(ctx));   // the warps stride over the listed runs
     HL_CUDA_TRY(launch(k_bwd_spans<G, NV>, span_grid, kThreads, stream, cache, keys, d_n_lookups, ctx->D / 4, n_slots, lr,
                        ctx->r.bwd_part, d_first, key_bias, span_count, (const int32_t*)span_list, max_chunks));
     note_launches(2);
