@@ -384,8 +384,16 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pairs(PairArgs a) {
 constexpr int kSpanLookahead = 32;      // chunks k_bwd_chunks looks ahead for the end of a run
 static_assert(kBwdChunk == 32, "one lookup of a chunk per lane");
 
-template <int G, int NV>
-__global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float* __restrict__ cache,
+//
+// CTAS: CTAs that fit a multiprocessor.  Rows of 36 to 64 fp32 (G = 16): a warp waits for its pairs, then for gradient rows,
+// and then puts two groups together, once per 32 lookups, so in a call of many chunks another warp should have something on
+// its way meanwhile: four CTAs of 64 registers with four rows a lane in flight, instead of three of 80 (and a spill) with
+// eight.  Rows of 256 bytes, alone, L2 flushed, three against four CTAs: Zipf over 26 tables 32 K lookups 11.5 / 13.0 us,
+// 106 K 14.1 / 15.1, 150 K 19.1 / 16.6, 426 K 35.7 / 33.9; uniform 9.6 / 10.0, 13.8 / 13.6, 19.0 / 16.6, 48.4 / 46.5; bags of
+// 20 lookups 8.4 / 8.8, 11.6 / 10.9, 15.7 / 12.8, 28.6 / 25.2.  So three as long as their warps have a chunk each at most.
+
+template <int G, int NV, int CTAS>
+__global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict__ cache,
                                                          const int32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ vals,
                                                          const int32_t* __restrict__ d_n_lookups,
@@ -400,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
     // (in any order): k_bwd_spans finishes those runs.
     static_assert(NV == 1 || G == 32, "several columns per lane only when a row fills the warp");
     constexpr int NG = 32 / G;                                              // groups per warp
-    constexpr int U = NV >= 4 ? 2 : (NV >= 2 ? 4 : (G >= 8 ? 8 : 4));       // lookups in flight per lane
+    constexpr int U = NV >= 4 ? 2 : (NV >= 2 || G == 4 || CTAS > 3 ? 4 : 8);        // lookups in flight per lane
     static_assert(G % U == 0, "batch must divide the group");
     // (positions are below 2^30: 32-bit arithmetic)
     const int first = d_first ? d_first[0] : 0;
@@ -443,6 +451,15 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
         // the slot before the previous chunk, and the first slot of the chunk after the next one
         const int32_t prev2_key = start - kBwdChunk > first ? keys[start - kBwdChunk - 1] : -3;
         const int32_t next2_key = start + 2 * kBwdChunk < n ? keys[start + 2 * kBwdChunk] : -2;
+        // the next chunk's pairs, for a run that ends there (narrow rows: asked for now, not when the sums are done)
+        int32_t k2 = -1, b2 = 0;
+        const auto load_next = [&]() {
+            if (end + lane < n) {
+                k2 = keys[end + lane];
+                b2 = vals[end + lane];
+            }
+        };
+        if (G < 32) load_next();
         // (a bag id outside the gradient array can only be what a given-up chain poll of the sort left behind; such a
         // call has its error status set, and reads bag 0 instead)
         bag = (uint32_t)bag < n_grad_u ? bag : 0;
@@ -547,20 +564,19 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
             // trailing sums that restarts at groups with a head.
             const unsigned upto = heads & (before_group | gmask);
             const int from = upto ? (31 - __clz((int)upto)) / G : 0, gi = g0 / G;
+            double in[1][4];          // what the run has collected in the groups before mine
 #pragma unroll
             for (int s = 1; s < NG; s <<= 1) {
                 const bool add = gi - s >= from;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const double o = __shfl_up_sync(0xffffffffu, acc[0][e], s * G);
-                    if (add) acc[0][e] += o;
+                    in[0][e] = __shfl_up_sync(0xffffffffu, acc[0][e], s * G);
+                    if (add) acc[0][e] += in[0][e];
                 }
             }
-            double in[1][4];          // what the run has collected in the groups before mine
+            if (NG > 2) {             // (of two groups, the scan's one step brought the first one's sum)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                in[0][e] = __shfl_up_sync(0xffffffffu, acc[0][e], G);
-                acc[0][e] = __shfl_sync(0xffffffffu, acc[0][e], 32 - G + sub);
+                for (int e = 0; e < 4; ++e) in[0][e] = __shfl_up_sync(0xffffffffu, acc[0][e], G);
             }
             const uint32_t row0 = __shfl_sync(0xffffffffu, row, 0, G);
             if (late) {
@@ -575,20 +591,19 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
             }
         }
         // the chunk's last lookup does not end its run: the run goes on in the next chunk (only a full chunk has a
-        // next one), and acc holds what it has collected here
+        // next one), and the last group's acc holds what it has collected here
+        const bool last_group = lane >= 32 - G;
         const int32_t last_key = __shfl_sync(0xffffffffu, key, 31);
         if ((tails >> 31) || (uint32_t)(last_key - key_bias) >= n_rows_u) continue;
         if (!heads) {
-            if (lane < G) store_piece(0, acc);
+            if (last_group) store_piece(0, acc);
         } else if (next2_key != last_key) {
             // it began in this chunk and ends in the next: its lookups there are summed here as well (they are a prefix
             // of that chunk: m of them), and the row gets its one update
             double more[NV][4];
 #pragma unroll
             for (int v = 0; v < NV; ++v) more[v][0] = more[v][1] = more[v][2] = more[v][3] = 0.0;
-            const int p = end + lane;
-            const int32_t k2 = p < n ? keys[p] : -1;
-            int32_t b2 = p < n ? vals[p] : 0;
+            if (G == 32) load_next();
             b2 = (uint32_t)b2 < n_grad_u ? b2 : 0;
             const int m = __popc(__ballot_sync(0xffffffffu, k2 == last_key));
             const int mine = m - g0;             // lookups of my group that belong to the run
@@ -614,9 +629,9 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 3 : 1) k_bwd_chunks(float*
                     for (int off = G; off < 32; off <<= 1) more[v][e] += __shfl_xor_sync(0xffffffffu, more[v][e], off);
                     more[v][e] += acc[v][e];
                 }
-            if (lane < G) apply((uint32_t)(last_key - key_bias), more);
+            if (last_group) apply((uint32_t)(last_key - key_bias), more);
         } else {
-            if (lane < G) store_piece(1, acc);
+            if (last_group) store_piece(1, acc);
             // List it, with its last chunk if that is among the next 32 (chunk c > chunk holds a piece of the run iff
             // its first slot is the run's; sorted keys: those chunks form a prefix).  Nearly every run ends there, and
             // k_bwd_spans then has nothing to search; the longer ones go to the list's other end.
@@ -803,9 +818,12 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
                    const float* grad, float lr, cudaStream_t stream, const int32_t* d_first = nullptr,
                    int32_t key_bias = 0) {
     const int64_t max_chunks = div_up(ctx->max_nnz, kBwdChunk);
-    // a fixed number of CTAs per multiprocessor (the groups stride over the chunks), so that kernels of other
-    // streams find room beside this one
-    const int grid = grid_for(max_chunks * 32, kThreads, bwd_ctas_per_sm(ctx) * ctx_sms(ctx));
+    // a fixed number of CTAs per multiprocessor (the warps stride over the chunks), so that kernels of other streams find
+    // room beside this one: two rounds of those that fit
+    const bool four = G == 16 && max_chunks > 3 * (kThreads / 32) * ctx_sms(ctx);
+    const auto sums = four ? k_bwd_chunks<G, NV, G == 16 ? 4 : NV == 1 ? 3 : 1> : k_bwd_chunks<G, NV, NV == 1 ? 3 : 1>;
+    const int per_sm = ctx->bwd_ctas > 0 ? ctx->bwd_ctas : four ? 8 : 6;
+    const int grid = grid_for(max_chunks * 32, kThreads, per_sm * ctx_sms(ctx));
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 0, stream);
     // the list of runs that cross a chunk border sits behind the partial sums: [count words (8 ints)] [entries].
@@ -817,7 +835,7 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
         HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(span_count), 8, stream));
         ctx->spans_suspect = 0;
     }
-    HL_CUDA_TRY(launch(k_bwd_chunks<G, NV>, grid, kThreads, stream, cache, keys, vals, d_n_lookups, grad, ctx->D / 4,
+    HL_CUDA_TRY(launch(sums, grid, kThreads, stream, cache, keys, vals, d_n_lookups, grad, ctx->D / 4,
                        n_slots, lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list, ctx->max_bags, max_chunks,
                        ctx->r.status));
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 1, stream);

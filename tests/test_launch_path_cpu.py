@@ -214,7 +214,7 @@ def test_a_graph_that_cannot_be_changed_or_built_gives_way_to_plain_launches(B, 
         k += 1
         lines = update(k)
         # whichever way: all kernels of the call, with this call's gradient
-        assert [_name(x) for x in lines if x[:5] in ("plain", "graph")][-2:] == ["k_bwd_chunks<4,1>", "k_bwd_spans<4,1>"]
+        assert [_name(x).split("<")[0] for x in lines if x[:5] in ("plain", "graph")][-2:] == ["k_bwd_chunks", "k_bwd_spans"]
         assert grads[k % 40].to_bytes(8, "little").hex() in [x for x in lines if "k_bwd_chunks" in x][0]
     lib.fake_fail(b"cudaGraphExecKernelNodeSetParams", 0)
     while not all(x.startswith("graph") for x in update(k)):
