@@ -171,7 +171,8 @@ HL_API int32_t hl_set_kernel_width(hl_ctx* ctx, int32_t fwd_ctas_per_sm, int32_t
  * and sort pass publishes nothing, and (stall_tile >= 0) the first stage of the movers' first CTA issues no copies.
  * The waits behind it then run out: the kernels return, the status word reads HL_ETIMEOUT, every position computed
  * from the incomplete data is range-checked before use, and the results of those calls are unspecified.
- * poll_limit = 0 restores production behaviour.  Nothing here can hang or fault the device. */
+ * poll_limit = 0 restores production behaviour.  Nothing here can hang or fault the device.
+ * (hl_profile_hot's selection and hl_wide_* have such tiles too; hl_wide_test_bounded_waits is the same for those.) */
 HL_API int32_t hl_test_bounded_waits(hl_ctx* ctx, int32_t poll_limit, int64_t stall_tile);
 
 /* Number of kernels this library has launched in this process so far (all contexts). */
@@ -546,6 +547,7 @@ HL_API int32_t hl_wide_create(hl_wide** out, const hl_geometry* geom, int32_t ma
                               void* d_workspace, size_t ws_bytes);
 HL_API int32_t hl_wide_destroy(hl_wide* w);
 HL_API int32_t hl_wide_status(hl_wide* w);     /* as hl_status */
+HL_API int32_t hl_wide_test_bounded_waits(hl_wide* w, int32_t poll_limit, int64_t stall_tile);   /* as hl_test_bounded_waits */
 /* As hl_profile_hot; d_hot_rows is int64 [hot_cap_rows]; row_bytes is the row payload HL_HOT_BUDGET_BYTES divides by. */
 HL_API int32_t hl_wide_profile_hot(hl_wide* w, const hl_batch* b, int32_t reset, int32_t finalize, int32_t policy,
                                    int64_t p_num, int64_t p_den, int32_t row_bytes, int64_t* d_hot_rows,

@@ -27,7 +27,7 @@ EXPORTS = (
     "hl_wide_workspace_bytes", "hl_wide_create", "hl_wide_destroy", "hl_wide_status", "hl_wide_profile_hot",
     "hl_wide_build_remap", "hl_wide_fragment", "hl_wide_index_cold",
     "hl_index_cold_begin", "hl_index_cold_end", "hl_index_cold_verdict",
-    "hl_embbag_bwd_prepare_merged", "hl_pipe_set_order", "hl_step",
+    "hl_embbag_bwd_prepare_merged", "hl_pipe_set_order", "hl_step", "hl_wide_test_bounded_waits",
 )
 
 
@@ -197,6 +197,8 @@ def _load() -> ctypes.CDLL:
     lib.hl_set_host_tables.argtypes = [vp, ctypes.POINTER(vp)]
     lib.hl_test_bounded_waits.restype = i32
     lib.hl_test_bounded_waits.argtypes = [vp, i32, i64]
+    lib.hl_wide_test_bounded_waits.restype = i32
+    lib.hl_wide_test_bounded_waits.argtypes = [vp, i32, i64]
     lib.hl_step.restype = i32
     lib.hl_step.argtypes = [vp, ctypes.POINTER(hl_batch), vp, i32, ctypes.POINTER(hl_step_buffers), vp, vp, vp, vp,
                             ctypes.c_float, i32, vp, vp]
@@ -523,6 +525,10 @@ def hl_wide_status(w: int, raise_on_error: bool = True) -> int:
     if raise_on_error:
         _check("hl_wide_status", st)
     return st
+
+
+def hl_wide_test_bounded_waits(w: int, poll_limit: int, stall_tile: int = -1) -> None:
+    _check("hl_wide_test_bounded_waits", _lib.hl_wide_test_bounded_waits(w, int(poll_limit), int(stall_tile)))
 
 
 def hl_wide_profile_hot(w: int, batch: Optional[hl_batch], reset: bool, finalize: bool, policy: int, p_num: int,

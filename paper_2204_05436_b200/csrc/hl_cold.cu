@@ -43,8 +43,8 @@ template <bool SUMMARY, int ITEMS>
 __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_words, int64_t staging_cap,
                                                         int32_t* __restrict__ cold_rows, int64_t* __restrict__ d_n_cold,
                                                         int32_t* __restrict__ verdict, unsigned long long* chain,
-                                                        int32_t* status, int max_polls, uint32_t* __restrict__ clear,
-                                                        int64_t n_clear) {
+                                                        int32_t* status, int max_polls, int64_t stall_tile,
+                                                        uint32_t* __restrict__ clear, int64_t n_clear) {
     constexpr int NW = kThreads / 32;
     __shared__ int s_sum[NW];
     __shared__ bool s_last;
@@ -86,8 +86,9 @@ __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_w
         if (k < warp) warp_start += s_sum[k];
         tile_sum += s_sum[k];
     }
-    chain_publish(chain + 1, tile, (unsigned long long)tile_sum);
-    const int before = (int)chain_before<kThreads>(chain + 1, tile, (unsigned long long)tile_sum, true, max_polls, status);
+    if (tile != stall_tile) chain_publish(chain + 1, tile, (unsigned long long)tile_sum);
+    const int before = (int)chain_before<kThreads>(chain + 1, tile, (unsigned long long)tile_sum, tile != stall_tile,
+                                                   max_polls, status);
     if (threadIdx.x == 0 && first + kThreads * ITEMS >= n_words) {       // the last tile knows the total
         int64_t distinct = (int64_t)before + tile_sum;
         if (distinct > staging_cap) {
@@ -442,8 +443,9 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
     const unsigned grid = (unsigned)div_up(words, kThreads * (many ? 4 : 1));
     const auto kernel = summary ? (many ? k_cold_rank<true, 4> : k_cold_rank<true, 1>)
                                 : (many ? k_cold_rank<false, 4> : k_cold_rank<false, 1>);
+    const WaitCfg w = wait_cfg(ctx);
     HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.cold_n + 1,
-                       r.cold_chain, r.status, wait_cfg(ctx).max_polls, clear, n_clear));
+                       r.cold_chain, r.status, w.max_polls, w.stall_tile, clear, n_clear));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;

@@ -141,6 +141,8 @@ struct hl_wide {
     int32_t* cold_n;                         // cold lookups of X
     unsigned long long* cold_chain;          // [max_nnz / 1024 + 1]
     hl::LaunchCache* launches;
+    int test_poll_limit;                     // as in hl_ctx
+    int64_t test_stall_tile;
 };
 
 namespace hl {
@@ -416,7 +418,8 @@ struct WaitCfg {
     int max_polls = 1 << 20;
     int64_t stall_tile = -1;
 };
-inline WaitCfg wait_cfg(const hl_ctx* ctx) {
+template <typename Ctx>                // hl_ctx or hl_wide
+inline WaitCfg wait_cfg(const Ctx* ctx) {
     WaitCfg w;
     if (ctx->test_poll_limit > 0) {
         w.max_polls = ctx->test_poll_limit;
@@ -561,7 +564,7 @@ int32_t fragment_and_mark(hl_ctx* ctx, const hl_batch* b, const float* d_dense, 
 // Selection of the rows with the k largest counts (implemented in hl_profile.cu; see there).
 int32_t select_rows_by_count(const uint32_t* counts, int64_t n, SelectState* sel, unsigned long long* chain, long long k,
                              long long share_num, long long share_den, int64_t cap, int32_t* out_idx, int64_t* d_n_out,
-                             int32_t* status, int sms, cudaStream_t stream);
+                             int32_t* status, int sms, WaitCfg w, cudaStream_t stream);
 
 // Process-wide count of kernels this library has launched (read by hl_launch_count).
 void note_launches(int n);

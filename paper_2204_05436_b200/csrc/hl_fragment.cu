@@ -492,7 +492,7 @@ extern "C" int32_t hl_wide_fragment(hl_wide* w, const hl_batch* b, int32_t* d_pe
     const HashProbe probe{w->r_keys, w->r_vals, (uint64_t)(w->remap_slots - 1)};
     return as_graph(w->launches, [&] {
         return fragment_launch<false, HashProbe, long long>(
-            b, w->T, w->S, w->sms, w->table_base, probe, w->frag_words, w->frag_chain, w->status, WaitCfg(), nullptr, 0,
+            b, w->T, w->S, w->sms, w->table_base, probe, w->frag_words, w->frag_chain, w->status, wait_cfg(w), nullptr, 0,
             d_perm, d_counts, pop, d_non_offsets, reinterpret_cast<long long*>(d_non_rows), non_cap, nullptr, ColdMarks{},
             static_cast<cudaStream_t>(stream_));
     });

@@ -141,7 +141,8 @@ __global__ void __launch_bounds__(kThreads) k_select_digit(const uint32_t* __res
 __global__ void __launch_bounds__(kThreads) k_select_emit(const uint32_t* __restrict__ counts, int64_t N,
                                                           const SelectState* __restrict__ sel, unsigned long long* chain,
                                                           int64_t hot_cap, int32_t* __restrict__ hot_rows,
-                                                          int64_t* __restrict__ n_hot, int max_polls, int32_t* status) {
+                                                          int64_t* __restrict__ n_hot, int max_polls, int64_t stall_tile,
+                                                          int32_t* status) {
     constexpr int kRows = kSelTile / kThreads / 4, NW = kThreads / 32, kHalf = 31;
     constexpr int kWords = kRows / 4;                        // eight fields of eight bits each
     static_assert(kRows % 4 == 0, "whole words");
@@ -204,8 +205,9 @@ __global__ void __launch_bounds__(kThreads) k_select_emit(const uint32_t* __rest
         if (w < warp) before_warp += s_sum[w];
         total += s_sum[w];
     }
-    chain_publish(chain, blockIdx.x, total);
-    const unsigned long long before = chain_before<kThreads>(chain, blockIdx.x, total, true, max_polls, status);
+    const bool publish = blockIdx.x != stall_tile;
+    if (publish) chain_publish(chain, blockIdx.x, total);
+    const unsigned long long before = chain_before<kThreads>(chain, blockIdx.x, total, publish, max_polls, status);
     // (32 bits are enough for numbers of rows)
     unsigned row_gt = (unsigned)((before + before_warp) >> kHalf);
     unsigned row_eq = (unsigned)((before + before_warp) & ((1ull << kHalf) - 1));
@@ -292,14 +294,14 @@ int32_t launch_gather_rows(hl_ctx* ctx, float* dst, int64_t dst_row0, const floa
 // ascending order, to out_idx [cap], their number to *d_n_out.  chain: div_up(n, kSelTile) words.  counts: 16-byte aligned.
 int32_t select_rows_by_count(const uint32_t* counts, int64_t n, SelectState* sel, unsigned long long* chain, long long k,
                              long long share_num, long long share_den, int64_t cap, int32_t* out_idx, int64_t* d_n_out,
-                             int32_t* status, int sms, cudaStream_t stream) {
+                             int32_t* status, int sms, WaitCfg w, cudaStream_t stream) {
     const int64_t n_tiles = div_up(n, kSelTile);
     HL_CUDA_TRY(launch(k_select_begin, 1, 256, stream, sel, (unsigned long long)k, share_num, share_den));
     for (int shift = 24; shift >= 0; shift -= 8)
         HL_CUDA_TRY(launch(k_select_digit, grid_for(n, kThreads * 16, sms * 8), kThreads, stream, counts, n, shift, sel,
                            chain, shift == 24 ? n_tiles : 0));
     HL_CUDA_TRY(launch(k_select_emit, n_tiles, kThreads, stream, counts, n, sel, chain, cap, out_idx, d_n_out,
-                       WaitCfg().max_polls, status));
+                       w.max_polls, w.stall_tile, status));
     note_launches(6);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -352,7 +354,7 @@ extern "C" int32_t hl_profile_hot(hl_ctx* ctx, const hl_batch* b, int32_t reset,
         if (k > ctx->hot_cap) k = ctx->hot_cap;
         return as_graph(ctx->launches, [&] {
             return select_rows_by_count(r.counts, ctx->N, r.sel, r.sel_chain, k, share_num, share_den, ctx->hot_cap,
-                                        d_hot_rows, d_n_hot, r.status, ctx_sms(ctx), stream);
+                                        d_hot_rows, d_n_hot, r.status, ctx_sms(ctx), wait_cfg(ctx), stream);
         });
     }
     return HL_OK;

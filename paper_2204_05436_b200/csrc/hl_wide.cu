@@ -162,6 +162,10 @@ __global__ void __launch_bounds__(kThreads) k_wide_entries(const long long* __re
     }
 }
 
+// What a sort gives as the number of one of n entries.  (It is one, unless a wait of the sort ran out and left the place as it
+// was: the status word says so, and the results are unspecified, but nothing outside the arrays may be read or written.)
+__device__ __forceinline__ int32_t entry_in(int32_t e, int64_t n) { return (uint32_t)e < (uint64_t)n ? e : 0; }
+
 // out_key[j] = table[val[j]]: the key of the second, stable sort
 __global__ void __launch_bounds__(kThreads) k_wide_gather_key(const int32_t* __restrict__ val,
                                                               const int32_t* __restrict__ table, const int32_t* d_n,
@@ -169,7 +173,7 @@ __global__ void __launch_bounds__(kThreads) k_wide_gather_key(const int32_t* __r
     int64_t n = *d_n;
     n = n < n_max ? n : n_max;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-        out_key[j] = table[val[j]];
+        out_key[j] = table[entry_in(val[j], n)];
 }
 
 // counts in row order (zero behind the last counted row), and the entry behind every position
@@ -180,14 +184,15 @@ __global__ void __launch_bounds__(kThreads) k_wide_row_order(const int32_t* __re
     int64_t n = *d_n;
     n = n < n_max ? n : n_max;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n_max; j += (int64_t)gridDim.x * blockDim.x) {
-        s_cnt[j] = j < n ? e_cnt[val[j]] : 0u;
-        s_ent[j] = j < n ? val[j] : -1;
+        const int32_t e = j < n ? entry_in(val[j], n) : -1;
+        s_cnt[j] = j < n ? e_cnt[e] : 0u;
+        s_ent[j] = e;
     }
 }
 
 __global__ void __launch_bounds__(kThreads) k_wide_hot_rows(const int32_t* __restrict__ sel_idx,
                                                             const int64_t* __restrict__ d_n_hot, int64_t hot_cap,
-                                                            const int32_t* __restrict__ s_ent,
+                                                            const int32_t* __restrict__ s_ent, int64_t n_entries,
                                                             const int32_t* __restrict__ e_tab,
                                                             const int32_t* __restrict__ e_idx,
                                                             const int64_t* __restrict__ table_base,
@@ -195,8 +200,8 @@ __global__ void __launch_bounds__(kThreads) k_wide_hot_rows(const int32_t* __res
     int64_t n = *d_n_hot;
     n = n < hot_cap ? n : hot_cap;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t e = s_ent[sel_idx[i]];
-        hot_rows[i] = table_base[e_tab[e]] + e_idx[e];
+        const int32_t e = s_ent[entry_in(sel_idx[i], n_entries)];
+        hot_rows[i] = e >= 0 ? table_base[e_tab[e]] + e_idx[e] : -1;
     }
 }
 
@@ -286,6 +291,13 @@ extern "C" int32_t hl_wide_create(hl_wide** out, const hl_geometry* geom, int32_
     return HL_OK;
 }
 
+extern "C" int32_t hl_wide_test_bounded_waits(hl_wide* w, int32_t poll_limit, int64_t stall_tile) {
+    if (!w || poll_limit < 0) return HL_EINVAL;
+    w->test_poll_limit = poll_limit;
+    w->test_stall_tile = poll_limit > 0 ? stall_tile : -1;
+    return HL_OK;
+}
+
 extern "C" int32_t hl_wide_destroy(hl_wide* w) {
     if (!w) return HL_EINVAL;
     delete w->launches;
@@ -312,7 +324,8 @@ namespace {
 int32_t sort_by_row(hl_wide* w, const int32_t* table_of_entry, const int32_t* d_n, int64_t n_max, int32_t** out_vals,
                     cudaStream_t stream) {
     int32_t *k1, *v1;
-    int32_t st = radix_sort_pairs(w->sort_keys, w->sort_vals, d_n, n_max, 31, w->sort_hist, w->status, &k1, &v1, stream);
+    int32_t st = radix_sort_pairs(w->sort_keys, w->sort_vals, d_n, n_max, 31, w->sort_hist, w->status, &k1, &v1, stream,
+                                  wait_cfg(w));
     if (st != HL_OK) return st;
     // the result sits in buffer `cur`; the second sort starts from buffer 0, so bring it there if needed
     const int cur = v1 == w->sort_vals[0] ? 0 : 1;
@@ -326,7 +339,7 @@ int32_t sort_by_row(hl_wide* w, const int32_t* table_of_entry, const int32_t* d_
     HL_LAUNCH_CHECK();
     int32_t* k2;
     return radix_sort_pairs(w->sort_keys, w->sort_vals, d_n, n_max, bits_for(w->T - 1), w->sort_hist, w->status, &k2,
-                            out_vals, stream);
+                            out_vals, stream, wait_cfg(w));
 }
 
 // ---- cold rows of X -----------------------------------------------------------------------------------------------
@@ -386,13 +399,13 @@ __global__ void __launch_bounds__(kThreads) k_wide_classify(const long long* __r
 
 // the upper bits of the rows, in the order of their lower bits
 __global__ void __launch_bounds__(kThreads) k_wide_upper_key(const int32_t* __restrict__ pos,
-                                                             const long long* __restrict__ rows, const int32_t* d_n,
-                                                             int64_t n_max, int32_t* __restrict__ key,
-                                                             int32_t* __restrict__ val) {
+                                                             const long long* __restrict__ rows, int64_t n_rows,
+                                                             const int32_t* d_n, int64_t n_max,
+                                                             int32_t* __restrict__ key, int32_t* __restrict__ val) {
     int64_t n = *d_n;
     n = n < n_max ? n : n_max;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t p = pos[j];
+        const int32_t p = entry_in(pos[j], n_rows);
         key[j] = (int32_t)(rows[p] >> 32);
         val[j] = p;
     }
@@ -408,7 +421,8 @@ __global__ void __launch_bounds__(kThreads) k_wide_ranks(const int32_t* __restri
                                                          int64_t n_max, unsigned long long* chain, int64_t slot0,
                                                          int64_t staging_cap, int64_t cap_ids,
                                                          int32_t* __restrict__ slots, long long* __restrict__ cold_rows,
-                                                         int64_t* __restrict__ d_n_cold, int max_polls, int32_t* status) {
+                                                         int64_t* __restrict__ d_n_cold, int max_polls, int64_t stall_tile,
+                                                         int32_t* status) {
     __shared__ int s_warp[kThreads / 32];
     int64_t n = *d_n;
     n = n < n_max ? n : n_max;
@@ -419,7 +433,9 @@ __global__ void __launch_bounds__(kThreads) k_wide_ranks(const int32_t* __restri
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t j0 = tile0 + threadIdx.x * kRankItems;
-    auto row_at = [&](int64_t j) -> long long { return UPPER ? rows[pos[j]] : (long long)(uint32_t)keys[j]; };
+    auto row_at = [&](int64_t j) -> long long {
+        return UPPER ? rows[entry_in(pos[j], cap_ids)] : (long long)(uint32_t)keys[j];
+    };
     long long g[kRankItems];
     int32_t at[kRankItems];
     long long prev = j0 > 0 && j0 < n ? row_at(j0 - 1) : -1;
@@ -450,8 +466,10 @@ __global__ void __launch_bounds__(kThreads) k_wide_ranks(const int32_t* __restri
         if (w < warp) before += s_warp[w];
         total += s_warp[w];
     }
-    chain_publish(chain, blockIdx.x, (unsigned long long)total);
-    const int64_t base = (int64_t)chain_before<kThreads>(chain, blockIdx.x, (unsigned long long)total, true, max_polls, status);
+    const bool publish = blockIdx.x != stall_tile;
+    if (publish) chain_publish(chain, blockIdx.x, (unsigned long long)total);
+    const int64_t base =
+        (int64_t)chain_before<kThreads>(chain, blockIdx.x, (unsigned long long)total, publish, max_polls, status);
     int64_t rank = base + before + (incl - mine) - 1;
 #pragma unroll
     for (int k = 0; k < kRankItems; ++k) {
@@ -539,10 +557,11 @@ extern "C" int32_t hl_wide_profile_hot(hl_wide* w, const hl_batch* b, int32_t re
     note_launches(1);
     HL_LAUNCH_CHECK();
     st = select_rows_by_count(w->s_cnt, E, w->sel, w->sel_chain, k, share_num, share_den, w->hot_cap,
-                              w->sel_idx, d_n_hot, w->status, w->sms, stream);
+                              w->sel_idx, d_n_hot, w->status, w->sms, wait_cfg(w), stream);
     if (st != HL_OK) return st;
     HL_CUDA_TRY(launch(k_wide_hot_rows, grid_for(w->hot_cap, kThreads, w->sms * 8), kThreads, stream, w->sel_idx, d_n_hot,
-                       w->hot_cap, w->s_ent, w->e_tab, w->e_idx, w->table_base, reinterpret_cast<long long*>(d_hot_rows)));
+                       w->hot_cap, w->s_ent, E, w->e_tab, w->e_idx, w->table_base,
+                       reinterpret_cast<long long*>(d_hot_rows)));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
@@ -577,7 +596,8 @@ extern "C" int32_t hl_wide_index_cold(hl_wide* w, const int32_t* d_non_offsets, 
     // Rows of up to 32 bits are sorted as they are; others by their lower 32 bits, then (stable) by the rest.
     const int upper_bits = (w->N - 1) >> 32 ? bits_for((w->N - 1) >> 32) : 0;
     const int lower_bits = upper_bits ? 32 : bits_for(w->N - 1);
-    const int64_t sort_words = sort_clear_words(w->max_nnz, lower_bits, WaitCfg());
+    const WaitCfg waits = wait_cfg(w);
+    const int64_t sort_words = sort_clear_words(w->max_nnz, lower_bits, waits);
     HL_CUDA_TRY(clear_words(w->cold_clear, (int64_t)(w->sort_hist - w->cold_clear) + sort_words, stream));
     HL_CUDA_TRY(launch(sort_words ? k_wide_classify<true> : k_wide_classify<false>,
                        grid_for(w->max_nnz, kThreads, 3 * w->sms), kThreads, stream,
@@ -587,22 +607,22 @@ extern "C" int32_t hl_wide_index_cold(hl_wide* w, const int32_t* d_non_offsets, 
     note_launches(1);
     int32_t *keys, *pos;
     int32_t st = radix_sort_pairs(w->sort_keys, w->sort_vals, w->cold_n, w->max_nnz, lower_bits, w->sort_hist, w->status,
-                                  &keys, &pos, stream, WaitCfg(), true);
+                                  &keys, &pos, stream, waits, true);
     if (st != HL_OK) return st;
     if (upper_bits) {
         const int other = pos == w->sort_vals[0] ? 1 : 0;
         int32_t* k2[2] = {w->sort_keys[other], w->sort_keys[other ^ 1]};
         int32_t* v2[2] = {w->sort_vals[other], w->sort_vals[other ^ 1]};
         HL_CUDA_TRY(launch(k_wide_upper_key, grid_for(w->max_nnz, kThreads, 8 * w->sms), kThreads, stream, pos,
-                           reinterpret_cast<const long long*>(d_non_rows), w->cold_n, w->max_nnz, k2[0], v2[0]));
+                           reinterpret_cast<const long long*>(d_non_rows), non_cap, w->cold_n, w->max_nnz, k2[0], v2[0]));
         note_launches(1);
-        st = radix_sort_pairs(k2, v2, w->cold_n, w->max_nnz, upper_bits, w->sort_hist, w->status, &keys, &pos, stream);
+        st = radix_sort_pairs(k2, v2, w->cold_n, w->max_nnz, upper_bits, w->sort_hist, w->status, &keys, &pos, stream, waits);
         if (st != HL_OK) return st;
     }
     HL_CUDA_TRY(launch(upper_bits ? k_wide_ranks<true> : k_wide_ranks<false>, div_up(w->max_nnz, kRankTile), kThreads,
                        stream, keys, pos, reinterpret_cast<const long long*>(d_non_rows), w->cold_n, w->max_nnz,
                        w->cold_chain, w->hot_cap, w->staging_cap, non_cap, d_non_slots,
-                       reinterpret_cast<long long*>(d_cold_rows), d_n_cold, WaitCfg().max_polls, w->status));
+                       reinterpret_cast<long long*>(d_cold_rows), d_n_cold, waits.max_polls, waits.stall_tile, w->status));
     note_launches(1);
     return batch.end();
 }
