@@ -143,7 +143,6 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
     if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_bits, 0, sizeof(uint32_t) * cold_bitmap_words(N));
     if (e == cudaSuccess && N > kColdDirectRows)
         e = cudaMemset(ctx->r.cold_summary, 0, sizeof(uint32_t) * cold_summary_words(N));
-    if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_chain, 0, sizeof(unsigned long long) * cold_chain_words(N));
     if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_n, 0, 4 * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(span_count_of(ctx), 0, 8 * sizeof(int32_t));   // kept zero between backward calls
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->step_ranked, cudaEventDisableTiming);

@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(kThreads) k_cold_classify(int32_t* __restrict_
                                                             const int32_t* __restrict__ d_n_non, int max_batch,
                                                             int bags_per_sample_all, int64_t cap_ids, int64_t N,
                                                             BitmapProbe remap, ColdMarks marks, int32_t* status) {
+    clear_cold_chain(marks);
     int n_non = *d_n_non;
     n_non = n_non < 0 ? 0 : (n_non > max_batch ? max_batch : n_non);
     int64_t L = offsets[(int64_t)n_non * bags_per_sample_all];
@@ -34,20 +35,17 @@ __global__ void __launch_bounds__(kThreads) k_cold_classify(int32_t* __restrict_
     }
 }
 
-// Tiles of kThreads * ITEMS words, chained (chain_before; chain[0] =
-// tally of finished CTAs, [1 + tile] = status word; zero on entry, and the CTA that finishes last clears them again).
+// Tiles of kThreads * ITEMS words, chained (chain_before; marks.chain is zero on entry).
 // SUMMARY: the words are those of the summary, which has a bit for every bitmap word that is not zero (models above
 // kColdDirectRows rows, whose bitmap would be megabytes of zeros to read); otherwise the bitmap's own.  Bitmap and summary
 // are left cleared; marks.ranked[word] keeps what k_cold_assign needs: the word's bits and the rank of its first one.
 template <bool SUMMARY, int ITEMS>
 __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_words, int64_t staging_cap,
                                                         int32_t* __restrict__ cold_rows, int64_t* __restrict__ d_n_cold,
-                                                        int32_t* __restrict__ verdict, unsigned long long* chain,
                                                         int32_t* status, int max_polls, int64_t stall_tile,
                                                         uint32_t* __restrict__ clear, int64_t n_clear) {
     constexpr int NW = kThreads / 32;
     __shared__ int s_sum[NW];
-    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x; i < n_clear / 4; i += (int64_t)gridDim.x * kThreads)
         reinterpret_cast<uint4*>(clear)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -86,8 +84,8 @@ __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_w
         if (k < warp) warp_start += s_sum[k];
         tile_sum += s_sum[k];
     }
-    if (tile != stall_tile) chain_publish(chain + 1, tile, (unsigned long long)tile_sum);
-    const int before = (int)chain_before<kThreads>(chain + 1, tile, (unsigned long long)tile_sum, tile != stall_tile,
+    if (tile != stall_tile) chain_publish(marks.chain, tile, (unsigned long long)tile_sum);
+    const int before = (int)chain_before<kThreads>(marks.chain, tile, (unsigned long long)tile_sum, tile != stall_tile,
                                                    max_polls, status);
     if (threadIdx.x == 0 && first + kThreads * ITEMS >= n_words) {       // the last tile knows the total
         int64_t distinct = (int64_t)before + tile_sum;
@@ -96,7 +94,6 @@ __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_w
             distinct = staging_cap;
         }
         *d_n_cold = distinct;
-        *verdict = 0;
     }
 #pragma unroll
     for (int i = 0; i < ITEMS; ++i) {
@@ -119,10 +116,6 @@ __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_w
             take(w, word[i]);
         }
     }
-    if (threadIdx.x == 0) s_last = atomicAdd(&chain[0], 1ull) == gridDim.x - 1;
-    __syncthreads();
-    if (s_last)                                              // (nobody reads the status words any more)
-        for (int i = threadIdx.x; i < (int)gridDim.x + 1; i += kThreads) chain[i] = 0ull;
 }
 
 // Every cold lookup of X (an id of -2 - g) gets the staging slot of its row: slot0 + rank (slot0 = start of the window).
@@ -444,8 +437,8 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
     const auto kernel = summary ? (many ? k_cold_rank<true, 4> : k_cold_rank<true, 1>)
                                 : (many ? k_cold_rank<false, 4> : k_cold_rank<false, 1>);
     const WaitCfg w = wait_cfg(ctx);
-    HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.cold_n + 1,
-                       r.cold_chain, r.status, w.max_polls, w.stall_tile, clear, n_clear));
+    HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.status,
+                       w.max_polls, w.stall_tile, clear, n_clear));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;

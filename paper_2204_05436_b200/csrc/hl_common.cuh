@@ -70,8 +70,8 @@ struct Regions {
     uint32_t* cold_bits;               // [cold_bitmap_words] one bit per row; zero between calls
     uint32_t* cold_summary;            // [cold_summary_words] one bit per bitmap word; zero between calls
     uint2* cold_ranked;                // [cold_bitmap_words] bits of the word, rank of its first row
-    unsigned long long* cold_chain;    // [cold_chain_words]; zero between calls
-    int32_t* cold_n;                   // [4]; [1] = hl_index_cold_verdict
+    unsigned long long* cold_chain;    // [cold_chain_words]
+    int32_t* cold_n;                   // [4]; [1] = hl_index_cold_verdict, which stays 0
 };
 
 class LaunchCache;
@@ -343,9 +343,9 @@ struct BitmapProbe {
 constexpr int64_t kColdDirectRows = int64_t(1) << 26;
 constexpr int64_t cold_bitmap_words(int64_t N) { return (N + 31) / 32; }
 constexpr int64_t cold_summary_words(int64_t N) { return (cold_bitmap_words(N) + 31) / 32; }
-// ticket, tally and one status word per tile of k_cold_rank (at least 256 words per tile)
+// one status word per tile of k_cold_rank (at least 256 words per tile)
 constexpr int64_t cold_chain_words(int64_t N) {
-    return 3 + (N > kColdDirectRows ? cold_summary_words(N) : cold_bitmap_words(N)) / 256;
+    return 1 + (N > kColdDirectRows ? cold_summary_words(N) : cold_bitmap_words(N)) / 256;
 }
 // tally, ticket and one status word per tile of k_frag_place (at least 256 bags per tile)
 constexpr int64_t frag_chain_words(int64_t max_bags) { return 3 + max_bags / 256 + 1; }
@@ -354,9 +354,19 @@ struct ColdMarks {
     uint32_t* bits;
     uint32_t* summary;                 // nullptr: no summary is kept
     uint2* ranked;
+    unsigned long long* chain;         // state of k_cold_rank's chained tiles, cleared by the kernel that marks
+    int64_t n_chain;
 };
 inline ColdMarks cold_marks(const hl_ctx* ctx) {
-    return {ctx->r.cold_bits, ctx->N > kColdDirectRows ? ctx->r.cold_summary : nullptr, ctx->r.cold_ranked};
+    return {ctx->r.cold_bits, ctx->N > kColdDirectRows ? ctx->r.cold_summary : nullptr, ctx->r.cold_ranked,
+            ctx->r.cold_chain, cold_chain_words(ctx->N)};
+}
+
+// The chain of the ranking that follows, cleared by the kernel that marks the rows.  (Not by the last CTA of the ranking
+// itself: nothing would order its clears behind what the other CTAs published.)
+__device__ __forceinline__ void clear_cold_chain(const ColdMarks& marks) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < marks.n_chain; i += (int64_t)gridDim.x * blockDim.x)
+        marks.chain[i] = 0ull;
 }
 
 // A lookup of X that addresses row g (inside the model): its cache slot if the row is popular; otherwise the row is

@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
                                                          ColdMarks marks) {
     constexpr int TB = kThreads * ITEMS, NW = kThreads / 32;
     __shared__ int32_t s_pop[NW], s_all[NW];         // lookups of O / lookups in the warps' bags
+    if (MARK) clear_cold_chain(marks);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int tile = blockIdx.x;
     const int B = a.B, S = a.S, n_pop = a.counts[0], n_non = B - n_pop;

@@ -54,7 +54,7 @@ size_t size_of(std::string t) {
     while (!t.empty() && t.front() == ' ') t.erase(0, 1);
     if (t.find('*') != std::string::npos) return 8;
     const std::pair<const char*, size_t> known[] = {
-        {"PairArgs", 64}, {"PlaceArgs", 64}, {"ForwardRows", 48}, {"TableMap", 32}, {"ColdMarks", 24}, {"BitmapProbe", 8},
+        {"PairArgs", 64}, {"PlaceArgs", 64}, {"ForwardRows", 48}, {"TableMap", 32}, {"ColdMarks", 40}, {"BitmapProbe", 8},
         {"HashProbe", 24}};
     for (const auto& k : known)
         if (t.find(k.first) != std::string::npos) return k.second;
