@@ -150,8 +150,7 @@ HL_API int32_t hl_set_host_tables(hl_ctx* ctx, float* const* h_table_bases);
 /* Width of the host-link movers inside a schedule: how many CTAs of hl_gather_cold / hl_stage_cold (read_ctas) and of
  * hl_scatter_cold (write_ctas) work when a mini-batch moves a DLRM-sized number of rows (the kernels decide on the
  * device, from the number of rows, whether more join in).  0 = the default (24 for reads, 16 for write-backs; 16 for
- * hl_stage_cold (24 again if the host table is larger than 32 GiB) and hl_scatter_cold_at while they move at most 65 536
- * lines of 128 bytes); at
+ * hl_stage_cold (24 again for more than 10 240 rows) and hl_scatter_cold_at while they move at most 65 536 lines of 128 bytes); at
  * most two per multiprocessor.  Wider movers finish sooner and slow the kernels that run beside them more.  Takes
  * effect with the next call. */
 HL_API int32_t hl_set_mover_ctas(hl_ctx* ctx, int32_t read_ctas, int32_t write_ctas);

@@ -251,13 +251,23 @@ constexpr int kBulkStagesPerCta = 200;    // stages of rows per working CTA befo
 constexpr int kPacedRequests = 40;
 constexpr int kPacedReadBytes = 8192;
 constexpr int64_t kPacedMost = 1 << 16;
-constexpr int64_t kFarTableBytes = int64_t(32) << 30;     // between the two sizes measured (move_cfg)
+// How many CTAs a paced read gets goes by its rows.  Up to some 10 thousand the rows are there in time with 16 CTAs, and more
+// of them only disturb the kernels beside them; beyond that the read is what the mini-batch waits for.  One pipeline, 16
+// against 24 CTAs, us per mini-batch (26 tables; rows read): rows of 256 bytes out of 2 GiB 5.0 K 83 / 84, 7.3 K 114 / 114,
+// 10.9 K 167 / 161; out of 24 GiB 4.7 K 82 / 85, 7.7 K 115 / 115, 12.5 K 183 / 170, 19.9 K 294 / 264; out of 6, 36, 48, 61 GiB
+// 15.5 K 236 / 210, 19.3 K 281 / 260, 18.5 K 281 / 251, 16.1 K 246 / 225.  Rows of 64 bytes: 3.7 K 56 / 56, 8.8 K 89 / 86, 13.3 K
+// 127 / 121 (2 GiB); 5.1 K 67 / 67, 8.6 K 91 / 90, 13.6 K 139 / 128, 22.3 K 221 / 200 (24 GiB).  Rows of 512 bytes: 3.7 K 110 /
+// 115, 5.3 K 150 / 153, 7.4 K 218 / 224 (2 GiB); 6.3 K 157 / 167, 9.5 K 237 / 236, 14.5 K 362 / 353 (24 GiB).  The size of the
+// table plays no part.  (32 CTAs: within 2 % of 24 for wide rows, 5 % faster for 20 K rows of 64 bytes.  Three pipelines in
+// turn on one chip, which no program runs, lose 1 to 4 % with 24: 12.4 K rows of 256 bytes 175 / 181.)
+constexpr int64_t kPacedFewRows = 10240;
 
 // What a launch of the mover needs to know about its context.
 struct MoveCfg {
     int sms;            // multiprocessors of the device: the launch has at most 2 CTAs per SM
     int min_ctas;       // CTAs that work however few rows there are (at full rate)
-    int paced_ctas;     // CTAs of a paced transfer; 0: never paced
+    int paced_ctas;     // CTAs of a paced transfer of up to kPacedFewRows rows; 0: never paced
+    int paced_more;     // ... of more rows
     int max_polls;      // poll limit of the wait for a stage to fill
     int stall;          // tests only: CTA 0 issues no loads for its first stage, whose wait then runs out
 };
@@ -271,7 +281,8 @@ __global__ void __launch_bounds__(kBulkThreads) k_move_rows_bulk(float* dense_si
                                                                  int64_t table_rows, int row_bytes,
                                                                  int rows_per_stage,
                                                                  const int32_t* __restrict__ skip, int32_t* status,
-                                                                 int min_ctas, int paced_ctas, int64_t paced_most,
+                                                                 int min_ctas, int paced_ctas, int paced_more,
+                                                                 int64_t paced_most,
                                                                  int paced_rows, int max_polls, int stall) {
     __shared__ __align__(128) unsigned char stage[kBulkStages][kBulkStageBytes];
     __shared__ __align__(8) uint64_t mbar[kBulkStages];
@@ -296,7 +307,7 @@ __global__ void __launch_bounds__(kBulkThreads) k_move_rows_bulk(float* dense_si
     // (the link is then all that matters): one more CTA for every kBulkStagesPerCta stages of rows.
     int64_t active = n_batches / kBulkStagesPerCta;
     active = active < min_ctas ? min_ctas : active;
-    if (paced) active = paced_ctas;
+    if (paced) active = n > kPacedFewRows ? paced_more : paced_ctas;
     active = active < (int64_t)gridDim.x ? active : (int64_t)gridDim.x;
     if ((int64_t)blockIdx.x >= active) return;
 
@@ -388,7 +399,8 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
         const int paced_rows = paced_fit > 1 ? paced_fit : 1;
         HL_CUDA_TRY(launch(k_move_rows_bulk<TO_TABLE>, grid, kBulkThreads, stream, dense_side, dense_row0, table, rows, d_n,
                            n_max, table_rows, row_bytes, rows_per_stage, skip, status,
-                           cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, kPacedMost / requests,
+                           cfg.min_ctas < grid ? cfg.min_ctas : grid, cfg.paced_ctas, cfg.paced_more,
+                           kPacedMost / requests,
                            paced_rows < rows_per_stage ? paced_rows : rows_per_stage, cfg.max_polls, cfg.stall));
         note_launches(1);
         HL_LAUNCH_CHECK();
@@ -461,11 +473,8 @@ static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false, 
     MoveCfg c;
     c.sms = ctx_sms(ctx);
     c.min_ctas = width > 0 ? width : 2 * c.sms;
-    // Reads out of a large host table answer later (their address translations miss), so more of them have to be on the way:
-    // 16 K rows of 256 bytes out of 61 GiB take 159 us with 16 CTAs and 135 us with 24 (a pass of the schedule 0.241 and
-    // 0.231 ms); out of 6 GiB 24 CTAs only disturb the others (three pipelines in turn: 159 and 167 us a pass).
-    const bool far = reads && ctx->N * ctx->D * 4 > kFarTableBytes;
-    c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : far ? kReadCtasDefault : kPacedCtas) : 0;
+    c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : kPacedCtas) : 0;
+    c.paced_more = in_schedule && reads && !ctx->mover_width_set ? kReadCtasDefault : c.paced_ctas;
     c.max_polls = ctx->test_poll_limit > 0 ? ctx->test_poll_limit : kBulkMaxPolls;
     c.stall = ctx->test_poll_limit > 0 && ctx->test_stall_tile >= 0;
     return c;
