@@ -62,9 +62,9 @@ size_t carve(char* base, const hl_geometry* g, int64_t N, int32_t max_batch, int
     r->bwd_part = c.take<float>(2 * div_up(nnz, kBwdChunk) * D + bwd_span_list_words(nnz));
     r->bwd_n = c.take<int32_t>(4);
     r->cold_bits = c.take<uint32_t>(cold_bitmap_words(N));
-    r->cold_summary = c.take<uint32_t>(N > kColdDirectRows ? cold_summary_words(N) : 1);
+    r->cold_summary = c.take<uint32_t>(cold_direct(N, max_nnz) ? 1 : cold_summary_words(N));
     r->cold_ranked = c.take<uint2>(cold_bitmap_words(N));
-    r->cold_chain = c.take<unsigned long long>(cold_chain_words(N));
+    r->cold_chain = c.take<unsigned long long>(cold_chain_words(N, max_nnz));
     r->cold_n = c.take<int32_t>(4);
     (void)hot_cap;
     (void)staging_cap;
@@ -141,7 +141,7 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
     if (e == cudaSuccess)
         e = cudaMemset(ctx->r.frag_chain, 0, sizeof(unsigned long long) * frag_chain_words(max_bags));
     if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_bits, 0, sizeof(uint32_t) * cold_bitmap_words(N));
-    if (e == cudaSuccess && N > kColdDirectRows)
+    if (e == cudaSuccess && !cold_direct(N, max_nnz))
         e = cudaMemset(ctx->r.cold_summary, 0, sizeof(uint32_t) * cold_summary_words(N));
     if (e == cudaSuccess) e = cudaMemset(ctx->r.cold_n, 0, 4 * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(span_count_of(ctx), 0, 8 * sizeof(int32_t));   // kept zero between backward calls

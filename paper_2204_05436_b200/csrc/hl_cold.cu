@@ -36,8 +36,8 @@ __global__ void __launch_bounds__(kThreads) k_cold_classify(int32_t* __restrict_
 }
 
 // Tiles of kThreads * ITEMS words, chained (chain_before; marks.chain is zero on entry).
-// SUMMARY: the words are those of the summary, which has a bit for every bitmap word that is not zero (models above
-// kColdDirectRows rows, whose bitmap would be megabytes of zeros to read); otherwise the bitmap's own.  Bitmap and summary
+// SUMMARY: the words are those of the summary, which has a bit for every bitmap word that is not zero (large models, whose
+// bitmap would be megabytes of zeros to read: cold_direct); otherwise the bitmap's own.  Bitmap and summary
 // are left cleared; marks.ranked[word] keeps what k_cold_assign needs: the word's bits and the rank of its first one.
 template <bool SUMMARY, int ITEMS>
 __global__ void __launch_bounds__(kThreads) k_cold_rank(ColdMarks marks, int n_words, int64_t staging_cap,

@@ -337,15 +337,22 @@ struct BitmapProbe {
 };
 
 // ---- the cold-row bitmap --------------------------------------------------------------------------------------
-// Above this many rows the bitmap is read through a summary.  Reading all of it costs little (64 M rows: 8 MB, 20 us), and
-// its words are dealt out evenly; behind a summary word the lookups of a table's first rows pile up on a few lanes (150 K
-// cold rows out of 18, 26 and 50 million: 36, 34 and 73 us through the summary, 15, 15 and 20 us without).
-constexpr int64_t kColdDirectRows = int64_t(1) << 26;
+// Whether the bitmap is read directly or through a summary.  Reading all of it costs 8 us and 0.28 us per million rows,
+// whatever it holds, and its words are dealt out evenly; behind a summary word the rows of small tables pile up on a few
+// lanes, so that its time goes by the cold lookups.  k_cold_rank alone, directly / through the summary, 26 tables, us:
+//   cold lookups     1.7 K        13 K         39 K         130 K        426 K
+//    18 M rows    13.1 / 10.7  13.2 / 22.6  14.3 / 28.8  13.5 / 45.0  14.4 / 60.0
+//    64 M         24.9 / 13.0  24.6 / 27.9  23.8 / 40.1  23.9 / 58.3  25.3 / 84.5
+//   100 M         36.6 / 13.5  33.2 / 23.6  33.9 / 34.0  37.2 / 52.6  36.0 / 93.0
+//   180 M         59.1 / 11.3  59.3 / 20.8  60.3 / 31.1  60.2 / 49.5  58.3 / 80.4
+//   257 M         80.1 / 14.9  78.2 / 34.2  75.9 / 48.4  79.2 / 77.0  82.2 / 123.8
+// What the host knows is how many lookups a mini-batch has at most.  (Of a learned model's 426 K some 22 K are cold.)
+constexpr bool cold_direct(int64_t N, int64_t max_nnz) { return N <= int64_t(1) << (max_nnz > 4096 ? 26 : 24); }
 constexpr int64_t cold_bitmap_words(int64_t N) { return (N + 31) / 32; }
 constexpr int64_t cold_summary_words(int64_t N) { return (cold_bitmap_words(N) + 31) / 32; }
 // one status word per tile of k_cold_rank (at least 256 words per tile)
-constexpr int64_t cold_chain_words(int64_t N) {
-    return 1 + (N > kColdDirectRows ? cold_summary_words(N) : cold_bitmap_words(N)) / 256;
+constexpr int64_t cold_chain_words(int64_t N, int64_t max_nnz) {
+    return 1 + (cold_direct(N, max_nnz) ? cold_bitmap_words(N) : cold_summary_words(N)) / 256;
 }
 // tally, ticket and one status word per tile of k_frag_place (at least 256 bags per tile)
 constexpr int64_t frag_chain_words(int64_t max_bags) { return 3 + max_bags / 256 + 1; }
@@ -358,8 +365,8 @@ struct ColdMarks {
     int64_t n_chain;
 };
 inline ColdMarks cold_marks(const hl_ctx* ctx) {
-    return {ctx->r.cold_bits, ctx->N > kColdDirectRows ? ctx->r.cold_summary : nullptr, ctx->r.cold_ranked,
-            ctx->r.cold_chain, cold_chain_words(ctx->N)};
+    return {ctx->r.cold_bits, cold_direct(ctx->N, ctx->max_nnz) ? nullptr : ctx->r.cold_summary, ctx->r.cold_ranked,
+            ctx->r.cold_chain, cold_chain_words(ctx->N, ctx->max_nnz)};
 }
 
 // The chain of the ranking that follows, cleared by the kernel that marks the rows.  (Not by the last CTA of the ranking
