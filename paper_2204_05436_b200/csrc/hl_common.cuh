@@ -164,11 +164,14 @@ namespace hl {
 // stream (an event, a memset).
 class LaunchCache {
 public:
-    explicit LaunchCache(int variants);              // graphs of the same kernels, with different arguments, worth keeping
+    // variants: graphs of the same kernels, with different arguments, worth keeping.  common: where there are graphs that a
+    // run of kernels without one here can be launched with (nullptr: kernel by kernel)
+    explicit LaunchCache(int variants, LaunchCache* common = nullptr);
     ~LaunchCache();
     LaunchCache(const LaunchCache&) = delete;
     LaunchCache& operator=(const LaunchCache&) = delete;
     cudaError_t launch(const void* recording, cudaStream_t stream);
+    void build(const void* recording);               // a graph of these kernels, if there is none; nothing is launched
 
 private:
     // (A context's calls make some 40 different runs of kernels, over all sizes of mini-batches; a program that had more than
@@ -177,7 +180,9 @@ private:
     struct Entry;
     struct List;
     List* list_of(const void* recording);
+    bool launch_kept(const void* recording, cudaStream_t stream, int* changed, cudaError_t* result);
     List* lists_ = nullptr;
+    LaunchCache* const common_;
     std::mutex mutex_;
     const int variants_;
     uint64_t tick_ = 0;
@@ -186,7 +191,8 @@ private:
 
 class LaunchBatch {
 public:
-    explicit LaunchBatch(LaunchCache* cache);        // nullptr, or inside another batch: nothing of its own
+    // cache: nullptr, or inside another batch: nothing of its own.  build_only: the kernels get graphs and are not launched
+    explicit LaunchBatch(LaunchCache* cache, bool build_only = false);
     ~LaunchBatch();
     int32_t end(int32_t st = HL_OK);                 // `st`, or HL_ECUDA if that is HL_OK and a launch failed
 
@@ -195,6 +201,7 @@ private:
 };
 
 cudaError_t launch_flush();
+bool launches_build_only();
 cudaError_t clear_words(uint32_t* p, int64_t n_words, cudaStream_t stream);      // p[0 .. n_words) = 0
 cudaError_t launch_kernel(const void* func, dim3 grid, dim3 block, size_t smem, int cluster, void** args,
                           const uint32_t* sizes, int n_args, cudaStream_t stream);

@@ -181,7 +181,8 @@ struct LaunchCache::List {
     }
 };
 
-LaunchCache::LaunchCache(int variants) : variants_(variants < kMaxVariants ? variants : kMaxVariants) {}
+LaunchCache::LaunchCache(int variants, LaunchCache* common)
+    : common_(common), variants_(variants < kMaxVariants ? variants : kMaxVariants) {}
 LaunchCache::~LaunchCache() {
     while (lists_) {
         List* l = lists_;
@@ -232,6 +233,7 @@ cudaError_t launch_one_by_one(Recording& r, cudaStream_t stream) {
 // what the calling thread is collecting
 struct Collecting {
     LaunchCache* cache = nullptr;
+    bool build_only = false;
     cudaStream_t stream = nullptr;
     cudaError_t failed = cudaSuccess;
     Recording rec;
@@ -246,7 +248,8 @@ thread_local Collecting t_now;
 // Building a graph costs as much as some 30 plain launches, in the call that does it.  So none is built before the plain
 // launches of this cache (and, for one more graph of kernels that have one, the arguments changed) have cost that much more
 // than graphs would have: a program that makes a call a few times never pays for a graph, one that makes it for ever pays for
-// plain launches twice at most, and graphs come one at a time, however many runs of kernels a call makes.
+// plain launches twice at most, and graphs come one at a time, however many runs of kernels a call makes.  (A cache with a
+// common one behind it launches with that one's graphs meanwhile, and what counts is what changing their arguments costs.)
 cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
     Recording& r = *const_cast<Recording*>(static_cast<const Recording*>(recording));
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -285,16 +288,56 @@ cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
         }
         if (l->graphs < variants_) lost = kUpdateNs * changed;
     }
-    if (!e) lost = (kPlainNs - kUpdateNs) * r.n - kGraphNs;
+    int changed = 0;
+    cudaError_t result = cudaSuccess;
+    const bool by_common = !e && common_ && common_->launch_kept(recording, stream, &changed, &result);
+    if (!e) lost = by_common ? kUpdateNs * changed : (kPlainNs - kUpdateNs) * r.n - kGraphNs;
     lost_ns_ = lost_ns_ + lost < kBuildNs ? lost_ns_ + lost : kBuildNs;
+    if (by_common) return result;
     if (!e) return launch_one_by_one(r, stream);
     e->used = ++tick_;
     return cudaGraphLaunch(e->exec, stream);
 }
 
+// with a graph that is here, its arguments brought up to date; false: there is none
+bool LaunchCache::launch_kept(const void* recording, cudaStream_t stream, int* changed, cudaError_t* result) {
+    const Recording& r = *static_cast<const Recording*>(recording);
+    std::lock_guard<std::mutex> lock(mutex_);
+    for (List* l = lists_; l; l = l->next) {
+        if (!l->has(r) || l->graphs == 0) continue;
+        Entry* e = l->graph[0];
+        if (e->update(r, changed) != cudaSuccess) {
+            l->drop(e);
+            cudaGetLastError();
+            return false;
+        }
+        *result = cudaGraphLaunch(e->exec, stream);
+        return true;
+    }
+    return false;
+}
+
+void LaunchCache::build(const void* recording) {
+    std::lock_guard<std::mutex> lock(mutex_);
+    List* l = list_of(recording);
+    if (!l || l->graphs) return;
+    Entry* e = new (std::nothrow) Entry();
+    if (e && e->build(*static_cast<const Recording*>(recording)) == cudaSuccess) {
+        l->graph[l->graphs++] = e;
+    } else {
+        delete e;
+        cudaGetLastError();
+    }
+}
+
 cudaError_t launch_flush() {
     Collecting& c = t_now;
     if (!c.cache || c.rec.n == 0) return cudaSuccess;
+    if (c.build_only) {
+        c.cache->build(&c.rec);
+        c.rec.clear();
+        return cudaSuccess;
+    }
     const cudaError_t e = c.cache->launch(&c.rec, c.stream);
     c.rec.clear();
     if (e != cudaSuccess && c.failed == cudaSuccess) c.failed = e;
@@ -312,9 +355,11 @@ cudaError_t launch_kernel(const void* func, dim3 grid, dim3 block, size_t smem, 
     if (c.rec.add(func, grid, block, smem, cluster, args, sizes, n_args)) return cudaSuccess;
     const cudaError_t e = launch_flush();
     if (e != cudaSuccess) return e;
-    if (c.rec.add(func, grid, block, smem, cluster, args, sizes, n_args)) return cudaSuccess;
+    if (c.rec.add(func, grid, block, smem, cluster, args, sizes, n_args) || c.build_only) return cudaSuccess;
     return launch_now(func, grid, block, smem, cluster, args, stream);
 }
+
+bool launches_build_only() { return t_now.cache && t_now.build_only; }
 
 namespace {
 __global__ void __launch_bounds__(256) k_clear_words(uint32_t* p, int64_t n) {
@@ -329,9 +374,10 @@ cudaError_t clear_words(uint32_t* p, int64_t n_words, cudaStream_t stream) {
     return launch(k_clear_words, grid_for(n_words, 256, 296), 256, stream, p, n_words);
 }
 
-LaunchBatch::LaunchBatch(LaunchCache* cache) : mine_(cache != nullptr && t_now.cache == nullptr) {
+LaunchBatch::LaunchBatch(LaunchCache* cache, bool build_only) : mine_(cache != nullptr && t_now.cache == nullptr) {
     if (!mine_) return;
     t_now.cache = cache;
+    t_now.build_only = build_only;
     t_now.stream = nullptr;
     t_now.failed = cudaSuccess;
     t_now.rec.clear();

@@ -1,6 +1,6 @@
-// Device-wide primitives used by several steps: single-pass exclusive scan and stable LSD radix sort of pairs
+// Device-wide primitive used by several steps: stable LSD radix sort of pairs
 // (few pairs: one kernel of one cluster; many: one kernel per digit, tiles chained through status words).
-// Both take their element count from device memory, so that no step has to synchronise the host.
+// It takes its element count from device memory, so that no step has to synchronise the host.
 #include <cooperative_groups.h>
 
 #include <atomic>
@@ -10,7 +10,9 @@
 namespace hl {
 
 static std::atomic<unsigned long long> g_launches{0};
-void note_launches(int n) { g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed); }
+void note_launches(int n) {
+    if (!launches_build_only()) g_launches.fetch_add((unsigned long long)n, std::memory_order_relaxed);
+}
 unsigned long long launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 
 namespace {

@@ -179,8 +179,9 @@ def test_many_runs_of_kernels_with_many_argument_sets_all_become_graphs(B, lib):
 
 
 def test_graphs_are_built_when_plain_launches_have_cost_as_much(B, lib):
-    """A graph costs as much as some 30 plain launches: the first repeats of a call pay for none, and a new pipeline's
-    mini-batches, of seven runs of kernels in each of four slots, pay for one now and then, never for several at once."""
+    """A graph costs as much as some 30 plain launches: the first repeats of a call pay for none.  A pipeline builds one for
+    each of its seven runs of kernels before its first mini-batch, launches them for every slot, and gives a slot graphs of
+    its own as the changed arguments add up, never several at once."""
     c = _Context(B)
     s, tags, rrpv, hits = c.mem(), c.mem(), c.mem(), c.mem()
     for k in range(5):
@@ -190,9 +191,16 @@ def test_graphs_are_built_when_plain_launches_have_cost_as_much(B, lib):
         B.hl_tracker_update(c.ctx, c.inputs(), tags, rrpv, 64, 16, hits, s)
     assert lib.fake_calls(b"cudaGraphInstantiate") >= 1
     c.close()
-    lib.fake_reset()
-    log, marks = _pipe_run(B, lib, 40)
-    assert lib.fake_calls(b"cudaGraphInstantiate") <= len([x for x in log if x.startswith("plain")]) / 30
+    for order, runs in ((0, 6), (1, 5)):                 # (the sort of 32 K lookups and more is a run of its own)
+        for batch, more in ((64, 0), (16384, 1)):
+            lib.fake_reset()
+            log, marks = _pipe_run(B, lib, 0, batch=batch, order=order)
+            assert lib.fake_calls(b"cudaGraphInstantiate") == runs + 2 * more
+            lib.fake_reset()
+            log, marks = _pipe_run(B, lib, 60, batch=batch, order=order)
+            assert lib.fake_calls(b"cudaGraphInstantiate") <= runs + 2 * more + 60 * 25 * 280 / 75000
+            # (the first two mini-batches have nothing to forward, and no sort before them to wait for)
+            assert len([x for x in log[marks[2]:] if x.startswith("plain")]) <= 2
 
 
 def test_a_graph_that_cannot_be_changed_or_built_gives_way_to_plain_launches(B, lib):
@@ -259,6 +267,7 @@ def test_marks_left_by_a_call_that_failed_are_cleared_before_the_next_ones(B, li
     """Cold rows are marked in the bitmap by one kernel and ranked (and the marks cleared) by another.  The launch of the
     second one fails: the call says so, and the next call on the context first clears the bitmap; the one after that
     does not."""
+    lib.fake_fail(b"cudaGraphInstantiate", -1)               # (kernel by kernel)
     c = _Context(B)
     s, side, st, b = c.mem(), c.mem(), c.one_set(), c.inputs()
     pipe = None
@@ -311,6 +320,7 @@ def test_marks_left_by_a_call_that_failed_are_cleared_before_the_next_ones(B, li
 def test_runs_listed_by_a_call_that_failed_are_taken_off_the_list(B, lib, which):
     """The sum kernel lists the runs that the span kernel finishes.  The span kernel's launch fails: the call says so, and
     the next update on the context starts with an empty list; the one after that clears nothing."""
+    lib.fake_fail(b"cudaGraphInstantiate", -1)               # (kernel by kernel)
     c = _Context(B)
     s, side, st, b, grad = c.mem(), c.mem(), c.one_set(), c.inputs(), c.mem()
     step_buffers = B.make_step_buffers(st["perm"], st["counts"], st["pop"], st["non"], None, st["cold_rows"], st["n_cold"],
