@@ -583,7 +583,7 @@ class PipelinedHotline(Hotline):
 
 
 class NativePipelinedHotline(Hotline):
-    """The default schedule of :class:`PipelinedHotline` (index work ``lookahead`` mini-batches ahead on three
+    """The default schedule of :class:`PipelinedHotline` (index work ``lookahead`` mini-batches ahead on two
     streams, one combined backward sort, host reads overlapping write-backs, shared rows forwarded), issued by the
     library itself (hl_pipe_*): one C call per mini-batch instead of some sixty Python-level calls, which is what
     bounds small mini-batches.  Same results, same buffers (``sets``), same call pattern:

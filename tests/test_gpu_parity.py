@@ -42,10 +42,9 @@ def test_arbitrary_hot_sets(hot):
 
 
 @pytest.mark.parametrize("batch", [2559, 2560, 2561, 3000, 5119, 5120, 5121, 6000])
-def test_cold_row_search_at_the_limit_of_its_one_cluster_path(batch):
-    """Empty hot set, 8 tables: every lookup is cold, 8 * batch of them.  The one-cluster kernel takes at most 40 960
-    (a cluster of 16 CTAs; 20 480 where the device places only 8); one more and the general path (tile sort, head
-    flags, scan, assignment), launched from the device, does the work."""
+def test_cold_row_search_with_every_lookup_cold(batch):
+    """Empty hot set, 8 tables: every lookup is cold, 8 * batch of them, on both sides of the 32 768 pairs up to which
+    the backward's sort is one cluster's."""
     spec = dataclasses.replace(gen.CONFIGS["tiny"], batch=batch, hot_policy=("topk", 80_000))
     stats = run_config_check(spec, steps=2, hot_override="empty", integer=True)
     assert stats["n_pop"] == 0 and stats["n_cold"] > 5_000        # distinct rows; the lookups are 8 * batch
@@ -177,16 +176,14 @@ def test_native_pipeline_equals_sequential_steps_integer_data():
     run_pipelined_check(spec, steps=4, integer=True, native=True)
 
 
-def test_native_pipeline_queues_the_same_launches_whichever_cold_row_search_runs():
-    """The host queues the same kernels for every mini-batch: when a mini-batch has more cold lookups than the
-    one-cluster kernel takes, that kernel launches the general search (tile sort, head flags, scan, assignment) from
-    the device.  Same results either way, and the host-side launch count does not depend on the data or on whether the
-    host waits between steps."""
+def test_native_pipeline_queues_the_same_launches_whatever_the_data():
+    """The host queues the same kernels for every mini-batch, however many cold lookups it has: the launch count does not
+    depend on the data, nor on whether the host waits between steps."""
     kw = dict(steps=6, scale_rows=0.02, integer=True, profile_batches=6, native=True)
     few = run_pipelined_check("dlrm_small", drain_between=True, **kw)      # a few thousand cold lookups per mini-batch
     spec = dataclasses.replace(gen.CONFIGS["multi_hot"], batch=2048, dim=32, rows=("fixed", 20000),
                                hot_policy=("fraction", 10, 100), profile_batches=2)
-    a = run_pipelined_check(spec, steps=4, integer=True, native=True)      # tens of thousands: the general search
+    a = run_pipelined_check(spec, steps=4, integer=True, native=True)      # tens of thousands
     b = run_pipelined_check(spec, steps=4, integer=True, native=True, drain_between=True)
     assert a["launches"] == b["launches"] and few["launches"] > 0
 
