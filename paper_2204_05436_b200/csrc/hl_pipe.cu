@@ -33,10 +33,9 @@ struct hl_pipe {
         cudaEvent_t inputs, pairs, index, gather, forward, x, scatter;
     };
     std::vector<Events> ev;
-    // one graph of every run of kernels, built before the first mini-batch is queued
-    std::unique_ptr<hl::LaunchCache> first_graphs;
     // the graphs of mini-batch j's kernels: slot j % slots, so that set and window, and with them nearly all arguments, are
-    // the same whenever a slot is used
+    // the same whenever a slot is used.  The first slot's are there before the first mini-batch is queued (build_graphs), and
+    // the other slots launch with them, the arguments changed, until graphs of their own are worth their price.
     std::vector<std::unique_ptr<hl::LaunchCache>> launches;
     // mini-batches whose index work is queued (indexed), whose host read is queued (submitted), whose main work is queued
     // (done)
@@ -129,7 +128,7 @@ hl::LaunchCache* launches_of(hl_pipe* p, int64_t j) {
 void build_graphs(hl_pipe* p, const hl_batch* b, const float* d_dense) {
     hl_ctx* ctx = p->ctx;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
-    if (!p->first_graphs || p->trace_mask || ctx->max_nnz == 0 || ctx->timing_on || ctx->mark_hook || ctx->marks_suspect ||
+    if (p->trace_mask || ctx->max_nnz == 0 || ctx->timing_on || ctx->mark_hook || ctx->marks_suspect ||
         ctx->spans_suspect)
         return;
     if (cudaStreamIsCapturing(p->main, &capturing) != cudaSuccess || capturing != cudaStreamCaptureStatusNone) {
@@ -143,7 +142,7 @@ void build_graphs(hl_pipe* p, const hl_batch* b, const float* d_dense) {
     const SortAside aside{p->sort, p->ev[0].pairs, 0};
     const SortAside* use = n_clear > 0 ? &aside : nullptr;
     const float* any = st.pooled_pop;                        // (some gradients)
-    LaunchBatch batch(p->first_graphs.get(), true);
+    LaunchBatch batch(p->launches[0].get(), true);
     if (fragment_and_mark(ctx, b, d_dense, d_dense ? p->n_dense : 0, st.perm, st.counts, &st.pop, &st.non,
                           d_dense ? st.dense_out : nullptr, p->index) != HL_OK)
         return;                                              // (the call itself will say so)
@@ -388,9 +387,8 @@ extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_t
                        cudaSuccess;
     }
     p->launches.resize(n_sets % 2 ? 2 * n_sets : n_sets);
-    p->first_graphs.reset(new (std::nothrow) LaunchCache(1));
     for (auto& l : p->launches) {
-        l.reset(new (std::nothrow) LaunchCache(1, p->first_graphs.get()));
+        l.reset(new (std::nothrow) LaunchCache(1, p->launches[0].get()));
         ok = ok && l;
     }
     p->ev.resize(n_sets);
