@@ -538,7 +538,7 @@ int32_t gather_impl(hl_ctx* ctx, hl_ubatch* non, const int32_t* d_n_non, const f
                     cudaEvent_t record_after_index, cudaEvent_t wait_a, cudaEvent_t wait_b, bool do_index,
                     bool do_move, cudaStream_t stream) {
     Regions& r = ctx->r;
-    LaunchBatch batch(ctx->launches);
+    LaunchBatch batch(kept_launches(ctx));
     if (!do_index) {
         if (ctx->max_nnz == 0) return HL_OK;
         timer_mark(ctx, HL_TIMER_GATHER_MOVE, 0, stream);
@@ -615,7 +615,7 @@ extern "C" int32_t hl_index_cold_begin(hl_ctx* ctx, hl_ubatch* non, const int32_
                                        int64_t stage_rows, int32_t* d_cold_rows, int64_t* d_n_cold, void* stream_) {
     if (!ctx || !non || !non->offsets || !d_n_non || !d_cold_rows || !d_n_cold) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
-    LaunchBatch batch(ctx->launches);
+    LaunchBatch batch(kept_launches(ctx));
     return scratch_kept(ctx, batch.end(index_begin(ctx, non, d_n_non, stage_row0, stage_rows, d_cold_rows, d_n_cold,
                                                  static_cast<cudaStream_t>(stream_))));
 }
@@ -674,7 +674,7 @@ static int32_t scatter_call(hl_ctx* ctx, const float* d_cache, int64_t stage_row
     if (!ctx || !d_cache || !d_cold_rows || !d_n_cold || !host_table) return HL_EINVAL;
     if (!window_ok(ctx, stage_row0, stage_rows)) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    LaunchBatch batch(ctx->launches);
+    LaunchBatch batch(kept_launches(ctx));
     timer_mark(ctx, HL_TIMER_SCATTER_MOVE, 0, stream);
     const int32_t st = launch_move_rows<true>(const_cast<float*>(d_cache), ctx->hot_cap + stage_row0,
                                               table_map(ctx, host_table),

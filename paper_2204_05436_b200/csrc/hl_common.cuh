@@ -234,6 +234,10 @@ int32_t as_graph(LaunchCache* cache, F f) {
     return batch.end(f());
 }
 
+// Where a call of this context keeps its graphs.  (A call whose kernels are traced launches them one by one, as its spans
+// show them, and does not pay for a graph inside a span.)
+inline LaunchCache* kept_launches(const hl_ctx* ctx) { return ctx && !ctx->mark_hook ? ctx->launches : nullptr; }
+
 // Records the start/end event of one of the optional kernel timers on `stream` (no-op unless enabled).
 inline void timer_mark(hl_ctx* ctx, int which, int end, cudaStream_t stream) {
     if (!ctx->timing_on && !ctx->mark_hook) return;

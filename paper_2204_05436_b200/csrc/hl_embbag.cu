@@ -896,7 +896,7 @@ int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, c
 
 extern "C" int32_t hl_embbag_fwd(hl_ctx* ctx, const float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples,
                                  float* d_out, void* stream) {
-    return as_graph(ctx ? ctx->launches : nullptr, [&] {
+    return as_graph(kept_launches(ctx), [&] {
         return fwd_call(ctx, d_cache, ub, d_n_samples, d_out, nullptr, static_cast<cudaStream_t>(stream));
     });
 }
@@ -983,7 +983,7 @@ extern "C" int32_t hl_embbag_bwd_sgd(hl_ctx* ctx, float* d_cache, const hl_ubatc
     if (ctx->max_nnz == 0) return HL_OK;
     if (!ub->ids) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    return scratch_kept(ctx, as_graph(ctx->launches, [&]() -> int32_t {
+    return scratch_kept(ctx, as_graph(kept_launches(ctx), [&]() -> int32_t {
         int32_t *keys, *vals;
         const int32_t st = sort_lookups(ctx, ub, d_n_samples, nullptr, nullptr, ctx->r.bwd_n, &keys, &vals, stream);
         if (st != HL_OK) return st;
@@ -1003,7 +1003,7 @@ extern "C" int32_t hl_embbag_bwd_prepare(hl_ctx* ctx, const hl_ubatch* ub, const
         return HL_OK;
     }
     if (!ub->ids || !d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
-    return as_graph(ctx->launches, [&] {
+    return as_graph(kept_launches(ctx), [&] {
         int32_t *keys, *vals;
         return sort_lookups(ctx, ub, d_n_samples, d_sorted_slots, d_sorted_bags, d_n_lookups, &keys, &vals, stream);
     });
@@ -1033,7 +1033,7 @@ int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, 
     a.bags_follow = merge;
     a.side[0] = {pop->ids, pop->offsets, d_n_pop, 0};
     a.side[1] = {non->ids, non->offsets, d_n_non, merge ? 0 : (int32_t)(n_slots + 1)};
-    return as_graph(ctx->launches, [&] {
+    return as_graph(kept_launches(ctx), [&] {
         int32_t *ok, *ov;
         return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, cleared, d_sorted_slots, d_sorted_bags,
                               d_n_lookups, out_slots ? out_slots : &ok, out_bags ? out_bags : &ov, stream, aside);
@@ -1092,7 +1092,7 @@ extern "C" int32_t hl_embbag_bwd_apply2(hl_ctx* ctx, float* d_cache, const int32
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
     const int32_t* d_first = which == 0 ? nullptr : d_n_lookups;             // X's block starts behind O's
     const int32_t bias = which == 0 ? 0 : (int32_t)(ctx->hot_cap + ctx->staging_cap + 1);
-    return scratch_kept(ctx, as_graph(ctx->launches, [&]() -> int32_t {
+    return scratch_kept(ctx, as_graph(kept_launches(ctx), [&]() -> int32_t {
 #define HL_BWD(G, NV) \
     launch_bwd<G, NV>(ctx, d_cache, d_sorted_slots, d_sorted_bags, d_n_lookups + which, d_grad_out, lr, stream, d_first, bias)
         HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
@@ -1107,7 +1107,7 @@ extern "C" int32_t hl_embbag_bwd_apply(hl_ctx* ctx, float* d_cache, const int32_
     if (ctx->max_nnz == 0) return HL_OK;
     if (!d_sorted_slots || !d_sorted_bags) return HL_EINVAL;
     cudaStream_t stream = static_cast<cudaStream_t>(stream_);
-    return scratch_kept(ctx, as_graph(ctx->launches, [&]() -> int32_t {
+    return scratch_kept(ctx, as_graph(kept_launches(ctx), [&]() -> int32_t {
 #define HL_BWD(G, NV) launch_bwd<G, NV>(ctx, d_cache, d_sorted_slots, d_sorted_bags, d_n_lookups, d_grad_out, lr, stream)
         HL_DISPATCH_ROW_SHAPE(ctx->D / 4, HL_BWD);
 #undef HL_BWD

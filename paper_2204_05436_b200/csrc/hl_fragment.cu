@@ -477,7 +477,7 @@ int32_t fragment_and_mark(hl_ctx* ctx, const hl_batch* b, const float* d_dense, 
 extern "C" int32_t hl_fragment(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t n_dense,
                                int32_t* d_perm, int32_t* d_counts, hl_ubatch* pop, hl_ubatch* non,
                                float* d_dense_out, void* stream) {
-    return as_graph(ctx ? ctx->launches : nullptr, [&] {
+    return as_graph(kept_launches(ctx), [&] {
         return fragment_call(ctx, b, d_dense, n_dense, d_perm, d_counts, pop, non, d_dense_out, false,
                              static_cast<cudaStream_t>(stream));
     });

@@ -98,8 +98,8 @@ class _Context:
         self.B.hl_destroy(self.ctx)
 
 
-def _pipe_run(B, lib, steps, n_sets=4, batch=64, order=0, same_inputs=3):
-    """A pipeline over ``steps`` mini-batches of two sizes; the log of what its steady state queued."""
+def _pipe_run(B, lib, steps, n_sets=4, batch=64, order=0, same_inputs=3, traced_from=None):
+    """A pipeline over ``steps`` mini-batches of two sizes (those from ``traced_from`` on traced); the log of what it queued."""
     c = _Context(B, batch=batch)
     sets = []
     for _ in range(n_sets):
@@ -116,6 +116,8 @@ def _pipe_run(B, lib, steps, n_sets=4, batch=64, order=0, same_inputs=3):
         B.hl_pipe_submit(p, inputs[j % same_inputs], None, "resident" if j % 2 else None)
     for j in range(steps):
         marks.append(lib.fake_lines())
+        if j == traced_from:
+            B.hl_pipe_trace_begin(p, 1000, B.HL_SPAN_ALL)
         gp, gn = grads[j % 3]
         B.hl_pipe_step(p, gp, gn, 0.1 + 0.01 * (j % 5), inputs[(j + n_sets - 2) % same_inputs], None, "resident")
     log = _log(lib)
@@ -260,6 +262,16 @@ def test_a_captured_stream_gets_plain_launches_only(B, lib):
         assert (lib.fake_calls(b"cudaGraphInstantiate"), lib.fake_calls(b"cudaGraphLaunch")) == (built, launched)
     assert launched > 100
     c.close()
+
+
+def test_traced_mini_batches_launch_kernel_by_kernel(B, lib):
+    """The spans of a trace bracket kernels: none of them holds the building of a graph."""
+    lib.fake_reset()
+    log, marks = _pipe_run(B, lib, 400, batch=16384, traced_from=100)
+    untraced, traced = log[marks[90]:marks[100]], log[marks[100]:]
+    assert any(x.startswith("graph") for x in untraced) and not any(x.startswith("graph") for x in traced)
+    kernels = [_name(x) for x in untraced if x[:5] in ("plain", "graph")]
+    assert sorted(kernels) == sorted(_name(x) for x in log[marks[300]:marks[310]] if x.startswith("plain"))
 
 
 @pytest.mark.parametrize("which", ["hl_index_cold", "hl_gather_cold", "hl_index_cold_begin", "hl_step", "hl_pipe_submit"])
