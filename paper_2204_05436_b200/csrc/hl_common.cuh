@@ -164,9 +164,7 @@ namespace hl {
 // stream (an event, a memset).
 class LaunchCache {
 public:
-    // variants: graphs of the same kernels, with different arguments, worth keeping.  common: where there are graphs that a
-    // run of kernels without one here can be launched with (nullptr: kernel by kernel)
-    explicit LaunchCache(int variants, LaunchCache* common = nullptr);
+    explicit LaunchCache(int variants);              // graphs of the same kernels, with different arguments, worth keeping
     ~LaunchCache();
     LaunchCache(const LaunchCache&) = delete;
     LaunchCache& operator=(const LaunchCache&) = delete;
@@ -180,9 +178,7 @@ private:
     struct Entry;
     struct List;
     List* list_of(const void* recording);
-    bool launch_kept(const void* recording, cudaStream_t stream, int* changed, cudaError_t* result);
     List* lists_ = nullptr;
-    LaunchCache* const common_;
     std::mutex mutex_;
     const int variants_;
     uint64_t tick_ = 0;

@@ -181,8 +181,7 @@ struct LaunchCache::List {
     }
 };
 
-LaunchCache::LaunchCache(int variants, LaunchCache* common)
-    : common_(common), variants_(variants < kMaxVariants ? variants : kMaxVariants) {}
+LaunchCache::LaunchCache(int variants) : variants_(variants < kMaxVariants ? variants : kMaxVariants) {}
 LaunchCache::~LaunchCache() {
     while (lists_) {
         List* l = lists_;
@@ -248,8 +247,7 @@ thread_local Collecting t_now;
 // Building a graph costs as much as some 30 plain launches, in the call that does it.  So none is built before the plain
 // launches of this cache (and, for one more graph of kernels that have one, the arguments changed) have cost that much more
 // than graphs would have: a program that makes a call a few times never pays for a graph, one that makes it for ever pays for
-// plain launches twice at most, and graphs come one at a time, however many runs of kernels a call makes.  (A cache with a
-// common one behind it launches with that one's graphs meanwhile, and what counts is what changing their arguments costs.)
+// plain launches twice at most, and graphs come one at a time, however many runs of kernels a call makes.
 cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
     Recording& r = *const_cast<Recording*>(static_cast<const Recording*>(recording));
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
@@ -288,33 +286,11 @@ cudaError_t LaunchCache::launch(const void* recording, cudaStream_t stream) {
         }
         if (l->graphs < variants_) lost = kUpdateNs * changed;
     }
-    int changed = 0;
-    cudaError_t result = cudaSuccess;
-    const bool by_common = !e && common_ && common_->launch_kept(recording, stream, &changed, &result);
-    if (!e) lost = by_common ? kUpdateNs * changed : (kPlainNs - kUpdateNs) * r.n - kGraphNs;
+    if (!e) lost = (kPlainNs - kUpdateNs) * r.n - kGraphNs;
     lost_ns_ = lost_ns_ + lost < kBuildNs ? lost_ns_ + lost : kBuildNs;
-    if (by_common) return result;
     if (!e) return launch_one_by_one(r, stream);
     e->used = ++tick_;
     return cudaGraphLaunch(e->exec, stream);
-}
-
-// with a graph that is here, its arguments brought up to date; false: there is none
-bool LaunchCache::launch_kept(const void* recording, cudaStream_t stream, int* changed, cudaError_t* result) {
-    const Recording& r = *static_cast<const Recording*>(recording);
-    std::lock_guard<std::mutex> lock(mutex_);
-    for (List* l = lists_; l; l = l->next) {
-        if (!l->has(r) || l->graphs == 0) continue;
-        Entry* e = l->graph[0];
-        if (e->update(r, changed) != cudaSuccess) {
-            l->drop(e);
-            cudaGetLastError();
-            return false;
-        }
-        *result = cudaGraphLaunch(e->exec, stream);
-        return true;
-    }
-    return false;
 }
 
 void LaunchCache::build(const void* recording) {

@@ -34,8 +34,7 @@ struct hl_pipe {
     };
     std::vector<Events> ev;
     // the graphs of mini-batch j's kernels: slot j % slots, so that set and window, and with them nearly all arguments, are
-    // the same whenever a slot is used.  The first slot's are there before the first mini-batch is queued (build_graphs), and
-    // the other slots launch with them, the arguments changed, until graphs of their own are worth their price.
+    // the same whenever a slot is used.  They are there before the first mini-batch is queued (build_graphs).
     std::vector<std::unique_ptr<hl::LaunchCache>> launches;
     // mini-batches whose index work is queued (indexed), whose host read is queued (submitted), whose main work is queued
     // (done)
@@ -122,10 +121,11 @@ hl::LaunchCache* launches_of(hl_pipe* p, int64_t j) {
     return p->trace_mask ? nullptr : p->launches[j % p->launches.size()].get();
 }
 
-// Before the first mini-batch is queued: a graph of every run of kernels that a mini-batch like this one makes, so that no
-// mini-batch has to launch them one by one (some 40 launches' worth of host time each until every slot has graphs of its own)
-// or to wait while one is built.  Nothing is launched.  The runs are those of queue_index and queue_mini_batch.
-void build_graphs(hl_pipe* p, const hl_batch* b, const float* d_dense) {
+// Before the first mini-batch is queued: a graph of every run of kernels that a mini-batch like this one makes in slot j, so
+// that no mini-batch has to launch them one by one or to wait while one is built (some 2 ms for the seven runs of four slots;
+// built when a slot's mini-batch came, they made mini-batches three to eight 200 to 600 us each).  Nothing is launched.  The
+// runs are those of queue_index and queue_mini_batch.
+void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense) {
     hl_ctx* ctx = p->ctx;
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (p->trace_mask || ctx->max_nnz == 0 || ctx->timing_on || ctx->mark_hook || ctx->marks_suspect ||
@@ -135,31 +135,34 @@ void build_graphs(hl_pipe* p, const hl_batch* b, const float* d_dense) {
         cudaGetLastError();
         return;
     }
-    hl_pipe_set &st = p->sets[0], &prev = p->sets[1];
-    const int64_t w = p->window_rows;
+    const int n = p->n_sets;
+    hl_pipe_set &st = p->sets[j % n], &prev = p->sets[(j + n - 1) % n];
+    const int64_t rows = p->window_rows, w = (j % 2) * rows, w_other = rows - w;
     const bool merge = p->order == HL_PIPE_ORDER_EQ5;
     const int64_t n_clear = backward_sort_clear_words(ctx, merge);
-    const SortAside aside{p->sort, p->ev[0].pairs, 0};
+    const SortAside aside{p->sort, p->ev[j % n].pairs, (int)(j % 2)};
     const SortAside* use = n_clear > 0 ? &aside : nullptr;
     const float* any = st.pooled_pop;                        // (some gradients)
-    LaunchBatch batch(p->launches[0].get(), true);
+    LaunchBatch batch(p->launches[j].get(), true);
     if (fragment_and_mark(ctx, b, d_dense, d_dense ? p->n_dense : 0, st.perm, st.counts, &st.pop, &st.non,
                           d_dense ? st.dense_out : nullptr, p->index) != HL_OK)
         return;                                              // (the call itself will say so)
     if (use) launch_flush();
-    (void)cold_rank(ctx, w, st.cold_rows, st.n_cold, p->index, ctx->r.bwd_hist[0], n_clear);
-    (void)assign_and_prepare(ctx, &st.pop, st.counts, &st.non, st.counts + 1, 0, w, st.cold_rows, st.n_cold, prev.cold_rows,
+    (void)cold_rank(ctx, rows, st.cold_rows, st.n_cold, p->index, ctx->r.bwd_hist[use ? j % 2 : 0], n_clear);
+    (void)assign_and_prepare(ctx, &st.pop, st.counts, &st.non, st.counts + 1, w, rows, st.cold_rows, st.n_cold, prev.cold_rows,
                              prev.n_cold, st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, p->index, use);
-    (void)hl_stage_cold(ctx, p->host_table, p->cache, 0, w, st.cold_rows, st.n_cold, st.fwd_src, p->link);
+    (void)hl_stage_cold(ctx, p->host_table, p->cache, w, rows, st.cold_rows, st.n_cold, st.fwd_src, p->link);
     launch_flush();
-    if (w > 0)
-        (void)fwd_and_forward_cold(ctx, p->cache, &st.pop, st.counts, st.pooled_pop, w, 0, w, st.fwd_src, st.n_cold, p->main);
+    if (rows > 0)
+        (void)fwd_and_forward_cold(ctx, p->cache, &st.pop, st.counts, st.pooled_pop, w_other, w, rows, st.fwd_src, st.n_cold,
+                                   p->main);
     launch_flush();
     if (!merge) (void)hl_embbag_bwd_apply2(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 0, any, 0.f, p->main);
     launch_flush();
     (void)hl_embbag_fwd(ctx, p->cache, &st.non, st.counts + 1, st.pooled_non, p->main);
-    (void)hl_embbag_bwd_apply2(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 1, any, 0.f, p->main);
-    (void)hl_scatter_cold_at(ctx, p->cache, 0, w, st.cold_rows, st.n_cold, p->host_table, p->wb);
+    if (!merge) (void)hl_embbag_bwd_apply2(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 1, any, 0.f, p->main);
+    else (void)hl_embbag_bwd_apply(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n + 2, any, 0.f, p->main);
+    (void)hl_scatter_cold_at(ctx, p->cache, w, rows, st.cold_rows, st.n_cold, p->host_table, p->wb);
 }
 
 // The index-only work of the next mini-batch (nothing here touches a row).
@@ -215,7 +218,8 @@ int32_t queue_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* i
 }
 
 int32_t submit_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* inputs_ready) {
-    if (p->j_indexed == 0) build_graphs(p, b, d_dense);
+    if (p->j_indexed == 0)
+        for (size_t j = 0; j < p->launches.size(); ++j) build_graphs(p, (int64_t)j, b, d_dense);
     return scratch_kept(p->ctx, queue_index(p, b, d_dense, inputs_ready));
 }
 
@@ -388,7 +392,7 @@ extern "C" hl_pipe* hl_pipe_create_ex(hl_ctx* ctx, float* d_cache, float* host_t
     }
     p->launches.resize(n_sets % 2 ? 2 * n_sets : n_sets);
     for (auto& l : p->launches) {
-        l.reset(new (std::nothrow) LaunchCache(1, p->launches[0].get()));
+        l.reset(new (std::nothrow) LaunchCache(1));
         ok = ok && l;
     }
     p->ev.resize(n_sets);

@@ -181,9 +181,8 @@ def test_many_runs_of_kernels_with_many_argument_sets_all_become_graphs(B, lib):
 
 
 def test_graphs_are_built_when_plain_launches_have_cost_as_much(B, lib):
-    """A graph costs as much as some 30 plain launches: the first repeats of a call pay for none.  A pipeline builds one for
-    each of its seven runs of kernels before its first mini-batch, launches them for every slot, and gives a slot graphs of
-    its own as the changed arguments add up, never several at once."""
+    """A graph costs as much as some 30 plain launches: the first repeats of a call pay for none.  A pipeline builds those of
+    all its slots before its first mini-batch, and none later."""
     c = _Context(B)
     s, tags, rrpv, hits = c.mem(), c.mem(), c.mem(), c.mem()
     for k in range(5):
@@ -195,14 +194,16 @@ def test_graphs_are_built_when_plain_launches_have_cost_as_much(B, lib):
     c.close()
     for order, runs in ((0, 6), (1, 5)):                 # (the sort of 32 K lookups and more is a run of its own)
         for batch, more in ((64, 0), (16384, 1)):
-            lib.fake_reset()
-            log, marks = _pipe_run(B, lib, 0, batch=batch, order=order)
-            assert lib.fake_calls(b"cudaGraphInstantiate") == runs + 2 * more
-            lib.fake_reset()
-            log, marks = _pipe_run(B, lib, 60, batch=batch, order=order)
-            assert lib.fake_calls(b"cudaGraphInstantiate") <= runs + 2 * more + 60 * 25 * 280 / 75000
-            # (the first two mini-batches have nothing to forward, and no sort before them to wait for)
-            assert len([x for x in log[marks[2]:] if x.startswith("plain")]) <= 2
+            for n_sets, slots in ((4, 4), (3, 6)):
+                lib.fake_reset()
+                log, marks = _pipe_run(B, lib, 0, n_sets, batch, order)
+                built = lib.fake_calls(b"cudaGraphInstantiate")
+                assert built == slots * (runs + 2 * more)
+                lib.fake_reset()
+                log, marks = _pipe_run(B, lib, 60, n_sets, batch, order)
+                # (the first two mini-batches have nothing to forward, and no sort before them to wait for)
+                assert lib.fake_calls(b"cudaGraphInstantiate") == built
+                assert len([x for x in log[marks[2]:] if x.startswith("plain")]) <= 2
 
 
 def test_a_graph_that_cannot_be_changed_or_built_gives_way_to_plain_launches(B, lib):
