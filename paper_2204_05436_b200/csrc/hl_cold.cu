@@ -262,9 +262,20 @@ constexpr int64_t kPacedMost = 1 << 16;
 // turn on one chip, which no program runs, lose 1 to 4 % with 24: 12.4 K rows of 256 bytes 175 / 181.)
 constexpr int64_t kPacedFewRows = 10240;
 
+// A transfer with nothing else on the chip (the popular rows, out and in) has 32 CTAs, which put 3 to 8 thousand requests on
+// the way; rows from 256 bytes on are read with two CTAs per multiprocessor.  More requests than that do not make the link
+// faster, and rows that are asked for far apart from one another miss more of what translates and holds their neighbours
+// (the rows of a transfer are in ascending order).  330 K rows, 2 GiB table, two CTAs per multiprocessor / 32 CTAs, us: rows of
+// 64 bytes read 732 / 610, written 759 / 624; 144 bytes (300 K) 1 822 / 1 685, 1 944 / 1 445; 192 bytes (250 K) 1 053 / 1 027,
+// 1 103 / 1 040; 256 bytes (200 K) 1 016 / 1 013, 1 065 / 1 062.  40 GiB table: 64 bytes 1 233 / 1 076, 1 224 / 1 125; 256 bytes
+// 1 664 / 1 814, 1 906 / 1 870; 512 bytes (200 K) 2 008 / 2 240, 2 116 / 2 098.
+constexpr int kAloneCtas = 32;
+constexpr int kAloneWideRow = 256;
+
 // What a launch of the mover needs to know about its context.
 struct MoveCfg {
     int sms;            // multiprocessors of the device: the launch has at most 2 CTAs per SM
+    bool alone;         // nothing else on the chip
     int min_ctas;       // CTAs that work however few rows there are (at full rate)
     int paced_ctas;     // CTAs of a paced transfer of up to kPacedFewRows rows; 0: never paced
     int paced_more;     // ... of more rows
@@ -393,7 +404,8 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
     const int row_bytes = D * 4;
     if (row_bytes <= kBulkStageBytes) {
         const int rows_per_stage = kBulkStageBytes / row_bytes < kBulkThreads ? kBulkStageBytes / row_bytes : kBulkThreads;
-        const int grid = grid_for(n_max, rows_per_stage, 2 * cfg.sms);
+        const bool few = cfg.alone && (TO_TABLE || row_bytes < kAloneWideRow);
+        const int grid = grid_for(n_max, rows_per_stage, few ? kAloneCtas : 2 * cfg.sms);
         const int requests = (row_bytes + 127) / 128;        // of one row
         const int paced_fit = TO_TABLE ? kPacedRequests / requests : kPacedReadBytes / row_bytes;
         const int paced_rows = paced_fit > 1 ? paced_fit : 1;
@@ -468,10 +480,11 @@ static TableMap table_map(const hl_ctx* ctx, const float* host_table) {
 }
 
 // how the movers of this context are launched: beside the kernels of other mini-batches (`width` = the context's setting),
-// or alone on the chip (`width` = 0: two CTAs per SM, the link's full rate)
+// or alone on the chip (`width` = 0: the link's full rate)
 static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false, bool reads = false) {
     MoveCfg c;
     c.sms = ctx_sms(ctx);
+    c.alone = width == 0;
     c.min_ctas = width > 0 ? width : 2 * c.sms;
     c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : kPacedCtas) : 0;
     c.paced_more = in_schedule && reads && !ctx->mover_width_set ? kReadCtasDefault : c.paced_ctas;
@@ -482,7 +495,7 @@ static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false, 
 
 int32_t launch_gather_rows(hl_ctx* ctx, float* dst, int64_t dst_row0, const float* table, const int32_t* rows,
                            const int64_t* d_n, int64_t n_max, int32_t* status, cudaStream_t stream) {
-    // loading the hot cache happens with nothing else on the chip: two mover CTAs per SM, for the link's full rate
+    // loading the hot cache happens with nothing else on the chip
     return launch_move_rows<false>(dst, dst_row0, table_map(ctx, table), rows, d_n, n_max, ctx->N, ctx->D, nullptr,
                                    move_cfg(ctx, 0), status, stream);
 }
@@ -700,7 +713,7 @@ extern "C" int32_t hl_scatter_cold(hl_ctx* ctx, const float* d_cache, const int3
 extern "C" int32_t hl_flush_hot(hl_ctx* ctx, const float* d_cache, const int32_t* d_hot_rows, const int64_t* d_n_hot,
                                 float* host_table, void* stream_) {
     if (!ctx || !d_cache || !d_hot_rows || !d_n_hot || !host_table) return HL_EINVAL;
-    // runs between learning phases, with nothing else on the chip: the mover at the link's full rate
+    // runs between learning phases, with nothing else on the chip
     return launch_move_rows<true>(const_cast<float*>(d_cache), 0, table_map(ctx, host_table), d_hot_rows, d_n_hot,
                                   ctx->hot_cap, ctx->N,
                                   ctx->D, nullptr, move_cfg(ctx, 0), ctx->r.status, static_cast<cudaStream_t>(stream_));
