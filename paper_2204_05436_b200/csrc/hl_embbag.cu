@@ -39,6 +39,33 @@ __device__ __forceinline__ int clamp_samples(const int32_t* d_n_samples, int max
 }
 
 // ---- forward ------------------------------------------------------------------------------------------------
+// FORWARD (both kernels): the launch also copies the staged rows that this mini-batch shares with the one before
+// (ForwardRows), which no bag of this launch reads.
+struct ForwardRows {
+    float* cache;
+    int64_t from_row0, to_row0;        // cache[to_row0 + i, :] = cache[from_row0 + src[i], :] where src[i] >= 0
+    const int32_t* src;
+    const int64_t* d_n;
+    int64_t n_max;
+};
+
+__device__ __forceinline__ void forward_rows(const ForwardRows& fr, int D4) {
+    int64_t n = *fr.d_n;
+    n = n < 0 ? 0 : (n < fr.n_max ? n : fr.n_max);
+    const int lane = threadIdx.x & 31;
+    float4* c4 = reinterpret_cast<float4*>(fr.cache);
+    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) - lane; i0 < n;
+         i0 += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t mine = i0 + lane < n ? fr.src[i0 + lane] : -1;
+        for (unsigned m = __ballot_sync(0xffffffffu, mine >= 0 && mine < fr.n_max); m; m &= m - 1) {
+            const int k = __ffs((int)m) - 1;
+            const int64_t from = fr.from_row0 + __shfl_sync(0xffffffffu, mine, k);
+            for (int c = lane; c < D4; c += 32) c4[(fr.to_row0 + i0 + k) * D4 + c] = c4[from * D4 + c];
+        }
+    }
+}
+
+// ---- bags of one lookup, as a rule (contexts of at most 1.5 lookups per bag)
 // A bag of several lookups, finished by one group of G lanes: rows are added in lookup order in fp64, four loads
 // in flight, and the sum is rounded once (so cancellation between the rows of a bag costs no accuracy).
 template <int G, int NV>
@@ -81,118 +108,22 @@ __device__ __forceinline__ void pool_long_bag(const float4* __restrict__ rows, c
     }
 }
 
-// The bags [bag0, bag1), one after the other, by one warp (rows wider than 64 fp32).  A warp reads 32 lookups with one load
-// and checks them with one vote, so that a row costs its load, its additions, a shuffle and an address; and the next 32 (of
-// the next bag, if this one ends) are on their way meanwhile, so that a bag starts without waiting for its ids.  2.6 M
-// lookups of 512-byte rows in bags of 20 on average: 154 us (8.9 TB/s out of the L2, which is what bounds it: neither 6 or 8
-// rows at a time nor a fifth CTA per multiprocessor gains anything, they lose 5-25 %); with every lane reading and
-// checking every id, four at a time and bag by bag (pool_long_bag), 183 us.
-template <int NV>
-__device__ __forceinline__ void pool_bags(const float4* __restrict__ rows, const int32_t* __restrict__ ids,
-                                          const int32_t* __restrict__ offsets, int64_t bag0, int64_t bag1, int lane, int D4,
-                                          int64_t n_slots, float4* __restrict__ out4, int32_t* status) {
-    constexpr int U = NV >= 4 ? 1 : 4 / NV;
-    int col[NV];                                   // (lanes past the row's end read its last column and store nothing)
-#pragma unroll
-    for (int v = 0; v < NV; ++v) col[v] = min(lane + v * 32, D4 - 1);
-    int32_t lo = __ldg(&offsets[bag0]), end = __ldg(&offsets[bag0 + 1]);
-    const int32_t all_end = __ldg(&offsets[bag1]);
-    auto ids_at = [&](int32_t q) { return q + lane < all_end ? __ldg(&ids[q + lane]) : -1; };
-    int32_t mine = ids_at(lo);
-    for (int64_t bag = bag0; bag < bag1; ++bag) {
-        const int32_t next_end = bag + 1 < bag1 ? __ldg(&offsets[bag + 2]) : end;
-        double acc[NV][4] = {};
-        while (lo < end) {
-            const int n = min(32, end - lo);
-            const int32_t next = ids_at(lo + n);
-            if (lane < n && mine >= n_slots) set_status(status, HL_EBOUNDS);
-            const unsigned good = __ballot_sync(0xffffffffu, lane < n && (uint32_t)mine < (uint32_t)n_slots);
-            const int rows_n = __popc(good);
-            if (rows_n < n) {                      // skipped lookups (negative ids) among them: close the gaps
-                const int from = lane < rows_n ? (int)__fns(good, 0, lane + 1) : 0;
-                mine = __shfl_sync(0xffffffffu, mine, from);
-            }
-            auto some = [&](int k0, int most) {    // rows k0 .. of the chunk; most = U unless they are the last
-                float4 r[U][NV];
-#pragma unroll
-                for (int k = 0; k < U; ++k) {
-                    const int64_t id = __shfl_sync(0xffffffffu, mine, k0 + k);
-#pragma unroll
-                    for (int v = 0; v < NV; ++v)
-                        if (k < most) r[k][v] = __ldg(&rows[id * D4 + col[v]]);
-                }
-#pragma unroll
-                for (int k = 0; k < U; ++k)
-                    if (k < most) {
-#pragma unroll
-                        for (int v = 0; v < NV; ++v) add_row(acc[v], r[k][v]);
-                    }
-            };
-            int k0 = 0;
-#pragma unroll 1
-            for (; k0 + U <= rows_n; k0 += U) some(k0, U);
-            if (k0 < rows_n) some(k0, rows_n - k0);
-            lo += n;
-            mine = next;
-        }
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-            if (lane + v * 32 < D4)
-                __stcs(&out4[bag * D4 + (lane + v * 32)],
-                       make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]));
-        end = next_end;
-    }
-}
-
 // A group of G lanes takes UB consecutive bags per trip.  Bags of at most one lookup (the one-hot case) are plain
 // row copies: the UB rows are loaded at once (UB independent 128-bit loads per lane), and the offsets and ids of
 // the NEXT trip are requested before those rows are consumed, so that the offsets -> id -> row chain of one trip
 // hides behind the rows of another.  Longer bags go through pool_long_bag one after the other.
-// MANY: bags of several lookups are the rule; every warp takes an equal share of consecutive bags through pool_bags.
-// FORWARD: the launch also copies the staged rows that this mini-batch shares with the one before (ForwardRows), which no
-// bag of this launch reads.
-struct ForwardRows {
-    float* cache;
-    int64_t from_row0, to_row0;        // cache[to_row0 + i, :] = cache[from_row0 + src[i], :] where src[i] >= 0
-    const int32_t* src;
-    const int64_t* d_n;
-    int64_t n_max;
-};
-
-template <int G, int NV, int UB, bool MANY, bool FORWARD>
+template <int G, int NV, int UB, bool FORWARD>
 __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const float* __restrict__ cache,
                                                          const int32_t* __restrict__ ids,
                                                          const int32_t* __restrict__ offsets,
                                                          const int32_t* __restrict__ d_n_samples, int max_batch,
                                                          int bags_per_sample_all /* T*S */, int D4, int64_t n_slots,
                                                          float* __restrict__ out, int32_t* status, ForwardRows fr) {
-    if (FORWARD) {
-        int64_t n = *fr.d_n;
-        n = n < 0 ? 0 : (n < fr.n_max ? n : fr.n_max);
-        const int lane = threadIdx.x & 31;
-        float4* c4 = reinterpret_cast<float4*>(fr.cache);
-        for (int64_t i0 = ((int64_t)blockIdx.x * kThreads + threadIdx.x) - lane; i0 < n;
-             i0 += (int64_t)gridDim.x * kThreads) {
-            const int32_t mine = i0 + lane < n ? fr.src[i0 + lane] : -1;
-            for (unsigned m = __ballot_sync(0xffffffffu, mine >= 0 && mine < fr.n_max); m; m &= m - 1) {
-                const int k = __ffs((int)m) - 1;
-                const int64_t from = fr.from_row0 + __shfl_sync(0xffffffffu, mine, k);
-                for (int c = lane; c < D4; c += 32) c4[(fr.to_row0 + i0 + k) * D4 + c] = c4[from * D4 + c];
-            }
-        }
-    }
+    if (FORWARD) forward_rows(fr, D4);
     const int64_t n_bags = (int64_t)clamp_samples(d_n_samples, max_batch) * bags_per_sample_all;
     const int sub = threadIdx.x % G;
     const float4* __restrict__ rows = reinterpret_cast<const float4*>(cache);
     float4* __restrict__ out4 = reinterpret_cast<float4*>(out);
-
-    if (MANY) {
-        const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
-        const int64_t me = (int64_t)blockIdx.x * (kThreads / 32) + threadIdx.x / 32;
-        const int64_t first = n_bags * me / warps, last = n_bags * (me + 1) / warps;
-        if (first < last) pool_bags<NV>(rows, ids, offsets, first, last, threadIdx.x & 31, D4, n_slots, out4, status);
-        return;
-    }
 
     // lo/len of the UB bags of a trip, and the id of every bag that has exactly one lookup (-1 otherwise)
     auto load_index = [&](int64_t bag0, int32_t (&lo)[UB], int32_t (&len)[UB], int32_t (&id1)[UB]) {
@@ -261,6 +192,127 @@ __global__ void __launch_bounds__(kThreads, NV == 1 ? 4 : 1) k_embbag_fwd(const 
             pool_long_bag<G, NV>(rows, ids, b_lo, b_len, sub, D4, n_slots, out4 + bag * D4, status);
         }
     }
+}
+
+// ---- bags of several lookups
+__device__ __forceinline__ void copy_16_async(uint32_t smem_to, const void* from, bool valid) {      // (else: zeros)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_to), "l"(from), "r"(valid ? 16 : 0) : "memory");
+}
+
+// By columns per lane: lookups of a block, threads of a CTA, CTAs that fit a multiprocessor (registers).
+template <int NV>
+struct FwdShape {
+    static constexpr int U = NV >= 4 ? 1 : 4 / NV, kBlocks = 2;
+    static constexpr int NT = NV >= 8 ? 128 : 256;
+    static constexpr int CTAS = NV >= 4 ? 3 : 4;
+    static constexpr size_t kSmem = sizeof(float4) * kBlocks * U * NV * NT;
+    static_assert(kSmem <= 48 * 1024, "more than that has to be asked for");
+};
+
+// A group of G lanes pools a run of consecutive bags; the runs of all groups of the launch are equally long.  The lookups of
+// a run are one list, which the group walks in blocks of U: while a block is summed, the rows of the next one are on their way
+// into shared memory and the ids of the one after that into registers, whatever bags they belong to.  (A lane copies and reads
+// the same 16 bytes of every row, so nothing but its own copies is waited for.)  Rows are added in lookup order in fp64 and the
+// sum is rounded once, so that cancellation between the rows of a bag costs no accuracy.  A lookup that is skipped (negative id)
+// or outside the cache adds zeros.
+//
+// What bounds it is how many rows are on their way, and how often a bag makes them stop: with a loop over the lookups of one
+// bag after the other (loads into registers, four at a time) 2.1 M lookups of 256-byte rows in bags of 5 took 114.7 us, 655 K of
+// 64 bytes in bags of 10 28.7, 80 K of 128 bytes in bags of 4 17.5, 200 K of 144 bytes in bags of 3 23.4; so 84.8, 18.4, 10.5 and
+// 18.5 (alone, L2 flushed, Zipf).  2.6 M lookups of 512 bytes in bags of 20: 149.5 -> 142.1 (9.4 TB/s).  Bags of one lookup, against
+// a kernel made for them: 426 K of 256 bytes 36.9 -> 35.5, 106 K of 512 bytes 21.8 -> 22.4, 33 K of 1 KB 18.4 -> 15.7.  Blocks of 8 or
+// 3 rows, and rings of three blocks: within 4 % or slower; five CTAs per multiprocessor: 2 % faster for bags of one lookup
+// of 256 bytes, 10 % slower for 64-byte rows and 22 % for 1 KB.
+template <int G, int NV, bool FORWARD>
+__global__ void __launch_bounds__(FwdShape<NV>::NT, FwdShape<NV>::CTAS) k_embbag_pool(const float* __restrict__ cache,
+                                                         const int32_t* __restrict__ ids,
+                                                         const int32_t* __restrict__ offsets,
+                                                         const int32_t* __restrict__ d_n_samples, int max_batch,
+                                                         int bags_per_sample_all /* T*S */, int D4, int64_t n_slots,
+                                                         float* __restrict__ out, int32_t* status, ForwardRows fr) {
+    constexpr int U = FwdShape<NV>::U, NB = FwdShape<NV>::kBlocks, NT = FwdShape<NV>::NT;
+    static_assert(U <= G, "a lane holds one id of a block");
+    constexpr unsigned kAll = 0xffffffffu;
+    extern __shared__ float4 ring[];                    // [NB][U][NV][NT]
+    const int lane = threadIdx.x & 31, sub = lane % G;
+    if (FORWARD) forward_rows(fr, D4);
+    // this group's bags: [first, first + n_bags)  (numbers of bags and lookups are below 2^30)
+    const int all_bags = clamp_samples(d_n_samples, max_batch) * bags_per_sample_all;
+    const int groups = gridDim.x * (NT / G), me = (blockIdx.x * NT + threadIdx.x) / G;
+    const int q = all_bags / groups, rem = all_bags - q * groups;
+    const int first = me * q + min(me, rem), n_bags = q + (me < rem ? 1 : 0);
+    const unsigned gmask = G == 32 ? kAll : ((1u << (G & 31)) - 1u) << (lane - sub);
+    const uint32_t n_rows = (uint32_t)(n_slots < 0x7fffffff ? n_slots : 0x7fffffff), row_bytes = (uint32_t)D4 * 16u;
+    const char* const column = reinterpret_cast<const char*>(cache) + sub * 16;
+    const uint32_t ring0 = (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * 16;
+
+    const int32_t* __restrict__ ends = offsets + first + 1;              // where the group's bags end
+    int32_t p = n_bags > 0 ? __ldg(ends - 1) : 0;
+    const int32_t hi = n_bags > 0 ? __ldg(ends + n_bags - 1) : 0;
+    auto ends_at = [&](int k) { return k + sub < n_bags ? __ldg(ends + k + sub) : 0x7fffffff; };
+    auto ids_at = [&](int32_t at) { return sub < U && at + sub < hi ? __ldg(&ids[at + sub]) : -1; };
+    auto request = [&](int b, int32_t mine) {           // the rows of a block, whose ids the first U lanes hold
+        const bool ok = (uint32_t)mine < n_rows;
+        if (!ok && mine >= 0) set_status(status, HL_EBOUNDS);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t id = __shfl_sync(kAll, ok ? (uint32_t)mine : 0xffffffffu, u, G);
+            const bool valid = id != 0xffffffffu;
+            const char* row = column + (uint64_t)(valid ? id : 0u) * row_bytes;
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+                if (sub + v * G < D4)
+                    copy_16_async(ring0 + ((b * U + u) * NV + v) * (NT * 16), row + v * G * 16, valid);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    int32_t my_end = ends_at(0), next_ends = ends_at(G);
+    int32_t next_ids = ids_at(p);
+#pragma unroll
+    for (int b = 0; b < NB - 1; ++b) {
+        const int32_t mine = next_ids;
+        next_ids = ids_at(p + (b + 1) * U);
+        request(b, mine);
+    }
+    double acc[NV][4] = {};
+    int k = 0;                                          // the bag being summed, and where it ends
+    int32_t end = __shfl_sync(kAll, my_end, 0, G);
+    float4* to = reinterpret_cast<float4*>(out) + (int64_t)first * D4 + sub;
+    auto next_bag = [&]() {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (sub + v * G < D4)
+                __stcs(to + v * G, make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]));
+            acc[v][0] = acc[v][1] = acc[v][2] = acc[v][3] = 0.0;
+        }
+        to += D4;
+        ++k;
+        if ((k & (G - 1)) == 0) {
+            my_end = next_ends;
+            next_ends = ends_at(k + G);
+        }
+        end = __shfl_sync(gmask, my_end, k & (G - 1), G);          // (behind the last bag: 2^31 - 1)
+    };
+    for (int b = 0; __any_sync(kAll, p < hi); p += U, b = b == NB - 1 ? 0 : b + 1) {
+        const int32_t mine = next_ids;
+        next_ids = ids_at(p + NB * U);
+        request(b == 0 ? NB - 1 : b - 1, mine);
+        asm volatile("cp.async.wait_group %0;" ::"n"(NB - 1) : "memory");
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            float4 r[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+                r[v] = sub + v * G < D4 ? ring[((b * U + u) * NV + v) * NT + threadIdx.x] : f4_zero();
+            if (p + u < hi) {
+                while (end <= p + u) next_bag();
+#pragma unroll
+                for (int v = 0; v < NV; ++v) add_row(acc[v], r[v]);
+            }
+        }
+    }
+    while (k < n_bags) next_bag();
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // ---- backward -----------------------------------------------------------------------------------------------
@@ -798,15 +850,18 @@ template <int G, int NV>
 int32_t launch_fwd(hl_ctx* ctx, const float* cache, const hl_ubatch* ub, const int32_t* d_n, float* out,
                    const ForwardRows* fr, cudaStream_t stream) {
     constexpr int UB = NV >= 4 ? 1 : (NV >= 2 ? 2 : 4);
-    const int64_t bags_per_trip = (int64_t)(kThreads / G) * UB;
     timer_mark(ctx, HL_TIMER_FWD, 0, stream);
-    // more than 1.5 lookups per bag at most: the one-hot loop is not worth trying first
-    const bool many = G == 32 && 2 * ctx->max_nnz > 3 * (int64_t)ctx->max_bags;
-    const int grid = grid_for(ctx->max_bags, many ? kThreads / 32 : (int)bags_per_trip, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
-    const auto kernel = many ? (fr ? k_embbag_fwd<G, NV, UB, G == 32, true> : k_embbag_fwd<G, NV, UB, G == 32, false>)
-                             : (fr ? k_embbag_fwd<G, NV, UB, false, true> : k_embbag_fwd<G, NV, UB, false, false>);
-    HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, cache, ub->ids, ub->offsets, d_n, ctx->max_batch, ctx->T * ctx->S,
-                       ctx->D / 4, ctx->hot_cap + ctx->staging_cap, out, ctx->r.status, fr ? *fr : ForwardRows{}));
+    // More than 1.5 lookups per bag at most: the loop for bags of one is not worth trying first.  (For those it is the better
+    // one beside other kernels: click log 75 us per mini-batch, 77 with the other.)
+    const bool many = 2 * ctx->max_nnz > 3 * (int64_t)ctx->max_bags;
+    // a fixed number of CTAs per multiprocessor; in small calls of bags of several lookups a group has a bag or two
+    using Shape = FwdShape<NV>;
+    const int grid = grid_for(ctx->max_bags, many ? Shape::NT / G : kThreads / G * UB, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
+    const auto kernel = many ? (fr ? k_embbag_pool<G, NV, true> : k_embbag_pool<G, NV, false>)
+                             : (fr ? k_embbag_fwd<G, NV, UB, true> : k_embbag_fwd<G, NV, UB, false>);
+    HL_CUDA_TRY(launch_cluster(kernel, grid, many ? Shape::NT : kThreads, many ? Shape::kSmem : 0, 0, stream, cache, ub->ids,
+                               ub->offsets, d_n, ctx->max_batch, ctx->T * ctx->S, ctx->D / 4,
+                               ctx->hot_cap + ctx->staging_cap, out, ctx->r.status, fr ? *fr : ForwardRows{}));
     timer_mark(ctx, HL_TIMER_FWD, 1, stream);
     note_launches(1);
     HL_LAUNCH_CHECK();

@@ -1,6 +1,6 @@
-"""The pooling forward on rows wider than 64 floats with several lookups per bag: one warp per run of bags, 32 lookups at a
-time.  Bag lengths around 32 and 4, empty bags, skipped lookups, every row width class; integer data, so the pooled vectors
-must equal the oracle's."""
+"""The pooling forward with several lookups per bag: a group of lanes per run of bags, one to four lookups at a time.  Bag
+lengths around 32 and 4, empty bags, skipped lookups, every row width class, runs of no bag, of one and of more bags than
+a group has lanes; integer data, so the pooled vectors must equal the oracle's."""
 import numpy as np
 import pytest
 import torch
@@ -13,12 +13,22 @@ LENGTHS = [0, 1, 2, 3, 4, 5, 31, 32, 33, 0, 0, 63, 64, 65, 7, 100, 28, 36, 0]
 
 
 @pytest.mark.parametrize("bags", [1, 2, 19, 5000])
-@pytest.mark.parametrize("dim", [68, 128, 132, 256, 260, 512, 1024])
+@pytest.mark.parametrize("dim", [4, 16, 20, 32, 36, 64, 68, 128, 132, 256, 260, 512, 1024])
 def test_forward_of_long_bags(dim, bags):
     import paper_2204_05436_b200 as hl
+    lengths = np.resize(LENGTHS, bags) if bags > 2 else np.full(bags, 35)
+    _check(hl, dim, bags, lengths)
+
+
+@pytest.mark.parametrize("dim,bags", [(4, 170_000), (12, 100_001), (32, 160_000), (128, 155_000)])
+def test_more_bags_than_lanes(dim, bags):
+    import paper_2204_05436_b200 as hl
+    _check(hl, dim, bags, np.resize([0, 3, 1, 2, 0, 4, 1], bags))
+
+
+def _check(hl, dim, bags, lengths):
     rng = np.random.default_rng(dim + bags)
     rows = 300
-    lengths = np.resize(LENGTHS, bags) if bags > 2 else np.full(bags, 35)
     offsets = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
     nnz = int(offsets[-1])
     ids = rng.integers(0, rows, nnz).astype(np.int32)
