@@ -411,11 +411,12 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pairs(PairArgs a) {
     }
 }
 
-// The sorted lookups are cut into chunks of 32.  One WARP per chunk sums, in order, the gradient rows of each run of
-// equal slots inside its chunk.  A run that lies wholly inside the chunk is finished here (one reduction into its row).
-// A run that crosses a chunk border leaves a partial sum: part[chunk][0] for the piece that continues a run from the
-// previous chunk, part[chunk][1] for the piece that starts a run continuing into the next chunk.  k_bwd_spans adds
-// those up.
+// The sorted lookups are cut into chunks of 32, and these into windows of 8.  A CTA takes a window, a WARP a chunk: it sums, in
+// order, the gradient rows of each run of equal slots inside its chunk.  A run that lies wholly inside the chunk is finished
+// there (one reduction into its row).  Of a run that goes on over several chunks of the window, the later chunks' warps leave
+// their sums in shared memory and the warp of the chunk it starts in adds them up.  A run that crosses a window's border
+// leaves a partial sum: part[window][0] for the piece that continues a run from the previous window, part[window][1] for the
+// piece that starts a run continuing into the next window.  k_bwd_spans adds those up.
 //
 // Every lane loads one (slot, bag) pair and the 32 / G groups of the warp take G consecutive lookups each, so that the
 // gradient rows of a chunk are requested by all groups at once: a chunk of narrow rows (64 bytes: G = 4) is a chain of
@@ -428,12 +429,17 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pairs(PairArgs a) {
 // 512 bytes: 183 -> 173 us; chunks of 64 / 128 / 256 lookups 177 / 190 / 197 us: the row updates of the warps at work
 // then lie further apart).
 //
-// A run that starts in one chunk and ends in the next (most runs that cross a border do) is finished by the warp of
-// the chunk it starts in, which reads on into the next chunk; the warp of that next chunk leaves the run's lookups
-// alone.  Both decide from the sorted slots alone and by the same test -- the run's head lies in the first of the two
-// chunks, and the chunk after the second does not begin with the run's slot -- so exactly one of them sums each
-// lookup.  Only runs over three or more chunks go through partial sums and k_bwd_spans.
-constexpr int kSpanLookahead = 32;      // chunks k_bwd_chunks looks ahead for the end of a run
+// A run that starts in one window and ends in the next one's first chunk is finished by the warp of the chunk it starts in,
+// which reads on into that chunk; the warp there leaves the run's lookups alone.  Both decide from the sorted slots alone and by
+// the same test -- the run's head lies in the first of the two windows, and what lies behind the second one's first chunk does not
+// begin with the run's slot -- so exactly one of them sums each lookup.  Only runs with more than 32 lookups in the next
+// window go through partial sums and k_bwd_spans.
+// (Without the windows, every run over three or more chunks went through them, a popular row's hundreds of pieces among them.
+// Sums and spans, alone, L2 flushed, Zipf, by chunks / by windows: 426 K lookups of 256 bytes 53.2 / 47.1 us, 312 K 43.1 / 40.8, 333 K
+// of 144 bytes 36.0 / 32.3, 129 K of 64 bytes 18.4 / 16.4, 2.6 M of 512 bytes 206.8 / 192.9, 262 K of 1 KB 70.1 / 59.3, 131 K of 2 KB
+// 101.2 / 88.1; uniform slots the same.  Of the 2.6 M the sums take 173 instead of 166, the spans 14 instead of 32.)
+constexpr int kWindowChunks = kThreads / 32, kBwdWindow = kWindowChunks * kBwdChunk;
+constexpr int kSpanLookahead = 32;      // windows k_bwd_chunks looks ahead for the end of a run
 static_assert(kBwdChunk == 32, "one lookup of a chunk per lane");
 
 //
@@ -470,7 +476,7 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
     constexpr unsigned gbits = G == 32 ? 0xffffffffu : ((1u << G) - 1u);
     const unsigned gmask = gbits << g0;
     const unsigned before_group = (1u << g0) - 1u;                          // lookups of the groups before mine
-    const int n_warps = gridDim.x * (kThreads / 32);
+    const int wib = threadIdx.x >> 5;
     float4* __restrict__ part4 = reinterpret_cast<float4*>(part);
     // slots and bags are 32-bit numbers, so one unsigned comparison tells whether one lies inside its array
     const uint32_t n_rows_u = (uint32_t)(n_slots < 0x7fffffff ? n_slots : 0x7fffffff);
@@ -481,6 +487,13 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
     const char* gcol[NV];
     const uint32_t row_bytes = (uint32_t)D4 * 16u;
     __shared__ double2 s_first[G == 32 ? 1 : 2][G == 32 ? 1 : kThreads];      // sums of the groups' first runs
+    // Of every chunk of the window that begins inside a run: what the run has there, and whether it ends there.  (Two sets, for
+    // windows in turn; rows of more than 256 fp32 have room for one, of fp32 sums.)
+    constexpr bool kTwo = NV <= 2;
+    using Piece = std::conditional_t<kTwo, double2, float4>;
+    constexpr int kParts = kTwo ? 2 : 1;
+    __shared__ Piece s_piece[kTwo ? 2 : 1][kWindowChunks][NV][kParts][G];
+    __shared__ int s_ends[kTwo ? 2 : 1][kWindowChunks];
     const float minus_lr = -lr;               // -(lr * G) and (-lr) * G are the same number
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -493,22 +506,23 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
         return __ldg(reinterpret_cast<const float4*>(gcol[v] + (uint64_t)(uint32_t)b * row_bytes));
     };
 
-    for (int chunk = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); chunk < n_chunks; chunk += n_warps) {
-        const int start = first + chunk * kBwdChunk;
-        const int end = min(start + kBwdChunk, n);
-        const int32_t key = start + lane < end ? keys[start + lane] : -1;     // -1: past the end; no slot has this key
-        int32_t bag = start + lane < end ? vals[start + lane] : 0;
-        const int32_t prev_key = start > first ? keys[start - 1] : -3;        // -3: equal to no key
-        const int32_t next_key = end < n ? keys[end] : -2;
-        // the slot before the previous chunk, and the first slot of the chunk after the next one
-        const int32_t prev2_key = start - kBwdChunk > first ? keys[start - kBwdChunk - 1] : -3;
-        const int32_t next2_key = start + 2 * kBwdChunk < n ? keys[start + 2 * kBwdChunk] : -2;
-        // the next chunk's pairs, for a run that ends there (narrow rows: asked for now, not when the sums are done)
+    for (int window = blockIdx.x, turn = 0; window * kWindowChunks < n_chunks; window += gridDim.x, ++turn) {
+        const int set = kTwo ? turn & 1 : 0;
+        const int start = first + (window * kWindowChunks + wib) * kBwdChunk;          // (may lie behind the last lookup)
+        const int window_end = first + (window + 1) * kBwdWindow;
+        const int32_t key = start + lane < n ? keys[start + lane] : -1;       // -1: past the end; no slot has this key
+        int32_t bag = start + lane < n ? vals[start + lane] : 0;
+        const int32_t prev_key = start > first && start <= n ? keys[start - 1] : -3;      // -3: equal to no key
+        const int32_t next_key = start + kBwdChunk < n ? keys[start + kBwdChunk] : -2;
+        // the slot before the previous window, and the first slot behind the next window's first chunk
+        const int32_t prev2_key = wib == 0 && window >= 2 ? keys[start - kBwdWindow - 1] : -3;
+        const int32_t next2_key = window_end + kBwdChunk < n ? keys[window_end + kBwdChunk] : -2;
+        // the next window's first pairs, for a run that ends there (narrow rows: asked for now, not when the sums are done)
         int32_t k2 = -1, b2 = 0;
         const auto load_next = [&]() {
-            if (end + lane < n) {
-                k2 = keys[end + lane];
-                b2 = vals[end + lane];
+            if (window_end + lane < n) {
+                k2 = keys[window_end + lane];
+                b2 = vals[window_end + lane];
             }
         };
         if (G < 32) load_next();
@@ -532,13 +546,46 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
                                make_float4(minus_lr * (float)acc[v][0], minus_lr * (float)acc[v][1],
                                            minus_lr * (float)acc[v][2], minus_lr * (float)acc[v][3]));
         };
-        // a piece of a run that crosses the chunk's border (which: 0 = it comes in from the left, 1 = it starts here)
+        // a piece of a run that crosses the window's border (which: 0 = it comes in from the left, 1 = it starts here)
         auto store_piece = [&](int which, const double (&acc)[NV][4]) {
 #pragma unroll
             for (int v = 0; v < NV; ++v)
                 if (on[v])
-                    part4[(int64_t)(chunk * 2 + which) * D4 + sub + v * G] =
+                    part4[(int64_t)(window * 2 + which) * D4 + sub + v * G] =
                         make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]);
+        };
+        // the same for a run that this chunk began inside: kept for the warp of the chunk it starts in
+        auto put_piece = [&](const double (&acc)[NV][4]) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                Piece* to = &s_piece[set][wib][v][0][sub];
+                if constexpr (kTwo) {
+                    to[0] = make_double2(acc[v][0], acc[v][1]);
+                    to[G] = make_double2(acc[v][2], acc[v][3]);
+                } else {
+                    to[0] = make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]);
+                }
+            }
+        };
+        // adds the pieces of a run in the chunks from `chunk` on; true: it ends in this window
+        auto add_pieces = [&](double (&sum)[NV][4], int chunk) {
+            for (; chunk < kWindowChunks; ++chunk) {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const Piece* from = &s_piece[set][chunk][v][0][sub];
+                    if constexpr (kTwo) {
+                        const double2 p = from[0], q = from[G];
+                        sum[v][0] += p.x;
+                        sum[v][1] += p.y;
+                        sum[v][2] += q.x;
+                        sum[v][3] += q.y;
+                    } else {
+                        add_row(sum[v], from[0]);
+                    }
+                }
+                if (s_ends[set][chunk]) return true;
+            }
+            return false;
         };
 
         int32_t l = __shfl_up_sync(0xffffffffu, key, 1), r = __shfl_down_sync(0xffffffffu, key, 1);
@@ -546,16 +593,16 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
         if (lane == 31) r = next_key;
         // bit q of `heads`: lookup q of the chunk begins a run; of `tails`: it ends one
         const unsigned heads = __ballot_sync(0xffffffffu, key != l), tails = __ballot_sync(0xffffffffu, key != r);
-        // A run that comes in from the previous chunk, began there and ends here was finished by that chunk's warp: its
-        // lookups count for nothing here, and a row that is loaded anyway stands in for theirs.
-        const bool skip = chunk >= 1 && !(heads & 1u) && tails != 0u && prev2_key != prev_key;
+        // A run that comes in from the previous window, began there and ends in this one's first chunk was finished there:
+        // its lookups count for nothing here, and a row that is loaded anyway stands in for theirs.
+        const bool skip = wib == 0 && window >= 1 && !(heads & 1u) && tails != 0u && prev2_key != prev_key;
         if (skip) {
             const int32_t other = __shfl_sync(0xffffffffu, bag, 31);
             if (key == prev_key) bag = other;
         }
         // Tails that end a run of a row inside the cache, begun in this chunk: one reduction each.  (A row outside is a
         // skipped lookup's sentinel, or past the end.)  The first tail of a chunk that begins inside a run leaves a
-        // piece instead, or nothing if the chunk before has seen to it.
+        // piece instead, or nothing if the window before has seen to it.
         const uint32_t row = (uint32_t)(key - key_bias);
         const unsigned valid = __ballot_sync(0xffffffffu, row < n_rows_u);
         unsigned piece = (heads & 1u) ? 0u : tails & (0u - tails);
@@ -581,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
                     for (int v = 0; v < NV; ++v) add_row(acc[v], x[u][v], hs & (1u << u));
                     if (es & (1u << u)) {
                         if (ds & (1u << u)) apply(__shfl_sync(0xffffffffu, row, j + u), acc);
-                        else store_piece(0, acc);
+                        else put_piece(acc);
                     }
                 }
                 hs >>= U;
@@ -639,87 +686,94 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
                 in[0][2] = q.x + (from_left ? in[0][2] : 0.0);
                 in[0][3] = q.y + (from_left ? in[0][3] : 0.0);
                 if (late & (done >> g0)) apply(row0, in);
-                else if (late & (piece >> g0)) store_piece(0, in);
+                else if (late & (piece >> g0)) put_piece(in);
             }
         }
-        // the chunk's last lookup does not end its run: the run goes on in the next chunk (only a full chunk has a
-        // next one), and the last group's acc holds what it has collected here
+        // The chunk's last lookup does not end its run: the run goes on in the next chunk (only a full chunk has a next
+        // one), and the last group's acc holds what it has collected here.
         const bool last_group = lane >= 32 - G;
         const int32_t last_key = __shfl_sync(0xffffffffu, key, 31);
-        if ((tails >> 31) || (uint32_t)(last_key - key_bias) >= n_rows_u) continue;
-        if (!heads) {
-            if (last_group) store_piece(0, acc);
-        } else if (next2_key != last_key) {
-            // it began in this chunk and ends in the next: its lookups there are summed here as well (they are a prefix
-            // of that chunk: m of them), and the row gets its one update
-            double more[NV][4];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) more[v][0] = more[v][1] = more[v][2] = more[v][3] = 0.0;
-            if (G == 32) load_next();
-            b2 = (uint32_t)b2 < n_grad_u ? b2 : 0;
-            const int m = __popc(__ballot_sync(0xffffffffu, k2 == last_key));
-            const int mine = m - g0;             // lookups of my group that belong to the run
+        const bool goes_on = !(tails >> 31) && (uint32_t)(last_key - key_bias) < n_rows_u;
+        if (goes_on && !heads && last_group) put_piece(acc);
+        if (lane == 0) s_ends[set][wib] = tails != 0u;
+        __syncthreads();
+        if (wib == 0 && !(heads & 1u) && !skip && (valid & 1u)) {       // what this window has of a run begun in one before
+            double sum[NV][4] = {};
+            add_pieces(sum, 0);
+            if (lane < G) store_piece(0, sum);
+        }
+        if (goes_on && heads) {
+            // The run began in this chunk: the next ones' pieces, if it ends among them, complete it.
+            if (add_pieces(acc, wib + 1)) {
+                if (last_group) apply((uint32_t)(last_key - key_bias), acc);
+            } else if (next2_key != last_key) {
+                // it ends in the next window's first chunk: its lookups there are summed here as well (they are a prefix of
+                // that chunk: m of them), and the row gets its one update
+                double more[NV][4] = {};
+                if (G == 32) load_next();
+                b2 = (uint32_t)b2 < n_grad_u ? b2 : 0;
+                const int m = __popc(__ballot_sync(0xffffffffu, k2 == last_key));
+                const int mine = m - g0;             // lookups of my group that belong to the run
 #pragma unroll 1
-            for (int j = 0; j < (G == 32 ? m : G); j += U) {
-                float4 x[U][NV];
+                for (int j = 0; j < (G == 32 ? m : G); j += U) {
+                    float4 x[U][NV];
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int32_t b = __shfl_sync(0xffffffffu, b2, j + u, G);
+                    for (int u = 0; u < U; ++u) {
+                        const int32_t b = __shfl_sync(0xffffffffu, b2, j + u, G);
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) x[u][v] = j + u < mine ? grad_row(v, b) : f4_zero();
+                        for (int v = 0; v < NV; ++v) x[u][v] = j + u < mine ? grad_row(v, b) : f4_zero();
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) add_row(more[v], x[u][v]);
                 }
 #pragma unroll
-                for (int u = 0; u < U; ++u)
+                for (int v = 0; v < NV; ++v)
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) add_row(more[v], x[u][v]);
-            }
+                    for (int e = 0; e < 4; ++e) {
 #pragma unroll
-            for (int v = 0; v < NV; ++v)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-#pragma unroll
-                    for (int off = G; off < 32; off <<= 1) more[v][e] += __shfl_xor_sync(0xffffffffu, more[v][e], off);
-                    more[v][e] += acc[v][e];
+                        for (int off = G; off < 32; off <<= 1)
+                            more[v][e] += __shfl_xor_sync(0xffffffffu, more[v][e], off);
+                        more[v][e] += acc[v][e];
+                    }
+                if (last_group) apply((uint32_t)(last_key - key_bias), more);
+            } else {
+                if (last_group) store_piece(1, acc);
+                // List it, with its last window if that is among the next 32 (window w > window holds a piece of the run iff
+                // its first slot is the run's; equal slots lie together: those windows form a prefix).  Nearly every run ends
+                // there, and k_bwd_spans then has nothing to search; the longer ones go to the list's other end.
+                const int64_t at = window_end + (int64_t)lane * kBwdWindow;
+                const bool there = at < n && keys[at] == last_key;
+                const int cnt = __popc(__ballot_sync(0xffffffffu, there));
+                if (lane == 0) {
+                    const bool is_long = cnt == kSpanLookahead;
+                    const int32_t i = atomicAdd(&span_count[is_long ? 1 : 0], 1);
+                    // (one entry per window at most, and the counts are zero when a call starts: the list cannot overflow
+                    // unless an earlier call was cut short between its two kernels)
+                    if (i >= 0 && i < max_entries)
+                        reinterpret_cast<int4*>(span_list)[is_long ? max_entries - 1 - i : i] =
+                            make_int4(window, last_key, is_long ? -1 : window + cnt, 0);
+                    else
+                        set_status(status, HL_ECAPACITY);
                 }
-            if (last_group) apply((uint32_t)(last_key - key_bias), more);
-        } else {
-            if (last_group) store_piece(1, acc);
-            // List it, with its last chunk if that is among the next 32 (chunk c > chunk holds a piece of the run iff
-            // its first slot is the run's; sorted keys: those chunks form a prefix).  Nearly every run ends there, and
-            // k_bwd_spans then has nothing to search; the longer ones go to the list's other end.
-            const int cc = chunk + 1 + lane;
-            const bool goes_on = cc < n_chunks && keys[first + cc * kBwdChunk] == last_key;
-            const int cnt = __popc(__ballot_sync(0xffffffffu, goes_on));
-            if (lane == 0) {
-                const bool is_long = cnt == kSpanLookahead;
-                const int32_t i = atomicAdd(&span_count[is_long ? 1 : 0], 1);
-                // (one entry per chunk at most, and the counts are zero when a call starts: the list cannot overflow
-                // unless an earlier call was cut short between its two kernels)
-                if (i >= 0 && i < max_entries)
-                    reinterpret_cast<int4*>(span_list)[is_long ? max_entries - 1 - i : i] =
-                        make_int4(chunk, last_key, is_long ? -1 : chunk + cnt, 0);
-                else
-                    set_status(status, HL_ECAPACITY);
             }
         }
+        if (!kTwo) __syncthreads();                 // (the one set of pieces is free for the next window's)
     }
 }
 
-// Finishes the listed runs: those that start in a chunk and go on over at least two more.  Two lists share one array.
+// Finishes the listed runs: those that start in a window and have more than 32 lookups in the next.  Two lists share one array.
 //
-// From its front: runs whose last chunk is known (up to kSpanLookahead chunks on).  One WARP per run: the 32/G groups add
+// From its front: runs whose last window is known (up to kSpanLookahead windows on).  One WARP per run: the 32/G groups add
 // the run's continuation pieces in an interleaved, fixed order in fp64, the group sums are combined by shuffles in a
 // fixed order, and group 0 applies the single SGD update of the row.
-// From its back: longer runs (a popular row can own hundreds of chunks).  One CTA per run, because they are what the
-// kernel's length depends on: its warps close in on the end with a 32-way search over the sorted keys, every group takes
-// every (8 * 32/G)-th piece, and one group combines the group sums in a fixed order.  (With both kinds in one list a CTA
-// met up to eight long runs one after the other: 2.6 M lookups of 512 bytes took 36.6 us.)
+// From its back: longer runs (a popular row can own hundreds of windows).  One CTA per run: its warps close in on the end with a
+// 32-way search over the sorted keys, every group takes every (8 * 32/G)-th piece, and one group combines the group sums in
+// a fixed order.
 //
-// A long run is a chain of round trips to the L2, so what helps is to have the pieces of the next trip on their way: two
-// CTAs per multiprocessor (the grid is no more than that) leave the compiler 120 registers for it; left alone it keeps to
-// 64 and asks for one trip at a time.  Zipf over 26 tables, alone, L2 flushed: 106 K / 426 K lookups of 256 bytes 9.6 / 15.7
-// us -> 6.3 / 11.0; 426 K of 64 bytes 11.5 -> 10.3, of 512 bytes 16.6 -> 13.8, of 2 KB 71.9 -> 33.9; 32 K of 256 bytes 5.9 ->
-// 4.8; no such run 3.2 either way.
+// A run is a chain of round trips to the L2 (entry, pieces, reduction), so what helps is to have the pieces of the next trip on
+// their way: two CTAs per multiprocessor (the grid is no more than that) leave the compiler 120 registers for it.
 template <int G, int NV>
 __global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ cache, const int32_t* __restrict__ keys,
                                                         const int32_t* __restrict__ d_n_lookups, int D4,
@@ -738,8 +792,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ c
     const float4* __restrict__ part4 = reinterpret_cast<const float4*>(part);
     const int4* __restrict__ list = reinterpret_cast<const int4*>(span_list);
     float4* cache4 = reinterpret_cast<float4*>(cache);
-    const int64_t n_chunks = (n - first + kBwdChunk - 1) / kBwdChunk;
-    const int64_t most = n_chunks < max_entries ? n_chunks : max_entries;
+    const int64_t n_windows = (n - first + kBwdWindow - 1) / kBwdWindow;
+    const int64_t most = n_windows < max_entries ? n_windows : max_entries;
     auto clamped = [&](int32_t c) { return c < 0 ? (int64_t)0 : ((int64_t)c < most ? (int64_t)c : most); };
     const int64_t n_short = clamped(span_count[0]), n_long = clamped(span_count[1]);
 
@@ -769,16 +823,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ c
     };
 
     for (int64_t i = blockIdx.x; i < n_long; i += gridDim.x) {
-        const int4 e = list[max_entries - 1 - i];            // (chunk, slot key of the run, -, -)
-        const int64_t chunk = e.x, row = (int64_t)e.y - key_bias;
-        if (chunk < 0 || chunk + 1 >= n_chunks || row < 0 || row >= n_slots) continue;     // the same for all threads
-        // last chunk that holds a piece of the run: chunk c > chunk holds one iff its first slot is the run's; chunk lo
-        // does, chunk hi (if any) does not
-        int64_t lo = chunk + 1, hi = n_chunks;
+        const int4 e = list[max_entries - 1 - i];            // (window, slot key of the run, -, -)
+        const int64_t window = e.x, row = (int64_t)e.y - key_bias;
+        if (window < 0 || window + 1 >= n_windows || row < 0 || row >= n_slots) continue;     // the same for all threads
+        // last window that holds a piece of the run: window w > window holds one iff its first slot is the run's; window lo
+        // does, window hi (if any) does not
+        int64_t lo = window + 1, hi = n_windows;
         while (hi - lo > 1) {
             const int64_t step = (hi - lo + 31) / 32;
             const int64_t cc = lo + (lane + 1) * step;
-            const bool t = cc < hi && keys[first + cc * kBwdChunk] == e.y;
+            const bool t = cc < hi && keys[first + cc * kBwdWindow] == e.y;
             const int cnt = __popc(__ballot_sync(0xffffffffu, t));     // sorted keys: a prefix of the lanes
             const int64_t new_hi = min(hi, lo + (cnt + 1) * step);
             lo += cnt * step;
@@ -787,7 +841,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ c
         double acc[NV][4];
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v][0] = acc[v][1] = acc[v][2] = acc[v][3] = 0.0;
-        add_pieces(acc, chunk + 1 + wib * GW + gi, lo, (int64_t)kWarps * GW);
+        add_pieces(acc, window + 1 + wib * GW + gi, lo, (int64_t)kWarps * GW);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
 #pragma unroll
@@ -795,7 +849,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ c
             __syncthreads();
             const int c = sub + v * G;
             if (threadIdx.x < G && c < D4) {       // group 0 of warp 0: lane sub owns column c
-                const float4 p = part4[(chunk * 2 + 1) * D4 + c];      // the piece in the run's first chunk
+                const float4 p = part4[(window * 2 + 1) * D4 + c];      // the piece in the run's first window
                 double a[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll 8
                 for (int g2 = 0; g2 < kWarps * GW; ++g2)
@@ -808,20 +862,20 @@ __global__ void __launch_bounds__(kThreads, 2) k_bwd_spans(float* __restrict__ c
     }
 
     for (int64_t i = (int64_t)blockIdx.x * kWarps + wib; i < n_short; i += (int64_t)gridDim.x * kWarps) {
-        const int4 e = list[i];                              // (chunk, slot key of the run, its last chunk, -)
-        const int64_t chunk = e.x, last = e.z, row = (int64_t)e.y - key_bias;
-        if (chunk < 0 || last <= chunk || last >= n_chunks || row < 0 || row >= n_slots) continue;
+        const int4 e = list[i];                              // (window, slot key of the run, its last window, -)
+        const int64_t window = e.x, last = e.z, row = (int64_t)e.y - key_bias;
+        if (window < 0 || last <= window || last >= n_windows || row < 0 || row >= n_slots) continue;
         double acc[NV][4];
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const int c = sub + v * G;
-            const float4 p = gi == 0 && c < D4 ? part4[(chunk * 2 + 1) * D4 + c] : f4_zero();
+            const float4 p = gi == 0 && c < D4 ? part4[(window * 2 + 1) * D4 + c] : f4_zero();
             acc[v][0] = p.x;
             acc[v][1] = p.y;
             acc[v][2] = p.z;
             acc[v][3] = p.w;
         }
-        add_pieces(acc, chunk + 1 + gi, last, GW);
+        add_pieces(acc, window + 1 + gi, last, GW);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
 #pragma unroll
