@@ -449,6 +449,10 @@ static_assert(kBwdChunk == 32, "one lookup of a chunk per lane");
 // eight.  Rows of 256 bytes, alone, L2 flushed, three against four CTAs: Zipf over 26 tables 32 K lookups 11.5 / 13.0 us,
 // 106 K 14.1 / 15.1, 150 K 19.1 / 16.6, 426 K 35.7 / 33.9; uniform 9.6 / 10.0, 13.8 / 13.6, 19.0 / 16.6, 48.4 / 46.5; bags of
 // 20 lookups 8.4 / 8.8, 11.6 / 10.9, 15.7 / 12.8, 28.6 / 25.2.  So three as long as their warps have a chunk each at most.
+// Rows of 68 to 128 fp32 (G = 32, one column per lane): four CTAs with four rows a lane in flight, instead of three with eight,
+// where most gradient rows come out of the L2, that is where bags have many lookups.  Rows of 512 bytes, sums and spans, three
+// against four CTAs: bags of 20 lookups, 2.6 M 193 / 184 us, 1.3 M 104.7 / 102.7; of 10, 1.6 M 125.6 / 119.6; of 5, 0.8 M 82.4 /
+// 79.9; of 3, 0.6 M 69.6 / 75.8; of 2, 0.4 M 55.8 / 58.6; of 1, 0.3 M 57.4 / 64.5.  (The host knows how many a bag has at most.)
 
 template <int G, int NV, int CTAS>
 __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict__ cache,
@@ -929,8 +933,10 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
     const int64_t max_chunks = div_up(ctx->max_nnz, kBwdChunk);
     // a fixed number of CTAs per multiprocessor (the warps stride over the chunks), so that kernels of other streams find
     // room beside this one: two rounds of those that fit
-    const bool four = G == 16 && max_chunks > 3 * (kThreads / 32) * ctx_sms(ctx);
-    const auto sums = four ? k_bwd_chunks<G, NV, G == 16 ? 4 : NV == 1 ? 3 : 1> : k_bwd_chunks<G, NV, NV == 1 ? 3 : 1>;
+    constexpr bool kFour = G >= 16 && NV == 1;
+    const bool four = kFour && max_chunks > 3 * (kThreads / 32) * ctx_sms(ctx) &&
+                      (G == 16 || ctx->max_nnz > 16 * ctx->max_bags);
+    const auto sums = four ? k_bwd_chunks<G, NV, kFour ? 4 : NV == 1 ? 3 : 1> : k_bwd_chunks<G, NV, NV == 1 ? 3 : 1>;
     const int per_sm = ctx->bwd_ctas > 0 ? ctx->bwd_ctas : four ? 8 : 6;
     const int grid = grid_for(max_chunks * 32, kThreads, per_sm * ctx_sms(ctx));
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
