@@ -8,7 +8,7 @@ namespace {
 constexpr int kThreads = 256;
 
 // ---- the distinct cold rows, in ascending order --------------------------------------------------------------
-// One bit per row of the model: classifying X's lookups sets the bits of its cold rows (classify_cold), k_cold_rank
+// One bit per row of the model: classifying X's lookups sets the bits of its cold rows (mark_cold), k_cold_rank
 // reads the bitmap in row order -- which is ascending order without a sort -- and hands out the ranks, and k_cold_assign
 // turns every cold lookup into the slot of its row's rank.  The work depends on the lookups and (a 32nd or a 1024th of
 // a word per row) on the size of the model, not on how many cold lookups there are, so there is one path for all
@@ -30,7 +30,10 @@ __global__ void __launch_bounds__(kThreads) k_cold_classify(int32_t* __restrict_
             set_status(status, HL_EBOUNDS);
             ids[j] = -1;
         } else if (g >= 0) {
-            ids[j] = classify_cold(remap, g, marks);
+            const uint32_t word = marks.bits[g >> 5];
+            const int32_t slot = remap.slot(remap.request(g), g);
+            ids[j] = slot >= 0 ? slot : cold_id(g);
+            if (slot < 0) mark_cold(marks, g, word);
         }
     }
 }

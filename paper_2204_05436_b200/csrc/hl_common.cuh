@@ -251,21 +251,29 @@ __device__ __forceinline__ void set_status(int32_t* status, int32_t code) {
     atomicCAS(status, 0, code);
 }
 
-// Hit test only: one 4-byte load.
-__device__ __forceinline__ bool remap_hit(const RemapBlock* __restrict__ remap, int64_t g) {
+// Popular rows are looked up in two halves, so that a thread with several lookups has all their loads on the way before it
+// waits for the first: `request` (or `request_hit`, for the hit test only) issues them, the other half uses what came.
+// Hit test: one 4-byte load.
+__device__ __forceinline__ uint32_t remap_word(const RemapBlock* __restrict__ remap, int64_t g) {
     const uint32_t blk = (uint32_t)(g / kRemapRowsPerBlock);
-    const uint32_t r = (uint32_t)(g - (int64_t)blk * kRemapRowsPerBlock);
-    const uint32_t word = __ldg(&remap[blk].w[1 + (r >> 5)]);
-    return (word >> (r & 31)) & 1u;
+    return __ldg(&remap[blk].w[1 + ((uint32_t)(g - (int64_t)blk * kRemapRowsPerBlock) >> 5)]);
 }
+__device__ __forceinline__ bool remap_hit(uint32_t word, int64_t g) {        // (a block's rows begin at a multiple of 32)
+    return (word >> (g & 31)) & 1u;
+}
+static_assert(kRemapRowsPerBlock % 32 == 0, "whole words");
 
 // Slot of global row g, or -1: one 32-byte sector.
-__device__ __forceinline__ int32_t remap_slot(const RemapBlock* __restrict__ remap, int64_t g) {
+struct RemapSector {
+    uint4 lo, hi;
+};
+__device__ __forceinline__ RemapSector remap_sector(const RemapBlock* __restrict__ remap, int64_t g) {
     const uint32_t blk = (uint32_t)(g / kRemapRowsPerBlock);
-    const uint32_t r = (uint32_t)(g - (int64_t)blk * kRemapRowsPerBlock);
-    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(&remap[blk].w[0]));
-    const uint4 hi = __ldg(reinterpret_cast<const uint4*>(&remap[blk].w[4]));
-    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    return {__ldg(reinterpret_cast<const uint4*>(&remap[blk].w[0])), __ldg(reinterpret_cast<const uint4*>(&remap[blk].w[4]))};
+}
+__device__ __forceinline__ int32_t remap_slot(const RemapSector& s, int64_t g) {
+    const uint32_t r = (uint32_t)(g % kRemapRowsPerBlock);
+    const uint32_t w[8] = {s.lo.x, s.lo.y, s.lo.z, s.lo.w, s.hi.x, s.hi.y, s.hi.z, s.hi.w};
     const uint32_t wi = 1 + (r >> 5), bit = r & 31;
     uint32_t slot = w[0];
     uint32_t word = 0;
@@ -318,29 +326,77 @@ __host__ __device__ __forceinline__ uint64_t randomize64(uint64_t g) {
     return ((uint64_t)l << 32) | r;
 }
 
-// Open-addressing table row id -> value (linear probing from randomize64(row) & mask; an empty entry holds -1).
+// Open-addressing table row id -> value (linear probing from randomize64(row) & mask; an empty entry holds -1).  A lookup asks
+// for the aligned four entries around its first one at a time -- one sector of keys, and their values with them --, so that
+// hardly any takes more than one trip to memory (one entry at a time: three or four, for the slowest lane of a warp).
 struct HashProbe {
-    const long long* keys;
+    const long long* keys;             // at least four entries
     const int32_t* vals;
     uint64_t mask;
-    __device__ __forceinline__ int32_t slot(int64_t g) const {
-        uint64_t h = randomize64((uint64_t)g) & mask;
-        for (uint64_t tries = 0; tries <= mask; ++tries) {
-            const long long k = __ldg(&keys[h]);
-            if (k == g) return __ldg(&vals[h]);
-            if (k < 0) return -1;
-            h = (h + 1) & mask;
+    struct HitRequest {
+        longlong2 k01, k23;
+    };
+    struct Request {
+        HitRequest k;
+        int4 v;
+    };
+    __device__ __forceinline__ uint64_t home(int64_t g) const { return randomize64((uint64_t)g) & mask; }
+    __device__ __forceinline__ HitRequest keys_at(uint64_t four) const {
+        const longlong2* p = reinterpret_cast<const longlong2*>(keys + four);
+        return {__ldg(p), __ldg(p + 1)};
+    }
+    __device__ __forceinline__ HitRequest request_hit(int64_t g) const { return keys_at(home(g) & ~3ull); }
+    __device__ __forceinline__ Request request(int64_t g) const {
+        const uint64_t four = home(g) & ~3ull;
+        return {keys_at(four), __ldg(reinterpret_cast<const int4*>(vals + four))};
+    }
+    // which of the four entries, from `from` on, is the first that holds g or nothing (4: none does); found: it holds g
+    static __device__ __forceinline__ int stop(const HitRequest& r, int from, int64_t g, bool* found) {
+        const long long k[4] = {r.k01.x, r.k01.y, r.k23.x, r.k23.y};
+        int at = 4;
+        *found = false;
+#pragma unroll
+        for (int i = 3; i >= 0; --i)
+            if (i >= from && (k[i] == g || k[i] < 0)) {
+                at = i;
+                *found = k[i] == g;
+            }
+        return at;
+    }
+    // where g is beyond its first four entries, or -1
+    __device__ __forceinline__ int64_t further(int64_t g) const {
+        uint64_t four = home(g) & ~3ull;
+        for (uint64_t seen = 0; seen <= mask; seen += 4) {           // (back at the first four: those in front of its home)
+            four = (four + 4) & mask;
+            bool found;
+            const int at = stop(keys_at(four), 0, g, &found);
+            if (at < 4) return found ? (int64_t)(four + at) : -1;
         }
         return -1;
     }
-    __device__ __forceinline__ bool hit(int64_t g) const { return slot(g) >= 0; }
+    __device__ __forceinline__ int32_t slot(const Request& r, int64_t g) const {
+        bool found;
+        const int at = stop(r.k, (int)(home(g) & 3), g, &found);
+        if (at < 4) return !found ? -1 : at == 0 ? r.v.x : at == 1 ? r.v.y : at == 2 ? r.v.z : r.v.w;
+        const int64_t h = further(g);
+        return h < 0 ? -1 : __ldg(&vals[h]);
+    }
+    __device__ __forceinline__ bool hit(const HitRequest& r, int64_t g) const {
+        bool found;
+        const int at = stop(r, (int)(home(g) & 3), g, &found);
+        return at < 4 ? found : further(g) >= 0;
+    }
 };
 
 // The dense form used by the 32-bit path: one 32-byte block per 224 rows (see RemapBlock).
 struct BitmapProbe {
     const RemapBlock* remap;
-    __device__ __forceinline__ int32_t slot(int64_t g) const { return remap_slot(remap, g); }
-    __device__ __forceinline__ bool hit(int64_t g) const { return remap_hit(remap, g); }
+    using Request = RemapSector;
+    using HitRequest = uint32_t;
+    __device__ __forceinline__ Request request(int64_t g) const { return remap_sector(remap, g); }
+    __device__ __forceinline__ HitRequest request_hit(int64_t g) const { return remap_word(remap, g); }
+    __device__ __forceinline__ int32_t slot(const Request& r, int64_t g) const { return remap_slot(r, g); }
+    __device__ __forceinline__ bool hit(HitRequest r, int64_t g) const { return remap_hit(r, g); }
 };
 
 // ---- the cold-row bitmap --------------------------------------------------------------------------------------
@@ -383,18 +439,19 @@ __device__ __forceinline__ void clear_cold_chain(const ColdMarks& marks) {
         marks.chain[i] = 0ull;
 }
 
-// A lookup of X that addresses row g (inside the model): its cache slot if the row is popular; otherwise the row is
-// marked in the bitmap and the result is -2 - g.  (A row that is marked already, as popular cold rows are, costs a load.)
-__device__ __forceinline__ int32_t classify_cold(const BitmapProbe& remap, int64_t g, const ColdMarks& marks) {
-    const int32_t slot = remap.slot(g);
-    if (slot >= 0) return slot;
-    const int64_t word = g >> 5;
+// A lookup of X that addresses row g (inside the model) becomes its cache slot if the row is popular; otherwise the row is
+// marked in the bitmap and the lookup becomes -2 - g.  (A row that is marked already, as popular cold rows are, costs a load:
+// marks.bits[g >> 5], `word` below.)
+__device__ __forceinline__ int32_t cold_id(int64_t g) { return (int32_t)(-2 - g); }
+__device__ __forceinline__ void mark_cold(const ColdMarks& marks, int64_t g, uint32_t word) {
     const uint32_t bit = 1u << (g & 31);
-    if (!(marks.bits[word] & bit)) {
-        const uint32_t old = atomicOr(&marks.bits[word], bit);
-        if (old == 0u && marks.summary) atomicOr(&marks.summary[word >> 5], 1u << (word & 31));
+    if (word & bit) return;
+    const int64_t at = g >> 5;
+    if (marks.summary == nullptr) {
+        atomicOr(&marks.bits[at], bit);              // (nothing comes back, so nothing is waited for)
+    } else if (atomicOr(&marks.bits[at], bit) == 0u) {
+        atomicOr(&marks.summary[at >> 5], 1u << (at & 31));
     }
-    return (int32_t)(-2 - g);
 }
 
 // Rows are marked and ranked in two kernels or two calls, and the marks must be gone when the next mini-batch's are set: a

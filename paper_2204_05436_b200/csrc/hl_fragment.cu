@@ -61,6 +61,7 @@ __device__ void partition_by_flags(const uint32_t* words, int B, int32_t* __rest
         s_before[threadIdx.x] = before + earlier + incl - __popc(word);
         __syncthreads();
         const int first = w0 * 32, last = min(B, first + NT * 32);
+#pragma unroll 8
         for (int b = first + threadIdx.x; b < last; b += NT) {
             const uint32_t m = s_word[(b - first) >> 5];
             const int bit = b & 31;
@@ -84,7 +85,7 @@ __device__ void partition_by_flags(const uint32_t* words, int B, int32_t* __rest
 // HashProbe: the hashed remap of the wide-id path).
 // chain / n_chain: the state of k_frag_place's chain, cleared here.
 template <bool SHORT_BAGS, class Probe>
-__global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __restrict__ indices,
+__global__ void __launch_bounds__(kFlagThreads, 4) k_frag_flags(const int32_t* __restrict__ indices,
                                                              const int32_t* __restrict__ offsets, int B, int T, int S,
                                                              const int64_t* __restrict__ table_base, Probe remap,
                                                              uint32_t* words, int32_t* __restrict__ perm,
@@ -117,19 +118,36 @@ __global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __re
                     base[u] = t < T ? table_base[t] : 0;
                     rows[u] = t < T ? table_base[t + 1] - base[u] : 0;
                 }
-                int32_t idx[U];
+                // the k-th lookups of the bags, the next ones on their way while these are looked up
+                int32_t idx[U], next[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u) idx[u] = lo[u] < hi[u] ? indices[lo[u]] : 0;
+                for (int u = 0; u < U; ++u) next[u] = lo[u] < hi[u] ? indices[lo[u]] : 0;
+                bool more = true;
+                for (int k = 0; more; ++k) {
+                    int64_t g[U];
+                    bool check[U];
+                    typename Probe::HitRequest found[U];
+                    more = false;
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    if (lo[u] < hi[u])
-                        miss |= idx[u] < 0 || idx[u] >= rows[u] || !remap.hit(base[u] + idx[u]);
-#pragma unroll
-                for (int u = 0; u < U; ++u)
-                    for (int32_t j = lo[u] + 1; j < hi[u]; ++j) {
-                        const int32_t i = indices[j];
-                        miss |= i < 0 || i >= rows[u] || !remap.hit(base[u] + i);
+                    for (int u = 0; u < U; ++u) {
+                        idx[u] = next[u];
+                        if (lo[u] + k + 1 < hi[u]) {
+                            next[u] = indices[lo[u] + k + 1];
+                            more = true;
+                        }
                     }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const bool in = lo[u] + k < hi[u];
+                        check[u] = in && idx[u] >= 0 && idx[u] < rows[u];
+                        miss |= in && !check[u];
+                        g[u] = base[u] + idx[u];
+                        if (check[u]) found[u] = remap.request_hit(g[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (check[u]) miss |= !remap.hit(found[u], g[u]);
+                }
             }
             const unsigned m = __ballot_sync(0xffffffffu, miss);
             if (lane == 0 && m) atomicOr(&s_miss, m);
@@ -149,13 +167,19 @@ __global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __re
                 for (int32_t j0 = lo + part * 32; j0 < hi; j0 += share * 32 * U) {
                     int32_t idx[U];
                     bool hit[U];
+                    typename Probe::HitRequest found[U];
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const int32_t j = j0 + u * share * 32 + lane;
                         idx[u] = j < hi ? indices[j] : -1;
                     }
 #pragma unroll
-                    for (int u = 0; u < U; ++u) hit[u] = idx[u] >= 0 && idx[u] < rows && remap.hit(base + idx[u]);
+                    for (int u = 0; u < U; ++u) {
+                        hit[u] = idx[u] >= 0 && idx[u] < rows;
+                        if (hit[u]) found[u] = remap.request_hit(base + idx[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < U; ++u) hit[u] = hit[u] && remap.hit(found[u], base + idx[u]);
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         const int32_t j = j0 + u * share * 32 + lane;
@@ -192,7 +216,7 @@ __global__ void __launch_bounds__(kFlagThreads) k_frag_flags(const int32_t* __re
 // ---- placing --------------------------------------------------------------------------------------------------
 // The lookups of X are written as global row ids (int64 on the wide path).  With MARK (the scheduler's calls) the first half
 // of the cold-row search is done on the way instead: a popular row becomes its slot, any other row g is marked in the
-// cold-row bitmap and written as -2 - g (classify_cold).
+// cold-row bitmap and written as -2 - g (mark_cold).
 //
 // The chain between tiles carries two sums, lookups of O and lookups of X: 31 bits each, below two flag bits.
 constexpr int kHalf = 31;
@@ -253,14 +277,36 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
     // what the first lookup of a short bag becomes (ready before the tile knows where it goes: the loads behind it, index and
     // popular-row block, are in flight while the tiles exchange their sums)
     NonId head[ITEMS];
-    auto resolve = [&](bool is_pop, int64_t base, int64_t rows, int32_t idx) -> NonId {
-        if (is_pop) return (NonId)remap.slot(base + idx);    // every lookup of a popular input is in range and popular
-        if (idx < 0 || idx >= rows) {
-            set_status(a.status, HL_EBOUNDS);
-            return (NonId)-1;
+    // What `n` lookups become; the loads of all of them are requested before the first is waited for.  in: there is one;
+    // is_pop: of a popular input (then it is in range and popular).
+    auto resolve = [&](auto count, const bool* in, const bool* is_pop, const int64_t* base, const int64_t* rows,
+                       const int32_t* idx, NonId* id) {
+        constexpr int n = decltype(count)::value;
+        typename Probe::Request found[n];
+        uint32_t word[n];
+        bool look[n];
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            id[i] = (NonId)-1;
+            look[i] = in[i] && (is_pop[i] || (idx[i] >= 0 && idx[i] < rows[i]));
+            if (in[i] && !look[i]) set_status(a.status, HL_EBOUNDS);
+            if (look[i] && (MARK || is_pop[i])) found[i] = remap.request(base[i] + idx[i]);
+            word[i] = 0;
+            if constexpr (MARK)
+                if (look[i] && !is_pop[i]) word[i] = marks.bits[(base[i] + idx[i]) >> 5];
         }
-        if constexpr (MARK) return (NonId)classify_cold(remap, base + idx, marks);
-        else return (NonId)(base + idx);
+#pragma unroll
+        for (int i = 0; i < n; ++i) {
+            if (!look[i]) continue;
+            const int64_t g = base[i] + idx[i];
+            if constexpr (MARK) {
+                const int32_t slot = remap.slot(found[i], g);
+                id[i] = slot >= 0 || is_pop[i] ? slot : cold_id(g);
+                if (slot < 0 && !is_pop[i]) mark_cold(marks, g, word[i]);
+            } else {
+                id[i] = is_pop[i] ? (NonId)remap.slot(found[i], g) : (NonId)g;
+            }
+        }
     };
     int32_t start[ITEMS], all = 0, pop = 0;          // where the bag's lookups go, counted from the warp's first one
 #pragma unroll
@@ -292,15 +338,16 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
     if (!LISTS) {
         int32_t idx[ITEMS];
         int64_t base[ITEMS], rows[ITEMS];
+        bool in[ITEMS], is_pop[ITEMS];
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-            idx[i] = len[i] > 0 ? a.indices[src_lo[i]] : 0;
+            in[i] = len[i] > 0;
+            is_pop[i] = first + (warp * ITEMS + i) * 32 + lane < pop_bags;
+            idx[i] = in[i] ? a.indices[src_lo[i]] : 0;
             base[i] = a.table_base[table[i]];
             rows[i] = a.table_base[table[i] + 1] - base[i];
         }
-#pragma unroll
-        for (int i = 0; i < ITEMS; ++i)
-            head[i] = len[i] > 0 ? resolve(first + (warp * ITEMS + i) * 32 + lane < pop_bags, base[i], rows[i], idx[i]) : 0;
+        resolve(std::integral_constant<int, ITEMS>(), in, is_pop, base, rows, idx, head);
     }
     // the dense features follow their inputs: dense_out[i, :] = dense[perm[i], :]
     if (a.dense != nullptr) {
@@ -333,7 +380,10 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
                 if (out >= 0) set_status(a.status, HL_ECAPACITY);
                 break;
             }
-            const NonId id = resolve(is_pop, base, rows, a.indices[lo + j]);
+            const bool in = true;
+            const int32_t idx = a.indices[lo + j];
+            NonId id;
+            resolve(std::integral_constant<int, 1>(), &in, &is_pop, &base, &rows, &idx, &id);
             if (is_pop) a.pop_ids[out + j] = (int32_t)id;
             else non_ids[out + j] = id;
         }
@@ -387,8 +437,7 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
                     rows[u] = a.table_base[t + 1] - base[u];
                 }
                 NonId id[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) id[u] = in[u] ? resolve(pop_bag[u], base[u], rows[u], idx[u]) : 0;
+                resolve(std::integral_constant<int, U>(), in, pop_bag, base, rows, idx, id);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     if (!in[u]) continue;
@@ -419,9 +468,9 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
     const int64_t n_bags = (int64_t)T * B * S;
     // one list per row of bags, unless nearly every bag has just one lookup
     const bool lists = 4 * b->nnz > 5 * n_bags;
-    // Bags per tile: 256 where there are few bags (the tiles are the parallelism) or lists of lookups, 1 024 from one tile
-    // per SM on.
-    const int items = lists || n_bags <= (int64_t)kThreads * sms ? 1 : 4;
+    // Bags per tile: 256 where there are few bags (the tiles are the parallelism) or lists of lookups, 512 from one tile
+    // per SM on (106 K bags 9.1 us, with 1 024 10.2, with 256 8.9; 426 K beside a pipeline's other kernels 31, 46, 42).
+    const int items = lists || n_bags <= (int64_t)kThreads * sms ? 1 : 2;
     const int n_tiles = (int)div_up(n_bags, kThreads * items);
     // the tally of finished CTAs of the flags kernel: word 0 of the chain words (zero between calls: cleared when the
     // context is created and by the CTA that counts to the end); the chain proper is cleared by the flags kernel
@@ -438,7 +487,7 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
                            table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles));
     const auto place = lists        ? k_frag_place<true, 1, MARK, Probe, NonId>
                        : items == 1 ? k_frag_place<false, 1, MARK, Probe, NonId>
-                                    : k_frag_place<false, 4, MARK, Probe, NonId>;
+                                    : k_frag_place<false, 2, MARK, Probe, NonId>;
     HL_CUDA_TRY(launch(place, n_tiles, kThreads, stream, a, probe, non_ids, marks));
     note_launches(2);
     HL_LAUNCH_CHECK();

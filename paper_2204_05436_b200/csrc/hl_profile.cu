@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(kThreads) k_remap_prefix(const int32_t* __rest
 __global__ void __launch_bounds__(kThreads) k_remap_dense(const RemapBlock* __restrict__ remap, int64_t N,
                                                           int32_t* __restrict__ out) {
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < N; g += (int64_t)gridDim.x * blockDim.x)
-        out[g] = remap_slot(remap, g);
+        out[g] = remap_slot(remap_sector(remap, g), g);
 }
 
 }  // namespace
