@@ -171,12 +171,13 @@ __global__ void __launch_bounds__(kThreads) k_sort_digit_hist(const int32_t* __r
 // One pass: stable scatter by one digit.  Order of the items of a tile: warp-major, then round, then lane.
 // ghist: this pass's 256 digit counts; tstat[tile][256]: status words, zero on entry.  A tile is the CTA's block index: CTAs
 // are dispatched in that order, so those of the tiles before have started.  With few tiles a pass is a chain of latencies:
-// everything that does not depend on another load is requested first, and the tile is put in order in shared memory while the
-// tiles before publish their sums.  With many it is bound by the instructions that rank the items.  (So indices are 32 bits,
-// a full tile checks no bounds, and a warp writes runs of one digit: 2.6 M pairs 32.8 -> 26.3 us a pass, 1.3 M 20.1 -> 17.4,
-// 426 K 12.0 -> 11.3, 333 K 11.1 -> 9.3, 42 K 9.2 -> 7.2; tiles of 3 072 pairs 26.1, 16.7, 10.6, 10.1, 7.6; of 4 096 in 512
-// threads 25.6, 17.4, 11.3, 11.2, 9.2.)
-__global__ void __launch_bounds__(kThreads, 4) k_sort_pass(const int32_t* __restrict__ keys_in,
+// everything that does not depend on another load is requested first.  With many it is bound by the instructions that rank the
+// items (so indices are 32 bits) and by the places that a warp writes to: ORDER checks no bounds in a full tile, puts the tile in
+// order in shared memory first, while the tiles before publish their sums, and writes runs of one digit.  us a pass, before /
+// without / with it: 42 K pairs 5.8 / 5.6 / 6.0, 106 K 6.8 / 6.6 / 6.9, 250 K 7.7 / 7.4 / 7.7, 426 K 10.2 / - / 9.3, 1.3 M 17.9 / - /
+// 15.0, 2.6 M 31.5 / - / 26.  (Ordered tiles of 3 072 pairs, or of 4 096 in 512 threads: within 5 %.)
+template <bool ORDER>
+__global__ void __launch_bounds__(kThreads, ORDER ? 4 : 1) k_sort_pass(const int32_t* __restrict__ keys_in,
                                                            const int32_t* __restrict__ vals_in,
                                                            int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out,
                                                            const int32_t* d_n, int64_t n_max, int shift,
@@ -185,7 +186,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_pass(const int32_t* __rest
                                                            int64_t stall_tile) {
     constexpr int kWarps = kThreads / 32;
     __shared__ uint32_t cnt[kWarps][256];
-    __shared__ uint2 ordered[kSortTile];
+    __shared__ uint2 ordered[ORDER ? kSortTile : 1];
     __shared__ uint32_t digit_base[256];
     __shared__ int scan_smem[40];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_pass(const int32_t* __rest
     const int here = min(kSortTile, n - first);
     const bool full = here == kSortTile;
     const int mine = warp * (32 * kItems) + lane;                    // this lane's items: mine + 32 * r
-    auto valid = [&](int r) { return full || mine + r * 32 < here; };
+    auto valid = [&](int r) { return (ORDER && full) || mine + r * 32 < here; };
     uint32_t key[kItems], val[kItems], rank[kItems];
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
@@ -230,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_pass(const int32_t* __rest
     uint32_t* my = tstat + (int64_t)tile * 256 + d;
     if (tile > 0 && tile != stall_tile) st_relaxed(my, kFlagAgg | total);
     int all;
-    const uint32_t start = (uint32_t)block_exclusive_scan((int)total, scan_smem, all);
+    const uint32_t start = ORDER ? (uint32_t)block_exclusive_scan((int)total, scan_smem, all) : 0u;
     uint32_t run = start;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {
@@ -238,9 +239,11 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_pass(const int32_t* __rest
         run += of_warp[w];
     }
     const uint32_t gbase = (uint32_t)block_exclusive_scan(of_digit, scan_smem, all);   // keys with a smaller digit
+    if (ORDER) {
 #pragma unroll
-    for (int r = 0; r < kItems; ++r)
-        if (valid(r)) ordered[my_cnt[(key[r] >> shift) & 255u] + rank[r]] = make_uint2(key[r], val[r]);
+        for (int r = 0; r < kItems; ++r)
+            if (valid(r)) ordered[my_cnt[(key[r] >> shift) & 255u] + rank[r]] = make_uint2(key[r], val[r]);
+    }
     uint32_t before = 0;                                             // items of the digit in earlier tiles
     if (tile > 0) {
         // walk back kLook tiles at a time (32 at a time was no faster and cost 16 registers): the kLook status
@@ -277,13 +280,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_sort_pass(const int32_t* __rest
 #pragma unroll
     for (int r = 0; r < kItems; ++r) {
         const int i = r * kThreads + threadIdx.x;
-        if (full || i < here) {
-            const uint2 x = ordered[i];
-            const uint32_t pos = digit_base[(x.x >> shift) & 255u] + i;
-            if (pos < (uint32_t)n) {             // always true unless a chain poll gave up
-                keys_out[pos] = (int32_t)x.x;
-                vals_out[pos] = (int32_t)x.y;
-            }
+        if (ORDER ? !(full || i < here) : !valid(r)) continue;
+        const uint2 x = ORDER ? ordered[i] : make_uint2(key[r], val[r]);
+        const uint32_t dg = (x.x >> shift) & 255u, pos = digit_base[dg] + (ORDER ? (uint32_t)i : my_cnt[dg] + rank[r]);
+        if (pos < (uint32_t)n) {                 // always true unless a chain poll gave up
+            keys_out[pos] = (int32_t)x.x;
+            vals_out[pos] = (int32_t)x.y;
         }
     }
 }
@@ -384,6 +386,7 @@ __global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__
 }
 
 constexpr int kClusterNT = 512, kClusterItems = 4;
+constexpr int64_t kOrderTiles = 148;              // tiles of a pass from which on they are put in order first (k_sort_pass)
 
 // CTAs of the widest cluster the current device can place: 16 (a non-portable size), 8, or 0; asked once per device.
 int sort_cluster_ctas() {
@@ -460,9 +463,9 @@ int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n,
         note_launches(1);
     }
     for (int p = 0; p < passes; ++p)
-        HL_CUDA_TRY(launch(k_sort_pass, (unsigned)n_tiles, kThreads, stream, keys[p & 1], vals[p & 1], keys[(p & 1) ^ 1],
-                           vals[(p & 1) ^ 1], d_n, n_max, 8 * p, ghist + 256 * p,
-                           tstat + (size_t)p * n_tiles * 256, status, w.max_polls, w.stall_tile));
+        HL_CUDA_TRY(launch(n_tiles > kOrderTiles ? k_sort_pass<true> : k_sort_pass<false>, (unsigned)n_tiles, kThreads,
+                           stream, keys[p & 1], vals[p & 1], keys[(p & 1) ^ 1], vals[(p & 1) ^ 1], d_n, n_max, 8 * p,
+                           ghist + 256 * p, tstat + (size_t)p * n_tiles * 256, status, w.max_polls, w.stall_tile));
     note_launches(passes);
     HL_LAUNCH_CHECK();
     return HL_OK;
