@@ -50,26 +50,43 @@ __global__ void __launch_bounds__(kThreads) k_trk_keys(const int32_t* __restrict
         }
         d_n[0] = (int32_t)(L < 0 ? 0 : L);
     }
-    for (int64_t bag = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; bag < n_bags;
-         bag += (int64_t)gridDim.x * blockDim.x) {
-        const int t = (int)(bag / bags_per_table);
-        const int64_t base = table_base[t], rows = table_base[t + 1] - base;
-        const int64_t lo = offsets[bag], hi = offsets[bag + 1];
-        for (int64_t j = lo; j < hi && j < max_nnz; ++j) {
-            const int32_t idx = indices[j];
-            uint32_t key = n_sets;
-            int32_t val = -1;
-            if (idx < 0 || idx >= rows) {
-                set_status(status, HL_EBOUNDS);
-            } else {
-                const uint32_t g = (uint32_t)(base + idx);
-                key = randomizer(g) % n_sets;
-                val = (int32_t)g;
-            }
-            keys[j] = (int32_t)key;
-            vals[j] = val;
-            if (HIST)
-                for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 255u], 1u);
+    // the lookup at position j, of table t (first row `base`, so many rows)
+    auto put = [&](int64_t j, int32_t idx, int64_t base, int64_t rows) {
+        uint32_t key = n_sets;
+        int32_t val = -1;
+        if (idx < 0 || idx >= rows) {
+            set_status(status, HL_EBOUNDS);
+        } else {
+            const uint32_t g = (uint32_t)(base + idx);
+            key = randomizer(g) % n_sets;
+            val = (int32_t)g;
+        }
+        keys[j] = (int32_t)key;
+        vals[j] = val;
+        if (HIST)
+            for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 255u], 1u);
+    };
+    // a thread's bags, U at a time: their offsets and first lookups are asked for together
+    constexpr int U = 4;
+    const int64_t n_threads = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t bag0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; bag0 < n_bags; bag0 += U * n_threads) {
+        int64_t lo[U], hi[U], base[U], rows[U];
+        int32_t idx[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t bag = min(bag0 + u * n_threads, n_bags - 1);
+            const uint32_t t = (uint32_t)bag / (uint32_t)bags_per_table;             // (fewer than 2^30 bags)
+            base[u] = table_base[t];
+            rows[u] = table_base[t + 1] - base[u];
+            lo[u] = offsets[bag];
+            hi[u] = bag0 + u * n_threads < n_bags ? min((int64_t)offsets[bag + 1], max_nnz) : lo[u];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) idx[u] = lo[u] < hi[u] ? indices[lo[u]] : 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (lo[u] < hi[u]) put(lo[u], idx[u], base[u], rows[u]);
+            for (int64_t j = lo[u] + 1; j < hi[u]; ++j) put(j, indices[j], base[u], rows[u]);
         }
     }
     if (HIST) {
@@ -82,27 +99,32 @@ __global__ void __launch_bounds__(kThreads) k_trk_keys(const int32_t* __restrict
 }
 
 // One warp per 32 positions of the sorted list: every position where a new set's run begins is a head, and the warp
-// replays, head after head, the accesses of that set (the run may reach far beyond the warp's own 32 positions; the
-// warps there find no head in it and leave it alone).  While a set is replayed lane w holds its way w.
+// replays, head after head, the accesses of that set (the run of the last head may reach far beyond the warp's own 32 positions;
+// the warps there find no head in it and leave it alone).  A set's ways are held one per lane; W lanes (the power of two that
+// holds the ways) replay a set, so that 32 / W sets go on side by side.  The last head's run is then replayed by its W lanes
+// alone, up to 32 lookups at a time.
 //
-// What bounds it is latency: of a set's blocks, which come from DRAM, and, in the set of a popular row (thousands of
-// lookups of a mini-batch), of the lookups themselves.  So the blocks of the next two heads are on their way while one is
-// replayed, the 64 lookups behind the warp's first stay in registers, and beyond them four groups of 32 are read at once.
-// 426 K lookups, 131 072 sets of 16: the whole update, with its sort, takes 78 us; with every load waited for where it is
-// needed, and the digits counted in a kernel of their own, 112 us.
+// What bounds it is the chain of votes per access, and latency: of a set's blocks, which come from DRAM, and, in the set of a
+// popular row (thousands of lookups of a mini-batch), of the lookups themselves.  So the blocks of the next rounds' sets are on
+// their way while one round's are replayed, the 64 lookups behind the warp's first stay in registers, and beyond them four
+// groups of 32 are read at once (eight: no faster).  426 K lookups, 131 072 sets of 16, the whole update: 72.9 us with a set per
+// warp, 66.2 so (replay 30.1 -> 26.7, keys 8.3 -> 7.2); sets of 8 74.0 -> 64.7; 10 K lookups 26.4 -> 21.6.  (Six CTAs per
+// multiprocessor, with the registers that leaves: 31.7.)
+template <int W>
 __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ vals,
                                                          const int32_t* __restrict__ d_n, int64_t n_max,
                                                          int32_t* __restrict__ tags, uint8_t* __restrict__ rrpv,
                                                          int64_t n_sets, int ways,
                                                          unsigned long long* __restrict__ d_hits) {
-    constexpr unsigned kAll = 0xffffffffu;
+    constexpr unsigned kAll = 0xffffffffu, kMine = W == 32 ? kAll : (1u << (W & 31)) - 1u;
+    constexpr int NG = 32 / W;                                   // sets side by side
     constexpr int kAhead = 4;                                    // groups of 32 lookups read at once
     int64_t n = d_n[0];
     n = n < 0 ? 0 : (n < n_max ? n : n_max);
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, way = lane % W, group = lane / W, shift = group * W;
     const int64_t n_warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    unsigned long long hits = 0;
+    unsigned hits = 0;                                           // of this lane's group
     struct Blocks {
         int64_t s;
         int tag, rr;
@@ -114,90 +136,122 @@ __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restri
         const int32_t k0 = key_at(p), k1 = key_at(p + 32), g0 = val_at(p), g1 = val_at(p + 32);
         const int32_t before = w0 > 0 ? keys[w0 - 1] : -1;
         const int32_t up = __shfl_up_sync(kAll, k0, 1);
-        unsigned heads = __ballot_sync(kAll, k0 >= 0 && k0 < n_sets && k0 != (lane ? up : before));
-        // a head's set and its blocks: -2 matches no row; RRPV -1 is never a victim and never aged
-        auto load = [&](unsigned hs) {
+        // positions where a run begins, of a set or of lookups that are skipped; heads: of a set
+        const unsigned begins = __ballot_sync(kAll, k0 != (lane ? up : before));
+        unsigned heads = begins & __ballot_sync(kAll, k0 >= 0 && k0 < n_sets);
+        if (!heads) continue;
+        const int last_head = 31 - __clz((int)heads);
+        // the next head of every group (32: none), and its blocks: -2 matches no row; RRPV -1 is never a victim and never aged
+        auto take = [&]() {
+            int mine = 32;
+#pragma unroll
+            for (int k = 0; k < NG; ++k) {
+                const int h = heads ? __ffs((int)heads) - 1 : 32;
+                heads &= heads - 1;
+                if (k == group) mine = h;
+            }
+            return mine;
+        };
+        auto load = [&](int h) {
             Blocks b{-1, -2, -1};
-            if (hs) {
-                b.s = __shfl_sync(kAll, k0, __ffs((int)hs) - 1);
-                if (lane < ways) {
-                    b.tag = tags[b.s * ways + lane];
-                    b.rr = (int)rrpv[b.s * ways + lane];
+            const int32_t s = __shfl_sync(kAll, k0, h & 31);
+            if (h < 32) {
+                b.s = s;
+                if (way < ways) {
+                    b.tag = tags[b.s * ways + way];
+                    b.rr = (int)rrpv[b.s * ways + way];
                 }
             }
             return b;
         };
-        Blocks next = load(heads), after = load(heads & (heads - 1));
-        while (heads) {
-            const int h = __ffs((int)heads) - 1;
-            heads &= heads - 1;
-            const Blocks now = next;
+        // one access of every group's set (active: it has one), row gg
+        auto access = [&](Blocks& b, int32_t gg, bool active) {
+            const unsigned hit = __ballot_sync(kAll, b.tag == gg) >> shift & kMine;
+            const unsigned r3 = __ballot_sync(kAll, b.rr == kRrpvMax) >> shift & kMine;
+            const unsigned r2 = __ballot_sync(kAll, b.rr == 2) >> shift & kMine;
+            const unsigned r1 = __ballot_sync(kAll, b.rr == 1) >> shift & kMine;
+            const unsigned r0 = __ballot_sync(kAll, b.rr == 0) >> shift & kMine;
+            if (!active) return;
+            if (hit) {
+                if (way == __ffs((int)hit) - 1) b.rr = 0;
+                hits += way == 0;
+            } else {                      // (no block at the maximum: the whole set ages until its oldest one is)
+                const int add = r3 ? 0 : r2 ? 1 : r1 ? 2 : 3;
+                const unsigned oldest = r3 ? r3 : r2 ? r2 : r1 ? r1 : r0;
+                if (b.rr >= 0) b.rr += add;
+                if (way == __ffs((int)oldest) - 1) {
+                    b.tag = gg;
+                    b.rr = kRrpvInsert;
+                }
+            }
+        };
+        auto store = [&](const Blocks& b) {
+            if (b.s >= 0 && way < ways) {
+                tags[b.s * ways + way] = b.tag;
+                rrpv[b.s * ways + way] = (uint8_t)b.rr;
+            }
+        };
+        int h = take(), h_next = take();
+        Blocks next = load(h), after = load(h_next);
+        while (__any_sync(kAll, h < 32)) {
+            Blocks now = next;
+            const int at = h;
             next = after;
-            const unsigned behind = heads & (heads - 1);
-            after = load(behind);
-            int32_t tag = now.tag;
-            int rr = now.rr;
-            int32_t last = -1;            // the row of the previous access
-            bool last_zero = false;       // ... which left that row at RRPV 0, so that repeating it changes nothing
-            // replays one group of up to 32 lookups; false: the run ended in it
-            auto replay = [&](int32_t k, int32_t g) {
-                const unsigned mine = __ballot_sync(kAll, k == (int32_t)now.s);
-                const int c = mine == kAll ? 32 : __ffs((int)~mine) - 1;                       // leading lanes of the run
-                if (last_zero && __all_sync(kAll, lane >= c || g == last)) {
-                    hits += c;                                                    // a burst of one popular row
+            h = h_next;
+            h_next = take();
+            after = load(h_next);
+            // its run: up to the next one's beginning, or, of the last head, what of it is among the 32
+            const unsigned behind = at < 31 ? begins & (kAll << (at + 1)) : 0u;
+            const int end = at < 32 ? (behind ? __ffs((int)behind) - 1 : 32) : 0;
+            for (int t = at; __any_sync(kAll, t < end); ++t) access(now, __shfl_sync(kAll, g0, t & 31), t < end);
+            // the last head's run may go on
+            const bool on = at == last_head && end == 32;
+            if (__any_sync(kAll, on)) {
+                const int from = __ffs((int)__ballot_sync(kAll, on)) - 1;            // a lane of the group it is in
+                const int32_t set = (int32_t)__shfl_sync(kAll, now.s, from);
+                // the row of the previous access, and whether that left it at RRPV 0, so that repeating it changes nothing
+                int32_t last = __shfl_sync(kAll, g0, 31);
+                bool last_zero = __any_sync(kAll, on && now.tag == last && now.rr == 0);
+                // replays one group of up to 32 lookups; false: the run ended in it
+                auto replay = [&](int32_t k, int32_t g) {
+                    const unsigned same = __ballot_sync(kAll, k == set);
+                    const int c = same == kAll ? 32 : __ffs((int)~same) - 1;                       // leading lanes of the run
+                    if (last_zero && __all_sync(kAll, lane >= c || g == last)) {
+                        if (on && way == 0) hits += c;                                // a burst of one popular row
+                        return c == 32;
+                    }
+                    for (int t = 0; t < c; ++t) {
+                        const int32_t gg = __shfl_sync(kAll, g, t);
+                        if (last_zero && gg == last) {
+                            hits += on && way == 0;
+                            continue;
+                        }
+                        access(now, gg, on);
+                        last = gg;
+                        last_zero = __any_sync(kAll, on && now.tag == gg && now.rr == 0);
+                    }
                     return c == 32;
-                }
-                for (int t = 0; t < c; ++t) {
-                    const int32_t gg = __shfl_sync(kAll, g, t);
-                    if (gg == last && last_zero) {
-                        ++hits;
-                        continue;
-                    }
-                    const unsigned hit = __ballot_sync(kAll, tag == gg);
-                    if (hit) {
-                        if (lane == __ffs((int)hit) - 1) rr = 0;
-                        last_zero = true;
-                        ++hits;
-                    } else {
-                        unsigned vm = __ballot_sync(kAll, rr == kRrpvMax);
-                        if (!vm) {   // age the whole set until its oldest block reaches the maximum
-                            const int add = __ballot_sync(kAll, rr == 2) ? 1 : __ballot_sync(kAll, rr == 1) ? 2 : 3;
-                            if (lane < ways) rr += add;
-                            vm = __ballot_sync(kAll, rr == kRrpvMax);
-                        }
-                        if (lane == __ffs((int)vm) - 1) {
-                            tag = gg;
-                            rr = kRrpvInsert;
-                        }
-                        last_zero = false;
-                    }
-                    last = gg;
-                }
-                return c == 32;
-            };
-            // the first 32 lookups of the run, out of the 64 at hand
-            const int from = (h + lane) & 31;
-            const int32_t ka = __shfl_sync(kAll, k0, from), kb = __shfl_sync(kAll, k1, from);
-            const int32_t ga = __shfl_sync(kAll, g0, from), gb = __shfl_sync(kAll, g1, from);
-            bool more = replay(h + lane < 32 ? ka : kb, h + lane < 32 ? ga : gb);
-            for (int64_t i = w0 + h + 32; more; i += 32 * kAhead) {
-                int32_t k[kAhead], g[kAhead];
+                };
+                bool more = replay(k1, g1);
+                for (int64_t i = w0 + 64; more; i += 32 * kAhead) {
+                    int32_t k[kAhead], g[kAhead];
 #pragma unroll
-                for (int u = 0; u < kAhead; ++u) {
-                    k[u] = key_at(i + 32 * u + lane);
-                    g[u] = val_at(i + 32 * u + lane);
-                }
+                    for (int u = 0; u < kAhead; ++u) {
+                        k[u] = key_at(i + 32 * u + lane);
+                        g[u] = val_at(i + 32 * u + lane);
+                    }
 #pragma unroll
-                for (int u = 0; u < kAhead; ++u)
-                    if (more) more = replay(k[u], g[u]);
+                    for (int u = 0; u < kAhead; ++u)
+                        if (more) more = replay(k[u], g[u]);
+                }
             }
-            if (lane < ways) {
-                tags[now.s * ways + lane] = tag;
-                rrpv[now.s * ways + lane] = (uint8_t)rr;
-            }
+            store(now);
         }
     }
-    if (lane == 0 && d_hits && hits) atomicAdd(d_hits, hits);
+    unsigned long long all = hits;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) all += __shfl_down_sync(kAll, all, d);
+    if (lane == 0 && d_hits && all) atomicAdd(d_hits, all);
 }
 
 // counts[row] = 4 - RRPV for every tracked row (the counters were cleared before).
@@ -275,7 +329,8 @@ extern "C" int32_t hl_tracker_update(hl_ctx* ctx, const hl_batch* b, int32_t* d_
     const int32_t st = radix_sort_pairs(r.bwd_keys, r.bwd_vals, r.bwd_n, ctx->max_nnz, key_bits, r.bwd_hist[0], r.status,
                                         &keys, &vals, stream, WaitCfg(), true);
     if (st != HL_OK) return st;
-    HL_CUDA_TRY(launch(k_trk_replay, grid_for(ctx->max_nnz, kThreads, kMaxGrid), kThreads, stream, keys, vals, r.bwd_n,
+    const auto replay = ways <= 8 ? k_trk_replay<8> : ways <= 16 ? k_trk_replay<16> : k_trk_replay<32>;
+    HL_CUDA_TRY(launch(replay, grid_for(ctx->max_nnz, kThreads, kMaxGrid), kThreads, stream, keys, vals, r.bwd_n,
                        ctx->max_nnz, d_tags, d_rrpv, n_sets, ways, d_hits));
     note_launches(1);
     HL_LAUNCH_CHECK();
