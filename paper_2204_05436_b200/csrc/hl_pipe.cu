@@ -153,14 +153,21 @@ void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense
                              prev.n_cold, st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, p->index, use);
     (void)hl_stage_cold(ctx, p->host_table, p->cache, w, rows, st.cold_rows, st.n_cold, st.fwd_src, p->link);
     launch_flush();
+    const auto update = [&](int which) {
+        (void)hl_embbag_bwd_apply2(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, which, any, 0.f, p->main);
+    };
     if (rows > 0)
         (void)fwd_and_forward_cold(ctx, p->cache, &st.pop, st.counts, st.pooled_pop, w_other, w, rows, st.fwd_src, st.n_cold,
                                    p->main);
+    else
+        (void)hl_embbag_fwd(ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main);
+    if (p->wb_mode == HL_PIPE_WB_AFTER_FORWARD) launch_flush();
+    if (!merge) update(0);
     launch_flush();
-    if (!merge) (void)hl_embbag_bwd_apply2(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 0, any, 0.f, p->main);
+    if (!merge) update(0);                                   // (by itself: what the first mini-batch launches)
     launch_flush();
     (void)hl_embbag_fwd(ctx, p->cache, &st.non, st.counts + 1, st.pooled_non, p->main);
-    if (!merge) (void)hl_embbag_bwd_apply2(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 1, any, 0.f, p->main);
+    if (!merge) update(1);
     else (void)hl_embbag_bwd_apply(ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n + 2, any, 0.f, p->main);
     (void)hl_scatter_cold_at(ctx, p->cache, w, rows, st.cold_rows, st.n_cold, p->host_table, p->wb);
 }
@@ -460,32 +467,44 @@ static int32_t queue_mini_batch(hl_pipe* p, const float* d_grad_pop, const float
     if (next && p->j_indexed - j >= n - 1) return HL_ECAPACITY;
     HL_PIPE_TRY(wait(p->main, e.index));
     if (p->wb_mode == HL_PIPE_WB_EXCLUSIVE && j >= 1) HL_PIPE_TRY(wait(p->main, p->ev[(j - 1) % n].scatter));
+    LaunchBatch popular(launches_of(p, j));
     {
         // with O's forward: the rows shared with mini-batch j-1, out of its staging window (its backward is done)
         Scope sc(p, HL_SPAN_FWD_POP, j, kMain);
-        LaunchBatch batch(launches_of(p, j));
         if (j >= 1 && p->window_rows > 0)
             HL_PIPE_TRY(fwd_and_forward_cold(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, w1, w0, p->window_rows,
                                              st.fwd_src, st.n_cold, p->main));
         else
             HL_PIPE_TRY(hl_embbag_fwd(p->ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main));
-        HL_PIPE_TRY(batch.end());
     }
-    HL_PIPE_TRY(record(e.forward, p->main));
-    if (p->wb_pending) {
-        // the write-back of j-1 starts when the popular forward of j is over: of all kernels of the main stream that
-        // one loses most next to a write-back
-        HL_PIPE_TRY(wait(p->wb, e.forward));
-        HL_PIPE_TRY(flush_scatter(p));
-    }
-    if (p->j_submitted == j + 1 && p->j_submitted < p->j_indexed) HL_PIPE_TRY(submit_link(p));   // mini-batch j+1
+    // The read of j+1's rows may start when those that j takes out of its window are gone.  It has to wait for the write-back of
+    // j-1 in any case, which began when this forward did and takes about as long as forward and update, so the event comes
+    // behind both, and they go out as one graph.  (In between it cost more than the 2 us from one graph to the next: the
+    // update waited behind what the read put on the chip.  One pipeline / three in turn on one chip, us per mini-batch: Tiny
+    // 36.3 -> 32.5 / 37.1 -> 32.7, click log 69.2 -> 68.3 / 77.4 -> 64.5, time series 58.3 -> 60.1 / 70.9 -> 57.4, DLRM-sized
+    // 146 -> 137 / 150 -> 132.)  The first mini-batch has no write-back before it, and one that is held over starts here.
+    const bool apart = j == 0 || p->wb_pending;
+    const auto read_next = [&]() -> int32_t {
+        HL_PIPE_TRY(popular.end());
+        HL_PIPE_TRY(record(e.forward, p->main));
+        if (p->wb_pending) {
+            // the write-back of j-1 starts when the popular forward of j is over: of all kernels of the main stream that
+            // one loses most next to a write-back
+            HL_PIPE_TRY(wait(p->wb, e.forward));
+            HL_PIPE_TRY(flush_scatter(p));
+        }
+        if (p->j_submitted == j + 1 && p->j_submitted < p->j_indexed) return submit_link(p);   // mini-batch j+1
+        return HL_OK;
+    };
+    if (apart) HL_PIPE_TRY(read_next());
     if (p->order == HL_PIPE_ORDER_FIG8) {
         Scope sc(p, HL_SPAN_BWD_POP, j, kMain);
-        LaunchBatch batch(launches_of(p, j));
+        LaunchBatch update(launches_of(p, j));               // (part of `popular`, unless that has ended)
         HL_PIPE_TRY(hl_embbag_bwd_apply2(p->ctx, p->cache, st.sorted_slots, st.sorted_bags, st.sorted_n, 0, d_grad_pop,
                                          lr, p->main));
-        HL_PIPE_TRY(batch.end());
+        HL_PIPE_TRY(update.end());
     }
+    if (!apart) HL_PIPE_TRY(read_next());
     HL_PIPE_TRY(wait(p->main, e.gather));
     LaunchBatch batch(launches_of(p, j));
     {
