@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__
     if (n == 0) return;                           // the same in all CTAs
     const int cta = (int)cluster.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int per = (n + CTAS - 1) / CTAS;        // pairs per CTA
+    const int per = max(2, (n + CTAS - 1) / CTAS);        // pairs per CTA (two at least: inv_per has 32 bits)
     const int rounds = (per + NT - 1) / NT;
     const uint32_t inv_per = (uint32_t)((0x100000000ull + per - 1) / per);       // pos / per = (pos * inv_per) >> 32
     const int here = max(0, min(n - cta * per, per));
