@@ -590,6 +590,27 @@ int32_t radix_sort_pairs(int32_t* keys[2], int32_t* vals[2], const int32_t* d_n,
 // counted = true.
 int64_t sort_clear_words(int64_t n_max, int key_bits, WaitCfg w);
 
+// Whether that many pairs are too many for one cluster, so that their sort is a chain of kernels or fills the chip.
+bool sort_is_long(int64_t n_max, WaitCfg w);
+
+// The sort of pairs that lie table by table (O's tables, then X's, or, merged, every table's of O and X together), each
+// table's by themselves: equal keys end up side by side, which is what the backward's sums need.
+struct SortSide {
+    const int32_t* offsets;
+    const int32_t* d_n_samples;
+    int32_t key_bias, unused;
+};
+struct SegmentArgs {
+    int32_t *keys_in, *vals_in;        // (scratch, if a table does not fit)
+    int32_t *keys_out, *vals_out;
+    SortSide side[2];
+    const int32_t* d_n_lookups;        // [0]: of the first side, [2]: of both
+    int32_t tables, max_batch, bags_per_sample, merge, passes, unused;
+    int64_t max_nnz;
+};
+bool sort_by_segments(int64_t n_max, int64_t n_bags, int tables, WaitCfg w);
+int32_t sort_segments(const SegmentArgs& a, cudaStream_t stream);
+
 // 32-bit words of histogram scratch radix_sort_pairs needs for at most max_nnz pairs.
 constexpr int64_t sort_hist_words(int64_t max_nnz) {
     const int64_t n_tiles = ((max_nnz > 0 ? max_nnz : 1) + kSortTile - 1) / kSortTile;
@@ -618,6 +639,7 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
 // sort's scratch, backward_sort_clear_words words of bwd_hist, is zero already.  d_sorted_slots / _bags may be null: the
 // result then stays in the context's scratch, at *out_slots / *out_bags.
 int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge);
+bool backward_sort_is_long(const hl_ctx* ctx);
 
 // The sort on a stream of its own, behind the pairs (event pairs_ready), with one of two sets of scratch (which): the
 // pairs of the next mini-batch, written with the other set, need not wait for it.

@@ -329,6 +329,8 @@ struct PairArgs {
     PairSide side[2];                  // the second one's pairs follow the first one's
     int sides;
     int bags_follow;                   // the second side's bags are numbered behind the first one's
+    int by_table;                      // the pairs lie table by table: of every table the first side's, then the second's
+    int bags_per_sample;               // ... and table
     int max_batch, bags_per_sample_all;
     int64_t n_slots, max_nnz;
     int32_t* keys;
@@ -378,7 +380,13 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pairs(PairArgs a) {
     for (int64_t all = thread / GROUP; all < bags0 + bags1; all += n_threads / GROUP) {
         const bool second = all >= bags0;
         const PairSide& s = a.side[second ? 1 : 0];
-        const int64_t bag = second ? all - bags0 : all, pos0 = second ? L0 : 0;
+        const int64_t bag = second ? all - bags0 : all;
+        int64_t pos0 = second ? L0 : 0;
+        if (a.by_table) {
+            const int tables = a.bags_per_sample_all / a.bags_per_sample;
+            const unsigned per_table = (unsigned)(second ? bags1 : bags0) / tables, t = (unsigned)bag / per_table;
+            pos0 = second ? a.side[0].offsets[(int64_t)(t + 1) * (bags0 / tables)] : a.side[1].offsets[(int64_t)t * (bags1 / tables)];
+        }
         const int32_t bag_value = (int32_t)(a.bags_follow ? all : bag);
         const int32_t lo = s.offsets[bag], hi = s.offsets[bag + 1];
         for (int32_t j = lo + (int)(thread % GROUP); j < hi; j += GROUP) {
@@ -1027,7 +1035,9 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
                        int32_t* caller_vals, int32_t* d_n_lookups, int32_t** out_keys, int32_t** out_vals,
                        cudaStream_t stream, const SortAside* aside = nullptr) {
     Regions& r = ctx->r;
-    const int key_bits = bits_for(max_key), passes = (key_bits + 7) / 8;
+    // (the schedules' pairs: fragment laid them out by table, and no row belongs to two)
+    const bool segments = assign && a.sides == 2 && sort_by_segments(ctx->max_nnz, ctx->max_bags, ctx->T, wait_cfg(ctx));
+    const int key_bits = bits_for(max_key), passes = segments ? 1 : (key_bits + 7) / 8;
     const int which = aside ? aside->which : 0;          // (with caller arrays, one of the two scratch buffers is free)
     uint32_t* sort_scratch = r.bwd_hist[which];
     int32_t* keys[2] = {r.bwd_keys[which], r.bwd_keys[which ^ 1]};
@@ -1042,6 +1052,8 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
     }
     a.max_batch = ctx->max_batch;
     a.bags_per_sample_all = ctx->T * ctx->S;
+    a.bags_per_sample = ctx->S;
+    a.by_table = segments && a.bags_follow;
     a.n_slots = ctx->hot_cap + ctx->staging_cap;
     a.max_nnz = ctx->max_nnz;
     a.keys = keys[0];
@@ -1051,7 +1063,7 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
     a.ghist = sort_scratch;
     a.passes = passes;
     // the tile sort wants its digit counts, which cost less here than in a sweep of their own
-    const int64_t clear_words = sort_clear_words(ctx->max_nnz, key_bits, wait_cfg(ctx));
+    const int64_t clear_words = segments ? 0 : sort_clear_words(ctx->max_nnz, key_bits, wait_cfg(ctx));
     const bool hist = clear_words > 0;
     if (hist && !cleared) HL_CUDA_TRY(hl::clear_words(sort_scratch, clear_words, stream));
     // lanes per bag: by the most lookups a bag has on average (bags of 20 out of at most 64: 20.8 us with 8 lanes, 22.2 with
@@ -1074,6 +1086,22 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
         HL_CUDA_TRY(cudaEventRecord(aside->pairs_ready, stream));
         HL_CUDA_TRY(cudaStreamWaitEvent(aside->stream, aside->pairs_ready, 0));
         stream = aside->stream;
+    }
+    if (segments) {
+        SegmentArgs g{};
+        g.keys_in = keys[0];
+        g.vals_in = vals[0];
+        g.keys_out = *out_keys = keys[1];
+        g.vals_out = *out_vals = vals[1];
+        for (int i = 0; i < 2; ++i) g.side[i] = {a.side[i].offsets, a.side[i].d_n_samples, a.side[i].key_bias, 0};
+        g.d_n_lookups = d_n_lookups;
+        g.tables = ctx->T;
+        g.max_batch = ctx->max_batch;
+        g.bags_per_sample = ctx->S;
+        g.merge = a.bags_follow;
+        g.passes = (bits_for(a.n_slots) + 7) / 8;
+        g.max_nnz = ctx->max_nnz;
+        return sort_segments(g, stream);
     }
     return radix_sort_pairs(keys, vals, d_n_lookups + (a.sides > 1 ? 2 : 0), ctx->max_nnz, key_bits, sort_scratch, r.status,
                             out_keys, out_vals, stream, wait_cfg(ctx), hist);
@@ -1157,7 +1185,10 @@ int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, 
 
 }  // namespace
 
+bool backward_sort_is_long(const hl_ctx* ctx) { return sort_is_long(ctx->max_nnz, wait_cfg(ctx)); }
+
 int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge) {
+    if (sort_by_segments(ctx->max_nnz, ctx->max_bags, ctx->T, wait_cfg(ctx))) return 0;
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     return sort_clear_words(ctx->max_nnz, bits_for(merge ? n_slots : 2 * n_slots + 1), wait_cfg(ctx));
 }

@@ -141,7 +141,7 @@ void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense
     const bool merge = p->order == HL_PIPE_ORDER_EQ5;
     const int64_t n_clear = backward_sort_clear_words(ctx, merge);
     const SortAside aside{p->sort, p->ev[j % n].pairs, (int)(j % 2)};
-    const SortAside* use = n_clear > 0 ? &aside : nullptr;
+    const SortAside* use = backward_sort_is_long(ctx) ? &aside : nullptr;
     const float* any = st.pooled_pop;                        // (some gradients)
     LaunchBatch batch(p->launches[j].get(), true);
     if (fragment_and_mark(ctx, b, d_dense, d_dense ? p->n_dense : 0, st.perm, st.counts, &st.pop, &st.non,
@@ -202,7 +202,7 @@ int32_t queue_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* i
     // set j % 2 was the sort's of mini-batch j-2.
     const int64_t n_clear = backward_sort_clear_words(p->ctx, merge);
     const SortAside aside{p->sort, e.pairs, (int)(j % 2)};
-    const SortAside* use = n_clear > 0 ? &aside : nullptr;
+    const SortAside* use = backward_sort_is_long(p->ctx) ? &aside : nullptr;
     if (use && j >= 2) {
         HL_PIPE_TRY(launch_flush() == cudaSuccess ? HL_OK : HL_ECUDA);
         HL_PIPE_TRY(wait(p->index, p->ev[(j - 2) % n].index));

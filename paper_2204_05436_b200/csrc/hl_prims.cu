@@ -94,6 +94,11 @@ __device__ __forceinline__ unsigned same_digit(uint32_t d, bool valid) {
     return peers;
 }
 
+constexpr size_t sort_smem_bytes(int threads, int items) {
+    return (size_t)threads / 32 * 256 * sizeof(uint32_t) + (size_t)threads * items * sizeof(uint2);
+}
+static_assert(sort_smem_bytes(512, 4) == sizeof(SortSmem<512, 4>), "the layout");
+
 // Ranks a warp's items among the warp's items of the same digit (order: round, then lane) and counts them into cnt.
 template <int ITEMS>
 __device__ __forceinline__ void rank_in_warp(const uint32_t (&key)[ITEMS], int rounds, int n_mine, int shift,
@@ -385,6 +390,171 @@ __global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__
     }
 }
 
+// ---- pairs that are grouped by table already ---------------------------------------------------------------------
+// Where the pairs of a mini-batch are written table by table and no slot belongs to two tables, equal slots lie in one
+// table's pairs, and all that the sums need is every table's pairs sorted by themselves: a cluster of CTAS CTAs per table (and
+// side, if O's and X's pairs are kept apart) does all passes as k_sort_cluster does, in one kernel for all tables.  What bounds
+// it is the chain count -> exchange -> scatter of a pass, with the larger tables' clusters on the chip together.  Alone, against
+// three chained passes: 86 K pairs of 21 tables 8.5 / 19 us, 107 K of 26 8.6 / 19, 129 K of 3 15.5 / 21, 333 K of 37 15.7 / 24, 426 K
+// of 26 18.5 / 28; 8 K of 8 tables 5.8, against 9.2 in one cluster.  (CTAs of 512 threads: 9.9, 9.9, 15.3, 21.5, 27.9, 7.6.)
+// A table with more pairs than the cluster holds (the host knows the average only) is sorted by one of its CTAs, tile by
+// tile through memory.
+template <int CTAS, int NT, int ITEMS>
+__global__ void __launch_bounds__(NT) k_sort_segments(SegmentArgs a) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    constexpr int PD = NT / 256;
+    extern __shared__ __align__(16) unsigned char sort_smem[];
+    SortSmem<NT, ITEMS>& sm = *reinterpret_cast<SortSmem<NT, ITEMS>*>(sort_smem);
+    __shared__ uint32_t cta_hist[256];            // this CTA's digit counts, read by the other CTAs
+    __shared__ uint32_t digit_base[256];
+    __shared__ int scan_smem[40];
+    // this cluster's pairs: [lo, lo + n)
+    const int segment = blockIdx.x / CTAS, cta = (int)cluster.block_rank();
+    const int which = a.merge ? 0 : segment / a.tables, table = a.merge ? segment : segment - which * a.tables;
+    auto starts = [&](const int32_t* offsets, const int32_t* d_n_samples, int t) {       // table t's first lookup of a side
+        const int samples = min(max(*d_n_samples, 0), a.max_batch);
+        return offsets[(int64_t)t * samples * a.bags_per_sample];
+    };
+    const int most = (int)min((int64_t)max(a.d_n_lookups[2], 0), a.max_nnz);
+    const int32_t* const offsets = which ? a.side[1].offsets : a.side[0].offsets;
+    const int32_t* const d_n_samples = which ? a.side[1].d_n_samples : a.side[0].d_n_samples;
+    int lo = starts(offsets, d_n_samples, table), hi = starts(offsets, d_n_samples, table + 1);
+    if (a.merge) {
+        lo += starts(a.side[1].offsets, a.side[1].d_n_samples, table);
+        hi += starts(a.side[1].offsets, a.side[1].d_n_samples, table + 1);
+    } else if (which) {
+        lo += a.d_n_lookups[0];
+        hi += a.d_n_lookups[0];
+    }
+    lo = min(max(lo, 0), most);
+    const int n = max(min(hi, most) - lo, 0);
+    const uint32_t bias = (uint32_t)(which ? a.side[1].key_bias : a.side[0].key_bias);
+    if (n == 0) return;                           // the same in all CTAs of the cluster
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int d = threadIdx.x / PD, q = threadIdx.x % PD;
+    if (n > CTAS * NT * ITEMS) {
+        if (cta != 0) return;
+        int32_t *kin = a.keys_in + lo, *vin = a.vals_in + lo, *kout = a.keys_out + lo, *vout = a.vals_out + lo;
+        constexpr int TILE = NT * ITEMS;
+        for (int p = 0; p < a.passes; ++p) {
+            const int shift = 8 * p;
+            if (threadIdx.x < 256) cta_hist[threadIdx.x] = 0;
+            __syncthreads();
+            for (int i = threadIdx.x; i < n; i += NT) atomicAdd(&cta_hist[((uint32_t)kin[i] - bias) >> shift & 255u], 1u);
+            __syncthreads();
+            const uint32_t smaller = scan_digits<PD>(cta_hist[d], scan_smem);
+            if (q == 0) digit_base[d] = smaller;
+            for (int tile = 0; tile < n; tile += TILE) {
+                const int n_mine = max(0, min(n - tile - warp * 32 * ITEMS, 32 * ITEMS)), at = tile + warp * 32 * ITEMS + lane;
+                uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
+#pragma unroll
+                for (int r = 0; r < ITEMS; ++r) {
+                    key[r] = r * 32 + lane < n_mine ? (uint32_t)kin[at + r * 32] - bias : 0u;
+                    val[r] = r * 32 + lane < n_mine ? (uint32_t)vin[at + r * 32] : 0u;
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) sm.cnt[warp][i * 32 + lane] = 0;
+                __syncwarp();
+                rank_in_warp<ITEMS>(key, ITEMS, n_mine, shift, sm.cnt[warp], rank);
+                __syncthreads();
+                const uint32_t total = prefix_over_warps<NT>(sm.cnt);
+                __syncthreads();
+#pragma unroll
+                for (int r = 0; r < ITEMS; ++r)
+                    if (r * 32 + lane < n_mine) {
+                        const uint32_t dg = (key[r] >> shift) & 255u, pos = digit_base[dg] + sm.cnt[warp][dg] + rank[r];
+                        kout[pos] = (int32_t)(key[r] + bias);
+                        vout[pos] = (int32_t)val[r];
+                    }
+                __syncthreads();
+                if (q == 0) digit_base[d] += total;
+                __syncthreads();
+            }
+            int32_t* const k = kin;
+            int32_t* const v = vin;
+            kin = kout;
+            vin = vout;
+            kout = k;
+            vout = v;
+        }
+        if (a.passes % 2 == 0)                    // (the last pass wrote the input's place)
+            for (int i = threadIdx.x; i < n; i += NT) {
+                kout[i] = kin[i];
+                vout[i] = vin[i];
+            }
+        return;
+    }
+    const int per = max(2, (n + CTAS - 1) / CTAS);        // pairs per CTA (two at least: inv_per has 32 bits)
+    const int rounds = (per + NT - 1) / NT;
+    const uint32_t inv_per = (uint32_t)((0x100000000ull + per - 1) / per);       // pos / per = (pos * inv_per) >> 32
+    const int here = max(0, min(n - cta * per, per));
+    const int first = warp * 32 * rounds;         // of this warp, within the CTA
+    const int n_mine = max(0, min(here - first, 32 * rounds));
+    uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        key[r] = val[r] = 0u;
+        if (r < rounds && r * 32 + lane < n_mine) {
+            key[r] = (uint32_t)a.keys_in[lo + cta * per + first + r * 32 + lane] - bias;
+            val[r] = (uint32_t)a.vals_in[lo + cta * per + first + r * 32 + lane];
+        }
+    }
+    for (int p = 0; p < a.passes; ++p) {
+        const int shift = 8 * p;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sm.cnt[warp][i * 32 + lane] = 0;
+        __syncwarp();
+        rank_in_warp<ITEMS>(key, rounds, n_mine, shift, sm.cnt[warp], rank);
+        __syncthreads();
+        const uint32_t total = prefix_over_warps<NT>(sm.cnt);
+        if (q == 0) cta_hist[d] = total;
+        cluster.sync();     // all counts published; all CTAs have taken the previous pass's pairs out of shared memory
+        uint32_t before = 0, all = 0;             // of this digit: in the CTAs before mine, in all CTAs
+#pragma unroll
+        for (int c = q; c < CTAS; c += PD) {
+            const uint32_t v = *cluster.map_shared_rank(&cta_hist[d], c);
+            if (c < cta) before += v;
+            all += v;
+        }
+#pragma unroll
+        for (int o = 1; o < PD; o <<= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+        const uint32_t smaller = scan_digits<PD>(all, scan_smem);
+        if (q == 0) digit_base[d] = smaller + before;
+        __syncthreads();
+        const bool last = p == a.passes - 1;
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            if (r >= rounds) break;
+            if (r * 32 + lane < n_mine) {
+                const uint32_t dg = (key[r] >> shift) & 255u;
+                const uint32_t pos = digit_base[dg] + sm.cnt[warp][dg] + rank[r];
+                if (last) {
+                    a.keys_out[lo + pos] = (int32_t)(key[r] + bias);
+                    a.vals_out[lo + pos] = (int32_t)val[r];
+                } else {
+                    const uint32_t owner = __umulhi(pos, inv_per);
+                    *cluster.map_shared_rank(&sm.pair[pos - owner * per], owner) = make_uint2(key[r], val[r]);
+                }
+            }
+        }
+        cluster.sync();     // every pair has arrived (after the last pass: no CTA leaves while others read its counts)
+        if (last) break;
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            if (r >= rounds) break;
+            if (r * 32 + lane < n_mine) {
+                const uint2 x = sm.pair[first + r * 32 + lane];
+                key[r] = x.x;
+                val[r] = x.y;
+            }
+        }
+    }
+}
+
 constexpr int kClusterNT = 512, kClusterItems = 4;
 constexpr int64_t kOrderTiles = 148;              // tiles of a pass from which on they are put in order first (k_sort_pass)
 
@@ -395,15 +565,15 @@ int sort_cluster_ctas() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
     const int k = known[dev].load(std::memory_order_acquire);
     if (k > 0) return k - 1;
-    auto can = [](auto* kernel, int ctas) {
-        constexpr size_t kBytes = sizeof(SortSmem<kClusterNT, kClusterItems>);
+    auto can = [](auto* kernel, int ctas, int threads, int items) {
+        const size_t kBytes = sort_smem_bytes(threads, items);
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = ctas;
         attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
         cfg.gridDim = dim3(ctas);
-        cfg.blockDim = dim3(kClusterNT);
+        cfg.blockDim = dim3(threads);
         cfg.dynamicSmemBytes = kBytes;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
@@ -412,9 +582,10 @@ int sort_cluster_ctas() {
                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBytes) == cudaSuccess &&
                cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1;
     };
-    const int ctas = can(k_sort_cluster<16, kClusterNT, kClusterItems>, 16)
+    const int ctas = can(k_sort_cluster<16, kClusterNT, kClusterItems>, 16, kClusterNT, kClusterItems) &&
+                             can(k_sort_segments<16, 256, 8>, 16, 256, 8) && can(k_sort_segments<16, 512, 8>, 16, 512, 8)
                          ? 16
-                         : (can(k_sort_cluster<8, kClusterNT, kClusterItems>, 8) ? 8 : 0);
+                         : (can(k_sort_cluster<8, kClusterNT, kClusterItems>, 8, kClusterNT, kClusterItems) ? 8 : 0);
     (void)cudaGetLastError();
     known[dev].store(ctas + 1, std::memory_order_release);
     return ctas;
@@ -427,6 +598,32 @@ int sort_cluster_ctas() {
 // (With a tile made to stall -- the test of the bounded waits -- the chained passes are what is asked for.)
 static bool sort_in_cluster(int64_t n_max, const WaitCfg& w) {
     return n_max <= (int64_t)sort_cluster_ctas() * kClusterNT * kClusterItems && w.stall_tile < 0;
+}
+
+bool sort_is_long(int64_t n_max, WaitCfg w) { return !sort_in_cluster(n_max, w); }
+
+// For contexts of one lookup per bag at most, on average: there the host knows how many pairs a table has, and takes a cluster
+// that holds them.  (Elsewhere it knows how many there could be.  Four times as many as there were, 37 clusters of 16 CTAs of 512
+// threads for 9 K pairs each took 67 us beside a pipeline's other kernels, where the chained passes take 3 x 15.)
+static int64_t segment_pairs(int64_t n_max, int tables) { return div_up(n_max, tables); }
+bool sort_by_segments(int64_t n_max, int64_t n_bags, int tables, WaitCfg w) {
+    const int64_t pairs = segment_pairs(n_max, tables);
+    return n_max > 0 && n_max <= n_bags && w.stall_tile < 0 &&
+           (pairs <= 16384 || (pairs <= 65536 && sort_cluster_ctas() == 16));
+}
+
+int32_t sort_segments(const SegmentArgs& a, cudaStream_t stream) {
+    const int64_t pairs = segment_pairs(a.max_nnz, a.tables);
+    const int ctas = pairs <= 8192 ? 4 : pairs <= 16384 ? 8 : 16, threads = pairs <= 32768 ? 256 : 512;
+    const auto kernel = pairs <= 8192    ? k_sort_segments<4, 256, 8>
+                        : pairs <= 16384 ? k_sort_segments<8, 256, 8>
+                        : pairs <= 32768 ? k_sort_segments<16, 256, 8>
+                                         : k_sort_segments<16, 512, 8>;
+    HL_CUDA_TRY(launch_cluster(kernel, (int64_t)a.tables * (a.merge ? 1 : 2) * ctas, threads, sort_smem_bytes(threads, 8), ctas,
+                               stream, a));
+    note_launches(1);
+    HL_LAUNCH_CHECK();
+    return HL_OK;
 }
 
 int64_t sort_clear_words(int64_t n_max, int key_bits, WaitCfg w) {
