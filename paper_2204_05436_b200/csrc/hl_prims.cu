@@ -400,7 +400,14 @@ __global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__
 // A table with more pairs than the cluster holds (the host knows the average only) is sorted by one of its CTAs, tile by
 // tile through memory.
 template <int CTAS, int NT, int ITEMS>
-__global__ void __launch_bounds__(NT) k_sort_segments(SegmentArgs a) {
+__global__ void __launch_bounds__(NT)
+    k_sort_segments(int32_t* keys_in, int32_t* vals_in, int32_t* keys_out, int32_t* vals_out, const int32_t* offsets_0,
+                    const int32_t* d_n_samples_0, int32_t key_bias_0, const int32_t* offsets_1, const int32_t* d_n_samples_1,
+                    int32_t key_bias_1, const int32_t* d_n_lookups, int32_t tables, int32_t max_batch, int32_t bags_per_sample,
+                    int32_t merge, int32_t passes, int64_t max_nnz) {
+    const SegmentArgs a{keys_in, vals_in, keys_out, vals_out,
+                        {{offsets_0, d_n_samples_0, key_bias_0, 0}, {offsets_1, d_n_samples_1, key_bias_1, 0}},
+                        d_n_lookups, tables, max_batch, bags_per_sample, merge, passes, 0, max_nnz};
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
     constexpr int PD = NT / 256;
@@ -620,7 +627,9 @@ int32_t sort_segments(const SegmentArgs& a, cudaStream_t stream) {
                         : pairs <= 32768 ? k_sort_segments<16, 256, 8>
                                          : k_sort_segments<16, 512, 8>;
     HL_CUDA_TRY(launch_cluster(kernel, (int64_t)a.tables * (a.merge ? 1 : 2) * ctas, threads, sort_smem_bytes(threads, 8), ctas,
-                               stream, a));
+                               stream, a.keys_in, a.vals_in, a.keys_out, a.vals_out, a.side[0].offsets, a.side[0].d_n_samples,
+                               a.side[0].key_bias, a.side[1].offsets, a.side[1].d_n_samples, a.side[1].key_bias, a.d_n_lookups,
+                               a.tables, a.max_batch, a.bags_per_sample, a.merge, a.passes, a.max_nnz));
     note_launches(1);
     HL_LAUNCH_CHECK();
     return HL_OK;
