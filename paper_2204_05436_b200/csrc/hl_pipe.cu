@@ -121,6 +121,14 @@ hl::LaunchCache* launches_of(hl_pipe* p, int64_t j) {
     return p->trace_mask ? nullptr : p->launches[j % p->launches.size()].get();
 }
 
+// Whether the read of the next mini-batch's rows may start beside O's update (else behind it: queue_mini_batch): where the
+// transfers of one mini-batch take hundreds of microseconds, so that the pipelines of a chip keep the link busy between them and
+// every wait of a read is lost.  What a mini-batch will move is not known here; its largest number of lookups is.  Three
+// pipelines in turn, behind / beside the update, us per mini-batch, bags of 20 lookups (64 at most), 8 tables, by lookups x row:
+// 0.5 M x 512 bytes 410 / 414, 1 M 569 / 563, 1.6 M 774 / 762, 2.1 M 974 / 957, 4.2 M 1 663 / 1 637; 2.1 M x 256 bytes 573 / 574
+// to 590, 4.2 M 931 / 922; 18 tables of bags of 2, 1.8 M x 336 bytes 382 / 385; all smaller ones 9 to 25 % faster behind it.
+bool read_beside_update(const hl_ctx* ctx) { return ctx->max_nnz * ctx->D > int64_t(160) << 20; }
+
 // Before the first mini-batch is queued: a graph of every run of kernels that a mini-batch like this one makes in slot j, so
 // that no mini-batch has to launch them one by one or to wait while one is built (some 2 ms for the seven runs of four slots;
 // built when a slot's mini-batch came, they made mini-batches three to eight 200 to 600 us each).  Nothing is launched.  The
@@ -161,7 +169,7 @@ void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense
                                    p->main);
     else
         (void)hl_embbag_fwd(ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main);
-    if (p->wb_mode == HL_PIPE_WB_AFTER_FORWARD) launch_flush();
+    if (p->wb_mode == HL_PIPE_WB_AFTER_FORWARD || read_beside_update(ctx)) launch_flush();
     if (!merge) update(0);
     launch_flush();
     if (!merge) update(0);                                   // (by itself: what the first mini-batch launches)
@@ -482,8 +490,9 @@ static int32_t queue_mini_batch(hl_pipe* p, const float* d_grad_pop, const float
     // behind both, and they go out as one graph.  (In between it cost more than the 2 us from one graph to the next: the
     // update waited behind what the read put on the chip.  One pipeline / three in turn on one chip, us per mini-batch: Tiny
     // 36.3 -> 32.5 / 37.1 -> 32.7, click log 69.2 -> 68.3 / 77.4 -> 64.5, time series 58.3 -> 60.1 / 70.9 -> 57.4, DLRM-sized
-    // 146 -> 137 / 150 -> 132.)  The first mini-batch has no write-back before it, and one that is held over starts here.
-    const bool apart = j == 0 || p->wb_pending;
+    // 146 -> 137 / 150 -> 132.)  The first mini-batch has no write-back before it, one that is held over starts here, and the
+    // longest transfers are better off beside the update (read_beside_update).
+    const bool apart = j == 0 || p->wb_pending || read_beside_update(p->ctx);
     const auto read_next = [&]() -> int32_t {
         HL_PIPE_TRY(popular.end());
         HL_PIPE_TRY(record(e.forward, p->main));
