@@ -407,7 +407,7 @@ HL_API int32_t hl_scatter_cold_at(hl_ctx* ctx, const float* d_cache, int64_t sta
 /* Buffers of one mini-batch in flight; all device memory, caller-owned, sized like the arguments of the calls
  * they are passed to (perm [max_batch]; counts [4]; pop / non as for hl_fragment; cold_rows, fwd_src [window_rows];
  * n_cold [1]; pooled_* [T*max_batch*S, D]; dense_out [max_batch, n_dense] or NULL; sorted_slots / sorted_bags
- * [max_nnz]; sorted_n [4]). */
+ * [max_nnz]: the (slot, bag) pairs with equal slots side by side, sorted as one list or table by table; sorted_n [4]). */
 typedef struct {
     int32_t*  perm;
     int32_t*  counts;

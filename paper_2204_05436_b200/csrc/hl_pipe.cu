@@ -3,7 +3,8 @@
 //   index stream  mini-batch j+L: fragment (X's lookups classified on the way), ranks of the cold rows, slots + match with
 //                 the cold rows of j+L-1 + (slot, bag) pairs, sort (more than 32 K lookups: on the sort stream)
 //   link stream   hl_stage_cold(j+1)           after the write-back of j-1 (host rows final, window free) and after
-//                                              mini-batch j took the rows it shares with j-1 out of that window
+//                                              mini-batch j took the rows it shares with j-1 out of that window and
+//                                              updated O (read_beside_update: or beside that)
 //   main stream   forward O (+ those rows), update O, [rows of j staged] forward X, update X            mini-batch j
 //   write-back    hl_scatter_cold_at(j)        after the update of X
 //
@@ -11,10 +12,10 @@
 //
 // Small mini-batches are bound by the host: what counts is the number of launches and event operations per mini-batch.
 // The index work is one stream (two), so that its steps need no events between them, and as few kernels as its data
-// dependences allow (five with at most 32 K lookups, otherwise four and one per sort digit); the rows forwarded between
-// windows ride on the popular forward.  13 to 15 launches, no memset and 12 to 15 event operations, where separate calls on
+// dependences allow (five where one kernel sorts, otherwise four and one per sort digit); the rows forwarded between
+// windows ride on the popular forward.  13 to 15 kernels, no memset and 12 to 15 event operations, where separate calls on
 // three streams made 22, 3 and 25 (8 K lookups: 88 us per mini-batch).  The kernels between two event operations go out as one
-// graph (hl_graph.cu): 17 us on the host instead of 41, 35 us per mini-batch instead of 54.
+// graph (hl_graph.cu), five to eight of them: 17 us on the host instead of 41; 30 to 35 us per mini-batch instead of 54.
 #include "hl_common.cuh"
 
 #include <memory>
@@ -130,7 +131,7 @@ hl::LaunchCache* launches_of(hl_pipe* p, int64_t j) {
 bool read_beside_update(const hl_ctx* ctx) { return ctx->max_nnz * ctx->D > int64_t(160) << 20; }
 
 // Before the first mini-batch is queued: a graph of every run of kernels that a mini-batch like this one makes in slot j, so
-// that no mini-batch has to launch them one by one or to wait while one is built (some 2 ms for the seven runs of four slots;
+// that no mini-batch has to launch them one by one or to wait while one is built (some 2 ms for the five to eight runs of four slots;
 // built when a slot's mini-batch came, they made mini-batches three to eight 200 to 600 us each).  Nothing is launched.  The
 // runs are those of queue_index and queue_mini_batch.
 void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense) {
