@@ -460,9 +460,14 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
     const int64_t words = summary ? cold_summary_words(ctx->N) : cold_bitmap_words(ctx->N);
     // words per thread: as in hl_fragment, one until there is a tile per multiprocessor
     const bool many = words > (int64_t)kThreads * ctx_sms(ctx);
-    const unsigned grid = (unsigned)div_up(words, kThreads * (many ? 4 : 1));
+    // and eight for large bitmaps, where a tile is mostly its wait for the one before it.  Four / eight, alone, us: 16.8 M rows
+    // with 10 K lookups 10.4 / 8.9, 26 K 11.0 / 9.0, 106 K 12.1 / 13.1, 426 K 14.8 / 15.8; 25 M 16.1 / 12.1, 14.1 / 12.0, 14.7 / 14.3,
+    // 13.6 / 14.8; 30 M 14.9 / 12.1, 16.4 / 11.7, 14.6 / 13.2, 14.9 / 16.1; 40 M 15.9 / 11.9, 16.2 / 11.4, 18.1 / 13.0, 20.7 / 14.8;
+    // 64 M 22.2 / 14.9, 21.4 / 14.0, 23.1 / 15.2, 21.0 / 15.9.  (7.7 M with 26 K 11.9 / 10.1, with 426 K 11.8 / 14.8.)
+    const bool most = !summary && ctx->N > int64_t(1) << (ctx->max_nnz > 65536 ? 25 : 24);
+    const unsigned grid = (unsigned)div_up(words, kThreads * (most ? 8 : many ? 4 : 1));
     const auto kernel = summary ? (many ? k_cold_rank<true, 4> : k_cold_rank<true, 1>)
-                                : (many ? k_cold_rank<false, 4> : k_cold_rank<false, 1>);
+                                : (most ? k_cold_rank<false, 8> : many ? k_cold_rank<false, 4> : k_cold_rank<false, 1>);
     const WaitCfg w = wait_cfg(ctx);
     HL_CUDA_TRY(launch(kernel, grid, kThreads, stream, marks, (int)words, stage_rows, d_cold_rows, d_n_cold, r.status,
                        w.max_polls, w.stall_tile, clear, n_clear));
