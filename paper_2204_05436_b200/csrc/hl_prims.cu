@@ -397,8 +397,9 @@ __global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__
 // it is the chain count -> exchange -> scatter of a pass, with the larger tables' clusters on the chip together.  Alone, against
 // three chained passes: 86 K pairs of 21 tables 8.5 / 19 us, 107 K of 26 8.6 / 19, 129 K of 3 15.5 / 21, 333 K of 37 15.7 / 24, 426 K
 // of 26 18.5 / 28; 8 K of 8 tables 5.8, against 9.2 in one cluster.  (CTAs of 512 threads: 9.9, 9.9, 15.3, 21.5, 27.9, 7.6.)
-// A table with more pairs than the cluster holds (the host knows the average only) is sorted by one of its CTAs, tile by
-// tile through memory.
+// A table with more pairs than the cluster holds (the host knows the average only) is sorted by it through memory, every CTA
+// taking a share of the pairs tile by tile.  (Pipelines of 20 tables with nearly all lookups in one, us per mini-batch, chained
+// passes / one CTA of the cluster / all of them: 24 K pairs 106 / 124 / 78, 74 K 154 / 366 / 137, 295 K 215 / 1 388 / 256.)
 template <int CTAS, int NT, int ITEMS>
 __global__ void __launch_bounds__(NT)
     k_sort_segments(int32_t* keys_in, int32_t* vals_in, int32_t* keys_out, int32_t* vals_out, const int32_t* offsets_0,
@@ -440,20 +441,37 @@ __global__ void __launch_bounds__(NT)
     if (n == 0) return;                           // the same in all CTAs of the cluster
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int d = threadIdx.x / PD, q = threadIdx.x % PD;
+    // q's part of a digit's counts over the CTAs (published by a cluster.sync()) into: those of the CTAs before mine, all
+    auto over_ctas = [&](uint32_t& before, uint32_t& all) {
+        before = all = 0;
+#pragma unroll
+        for (int c = q; c < CTAS; c += PD) {
+            const uint32_t v = *cluster.map_shared_rank(&cta_hist[d], c);
+            if (c < cta) before += v;
+            all += v;
+        }
+#pragma unroll
+        for (int o = 1; o < PD; o <<= 1) {
+            before += __shfl_xor_sync(0xffffffffu, before, o);
+            all += __shfl_xor_sync(0xffffffffu, all, o);
+        }
+    };
+    uint32_t before, all;                         // of this thread's digit
     if (n > CTAS * NT * ITEMS) {
-        if (cta != 0) return;
         int32_t *kin = a.keys_in + lo, *vin = a.vals_in + lo, *kout = a.keys_out + lo, *vout = a.vals_out + lo;
         constexpr int TILE = NT * ITEMS;
+        const int share = (n + CTAS - 1) / CTAS, from = min(n, cta * share), to = min(n, from + share);     // of this CTA
         for (int p = 0; p < a.passes; ++p) {
             const int shift = 8 * p;
             if (threadIdx.x < 256) cta_hist[threadIdx.x] = 0;
             __syncthreads();
-            for (int i = threadIdx.x; i < n; i += NT) atomicAdd(&cta_hist[((uint32_t)kin[i] - bias) >> shift & 255u], 1u);
-            __syncthreads();
-            const uint32_t smaller = scan_digits<PD>(cta_hist[d], scan_smem);
-            if (q == 0) digit_base[d] = smaller;
-            for (int tile = 0; tile < n; tile += TILE) {
-                const int n_mine = max(0, min(n - tile - warp * 32 * ITEMS, 32 * ITEMS)), at = tile + warp * 32 * ITEMS + lane;
+            for (int i = from + threadIdx.x; i < to; i += NT) atomicAdd(&cta_hist[((uint32_t)kin[i] - bias) >> shift & 255u], 1u);
+            cluster.sync();                       // all counts published
+            over_ctas(before, all);
+            const uint32_t smaller = scan_digits<PD>(all, scan_smem);
+            if (q == 0) digit_base[d] = smaller + before;
+            for (int tile = from; tile < to; tile += TILE) {
+                const int n_mine = max(0, min(to - tile - warp * 32 * ITEMS, 32 * ITEMS)), at = tile + warp * 32 * ITEMS + lane;
                 uint32_t key[ITEMS], val[ITEMS], rank[ITEMS];
 #pragma unroll
                 for (int r = 0; r < ITEMS; ++r) {
@@ -478,6 +496,7 @@ __global__ void __launch_bounds__(NT)
                 if (q == 0) digit_base[d] += total;
                 __syncthreads();
             }
+            cluster.sync();                       // all pairs written; no CTA clears its counts, or leaves, while others read them
             int32_t* const k = kin;
             int32_t* const v = vin;
             kin = kout;
@@ -486,7 +505,7 @@ __global__ void __launch_bounds__(NT)
             vout = v;
         }
         if (a.passes % 2 == 0)                    // (the last pass wrote the input's place)
-            for (int i = threadIdx.x; i < n; i += NT) {
+            for (int i = from + threadIdx.x; i < to; i += NT) {
                 kout[i] = kin[i];
                 vout[i] = vin[i];
             }
@@ -517,18 +536,7 @@ __global__ void __launch_bounds__(NT)
         const uint32_t total = prefix_over_warps<NT>(sm.cnt);
         if (q == 0) cta_hist[d] = total;
         cluster.sync();     // all counts published; all CTAs have taken the previous pass's pairs out of shared memory
-        uint32_t before = 0, all = 0;             // of this digit: in the CTAs before mine, in all CTAs
-#pragma unroll
-        for (int c = q; c < CTAS; c += PD) {
-            const uint32_t v = *cluster.map_shared_rank(&cta_hist[d], c);
-            if (c < cta) before += v;
-            all += v;
-        }
-#pragma unroll
-        for (int o = 1; o < PD; o <<= 1) {
-            before += __shfl_xor_sync(0xffffffffu, before, o);
-            all += __shfl_xor_sync(0xffffffffu, all, o);
-        }
+        over_ctas(before, all);
         const uint32_t smaller = scan_digits<PD>(all, scan_smem);
         if (q == 0) digit_base[d] = smaller + before;
         __syncthreads();

@@ -22,6 +22,8 @@ CASES = {
     "one_large_table_one_pass": ([3] * 20, 2000, [(0, 1), (8, 14)] + [(0, 0)] * 16 + [(0, 1)] * 2, 0.9),
     "one_large_table_two_passes": ([700, 6000] + [10] * 20, 2000, [(1, 1), (8, 14), (0, 1)] + [(0, 0)] * 19, 0.99),
     "one_large_table_three_passes": ([90_000] + [500] * 19, 2000, [(8, 14), (1, 1)] + [(0, 0)] * 17 + [(0, 1)], 0.5),
+    "one_large_table_8_ctas": ([50_000, 5], 16_384, [(2, 2), (0, 0)], 0.9),
+    "one_large_table_16_ctas": ([50_000, 5], 20_001, [(2, 2), (0, 0)], 0.95),
     "all_popular": ([9000] + [10] * 15, 3000, [(5, 9), (1, 1), (0, 1)] + [(0, 0)] * 13, 1.0),
     "one_table": ([20_000], 5000, [(1, 1)], 0.5),
 }
