@@ -115,7 +115,8 @@ extern "C" int32_t hl_create(hl_ctx** out, const hl_geometry* geom, int32_t max_
         return HL_ECAPACITY;
     }
     if (cudaGetDevice(&ctx->device) != cudaSuccess ||
-        cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess) {
+        cudaDeviceGetAttribute(&ctx->sms, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
+        !piece_memory_granted(ctx->D)) {
         free(ctx);
         return HL_ECUDA;
     }

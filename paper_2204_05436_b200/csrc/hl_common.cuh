@@ -655,6 +655,9 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
                            bool merge, cudaStream_t stream, const SortAside* aside, int32_t** out_slots = nullptr,
                            int32_t** out_bags = nullptr);
 
+// Asks for what the backward's sum kernel needs of shared memory for rows of D fp32, on the current device (hl_embbag.cu).
+bool piece_memory_granted(int D);
+
 // hl_embbag_fwd and hl_forward_cold in one launch (the bags read no staged row).
 int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples, float* d_out,
                              int64_t from_stage_row0, int64_t to_stage_row0, int64_t stage_rows, const int32_t* d_fwd_src,

@@ -450,6 +450,17 @@ constexpr int kWindowChunks = kThreads / 32, kBwdWindow = kWindowChunks * kBwdCh
 constexpr int kSpanLookahead = 32;      // windows k_bwd_chunks looks ahead for the end of a run
 static_assert(kBwdChunk == 32, "one lookup of a chunk per lane");
 
+// Shared memory for the pieces of a window's runs, in fp64 whatever the width of a row, so that what a run adds up to inside a window
+// is rounded nowhere: two sets, for windows in turn, where they fit (rows of up to 256 fp32), else one; rows of more than 512
+// fp32 need more than the 48 KB that a kernel has without asking (piece_memory_granted).
+template <int G, int NV>
+struct PieceShape {
+    static constexpr int kSets = NV <= 2 ? 2 : 1;
+    static constexpr int kCount = kSets * kWindowChunks * NV * 2 * G;               // double2
+    static constexpr bool kDynamic = NV >= 8;
+    static constexpr size_t kDynamicBytes = kDynamic ? kCount * sizeof(double2) : 0;
+};
+
 //
 // CTAS: CTAs that fit a multiprocessor.  Rows of 36 to 64 fp32 (G = 16): a warp waits for its pairs, then for gradient rows,
 // and then puts two groups together, once per 32 lookups, so in a call of many chunks another warp should have something on
@@ -499,13 +510,16 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
     const char* gcol[NV];
     const uint32_t row_bytes = (uint32_t)D4 * 16u;
     __shared__ double2 s_first[G == 32 ? 1 : 2][G == 32 ? 1 : kThreads];      // sums of the groups' first runs
-    // Of every chunk of the window that begins inside a run: what the run has there, and whether it ends there.  (Two sets, for
-    // windows in turn; rows of more than 256 fp32 have room for one, of fp32 sums.)
-    constexpr bool kTwo = NV <= 2;
-    using Piece = std::conditional_t<kTwo, double2, float4>;
-    constexpr int kParts = kTwo ? 2 : 1;
-    __shared__ Piece s_piece[kTwo ? 2 : 1][kWindowChunks][NV][kParts][G];
-    __shared__ int s_ends[kTwo ? 2 : 1][kWindowChunks];
+    // Of every chunk of the window that begins inside a run: what the run has there, and whether it ends there.
+    using Shape = PieceShape<G, NV>;
+    constexpr bool kTwo = Shape::kSets == 2;
+    __shared__ double2 s_piece_static[Shape::kDynamic ? 1 : Shape::kCount];
+    extern __shared__ double2 s_piece_dynamic[];
+    double2* const s_piece = Shape::kDynamic ? s_piece_dynamic : s_piece_static;    // [set][chunk][NV][2][G]
+    __shared__ int s_ends[Shape::kSets][kWindowChunks];
+    const auto piece_at = [&](int set, int chunk, int v) {
+        return s_piece + ((set * kWindowChunks + chunk) * NV + v) * 2 * G + sub;
+    };
     const float minus_lr = -lr;               // -(lr * G) and (-lr) * G are the same number
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -570,13 +584,9 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
         auto put_piece = [&](const double (&acc)[NV][4]) {
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                Piece* to = &s_piece[set][wib][v][0][sub];
-                if constexpr (kTwo) {
-                    to[0] = make_double2(acc[v][0], acc[v][1]);
-                    to[G] = make_double2(acc[v][2], acc[v][3]);
-                } else {
-                    to[0] = make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]);
-                }
+                double2* to = piece_at(set, wib, v);
+                to[0] = make_double2(acc[v][0], acc[v][1]);
+                to[G] = make_double2(acc[v][2], acc[v][3]);
             }
         };
         // adds the pieces of a run in the chunks from `chunk` on; true: it ends in this window
@@ -584,16 +594,12 @@ __global__ void __launch_bounds__(kThreads, CTAS) k_bwd_chunks(float* __restrict
             for (; chunk < kWindowChunks; ++chunk) {
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
-                    const Piece* from = &s_piece[set][chunk][v][0][sub];
-                    if constexpr (kTwo) {
-                        const double2 p = from[0], q = from[G];
-                        sum[v][0] += p.x;
-                        sum[v][1] += p.y;
-                        sum[v][2] += q.x;
-                        sum[v][3] += q.y;
-                    } else {
-                        add_row(sum[v], from[0]);
-                    }
+                    const double2* from = piece_at(set, chunk, v);
+                    const double2 p = from[0], q = from[G];
+                    sum[v][0] += p.x;
+                    sum[v][1] += p.y;
+                    sum[v][2] += q.x;
+                    sum[v][3] += q.y;
                 }
                 if (s_ends[set][chunk]) return true;
             }
@@ -958,9 +964,9 @@ int32_t launch_bwd(hl_ctx* ctx, float* cache, const int32_t* keys, const int32_t
         HL_CUDA_TRY(clear_words(reinterpret_cast<uint32_t*>(span_count), 8, stream));
         ctx->spans_suspect = 0;
     }
-    HL_CUDA_TRY(launch(sums, grid, kThreads, stream, cache, keys, vals, d_n_lookups, grad, ctx->D / 4,
-                       n_slots, lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list, ctx->max_bags, max_chunks,
-                       ctx->r.status));
+    HL_CUDA_TRY(launch_cluster(sums, grid, kThreads, PieceShape<G, NV>::kDynamicBytes, 0, stream, cache, keys, vals, d_n_lookups,
+                               grad, ctx->D / 4, n_slots, lr, ctx->r.bwd_part, d_first, key_bias, span_count, span_list,
+                               ctx->max_bags, max_chunks, ctx->r.status));
     timer_mark(ctx, HL_TIMER_BWD_REDUCE, 1, stream);
     const int span_grid = grid_for(max_chunks * 32, kThreads, 2 * ctx_sms(ctx));   // the warps stride over the listed runs
     HL_CUDA_TRY(launch(k_bwd_spans<G, NV>, span_grid, kThreads, stream, cache, keys, d_n_lookups, ctx->D / 4, n_slots, lr,
@@ -1006,6 +1012,13 @@ int32_t fwd_call(hl_ctx* ctx, const float* d_cache, const hl_ubatch* ub, const i
 }
 
 }  // namespace
+
+bool piece_memory_granted(int D) {
+    using Shape = PieceShape<32, 8>;
+    if (D / 4 <= 128) return true;
+    return cudaFuncSetAttribute(k_bwd_chunks<32, 8, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)Shape::kDynamicBytes) == cudaSuccess;
+}
 
 int32_t fwd_and_forward_cold(hl_ctx* ctx, float* d_cache, const hl_ubatch* ub, const int32_t* d_n_samples, float* d_out,
                              int64_t from_stage_row0, int64_t to_stage_row0, int64_t stage_rows, const int32_t* d_fwd_src,
