@@ -199,12 +199,16 @@ __device__ __forceinline__ void copy_16_async(uint32_t smem_to, const void* from
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(smem_to), "l"(from), "r"(valid ? 16 : 0) : "memory");
 }
 
-// By columns per lane: lookups of a block, threads of a CTA, CTAs that fit a multiprocessor (registers).
+// By columns per lane: lookups of a block, blocks of the ring, threads of a CTA, CTAs that fit a multiprocessor (registers).  Rows
+// of 260 to 512 fp32: three CTAs of 80 registers spill 72 bytes; two, with a block more on its way instead, do not.  Rows of
+// 2 KB, alone, L2 flushed, three CTAs / two / two and three blocks: 655 K lookups in bags of 20 268 / 147 / 137 us, 197 K in bags of
+// 3 98 / 65 / 60, 82 K in bags of 20 47.8 / 30.0 / 27.4, 10 K 18.5 / 14.9 / 12.9; of 1 040 bytes 241 / 141 / 131, 84.5 / 57.8 / 54.5,
+// 43.4 / 28.2 / 25.4, 18.2 / 15.3 / 12.8.  (CTAs of 128 threads, four or five of them: 3 to 20 % slower in the large calls.)
 template <int NV>
 struct FwdShape {
-    static constexpr int U = NV >= 4 ? 1 : 4 / NV, kBlocks = 2;
+    static constexpr int U = NV >= 4 ? 1 : 4 / NV, kBlocks = NV == 4 ? 3 : 2;
     static constexpr int NT = NV >= 8 ? 128 : 256;
-    static constexpr int CTAS = NV >= 4 ? 3 : 4;
+    static constexpr int CTAS = NV == 4 ? 2 : NV >= 8 ? 3 : 4;
     static constexpr size_t kSmem = sizeof(float4) * kBlocks * U * NV * NT;
     static_assert(kSmem <= 48 * 1024, "more than that has to be asked for");
 };
@@ -928,7 +932,9 @@ int32_t launch_fwd(hl_ctx* ctx, const float* cache, const hl_ubatch* ub, const i
     const bool many = 2 * ctx->max_nnz > 3 * (int64_t)ctx->max_bags;
     // a fixed number of CTAs per multiprocessor; in small calls of bags of several lookups a group has a bag or two
     using Shape = FwdShape<NV>;
-    const int grid = grid_for(ctx->max_bags, many ? Shape::NT / G : kThreads / G * UB, fwd_ctas_per_sm(ctx) * ctx_sms(ctx));
+    int per_sm = fwd_ctas_per_sm(ctx);
+    if (many && ctx->fwd_ctas <= 0 && per_sm > Shape::CTAS) per_sm = Shape::CTAS;
+    const int grid = grid_for(ctx->max_bags, many ? Shape::NT / G : kThreads / G * UB, per_sm * ctx_sms(ctx));
     const auto kernel = many ? (fr ? k_embbag_pool<G, NV, true> : k_embbag_pool<G, NV, false>)
                              : (fr ? k_embbag_fwd<G, NV, UB, true> : k_embbag_fwd<G, NV, UB, false>);
     HL_CUDA_TRY(launch_cluster(kernel, grid, many ? Shape::NT : kThreads, many ? Shape::kSmem : 0, 0, stream, cache, ub->ids,
