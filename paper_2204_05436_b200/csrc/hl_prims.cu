@@ -489,8 +489,10 @@ __global__ void __launch_bounds__(NT)
                 for (int r = 0; r < ITEMS; ++r)
                     if (r * 32 + lane < n_mine) {
                         const uint32_t dg = (key[r] >> shift) & 255u, pos = digit_base[dg] + sm.cnt[warp][dg] + rank[r];
-                        kout[pos] = (int32_t)(key[r] + bias);
-                        vout[pos] = (int32_t)val[r];
+                        if (pos < (uint32_t)n) {     // always, unless a wait gave up when the pairs' places were worked out:
+                            kout[pos] = (int32_t)(key[r] + bias);        // tables' shares may overlap then, and what is read
+                            vout[pos] = (int32_t)val[r];                 // here not be what was counted
+                        }
                     }
                 __syncthreads();
                 if (q == 0) digit_base[d] += total;

@@ -24,6 +24,13 @@ CASES = {
     "one_large_table_three_passes": ([90_000] + [500] * 19, 2000, [(8, 14), (1, 1)] + [(0, 0)] * 17 + [(0, 1)], 0.5),
     "one_large_table_8_ctas": ([50_000, 5], 16_384, [(2, 2), (0, 0)], 0.9),
     "one_large_table_16_ctas": ([50_000, 5], 20_001, [(2, 2), (0, 0)], 0.95),
+    # (as many lookups as bags, all of them in one table: through memory, one to four digits, CTAs of 256 and of 512 threads)
+    "one_full_table_one_pass": ([3] * 20, 2000, [(20, 20)] + [(0, 0)] * 19, 0.9),
+    "one_full_table_two_passes": ([700, 6000] + [10] * 18, 2000, [(0, 0), (20, 20)] + [(0, 0)] * 18, 0.99),
+    "one_full_table_three_passes": ([90_000] + [500] * 19, 2001, [(20, 20)] + [(0, 0)] * 19, 0.5),
+    "one_full_table_four_passes": ([30] * 3 + [17_000_000] + [30] * 4, 2000, [(0, 0)] * 3 + [(8, 8)] + [(0, 0)] * 4, 1.0),
+    "one_full_table_512_threads": ([90_000, 700], 33_000, [(2, 2), (0, 0)], 0.9),
+    "one_full_table_512_threads_last": ([700, 90_000], 65_536, [(0, 0), (2, 2)], 0.6),
     "all_popular": ([9000] + [10] * 15, 3000, [(5, 9), (1, 1), (0, 1)] + [(0, 0)] * 13, 1.0),
     "one_table": ([20_000], 5000, [(1, 1)], 0.5),
 }
