@@ -608,7 +608,7 @@ struct SegmentArgs {
     int32_t tables, max_batch, bags_per_sample, merge, passes, unused;
     int64_t max_nnz;
 };
-bool sort_by_segments(int64_t n_max, int64_t n_bags, int tables, WaitCfg w);
+bool sort_by_segments(int64_t n_max, int64_t n_bags, int tables, bool merge, WaitCfg w);
 int32_t sort_segments(const SegmentArgs& a, cudaStream_t stream);
 
 // 32-bit words of histogram scratch radix_sort_pairs needs for at most max_nnz pairs.
@@ -637,8 +637,10 @@ int32_t cold_rank(hl_ctx* ctx, int64_t stage_rows, int32_t* d_cold_rows, int64_t
 // hl_embbag_bwd_prepare2 / _merged on what fragment_and_mark and cold_rank left behind (hl_embbag.cu): X's cold lookups
 // get their slots, the cold rows are matched against the previous ones, and the pairs are sorted (aside: may be null).  The
 // sort's scratch, backward_sort_clear_words words of bwd_hist, is zero already.  d_sorted_slots / _bags may be null: the
-// result then stays in the context's scratch, at *out_slots / *out_bags.
-int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge);
+// result then stays in the context's scratch, at *out_slots / *out_bags.  by_table: backward_sorts_tables, asked once for a
+// mini-batch, since its ranks (which clear the scratch), pairs and sort have to go the same way.
+bool backward_sorts_tables(const hl_ctx* ctx, const hl_batch* b, bool merge);
+int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge, bool by_table);
 bool backward_sort_is_long(const hl_ctx* ctx);
 
 // The sort on a stream of its own, behind the pairs (event pairs_ready), with one of two sets of scratch (which): the
@@ -652,8 +654,8 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
                            const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows, const int32_t* d_cold_rows,
                            const int64_t* d_n_cold, const int32_t* d_prev_rows, const int64_t* d_n_prev,
                            int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
-                           bool merge, cudaStream_t stream, const SortAside* aside, int32_t** out_slots = nullptr,
-                           int32_t** out_bags = nullptr);
+                           bool merge, bool by_table, cudaStream_t stream, const SortAside* aside,
+                           int32_t** out_slots = nullptr, int32_t** out_bags = nullptr);
 
 // Asks for what the backward's sum kernel needs of shared memory for rows of D fp32, on the current device (hl_embbag.cu).
 bool piece_memory_granted(int D);

@@ -1050,13 +1050,12 @@ namespace {
 // out_keys / out_vals: either the caller's arrays (which then serve as one half of the sort's ping-pong buffers) or, if
 // they are null, whichever scratch buffer the last pass wrote.  cleared: the sort's scratch (sort_clear_words words of
 // bwd_hist) is zero already.  aside: see SortAside.
-int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bool cleared, int32_t* caller_keys,
+// by_table: every table's pairs by themselves (the schedules' pairs: fragment laid them out by table, and no row belongs to two).
+int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bool by_table, bool cleared, int32_t* caller_keys,
                        int32_t* caller_vals, int32_t* d_n_lookups, int32_t** out_keys, int32_t** out_vals,
                        cudaStream_t stream, const SortAside* aside = nullptr) {
     Regions& r = ctx->r;
-    // (the schedules' pairs: fragment laid them out by table, and no row belongs to two)
-    const bool segments = assign && a.sides == 2 && sort_by_segments(ctx->max_nnz, ctx->max_bags, ctx->T, wait_cfg(ctx));
-    const int key_bits = bits_for(max_key), passes = segments ? 1 : (key_bits + 7) / 8;
+    const int key_bits = bits_for(max_key), passes = by_table ? 1 : (key_bits + 7) / 8;
     const int which = aside ? aside->which : 0;          // (with caller arrays, one of the two scratch buffers is free)
     uint32_t* sort_scratch = r.bwd_hist[which];
     int32_t* keys[2] = {r.bwd_keys[which], r.bwd_keys[which ^ 1]};
@@ -1072,7 +1071,7 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
     a.max_batch = ctx->max_batch;
     a.bags_per_sample_all = ctx->T * ctx->S;
     a.bags_per_sample = ctx->S;
-    a.by_table = segments && a.bags_follow;
+    a.by_table = by_table && a.bags_follow;
     a.n_slots = ctx->hot_cap + ctx->staging_cap;
     a.max_nnz = ctx->max_nnz;
     a.keys = keys[0];
@@ -1082,7 +1081,7 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
     a.ghist = sort_scratch;
     a.passes = passes;
     // the tile sort wants its digit counts, which cost less here than in a sweep of their own
-    const int64_t clear_words = segments ? 0 : sort_clear_words(ctx->max_nnz, key_bits, wait_cfg(ctx));
+    const int64_t clear_words = by_table ? 0 : sort_clear_words(ctx->max_nnz, key_bits, wait_cfg(ctx));
     const bool hist = clear_words > 0;
     if (hist && !cleared) HL_CUDA_TRY(hl::clear_words(sort_scratch, clear_words, stream));
     // lanes per bag: by the most lookups a bag has on average (bags of 20 out of at most 64: 20.8 us with 8 lanes, 22.2 with
@@ -1106,7 +1105,7 @@ int32_t pairs_and_sort(hl_ctx* ctx, PairArgs a, int64_t max_key, bool assign, bo
         HL_CUDA_TRY(cudaStreamWaitEvent(aside->stream, aside->pairs_ready, 0));
         stream = aside->stream;
     }
-    if (segments) {
+    if (by_table) {
         SegmentArgs g{};
         g.keys_in = keys[0];
         g.vals_in = vals[0];
@@ -1132,7 +1131,7 @@ int32_t sort_lookups(hl_ctx* ctx, const hl_ubatch* ub, const int32_t* d_n_sample
     PairArgs a{};
     a.sides = 1;
     a.side[0] = {ub->ids, ub->offsets, d_n_samples, 0};
-    return pairs_and_sort(ctx, a, ctx->hot_cap + ctx->staging_cap, false, false, caller_keys, caller_vals, d_n_lookups,
+    return pairs_and_sort(ctx, a, ctx->hot_cap + ctx->staging_cap, false, false, false, caller_keys, caller_vals, d_n_lookups,
                           out_keys, out_vals, stream);
 }
 
@@ -1180,7 +1179,7 @@ namespace {
 // run, over one gradient array [bags of O; bags of X]
 int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, const hl_ubatch* non,
                      const int32_t* d_n_non, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
-                     bool merge, PairArgs a, bool assign, bool cleared, cudaStream_t stream,
+                     bool merge, PairArgs a, bool assign, bool by_table, bool cleared, cudaStream_t stream,
                      const SortAside* aside = nullptr, int32_t** out_slots = nullptr, int32_t** out_bags = nullptr) {
     if (!ctx || !pop || !non || !pop->offsets || !non->offsets || !d_n_pop || !d_n_non || !d_n_lookups)
         return HL_EINVAL;
@@ -1197,7 +1196,7 @@ int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, 
     a.side[1] = {non->ids, non->offsets, d_n_non, merge ? 0 : (int32_t)(n_slots + 1)};
     return as_graph(kept_launches(ctx), [&] {
         int32_t *ok, *ov;
-        return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, cleared, d_sorted_slots, d_sorted_bags,
+        return pairs_and_sort(ctx, a, merge ? n_slots : 2 * n_slots + 1, assign, by_table, cleared, d_sorted_slots, d_sorted_bags,
                               d_n_lookups, out_slots ? out_slots : &ok, out_bags ? out_bags : &ov, stream, aside);
     });
 }
@@ -1206,8 +1205,15 @@ int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, 
 
 bool backward_sort_is_long(const hl_ctx* ctx) { return sort_is_long(ctx->max_nnz, wait_cfg(ctx)); }
 
-int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge) {
-    if (sort_by_segments(ctx->max_nnz, ctx->max_bags, ctx->T, wait_cfg(ctx))) return 0;
+// As many lookups as bags: one in every bag, in all likelihood, so that the tables have equally many.  (Otherwise some bags are
+// empty and others long, and one table may have most of the lookups: k_sort_segments.)
+bool backward_sorts_tables(const hl_ctx* ctx, const hl_batch* b, bool merge) {
+    return b->nnz == (int64_t)ctx->T * b->batch * ctx->S &&
+           sort_by_segments(ctx->max_nnz, ctx->max_bags, ctx->T, merge, wait_cfg(ctx));
+}
+
+int64_t backward_sort_clear_words(const hl_ctx* ctx, bool merge, bool by_table) {
+    if (by_table) return 0;
     const int64_t n_slots = ctx->hot_cap + ctx->staging_cap;
     return sort_clear_words(ctx->max_nnz, bits_for(merge ? n_slots : 2 * n_slots + 1), wait_cfg(ctx));
 }
@@ -1216,7 +1222,7 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
                            const int32_t* d_n_non, int64_t stage_row0, int64_t stage_rows, const int32_t* d_cold_rows,
                            const int64_t* d_n_cold, const int32_t* d_prev_rows, const int64_t* d_n_prev,
                            int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
-                           bool merge, cudaStream_t stream, const SortAside* aside, int32_t** out_slots,
+                           bool merge, bool by_table, cudaStream_t stream, const SortAside* aside, int32_t** out_slots,
                            int32_t** out_bags) {
     PairArgs a{};
     a.ranked = ctx->r.cold_ranked;
@@ -1228,8 +1234,8 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
     a.d_n_prev = d_n_prev;
     a.n_prev_max = ctx->staging_cap;
     a.fwd_src = d_fwd_src;
-    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, merge, a, true, true,
-                        stream, aside, out_slots, out_bags);
+    return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, merge, a, true,
+                        by_table, true, stream, aside, out_slots, out_bags);
 }
 
 }  // namespace hl
@@ -1238,14 +1244,14 @@ extern "C" int32_t hl_embbag_bwd_prepare2(hl_ctx* ctx, const hl_ubatch* pop, con
                                           const hl_ubatch* non, const int32_t* d_n_non, int32_t* d_sorted_slots,
                                           int32_t* d_sorted_bags, int32_t* d_n_lookups, void* stream) {
     return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, false, PairArgs{}, false,
-                        false, static_cast<cudaStream_t>(stream));
+                        false, false, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int32_t hl_embbag_bwd_prepare_merged(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop,
                                                 const hl_ubatch* non, const int32_t* d_n_non, int32_t* d_sorted_slots,
                                                 int32_t* d_sorted_bags, int32_t* d_n_lookups, void* stream) {
     return prepare_both(ctx, pop, d_n_pop, non, d_n_non, d_sorted_slots, d_sorted_bags, d_n_lookups, true, PairArgs{}, false,
-                        false, static_cast<cudaStream_t>(stream));
+                        false, false, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int32_t hl_embbag_bwd_apply2(hl_ctx* ctx, float* d_cache, const int32_t* d_sorted_slots,

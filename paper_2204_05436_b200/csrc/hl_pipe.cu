@@ -148,7 +148,8 @@ void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense
     hl_pipe_set &st = p->sets[j % n], &prev = p->sets[(j + n - 1) % n];
     const int64_t rows = p->window_rows, w = (j % 2) * rows, w_other = rows - w;
     const bool merge = p->order == HL_PIPE_ORDER_EQ5;
-    const int64_t n_clear = backward_sort_clear_words(ctx, merge);
+    const bool by_table = backward_sorts_tables(ctx, b, merge);
+    const int64_t n_clear = backward_sort_clear_words(ctx, merge, by_table);
     const SortAside aside{p->sort, p->ev[j % n].pairs, (int)(j % 2)};
     const SortAside* use = backward_sort_is_long(ctx) ? &aside : nullptr;
     const float* any = st.pooled_pop;                        // (some gradients)
@@ -159,7 +160,7 @@ void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense
     if (use) launch_flush();
     (void)cold_rank(ctx, rows, st.cold_rows, st.n_cold, p->index, ctx->r.bwd_hist[use ? j % 2 : 0], n_clear);
     (void)assign_and_prepare(ctx, &st.pop, st.counts, &st.non, st.counts + 1, w, rows, st.cold_rows, st.n_cold, prev.cold_rows,
-                             prev.n_cold, st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, p->index, use);
+                             prev.n_cold, st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, by_table, p->index, use);
     (void)hl_stage_cold(ctx, p->host_table, p->cache, w, rows, st.cold_rows, st.n_cold, st.fwd_src, p->link);
     launch_flush();
     const auto update = [&](int which) {
@@ -209,7 +210,8 @@ int32_t queue_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* i
     }
     // A sort of many pairs goes to a stream of its own, so that its passes overlap the next mini-batch's fragment; scratch
     // set j % 2 was the sort's of mini-batch j-2.
-    const int64_t n_clear = backward_sort_clear_words(p->ctx, merge);
+    const bool by_table = backward_sorts_tables(p->ctx, b, merge);
+    const int64_t n_clear = backward_sort_clear_words(p->ctx, merge, by_table);
     const SortAside aside{p->sort, e.pairs, (int)(j % 2)};
     const SortAside* use = backward_sort_is_long(p->ctx) ? &aside : nullptr;
     if (use && j >= 2) {
@@ -225,7 +227,8 @@ int32_t queue_index(hl_pipe* p, const hl_batch* b, const float* d_dense, void* i
         Scope sc(p, HL_SPAN_SORT, j, kIndex);
         HL_PIPE_TRY(assign_and_prepare(p->ctx, &st.pop, st.counts, &st.non, st.counts + 1, w, p->window_rows, st.cold_rows,
                                        st.n_cold, prev ? prev->cold_rows : nullptr, prev ? prev->n_cold : nullptr,
-                                       st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, p->index, use));
+                                       st.fwd_src, st.sorted_slots, st.sorted_bags, st.sorted_n, merge, by_table, p->index,
+                                       use));
     }
     HL_PIPE_TRY(batch.end());
     HL_PIPE_TRY(record(e.index, use ? p->sort : p->index));
@@ -317,17 +320,18 @@ int32_t queue_step(hl_ctx* ctx, const hl_batch* b, const float* d_dense, int32_t
         return record(ctx->step_staged, side);
     };
     if (one_sort) {
+        const bool by_table = backward_sorts_tables(ctx, b, false);
         HL_PIPE_TRY(fragment_and_mark(ctx, b, d_dense, d_dense ? n_dense : 0, s->perm, s->counts, &pop, &non,
                                       d_dense ? s->dense_out : nullptr, main));
         HL_PIPE_TRY(cold_rank(ctx, ctx->staging_cap, s->cold_rows, s->n_cold, main, ctx->r.bwd_hist[0],
-                              backward_sort_clear_words(ctx, false)));
+                              backward_sort_clear_words(ctx, false, by_table)));
         HL_PIPE_TRY(to_side());
         HL_PIPE_TRY(hl_stage_cold(ctx, host_table, d_cache, 0, ctx->staging_cap, s->cold_rows, s->n_cold, nullptr, side));
         HL_PIPE_TRY(side_done());
         HL_PIPE_TRY(hl_embbag_fwd(ctx, d_cache, &pop, s->counts, s->pooled_pop, main));
         HL_PIPE_TRY(assign_and_prepare(ctx, &pop, s->counts, &non, d_n_non, 0, ctx->staging_cap, s->cold_rows, s->n_cold,
-                                       nullptr, nullptr, nullptr, nullptr, nullptr, ctx->r.bwd_n, false, main, nullptr,
-                                       &slots, &bags));
+                                       nullptr, nullptr, nullptr, nullptr, nullptr, ctx->r.bwd_n, false, by_table, main,
+                                       nullptr, &slots, &bags));
     } else {
         HL_PIPE_TRY(hl_fragment(ctx, b, d_dense, d_dense ? n_dense : 0, s->perm, s->counts, &pop, &non,
                                 d_dense ? s->dense_out : nullptr, main));

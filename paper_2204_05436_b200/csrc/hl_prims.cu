@@ -398,8 +398,9 @@ __global__ void __launch_bounds__(NT) k_sort_cluster(const int32_t* __restrict__
 // three chained passes: 86 K pairs of 21 tables 8.5 / 19 us, 107 K of 26 8.6 / 19, 129 K of 3 15.5 / 21, 333 K of 37 15.7 / 24, 426 K
 // of 26 18.5 / 28; 8 K of 8 tables 5.8, against 9.2 in one cluster.  (CTAs of 512 threads: 9.9, 9.9, 15.3, 21.5, 27.9, 7.6.)
 // A table with more pairs than the cluster holds (the host knows the average only) is sorted by it through memory, every CTA
-// taking a share of the pairs tile by tile.  (Pipelines of 20 tables with nearly all lookups in one, us per mini-batch, chained
-// passes / one CTA of the cluster / all of them: 24 K pairs 106 / 124 / 78, 74 K 154 / 366 / 137, 295 K 215 / 1 388 / 256.)
+// taking a share of the pairs tile by tile: right, and slow (nearly all lookups in one of 20 to 26 tables, the sort alone, chained
+// passes / this: 76 K pairs 21 / 100 us, 204 K 28 / 256, 1.7 M 71 / 474), so the mini-batches that come here are those that have
+// as many lookups as bags (backward_sorts_tables).
 template <int CTAS, int NT, int ITEMS>
 __global__ void __launch_bounds__(NT)
     k_sort_segments(int32_t* keys_in, int32_t* vals_in, int32_t* keys_out, int32_t* vals_out, const int32_t* offsets_0,
@@ -619,25 +620,45 @@ static bool sort_in_cluster(int64_t n_max, const WaitCfg& w) {
 
 bool sort_is_long(int64_t n_max, WaitCfg w) { return !sort_in_cluster(n_max, w); }
 
-// For contexts of one lookup per bag at most, on average: there the host knows how many pairs a table has, and takes a cluster
-// that holds them.  (Elsewhere it knows how many there could be.  Four times as many as there were, 37 clusters of 16 CTAs of 512
-// threads for 9 K pairs each took 67 us beside a pipeline's other kernels, where the chained passes take 3 x 15.)
+// For contexts of one lookup per bag at most, on average: the cluster of a table holds the pairs that an average table of the
+// context can have.  (In contexts of several lookups per bag that is far more than a mini-batch's tables have: four times as many,
+// 37 clusters of 16 CTAs of 512 threads for 9 K pairs each took 67 us beside a pipeline's other kernels, where the chained passes
+// take 3 x 15.)
+//
+// There may be as many clusters as run side by side, more or less: the later ones wait for the first, and thousands of CTAs that
+// find a few pairs each take longer to start than the list to sort.  Mini-batches one after the other (hl_step), us each, the sort
+// alone in brackets, chained passes or one cluster / clusters per table.  Of 4 CTAs: 8 K pairs of 37 tables 62.5 (11) / 58.7 (8.4), of
+// 100 65.5 (11) / 62 (10), of 128 61.0 (11) / 62.3 (15), of 300 77 (11) / 83 (25), of 1 000 108 (11) / 154 (76); 33 K of 100 76 (16) /
+// 69 (11), of 200 81 (16) / 77 (18), of 300 90 (16) / 93 (25); 131 K of 200 108 (19) / 104 (22), of 300 117 (20) / 117 (29).  Of 8: 40
+// tables of 16 384 184 (34) / 180 (41), 60 219 (43) / 213 (42), 80 of 8 193 180 (34) / 181 (41).  Of 16, which find few places: 6
+// tables of 16 385 104 (19) / 91 (13), 12 125 (21) / 125 (27), 20 146 (27) / 153 (44), 40 184 (34) / 215 (81); pipelined, 9 of 30 000
+// 64 / 71.  Of 16 with 512 threads, one to a multiprocessor: 3 of 32 769 114 (20) / 99 (14), 4 pipelined 82 / 81, 7 132 (22) / 134
+// (37), 26 205 (38) / 262 (101).
 static int64_t segment_pairs(int64_t n_max, int tables) { return div_up(n_max, tables); }
-bool sort_by_segments(int64_t n_max, int64_t n_bags, int tables, WaitCfg w) {
+struct SegmentShape {
+    int ctas, threads, most_ctas;      // of a cluster, of a CTA, of the launch
+};
+static SegmentShape segment_shape(int64_t pairs) {
+    if (pairs <= 16384) return {pairs <= 8192 ? 4 : 8, 256, 960};
+    return pairs <= 32768 ? SegmentShape{16, 256, 192} : SegmentShape{16, 512, 96};
+}
+bool sort_by_segments(int64_t n_max, int64_t n_bags, int tables, bool merge, WaitCfg w) {
     const int64_t pairs = segment_pairs(n_max, tables);
-    return n_max > 0 && n_max <= n_bags && w.stall_tile < 0 &&
-           (pairs <= 16384 || (pairs <= 65536 && sort_cluster_ctas() == 16));
+    if (n_max <= 0 || n_max > n_bags || w.stall_tile >= 0 || pairs > 65536) return false;
+    const SegmentShape s = segment_shape(pairs);
+    const int64_t launched = (int64_t)tables * (merge ? 1 : 2) * s.ctas;
+    if (launched > s.most_ctas || (launched > 800 && sort_in_cluster(n_max, w))) return false;
+    return s.ctas < 16 || sort_cluster_ctas() == 16;
 }
 
 int32_t sort_segments(const SegmentArgs& a, cudaStream_t stream) {
-    const int64_t pairs = segment_pairs(a.max_nnz, a.tables);
-    const int ctas = pairs <= 8192 ? 4 : pairs <= 16384 ? 8 : 16, threads = pairs <= 32768 ? 256 : 512;
-    const auto kernel = pairs <= 8192    ? k_sort_segments<4, 256, 8>
-                        : pairs <= 16384 ? k_sort_segments<8, 256, 8>
-                        : pairs <= 32768 ? k_sort_segments<16, 256, 8>
-                                         : k_sort_segments<16, 512, 8>;
-    HL_CUDA_TRY(launch_cluster(kernel, (int64_t)a.tables * (a.merge ? 1 : 2) * ctas, threads, sort_smem_bytes(threads, 8), ctas,
-                               stream, a.keys_in, a.vals_in, a.keys_out, a.vals_out, a.side[0].offsets, a.side[0].d_n_samples,
+    const SegmentShape s = segment_shape(segment_pairs(a.max_nnz, a.tables));
+    const auto kernel = s.threads == 512 ? k_sort_segments<16, 512, 8>
+                        : s.ctas == 16   ? k_sort_segments<16, 256, 8>
+                        : s.ctas == 8    ? k_sort_segments<8, 256, 8>
+                                         : k_sort_segments<4, 256, 8>;
+    HL_CUDA_TRY(launch_cluster(kernel, (int64_t)a.tables * (a.merge ? 1 : 2) * s.ctas, s.threads,
+                               sort_smem_bytes(s.threads, 8), s.ctas, stream, a.keys_in, a.vals_in, a.keys_out, a.vals_out, a.side[0].offsets, a.side[0].d_n_samples,
                                a.side[0].key_bias, a.side[1].offsets, a.side[1].d_n_samples, a.side[1].key_bias, a.d_n_lookups,
                                a.tables, a.max_batch, a.bags_per_sample, a.merge, a.passes, a.max_nnz));
     note_launches(1);

@@ -33,6 +33,9 @@ CASES = {
     "one_full_table_512_threads_last": ([700, 90_000], 65_536, [(0, 0), (2, 2)], 0.6),
     "all_popular": ([9000] + [10] * 15, 3000, [(5, 9), (1, 1), (0, 1)] + [(0, 0)] * 13, 1.0),
     "one_table": ([20_000], 5000, [(1, 1)], 0.5),
+    # (mini-batches in turn: as many lookups as bags, and fewer, which the chained passes or one cluster sort)
+    "both_ways_short": ([4000, 60, 900], 3000, [[(1, 1)] * 3, [(3, 5), (0, 0), (0, 0)]], 0.9),
+    "both_ways_long": ([40_000, 50, 3000], 14_000, [[(0, 1), (1, 1), (0, 1)], [(1, 1)] * 3], 0.8),
 }
 
 
@@ -45,8 +48,8 @@ def test_pipeline_over_tables_of_many_sizes(case, order):
     rng = np.random.default_rng(len(case))
     base = np.concatenate([[0], np.cumsum(rows)])
     batches = []
-    for _ in range(steps):
-        lengths = np.concatenate([rng.integers(lo, hi + 1, B) for lo, hi in spans])
+    for k in range(steps):
+        lengths = np.concatenate([rng.integers(lo, hi + 1, B) for lo, hi in (spans[k % 2] if isinstance(spans[0], list) else spans)])
         offsets = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
         r = np.repeat(np.repeat(rows, B), lengths)
         limit = np.where(rng.random(len(r)) < 0.5, np.minimum(r, 20), r)          # half of them on a few rows

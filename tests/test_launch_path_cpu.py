@@ -145,6 +145,29 @@ def test_graphs_queue_what_plain_launches_queue(B, lib, batch, order, n_sets):
     assert sum(x.startswith("graph") for x in late) > 100 and not any(x.startswith("plain") for x in late)
 
 
+@pytest.mark.parametrize("tables, batch, lookups, sort", [
+    (21, 4096, 21 * 4096, ["k_sort_segments"]), (3, 43008, 3 * 43008, ["k_sort_segments"]), (60, 16384, 60 * 16384, ["k_sort_segments"]),
+    (21, 4096, 21 * 4096 - 1, ["k_sort_pass"] * 3), (21, 1000, 21 * 1000 - 1, ["k_sort_cluster"]),    # some bags empty, others long?
+    (100, 82, 8200, ["k_sort_segments"]), (101, 81, 8181, ["k_sort_cluster"]), (1000, 8, 8000, ["k_sort_cluster"]),
+    (120, 400, 48_000, ["k_sort_segments"]), (121, 400, 48_400, ["k_sort_pass"] * 3), (61, 8193, 61 * 8193, ["k_sort_pass"] * 3),
+    (6, 16385, 6 * 16385, ["k_sort_segments"]), (7, 16385, 7 * 16385, ["k_sort_pass"] * 3),
+    (3, 32769, 3 * 32769, ["k_sort_segments"]), (4, 32769, 4 * 32769, ["k_sort_pass"] * 3), (1, 65537, 65537, ["k_sort_pass"] * 3)])
+def test_tables_are_sorted_by_themselves_where_their_clusters_fit_the_chip(B, lib, tables, batch, lookups, sort):
+    """And where a mini-batch has as many lookups as bags: otherwise one table may have most of them."""
+    c = _Context(B, tables=tables, batch=batch, rows=20, dim=4, hot=60_000, staging=60_000)
+    s, side, st = c.mem(), c.mem(), c.one_set()
+    step_buffers = B.make_step_buffers(st["perm"], st["counts"], st["pop"], st["non"], None, st["cold_rows"], st["n_cold"],
+                                       st["pooled_pop"], st["pooled_non"])
+    for n in (lookups, tables * batch - 1, lookups):         # (a mini-batch of the other kind in between)
+        at = lib.fake_lines()
+        B.hl_step(c.ctx, B.make_batch(c.mem(), c.mem(), batch, n), None, 0, step_buffers, c.cache, c.table, c.mem(), c.mem(),
+                  0.1, False, s, side)
+        if n == lookups:
+            names = [_name(x).split("<")[0] for x in _log(lib, at)]
+            assert [x for x in names if x.startswith("k_sort")] == sort
+    c.close()
+
+
 def test_many_runs_of_kernels_with_many_argument_sets_all_become_graphs(B, lib):
     """A pipeline issued call by call: nine calls per mini-batch, four buffer sets, inputs that change.  No run of kernels
     may push out another's graph for ever: in the steady state nothing is built and nothing is launched plainly."""
