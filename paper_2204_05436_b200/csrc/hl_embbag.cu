@@ -217,8 +217,9 @@ struct FwdShape {
 // a run are one list, which the group walks in blocks of U: while a block is summed, the rows of the next one are on their way
 // into shared memory and the ids of the one after that into registers, whatever bags they belong to.  (A lane copies and reads
 // the same 16 bytes of every row, so nothing but its own copies is waited for.)  Rows are added in lookup order in fp64 and the
-// sum is rounded once, so that cancellation between the rows of a bag costs no accuracy.  A lookup that is skipped (negative id)
-// or outside the cache adds zeros.
+// sum is rounded once, so that cancellation between the rows of a bag costs no accuracy; the row of a bag of one lookup is copied
+// as it is where rows have up to 64 fp32 (the sign of a zero and the bits of a NaN with it), and added to zero in wider ones.  A
+// lookup that is skipped (negative id) or outside the cache adds zeros.
 //
 // What bounds it is how many rows are on their way, and how often a bag makes them stop: with a loop over the lookups of one
 // bag after the other (loads into registers, four at a time) 2.1 M lookups of 256-byte rows in bags of 5 took 114.7 us, 655 K of
@@ -281,11 +282,12 @@ __global__ void __launch_bounds__(FwdShape<NV>::NT, FwdShape<NV>::CTAS) k_embbag
     double acc[NV][4] = {};
     int k = 0;                                          // the bag being summed, and where it ends
     int32_t end = __shfl_sync(kAll, my_end, 0, G);
+    bool copied = G < 32 && end - p == 1;               // its one row is copied, bit for bit, and not summed
     float4* to = reinterpret_cast<float4*>(out) + (int64_t)first * D4 + sub;
     auto next_bag = [&]() {
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-            if (sub + v * G < D4)
+            if (sub + v * G < D4 && !copied)
                 __stcs(to + v * G, make_float4((float)acc[v][0], (float)acc[v][1], (float)acc[v][2], (float)acc[v][3]));
             acc[v][0] = acc[v][1] = acc[v][2] = acc[v][3] = 0.0;
         }
@@ -295,7 +297,9 @@ __global__ void __launch_bounds__(FwdShape<NV>::NT, FwdShape<NV>::CTAS) k_embbag
             my_end = next_ends;
             next_ends = ends_at(k + G);
         }
+        const int32_t begin = end;
         end = __shfl_sync(gmask, my_end, k & (G - 1), G);          // (behind the last bag: 2^31 - 1)
+        copied = G < 32 && end - begin == 1;
     };
     for (int b = 0; __any_sync(kAll, p < hi); p += U, b = b == NB - 1 ? 0 : b + 1) {
         const int32_t mine = next_ids;
@@ -310,8 +314,12 @@ __global__ void __launch_bounds__(FwdShape<NV>::NT, FwdShape<NV>::CTAS) k_embbag
                 r[v] = sub + v * G < D4 ? ring[((b * U + u) * NV + v) * NT + threadIdx.x] : f4_zero();
             if (p + u < hi) {
                 while (end <= p + u) next_bag();
+                if (copied) {
+                    if (sub < D4) __stcs(to, r[0]);
+                } else {
 #pragma unroll
-                for (int v = 0; v < NV; ++v) add_row(acc[v], r[v]);
+                    for (int v = 0; v < NV; ++v) add_row(acc[v], r[v]);
+                }
             }
         }
     }
