@@ -171,7 +171,8 @@ extern "C" int32_t hl_set_host_tables(hl_ctx* ctx, float* const* h_table_bases) 
         if (!h_table_bases[t] || (reinterpret_cast<uintptr_t>(h_table_bases[t]) & 15)) return HL_EINVAL;
     HL_CUDA_TRY(cudaDeviceSynchronize());      // no kernel may still be reading the previous addresses
     HL_CUDA_TRY(cudaMemcpy(ctx->r.table_ptrs, h_table_bases, sizeof(float*) * ctx->T, cudaMemcpyHostToDevice));
-    ctx->per_table = 1;
+    ctx->per_table = ctx->tables_on_device = 1;
+    for (int t = 0; t < ctx->T && ctx->tables_on_device; ++t) ctx->tables_on_device = in_device_memory(h_table_bases[t]);
     return HL_OK;
 }
 

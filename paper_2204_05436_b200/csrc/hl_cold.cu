@@ -272,13 +272,15 @@ constexpr int64_t kPacedFewRows = 10240;
 // 64 bytes read 732 / 610, written 759 / 624; 144 bytes (300 K) 1 822 / 1 685, 1 944 / 1 445; 192 bytes (250 K) 1 053 / 1 027,
 // 1 103 / 1 040; 256 bytes (200 K) 1 016 / 1 013, 1 065 / 1 062.  40 GiB table: 64 bytes 1 233 / 1 076, 1 224 / 1 125; 256 bytes
 // 1 664 / 1 814, 1 906 / 1 870; 512 bytes (200 K) 2 008 / 2 240, 2 116 / 2 098.
+// (A table in device memory has no link in between: two CTAs per multiprocessor, 1 M of 2 M rows of 64 bytes written 86 us, read 106,
+// with 32 CTAs 645 and 645; of 256 bytes 201 and 222, written with 32 CTAs 1 697.)
 constexpr int kAloneCtas = 32;
 constexpr int kAloneWideRow = 256;
 
 // What a launch of the mover needs to know about its context.
 struct MoveCfg {
     int sms;            // multiprocessors of the device: the launch has at most 2 CTAs per SM
-    bool alone;         // nothing else on the chip
+    bool link_alone;    // nothing else on the chip, and the table is behind the link
     int min_ctas;       // CTAs that work however few rows there are (at full rate)
     int paced_ctas;     // CTAs of a paced transfer of up to kPacedFewRows rows; 0: never paced
     int paced_more;     // ... of more rows
@@ -407,7 +409,7 @@ int32_t launch_move_rows(float* dense_side, int64_t dense_row0, TableMap table, 
     const int row_bytes = D * 4;
     if (row_bytes <= kBulkStageBytes) {
         const int rows_per_stage = kBulkStageBytes / row_bytes < kBulkThreads ? kBulkStageBytes / row_bytes : kBulkThreads;
-        const bool few = cfg.alone && (TO_TABLE || row_bytes < kAloneWideRow);
+        const bool few = cfg.link_alone && (TO_TABLE || row_bytes < kAloneWideRow);
         const int grid = grid_for(n_max, rows_per_stage, few ? kAloneCtas : 2 * cfg.sms);
         const int requests = (row_bytes + 127) / 128;        // of one row
         const int paced_fit = TO_TABLE ? kPacedRequests / requests : kPacedReadBytes / row_bytes;
@@ -487,12 +489,20 @@ static TableMap table_map(const hl_ctx* ctx, const float* host_table) {
     return m;
 }
 
+bool in_device_memory(const void* p) {
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type == cudaMemoryTypeDevice;
+    (void)cudaGetLastError();
+    return false;
+}
+
 // how the movers of this context are launched: beside the kernels of other mini-batches (`width` = the context's setting),
-// or alone on the chip (`width` = 0: the link's full rate)
-static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false, bool reads = false) {
+// or alone on the chip (`alone`, for the table they move to or from)
+static MoveCfg move_cfg(const hl_ctx* ctx, int width, bool in_schedule = false, bool reads = false,
+                        const float* alone = nullptr) {
     MoveCfg c;
     c.sms = ctx_sms(ctx);
-    c.alone = width == 0;
+    c.link_alone = alone && !(ctx->per_table ? ctx->tables_on_device != 0 : in_device_memory(alone));
     c.min_ctas = width > 0 ? width : 2 * c.sms;
     c.paced_ctas = in_schedule ? (ctx->mover_width_set ? width : kPacedCtas) : 0;
     c.paced_more = in_schedule && reads && !ctx->mover_width_set ? kReadCtasDefault : c.paced_ctas;
@@ -505,7 +515,7 @@ int32_t launch_gather_rows(hl_ctx* ctx, float* dst, int64_t dst_row0, const floa
                            const int64_t* d_n, int64_t n_max, int32_t* status, cudaStream_t stream) {
     // loading the hot cache happens with nothing else on the chip
     return launch_move_rows<false>(dst, dst_row0, table_map(ctx, table), rows, d_n, n_max, ctx->N, ctx->D, nullptr,
-                                   move_cfg(ctx, 0), status, stream);
+                                   move_cfg(ctx, 0, false, true, table), status, stream);
 }
 
 }  // namespace hl
@@ -724,5 +734,6 @@ extern "C" int32_t hl_flush_hot(hl_ctx* ctx, const float* d_cache, const int32_t
     // runs between learning phases, with nothing else on the chip
     return launch_move_rows<true>(const_cast<float*>(d_cache), 0, table_map(ctx, host_table), d_hot_rows, d_n_hot,
                                   ctx->hot_cap, ctx->N,
-                                  ctx->D, nullptr, move_cfg(ctx, 0), ctx->r.status, static_cast<cudaStream_t>(stream_));
+                                  ctx->D, nullptr, move_cfg(ctx, 0, false, false, host_table), ctx->r.status,
+                                  static_cast<cudaStream_t>(stream_));
 }

@@ -94,6 +94,7 @@ struct hl_ctx {
     int64_t test_stall_tile;           // with it: the tile / mover stage that never delivers (-1: none)
     int64_t* h_table_base;             // host copy [T+1]
     int per_table;                     // 1: the host table is one allocation per table (r.table_ptrs is set)
+    int tables_on_device;              // ... and all of them are device memory
     hl::Regions r;
     int timing_on;                     // optional kernel timers (hl_timing_enable)
     cudaEvent_t timer[HL_TIMER_COUNT][2];
@@ -656,6 +657,9 @@ int32_t assign_and_prepare(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n
                            int32_t* d_fwd_src, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
                            bool merge, bool by_table, cudaStream_t stream, const SortAside* aside,
                            int32_t** out_slots = nullptr, int32_t** out_bags = nullptr);
+
+// Whether p is device memory (hl_cold.cu).
+bool in_device_memory(const void* p);
 
 // Asks for what the backward's sum kernel needs of shared memory for rows of D fp32, on the current device (hl_embbag.cu).
 bool piece_memory_granted(int D);

@@ -39,7 +39,7 @@ std::map<const void*, Kernel> kernels;
 std::vector<std::string> lines;
 std::map<std::string, int> calls, fail_at;  // calls of a function so far; which of them fails (-1: every one)
 std::string fail_kernel;                    // launches of this kernel fail
-std::set<const void*> capturing;
+std::set<const void*> capturing, device_memory;
 long handles = 0x1000;
 
 bool fails(const char* name) {
@@ -137,6 +137,7 @@ void fake_reset() {
     fail_at.clear();
     fail_kernel.clear();
     capturing.clear();
+    device_memory.clear();
     handles = 0x1000;                       // (streams and events of two runs have the same names)
 }
 void fake_fail(const char* function, int nth) {
@@ -149,6 +150,7 @@ void fake_capture(void* stream, int on) {
     if (on) capturing.insert(stream);
     else capturing.erase(stream);
 }
+void fake_device_memory(const void* p) { device_memory.insert(p); }
 int fake_calls(const char* function) { return calls[function]; }
 int fake_lines() { return (int)lines.size(); }
 const char* fake_line(int i) { return lines[i].c_str(); }
@@ -185,7 +187,12 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
     return cudaSuccess;
 }
 cudaError_t cudaGetSymbolAddress(void**, const void*) { return cudaErrorUnknown; }
-cudaError_t cudaPointerGetAttributes(cudaPointerAttributes*, const void*) { return cudaErrorUnknown; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+    if (!device_memory.count(p)) return cudaErrorUnknown;
+    memset(a, 0, sizeof(*a));
+    a->type = cudaMemoryTypeDevice;
+    return cudaSuccess;
+}
 cudaError_t cudaMallocManaged(void**, size_t, unsigned) { return cudaErrorMemoryAllocation; }
 cudaError_t cudaHostAlloc(void**, size_t, unsigned) { return cudaErrorMemoryAllocation; }
 cudaError_t cudaMemAdvise(const void*, size_t, cudaMemoryAdvise, int) { return cudaErrorUnknown; }

@@ -37,6 +37,7 @@ def lib(tmp_path_factory):
         lib = B._load()
     lib.fake_line.restype = ctypes.c_char_p
     lib.fake_capture.argtypes = [ctypes.c_void_p, ctypes.c_int]
+    lib.fake_device_memory.argtypes = [ctypes.c_void_p]
     return lib
 
 
@@ -165,6 +166,30 @@ def test_tables_are_sorted_by_themselves_where_their_clusters_fit_the_chip(B, li
         if n == lookups:
             names = [_name(x).split("<")[0] for x in _log(lib, at)]
             assert [x for x in names if x.startswith("k_sort")] == sort
+    c.close()
+
+
+@pytest.mark.parametrize("dim, written, read", [(16, 32, 32), (64, 32, 296)])
+def test_popular_rows_of_a_table_in_device_memory_move_with_the_whole_chip(B, lib, dim, written, read):
+    """Few CTAs are for the host link: a table on the device, as one allocation or one per table, has none in its way."""
+    c = _Context(B, dim=dim, hot=100_000, batch=16)
+    s, hot_rows, n_hot = c.mem(), c.mem(), c.mem()
+
+    def grids():
+        at = lib.fake_lines()
+        B.hl_flush_hot(c.ctx, c.cache, hot_rows, n_hot, c.table, s)
+        B.hl_build_remap(c.ctx, hot_rows, n_hot, c.table, c.cache, None, s)
+        return [int(x.split("grid=")[1].split(" ")[0]) for x in _log(lib, at) if _name(x).startswith("k_move_rows")]
+
+    assert grids() == [written, read]
+    lib.fake_device_memory(c.table)
+    assert grids() == [296, 296]
+    per_table = [c.mem() for _ in range(c.T)]
+    for on_device in range(c.T + 1):             # (all of them have to be)
+        B.hl_set_host_tables(c.ctx, per_table)
+        assert grids() == ([296, 296] if on_device == c.T else [written, read])
+        if on_device < c.T:
+            lib.fake_device_memory(per_table[on_device])
     c.close()
 
 
