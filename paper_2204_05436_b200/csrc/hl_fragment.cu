@@ -84,6 +84,11 @@ __device__ void partition_by_flags(const uint32_t* words, int B, int32_t* __rest
 // Probe: how a global row is looked up in the popular set (BitmapProbe: the dense bitmap of the 32-bit path;
 // HashProbe: the hashed remap of the wide-id path).
 // chain / n_chain: the state of k_frag_place's chain, cleared here.
+// Lookups asked for together: four, or two where a lookup takes a sector of 64-bit keys (with four the hash probe's kernels spilled
+// up to 160 bytes).  Hash probe, one after the other / four / two together: 426 K bags of one 12.1 / 14.0 / 11.6 us, 416 K lookups
+// in bags of 4 24.7 / 19.8 / 17.0, 31 K in bags of 3 18.9 / 17.6 / 13.9, 1 200 8.4 / 11.3 / 8.2, 320 K in bags of 20 29.2 / 20.7 / 20.8.
+template <class Probe>
+constexpr int kFlagLookups = std::is_same_v<Probe, HashProbe> ? 2 : 4;
 template <bool SHORT_BAGS, class Probe>
 __global__ void __launch_bounds__(kFlagThreads, 4) k_frag_flags(const int32_t* __restrict__ indices,
                                                              const int32_t* __restrict__ offsets, int B, int T, int S,
@@ -103,7 +108,7 @@ __global__ void __launch_bounds__(kFlagThreads, 4) k_frag_flags(const int32_t* _
         if (threadIdx.x == 0) s_miss = 0;
         __syncthreads();
         if (SHORT_BAGS) {
-            constexpr int U = 4;
+            constexpr int U = kFlagLookups<Probe>;
             bool miss = false;
             for (int t0 = warp; t0 < T; t0 += NW * U) {
                 int32_t lo[U], hi[U];
@@ -163,7 +168,7 @@ __global__ void __launch_bounds__(kFlagThreads, 4) k_frag_flags(const int32_t* _
                 __syncwarp();
                 const int32_t lo = s_start[warp][0], hi = s_start[warp][in_group];
                 const int64_t base = table_base[t], rows = table_base[t + 1] - base;
-                constexpr int U = 4;
+                constexpr int U = kFlagLookups<Probe>;
                 for (int32_t j0 = lo + part * 32; j0 < hi; j0 += share * 32 * U) {
                     int32_t idx[U];
                     bool hit[U];
