@@ -249,8 +249,12 @@ struct PlaceArgs {
 
 // ITEMS destination bags per thread, in rows of 32 bags per warp.
 // LISTS: bags of several lookups; a warp takes the lookups of a row's 32 bags as one list (which they are at their
-// destination), 128 at a time, so that every lane has one and four loads are on their way: 333 K lookups in 111 K bags
-// 11.5 us, 1.3 M in 65 K bags 24 us; with 4 or 16 lanes for one bag after the other 26 and 89 us.
+// destination), 128 at a time, so that every lane has one and four loads are on their way (with 4 or 16 lanes for one bag after
+// the other the kernel takes two to four times as long).  What a lookup needs of the popular rows is asked for four lookups at a
+// time with MARK, where every lookup of X needs it too (80 registers; one after the other / together: 333 K lookups in 111 K bags
+// 15.2 / 14.8 us, 1.3 M in 65 K bags 42.5 / 33.0), and one after the other without, where X's lookups need nothing (54 registers, and
+// 57 with the hash probe; together, with 78 and 96 / one after the other: 1.3 M 17.6 / 15.9, 130 K in bags of 5 7.6 / 7.0; hash probe,
+// 416 K in bags of 4 14.9 / 10.8, 320 K in bags of 20 13.7 / 12.4).
 template <bool LISTS, int ITEMS, bool MARK, class Probe, typename NonId>
 __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe remap, NonId* __restrict__ non_ids,
                                                          ColdMarks marks) {
@@ -442,7 +446,19 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
                     rows[u] = a.table_base[t + 1] - base[u];
                 }
                 NonId id[U];
-                resolve(std::integral_constant<int, U>(), in, pop_bag, base, rows, idx, id);
+                if constexpr (MARK) {
+                    resolve(std::integral_constant<int, U>(), in, pop_bag, base, rows, idx, id);
+                } else {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int64_t g = base[u] + idx[u];
+                        id[u] = (NonId)-1;
+                        if (!in[u]) continue;
+                        if (pop_bag[u]) id[u] = (NonId)remap.slot(remap.request(g), g);
+                        else if (idx[u] >= 0 && idx[u] < rows[u]) id[u] = (NonId)g;
+                        else set_status(a.status, HL_EBOUNDS);
+                    }
+                }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     if (!in[u]) continue;
