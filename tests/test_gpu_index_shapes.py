@@ -1,5 +1,5 @@
-"""The index-only calls (fragment, cold-row search, sort) at the sizes where they change their launch: bags per tile (1 024
-once there is a 256-bag tile per multiprocessor), lists of lookups for bags of several, long bags in the popularity test,
+"""The index-only calls (fragment, cold-row search, sort) at the sizes where they change their launch: bags per tile (512
+once there is a 256-bag tile per multiprocessor, 1 024 once there is one of those), lists of lookups for bags of several, long bags in the popularity test,
 words per thread and the summary bitmap of the cold-row ranking, and the sort in one cluster (up to 32 768 lookups) or in
 tiles.  All outputs are integers and must equal the oracle's."""
 import numpy as np
@@ -17,6 +17,9 @@ CASES = {
     "inputs_33_ragged": ([100, 7, 3000], 33, 1, 0, 3, 0.8),
     "tiles_of_256_last_full": ([997] * 37, 1024, 1, 1, 1, 0.97),        # 37 888 bags: 148 tiles of 256
     "tiles_of_1024": ([997] * 37, 1025, 1, 0, 2, 0.97),
+    "tiles_of_512_last_full": ([997] * 37, 4096, 1, 1, 1, 0.97),         # 151 552 bags: 148 tiles of 1 024
+    "tiles_of_1024_from_here": ([997] * 37, 4097, 1, 0, 2, 0.97),
+    "tiles_of_1024_mostly_popular": ([997] * 37, 4099, 1, 1, 1, 0.9999),
     "tiles_of_256_some_longer": ([997] * 3, 1025, 1, 0, 2, 0.9),
     "lists_short": ([997] * 20, 2049, 1, 0, 9, 0.98),
     "lists_of_up_to_129": ([997] * 2, 333, 2, 0, 4, 0.98),
