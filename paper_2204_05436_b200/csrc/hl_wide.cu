@@ -366,50 +366,58 @@ __global__ void __launch_bounds__(kThreads) k_wide_classify(const long long* __r
     n_non = n_non < 0 ? 0 : (n_non > max_batch ? max_batch : n_non);
     int64_t L = offsets[(int64_t)n_non * bags_per_sample_all];
     if (L > cap) L = cap;
-    // a warp takes 32 * U lookups at a time, whose loads go out together, and one place in the list for all their cold ones
-    constexpr int U = 4;
+    // A warp takes 32 * U lookups at a time, whose loads go out together, and one place in the list for all their cold ones: four a
+    // lane where there are many, one where that leaves the chip idle.  One / four a lane, half of them cold and nearly all: 1 K lookups
+    // 3.0 / 4.6, 3.1 / 5.0 us, 10 K 3.3 / 4.7, 3.8 / 6.6, 39 K 4.1 / 5.8, 4.9 / 7.8, 78 K 5.9 / 6.1, 7.0 / 7.8, 91 K 6.1 / 5.8, 7.6 / 7.8,
+    // 112 K 7.1 / 6.1, 8.9 / 7.9, 426 K 14.8 / 10.5, 15.5 / 12.0.
+    constexpr int64_t kFew = 81920;
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (int64_t)gridDim.x * (kThreads / 32);
-    for (int64_t j0 = warp * 32 * U + lane; j0 - lane < L; j0 += n_warps * 32 * U) {
-        long long g[U];
-        HashProbe::Request found[U];
-        bool cold[U];
-        unsigned m[U];
-        int n_cold = 0;
+    const auto classify = [&](auto per_lane) {
+        constexpr int U = decltype(per_lane)::value;
+        for (int64_t j0 = warp * 32 * U + lane; j0 - lane < L; j0 += n_warps * 32 * U) {
+            long long g[U];
+            HashProbe::Request found[U];
+            bool cold[U];
+            unsigned m[U];
+            int n_cold = 0;
 #pragma unroll
-        for (int u = 0; u < U; ++u) g[u] = j0 + u * 32 < L ? rows[j0 + u * 32] : -1;
+            for (int u = 0; u < U; ++u) g[u] = j0 + u * 32 < L ? rows[j0 + u * 32] : -1;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (g[u] >= N) {
-                set_status(status, HL_EBOUNDS);
-                g[u] = -1;
+            for (int u = 0; u < U; ++u) {
+                if (g[u] >= N) {
+                    set_status(status, HL_EBOUNDS);
+                    g[u] = -1;
+                }
+                if (g[u] >= 0) found[u] = probe.request(g[u]);
             }
-            if (g[u] >= 0) found[u] = probe.request(g[u]);
-        }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int32_t s = g[u] >= 0 ? probe.slot(found[u], g[u]) : -1;
-            cold[u] = g[u] >= 0 && s < 0;
-            if (j0 + u * 32 < L && !cold[u]) slots[j0 + u * 32] = s;
-            m[u] = __ballot_sync(0xffffffffu, cold[u]);
-            n_cold += __popc(m[u]);
-        }
-        int32_t first = 0;
-        if (lane == 0 && n_cold) first = atomicAdd(d_n_cold_lookups, n_cold);
-        int64_t i = __shfl_sync(0xffffffffu, first, 0);
+            for (int u = 0; u < U; ++u) {
+                const int32_t s = g[u] >= 0 ? probe.slot(found[u], g[u]) : -1;
+                cold[u] = g[u] >= 0 && s < 0;
+                if (j0 + u * 32 < L && !cold[u]) slots[j0 + u * 32] = s;
+                m[u] = __ballot_sync(0xffffffffu, cold[u]);
+                n_cold += __popc(m[u]);
+            }
+            int32_t first = 0;
+            if (lane == 0 && n_cold) first = atomicAdd(d_n_cold_lookups, n_cold);
+            int64_t i = __shfl_sync(0xffffffffu, first, 0);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int64_t at = i + __popc(m[u] & ((1u << lane) - 1u));
-            i += __popc(m[u]);
-            if (cold[u] && at < max_nnz) {
-                const uint32_t key = (uint32_t)g[u];
-                sort_key[at] = (int32_t)key;
-                sort_val[at] = (int32_t)(j0 + u * 32);
-                if (HIST)
-                    for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 255u], 1u);
+            for (int u = 0; u < U; ++u) {
+                const int64_t at = i + __popc(m[u] & ((1u << lane) - 1u));
+                i += __popc(m[u]);
+                if (cold[u] && at < max_nnz) {
+                    const uint32_t key = (uint32_t)g[u];
+                    sort_key[at] = (int32_t)key;
+                    sort_val[at] = (int32_t)(j0 + u * 32);
+                    if (HIST)
+                        for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(key >> (8 * p)) & 255u], 1u);
+                }
             }
         }
-    }
+    };
+    if (L > kFew) classify(std::integral_constant<int, 4>());
+    else classify(std::integral_constant<int, 1>());
     if (HIST) {
         __syncthreads();
         for (int i = threadIdx.x; i < passes * 256; i += kThreads) {
@@ -622,7 +630,7 @@ extern "C" int32_t hl_wide_index_cold(hl_wide* w, const int32_t* d_non_offsets, 
     const int64_t sort_words = sort_clear_words(w->max_nnz, lower_bits, waits);
     HL_CUDA_TRY(clear_words(w->cold_clear, (int64_t)(w->sort_hist - w->cold_clear) + sort_words, stream));
     HL_CUDA_TRY(launch(sort_words ? k_wide_classify<true> : k_wide_classify<false>,
-                       grid_for(w->max_nnz, kThreads * 4, 3 * w->sms), kThreads, stream,
+                       grid_for(w->max_nnz, kThreads, 3 * w->sms), kThreads, stream,
                        reinterpret_cast<const long long*>(d_non_rows), d_non_offsets, d_n_non, w->max_batch, w->T * w->S,
                        non_cap, w->N, probe, d_non_slots, w->sort_keys[0], w->sort_vals[0], w->cold_n, w->max_nnz,
                        w->sort_hist, (lower_bits + 7) / 8, w->status));

@@ -17,6 +17,9 @@ CASES = {
     "upper_bits_cluster": ([2_147_483_647, 2_147_483_647, 3], 2000, 0.3, 4000),  # 2^32 + 1 rows
     "upper_bits_tiles": ([2_000_000_000] * 9, 4097, 0.2, 20_000),
     "lower_bits_tiles": ([500_000_000] * 8, 4097, 0.2, 20_000),
+    "one_a_lane_last": ([500_000_000] * 8, 10_240, 0.3, 20_000),                 # classified: one lookup a lane up to 81 920
+    "four_a_lane_first": ([500_000_000] * 8, 10_241, 0.3, 20_000),
+    "four_a_lane": ([2_000_000_000] * 3, 65_537, 0.1, 1 << 30),
     "many_upper_values": ([2_147_483_647] * 255, 300, 0.1, 500),
 }
 
