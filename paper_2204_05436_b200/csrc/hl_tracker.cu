@@ -108,8 +108,10 @@ __global__ void __launch_bounds__(kThreads) k_trk_keys(const int32_t* __restrict
 // popular row (thousands of lookups of a mini-batch), of the lookups themselves.  So the blocks of the next rounds' sets are on
 // their way while one round's are replayed, the 64 lookups behind the warp's first stay in registers, and beyond them four
 // groups of 32 are read at once (eight: no faster).  426 K lookups, 131 072 sets of 16, the whole update: 72.9 us with a set per
-// warp, 66.2 so (replay 30.1 -> 26.7, keys 8.3 -> 7.2); sets of 8 74.0 -> 64.7; 10 K lookups 26.4 -> 21.6.  (Six CTAs per
-// multiprocessor, with the registers that leaves: 31.7.)
+// warp, 66.2 so (replay 30.1 -> 26.7, keys 8.3 -> 7.2); sets of 8 74.0 -> 64.7; 10 K lookups 26.4 -> 21.6.  A set that is replayed
+// alone -- more than 16 ways, or the last head's run -- is asked for its oldest blocks only after a miss: with all five votes per
+// access, as sets side by side have to, 10 K lookups, 20 ways 17.7 us instead of 14.1 (32 ways 14.5 / 11.2), 426 K of 6 250 sets of 16
+// 49.3 / 43.5, of 65 536 sets of 32 42.3 / 38.4.  (16 ways with 48 registers instead of 40, five CTAs instead of six: 28.7 / 27.8.)
 template <int W>
 __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restrict__ keys,
                                                          const int32_t* __restrict__ vals,
@@ -164,8 +166,29 @@ __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restri
             }
             return b;
         };
+        // One access of one set, whose lanes are on, row gg: asked for its oldest blocks only where the row is not among them (the
+        // votes are what an access takes).
+        auto access_one = [&](Blocks& b, int32_t gg, bool on) {
+            const unsigned hit = __ballot_sync(kAll, on && b.tag == gg);
+            if (hit) {
+                if (lane == __ffs((int)hit) - 1) b.rr = 0;
+                hits += on && way == 0;
+                return;
+            }
+            unsigned oldest = __ballot_sync(kAll, on && b.rr == kRrpvMax);
+            if (!oldest) {
+                const int add = __any_sync(kAll, on && b.rr == 2) ? 1 : __any_sync(kAll, on && b.rr == 1) ? 2 : 3;
+                if (on && b.rr >= 0) b.rr += add;
+                oldest = __ballot_sync(kAll, on && b.rr == kRrpvMax);
+            }
+            if (lane == __ffs((int)oldest) - 1) {
+                b.tag = gg;
+                b.rr = kRrpvInsert;
+            }
+        };
         // one access of every group's set (active: it has one), row gg
         auto access = [&](Blocks& b, int32_t gg, bool active) {
+            if constexpr (NG == 1) return access_one(b, gg, true);
             const unsigned hit = __ballot_sync(kAll, b.tag == gg) >> shift & kMine;
             const unsigned r3 = __ballot_sync(kAll, b.rr == kRrpvMax) >> shift & kMine;
             const unsigned r2 = __ballot_sync(kAll, b.rr == 2) >> shift & kMine;
@@ -191,9 +214,10 @@ __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restri
                 rrpv[b.s * ways + way] = (uint8_t)b.rr;
             }
         };
+        const auto any = [&](bool x) { return NG == 1 ? x : (bool)__any_sync(kAll, x); };      // (of one group: the same in all)
         int h = take(), h_next = take();
         Blocks next = load(h), after = load(h_next);
-        while (__any_sync(kAll, h < 32)) {
+        while (any(h < 32)) {
             Blocks now = next;
             const int at = h;
             next = after;
@@ -203,10 +227,10 @@ __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restri
             // its run: up to the next one's beginning, or, of the last head, what of it is among the 32
             const unsigned behind = at < 31 ? begins & (kAll << (at + 1)) : 0u;
             const int end = at < 32 ? (behind ? __ffs((int)behind) - 1 : 32) : 0;
-            for (int t = at; __any_sync(kAll, t < end); ++t) access(now, __shfl_sync(kAll, g0, t & 31), t < end);
+            for (int t = at; any(t < end); ++t) access(now, __shfl_sync(kAll, g0, t & 31), t < end);
             // the last head's run may go on
             const bool on = at == last_head && end == 32;
-            if (__any_sync(kAll, on)) {
+            if (any(on)) {
                 const int from = __ffs((int)__ballot_sync(kAll, on)) - 1;            // a lane of the group it is in
                 const int32_t set = (int32_t)__shfl_sync(kAll, now.s, from);
                 // the row of the previous access, and whether that left it at RRPV 0, so that repeating it changes nothing
@@ -226,7 +250,7 @@ __global__ void __launch_bounds__(kThreads) k_trk_replay(const int32_t* __restri
                             hits += on && way == 0;
                             continue;
                         }
-                        access(now, gg, on);
+                        access_one(now, gg, on);
                         last = gg;
                         last_zero = __any_sync(kAll, on && now.tag == gg && now.rr == 0);
                     }

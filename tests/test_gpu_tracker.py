@@ -56,7 +56,7 @@ def _run(spec, n_sets, ways, n_batches=3, scale_rows=1.0, corrupt=False, select_
         h.close()
 
 
-@pytest.mark.parametrize("n_sets,ways", [(257, 4), (64, 16), (1, 32), (4096, 1), (1000, 7)])
+@pytest.mark.parametrize("n_sets,ways", [(257, 4), (64, 16), (1, 32), (4096, 1), (1000, 7), (61, 17), (333, 32)])
 def test_tracker_state_matches_the_oracle_access_by_access_order(n_sets, ways):
     stats = _run(gen.CONFIGS["tiny"], n_sets, ways)
     assert stats["hits"] > 0 and stats["tracked"] > 0
