@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(kThreads) k_bwd_pairs(PairArgs a) {
         const PairSide& s = a.side[second ? 1 : 0];
         const int64_t bag = second ? all - bags0 : all;
         int64_t pos0 = second ? L0 : 0;
-        if (a.by_table) {
+        if (ASSIGN && a.by_table) {
             const int tables = a.bags_per_sample_all / a.bags_per_sample;
             const unsigned per_table = (unsigned)(second ? bags1 : bags0) / tables, t = (unsigned)bag / per_table;
             pos0 = second ? a.side[0].offsets[(int64_t)(t + 1) * (bags0 / tables)] : a.side[1].offsets[(int64_t)t * (bags1 / tables)];
