@@ -286,8 +286,8 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
     // what the first lookup of a short bag becomes (ready before the tile knows where it goes: the loads behind it, index and
     // popular-row block, are in flight while the tiles exchange their sums)
     NonId head[ITEMS];
-    // What `n` lookups become, with MARK; the loads of all of them are requested before the first is waited for.  in: there is
-    // one; is_pop: of a popular input (then it is in range and popular).
+    // What `n` lookups become; the loads of all of them are requested before the first is waited for.  in: there is one;
+    // is_pop: of a popular input (then it is in range and popular).
     auto resolve = [&](auto count, const bool* in, const bool* is_pop, const int64_t* base, const int64_t* rows,
                        const int32_t* idx, NonId* id) {
         constexpr int n = decltype(count)::value;
@@ -299,19 +299,27 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
             id[i] = (NonId)-1;
             look[i] = in[i] && (is_pop[i] || (idx[i] >= 0 && idx[i] < rows[i]));
             if (in[i] && !look[i]) set_status(a.status, HL_EBOUNDS);
-            if (look[i]) found[i] = remap.request(base[i] + idx[i]);
-            word[i] = look[i] && !is_pop[i] ? marks.bits[(base[i] + idx[i]) >> 5] : 0;
+            if (look[i] && (MARK || is_pop[i])) found[i] = remap.request(base[i] + idx[i]);
+            word[i] = 0;
+            if constexpr (MARK)
+                if (look[i] && !is_pop[i]) word[i] = marks.bits[(base[i] + idx[i]) >> 5];
         }
 #pragma unroll
         for (int i = 0; i < n; ++i) {
             if (!look[i]) continue;
             const int64_t g = base[i] + idx[i];
-            const int32_t slot = remap.slot(found[i], g);
-            id[i] = slot >= 0 || is_pop[i] ? slot : cold_id(g);
-            if (slot < 0 && !is_pop[i]) mark_cold(marks, g, word[i]);
+            if constexpr (MARK) {
+                const int32_t slot = remap.slot(found[i], g);
+                id[i] = slot >= 0 || is_pop[i] ? slot : cold_id(g);
+                if (slot < 0 && !is_pop[i]) mark_cold(marks, g, word[i]);
+            } else {
+                id[i] = is_pop[i] ? (NonId)remap.slot(found[i], g) : (NonId)g;
+            }
         }
     };
-    // The same without MARK, one lookup after the other: those of X need nothing.
+    // The same without MARK, one lookup after the other: those of X need nothing.  (Of bags of one lookup, the hash probe's are
+    // asked for together all the same: its keys and values come from far away, now and then from twice as far.)
+    constexpr bool kTogether = MARK || std::is_same_v<Probe, HashProbe>;
     auto resolve_each = [&](auto count, const bool* in, const bool* is_pop, const int64_t* base, const int64_t* rows,
                             const int32_t* idx, NonId* id) {
         constexpr int n = decltype(count)::value;
@@ -364,7 +372,7 @@ __global__ void __launch_bounds__(kThreads) k_frag_place(PlaceArgs a, Probe rema
             base[i] = a.table_base[table[i]];
             rows[i] = a.table_base[table[i] + 1] - base[i];
         }
-        if constexpr (MARK) resolve(std::integral_constant<int, ITEMS>(), in, is_pop, base, rows, idx, head);
+        if constexpr (kTogether) resolve(std::integral_constant<int, ITEMS>(), in, is_pop, base, rows, idx, head);
         else resolve_each(std::integral_constant<int, ITEMS>(), in, is_pop, base, rows, idx, head);
     }
     // the dense features follow their inputs: dense_out[i, :] = dense[perm[i], :]
@@ -490,9 +498,10 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
     const bool lists = 4 * b->nnz > 5 * n_bags;
     // Bags per tile: 256 where there are few bags (the tiles are the parallelism) or lists of lookups, 512 from one tile
     // per SM on (with MARK: 106 K bags 9.1 us, with 1 024 10.2, with 256 8.9; 426 K beside a pipeline's other kernels 31, 46, 42).
-    // Without MARK, 1 024 from a tile of those per SM on: of 512 / 1 024, 426 K bags 12.1 / 10.2 us, most of them X's 11.6 / 9.3; 64-bit
-    // path 12.3 / 10.2 and 11.3 / 9.9; 208 K 7.4 / 7.1, 7.3 / 6.9, 6.7 / 8.0, 7.5 / 6.4.
-    const int items = lists || n_bags <= (int64_t)kThreads * sms ? 1 : MARK || n_bags <= (int64_t)4 * kThreads * sms ? 2 : 4;
+    // Without MARK, 1 024 from a tile of those per SM on: of 512 / 1 024, 426 K bags 12.1 / 10.2 us, most of them X's 11.6 / 9.3; 208 K
+    // 7.4 / 7.1 and 7.3 / 6.9.  (64-bit path: 426 K 11.5 to 12.3 / 10.2 to 14.8, by where its tables happen to lie; 512.)
+    constexpr bool kLargeTiles = !MARK && std::is_same_v<Probe, BitmapProbe>;
+    const int items = lists || n_bags <= (int64_t)kThreads * sms ? 1 : kLargeTiles && n_bags > (int64_t)4 * kThreads * sms ? 4 : 2;
     const int n_tiles = (int)div_up(n_bags, kThreads * items);
     // the tally of finished CTAs of the flags kernel: word 0 of the chain words (zero between calls: cleared when the
     // context is created and by the CTA that counts to the end); the chain proper is cleared by the flags kernel
@@ -507,7 +516,7 @@ int32_t fragment_launch(const hl_batch* b, int T, int S, int sms, const int64_t*
     else
         HL_CUDA_TRY(launch(k_frag_flags<false, Probe>, flag_grid, kFlagThreads, stream, b->indices, b->offsets, B, T, S,
                            table_base, probe, words, d_perm, d_counts, finished, chain + 1, n_tiles));
-    constexpr int kMost = MARK ? 2 : 4;
+    constexpr int kMost = kLargeTiles ? 4 : 2;
     const auto place = lists        ? k_frag_place<true, 1, MARK, Probe, NonId>
                        : items == 1 ? k_frag_place<false, 1, MARK, Probe, NonId>
                        : items == 2 ? k_frag_place<false, 2, MARK, Probe, NonId>
