@@ -238,7 +238,8 @@ constexpr int kBulkStageBytes = 12288;
 constexpr int kBulkMaxPolls = 1 << 22;
 constexpr int kBulkStagesPerCta = 200;    // stages of rows per working CTA before another CTA joins in
 // How many rows are on the link at a time decides what the transfer costs everything else on the chip.  The link takes
-// some 300 M requests a second (a request: a row's 128-byte line, or what there is of it) and answers in about 1.5 us, so
+// some 300 M requests a second of a mini-batch's rows (a request: a row's 128-byte line, or what there is of it; rows that lie
+// close to one another, as a popular set's do, up to 580 M a second) and answers in about 1.5 us, so
 // 400 to 500 outstanding requests fill it; any more queue up in front of it, and the memory system behind the queue comes
 // to a near standstill.  Measured beside write-backs of random rows of 64 bytes (256 bytes): 16 CTAs that put up to 32 KB
 // each on the way move 288 M (302 M) requests a second, a streaming read of 256 MB takes 217 us (104) instead of 62, and a

@@ -1181,10 +1181,11 @@ extern "C" int32_t hl_embbag_bwd_prepare(hl_ctx* ctx, const hl_ubatch* ub, const
 namespace hl {
 namespace {
 
-// merge = false: X's keys are offset by the number of slots + 1, so that the sorted list is O's pairs (skipped lookups of
-// O, key n_slots, last among them), then X's (its skipped lookups, key 2 * n_slots + 1, at the very end);
+// merge = false: X's keys are offset by the number of slots + 1, so that the sorted list is O's pairs, then X's;
 // merge = true: one key space, and X's bags are numbered behind O's: the lookups of a row from both micro-batches form one
-// run, over one gradient array [bags of O; bags of X]
+// run, over one gradient array [bags of O; bags of X].
+// Skipped lookups have the key n_slots (of X, merge = false: 2 * n_slots + 1): they are last among O's, or X's, pairs, or, where
+// every table's pairs are sorted by themselves, last among each table's.
 int32_t prepare_both(hl_ctx* ctx, const hl_ubatch* pop, const int32_t* d_n_pop, const hl_ubatch* non,
                      const int32_t* d_n_non, int32_t* d_sorted_slots, int32_t* d_sorted_bags, int32_t* d_n_lookups,
                      bool merge, PairArgs a, bool assign, bool by_table, bool cleared, cudaStream_t stream,

@@ -1,7 +1,8 @@
 """The schedules' sort of every table's pairs by themselves, at the sizes where it changes: pairs of a table for a cluster of 4,
-8 and 16 CTAs, of CTAs with 512 threads, and for the chained passes; tables that hold many more lookups than the others (more
-than their cluster does: sorted through memory, in one, two and three passes), and tables without any.  Whole pipelines with
-both orders of a step, integer data, so that every row must equal the oracle's bit for bit."""
+8 and 16 CTAs, of CTAs with 512 threads, and for the chained passes; tables that hold more lookups than their cluster, in mini-batches of
+as many lookups as bags (sorted through memory, in one to four passes), and others of uneven tables, which the chained passes or one
+cluster sort; tables without any lookup; mini-batches that go one way and the other in turn.  Whole pipelines with both orders of a
+step, integer data, so that every row must equal the oracle's bit for bit."""
 import numpy as np
 import pytest
 import torch
