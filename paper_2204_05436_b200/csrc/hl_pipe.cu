@@ -171,10 +171,12 @@ void build_graphs(hl_pipe* p, int64_t j, const hl_batch* b, const float* d_dense
                                    p->main);
     else
         (void)hl_embbag_fwd(ctx, p->cache, &st.pop, st.counts, st.pooled_pop, p->main);
-    if (p->wb_mode == HL_PIPE_WB_AFTER_FORWARD || read_beside_update(ctx)) launch_flush();
+    const bool apart = p->wb_mode == HL_PIPE_WB_AFTER_FORWARD || read_beside_update(ctx);
+    if (apart) launch_flush();
     if (!merge) update(0);
     launch_flush();
-    if (!merge) update(0);                                   // (by itself: what the first mini-batch launches)
+    // the first mini-batch launches the update by itself, no later one of its slot or of another does
+    if (!merge && !apart && j == 0) update(0);
     launch_flush();
     (void)hl_embbag_fwd(ctx, p->cache, &st.non, st.counts + 1, st.pooled_non, p->main);
     if (!merge) update(1);
